@@ -37,7 +37,10 @@ def nvcc() -> str:
 def _flags(src: str):
     common = ["-O3", "-std=c++17", "-I" + INCLUDE, "-I" + CSRC, "-Xcompiler", "-fPIC"]
     if src.endswith(".cu"):
-        return common + ARCH + ["-lineinfo", "-Xptxas", "-O3"]
+        flags = common + ARCH + ["-lineinfo", "-Xptxas", "-O3"]
+        # the step kernels write every fused multiply-add out: no contraction
+        # by the compiler, so all launch shapes round alike
+        return flags + (["-fmad=false"] if src.startswith("kernels_") else [])
     # host-only C++: keep double-double arithmetic free of contraction
     return common + ["-x", "cu", "-Xcompiler", "-ffp-contract=off"] + ARCH
 

@@ -332,29 +332,14 @@ __device__ __forceinline__ void warp_reduce_add2(double a, double b, double* acc
 
 // New relative deviations of the four shells of a direction from its cubic:
 // out_j = (1 - omega) g_j + R0 + R1 p0_j + R2 p0_j^2 + R3 p0_j^3
-// (delta = w g: the weight w_j drops out of the update).
+// (delta = w g: the weight w_j drops out of the update).  omc = 1 - omega.
 template <typename R, class C>
-__device__ __forceinline__ void relax_shells(const R (&Rm)[4], R omega, int kind, const C& qc,
-                                             R* f) {
-  const R omc = R(1) - omega;
+__device__ __forceinline__ void relax_shells(const R (&Rm)[4], R omc, const C& qc, R* f) {
 #pragma unroll
   for (int j = 0; j < kShells; ++j) {
     const R p = qc.p0[j];
     const R val = fma(fma(fma(Rm[3], p, Rm[2]), p, Rm[1]), p, Rm[0]);
     f[j] = fma(omc, f[j], val);
-  }
-}
-
-// Adds sum_j w_j (out_j - in_j) p0_j and sum_j w_j (out_j - in_j) p0_j^2 of one
-// direction (relative deviations in / out).
-template <typename R, class C>
-__device__ __forceinline__ void balance(const R* in, const R* out, int kind, const C& qc, R& aN,
-                                        R& aE) {
-#pragma unroll
-  for (int j = 0; j < kShells; ++j) {
-    const R dlt = out[j] - in[j];
-    aN = fma(dlt, qc.wp0[kind][j], aN);
-    aE = fma(dlt, qc.wp0sq[kind][j], aE);
   }
 }
 
@@ -400,84 +385,47 @@ __device__ __forceinline__ void gather(const S* __restrict__ fin, const DevSampl
   }
 }
 
-// Per-direction cubic coefficients of a direction pair, on lanes (d, d + 1):
-// the quantities pair_cubics() computes, written on register pairs.  Every
-// polynomial in v is split into even and odd parts, and the odd parts take
-// the constant pairs (a, -a) of QuadConsts::odd, so each instruction serves
-// both directions.  nT, nmT as in pair_cubics; FxT, FyT = (Fx, Fy) nT.
-// Returns R0..R3 (lanes p, n) and om = (omega_p, omega_n).
+// pair_cubics() on register pairs, lanes (d, d + 1): the two lanes differ only
+// in the sign of v, which the constant pairs (vx, -vx), (vy, -vy) carry, so
+// each instruction serves both directions.  Returns R0..R3 and 1 - omega.
 template <bool FORCE, class C>
 __device__ __forceinline__ void pair_cubics_paired(const int d, const EqCoeffs<float>& c,
-                                                   float nT, float nmT, float gt, float gux,
-                                                   float guy, float FxT, float FyT, const C& qc,
-                                                   float2 (&R)[4], float2& om) {
+                                                   const ForceCoeffs<float>& k,
+                                                   const RelaxSite<float>& s, const C& qc,
+                                                   float2 (&R)[4], float2& omc) {
   const int q = d / 2;
   const bool hx = hop_x(d) != 0, hy = hop_y(d) != 0;
-  const float vx = float(hop_x(d)) / 5.f, vy = float(hop_y(d)) / 5.f;
-  const float2* od = qc.odd[q];
-  // omega = gamma (1 -+ v.u) / tau on the two lanes
-  om = S2(gt);
-  if (hx) om = fma2(S2(gux), od[kONVx], om);
-  if (hy) om = fma2(S2(guy), od[kONVy], om);
-  const float2 on = mul2(om, S2(nT));
-  float2 q1 = S2(c.c1_0);
-  if (hx) q1 = fma2(S2(c.c1_x), od[kOVx], q1);
-  if (hy) q1 = fma2(S2(c.c1_y), od[kOVy], q1);
-  float2 q2 = S2(c.c2_0);
-  if (hx) q2 = fma2(S2(c.c2_xx), S2(vx * vx), q2);
-  if (hx && hy) q2 = fma2(S2(c.c2_xy), S2(vx * vy), q2);
-  if (hx) q2 = fma2(S2(c.c2_x), od[kOVx], q2);
-  if (hy) q2 = fma2(S2(c.c2_y), od[kOVy], q2);
-  float2 q3 = S2(c.c3_0);
-  if (hx) q3 = fma2(S2(c.c3_xx), S2(vx * vx), q3);
-  if (hx && hy) q3 = fma2(S2(c.c3_xy), S2(vx * vy), q3);
-  if (hx) q3 = fma2(S2(c.c3_x), od[kOVx], q3);
-  if (hy) q3 = fma2(S2(c.c3_y), od[kOVy], q3);
-  if (hx) q3 = fma2(S2(c.c3_xxx), od[kOVx3], q3);
-  if (hx && hy) q3 = fma2(S2(c.c3_xxy), od[kOVx2y], q3);
-  R[0] = fma2(on, S2(c.q0m1), mul2(om, S2(nmT)));
-  R[1] = mul2(on, q1);
-  R[2] = mul2(on, q2);
-  R[3] = mul2(on, q3);
-  if (FORCE) {
-    // lanes (F.v, -F.v) and (F.t, -F.t) times n/T, t = (-vy, vx)
-    float2 Fv, Ft;
-    if (hx && hy) {
-      Fv = fma2(S2(FxT), od[kOVx], mul2(S2(FyT), od[kOVy]));
-      Ft = fma2(S2(FyT), od[kOVx], mul2(S2(FxT), od[kONVy]));
-    } else if (hx) {
-      Fv = mul2(S2(FxT), od[kOVx]);
-      Ft = mul2(S2(FyT), od[kOVx]);
-    } else {
-      Fv = mul2(S2(FyT), od[kOVy]);
-      Ft = mul2(S2(FxT), od[kONVy]);
-    }
-    // minus the shell derivatives dq_m/dtheta on the two lanes
-    float2 nD1;
-    if (hx && hy) nD1 = fma2(S2(c.c1_x), od[kOVy], mul2(S2(c.c1_y), od[kONVx]));
-    else if (hx) nD1 = mul2(S2(c.c1_y), od[kONVx]);
-    else nD1 = mul2(S2(c.c1_x), od[kOVy]);
-    // even part of -dq2/dtheta: 2 vx vy c2_xx + (vy^2 - vx^2) c2_xy
-    float2 nD2 = mul2(S2(c.c2_xy), S2(vy * vy - vx * vx));
-    if (hx && hy) nD2 = fma2(S2(c.c2_xx), S2(2.f * vx * vy), nD2);
-    if (hy) nD2 = fma2(S2(c.c2_x), od[kOVy], nD2);
-    if (hx) nD2 = fma2(S2(c.c2_y), od[kONVx], nD2);
-    float2 nD3 = mul2(S2(c.c3_xy), S2(vy * vy - vx * vx));
-    if (hx && hy) nD3 = fma2(S2(c.c3_xx), S2(2.f * vx * vy), nD3);
-    if (hy) nD3 = fma2(S2(c.c3_x), od[kOVy], nD3);
-    if (hx) nD3 = fma2(S2(c.c3_y), od[kONVx], nD3);
-    if (hx && hy) nD3 = fma2(S2(c.c3_xxx), od[kO3x2y], nD3);
-    if (hx) nD3 = fma2(S2(c.c3_xxy), od[kOX3m2xy2], nD3);
-    const float q0 = 1.f + c.q0m1;
-    // s_m = (F.v)(q_m - (m + 1) q_{m+1}) - (F.t) dq_{m+1}/dtheta
-    R[0] = fma2(Fv, fma2(q1, S2(-1.f), S2(q0)), R[0]);
-    R[0] = fma2(Ft, nD1, R[0]);
-    R[1] = fma2(Fv, fma2(q2, S2(-2.f), q1), R[1]);
-    R[1] = fma2(Ft, nD2, R[1]);
-    R[2] = fma2(Fv, fma2(q3, S2(-3.f), q2), R[2]);
-    R[2] = fma2(Ft, nD3, R[2]);
-    R[3] = fma2(Fv, q3, R[3]);
+  const float2 vx = qc.vxo[q], vy = qc.vyo[q];
+  float2 z = S2(c.W);
+  omc = S2(s.omgt);
+  if (hx) {
+    z = fma2(S2(c.X), vx, z);
+    omc = fma2(S2(s.gux), vx, omc);
   }
+  if (hy) {
+    z = fma2(S2(c.Y), vy, z);
+    omc = fma2(S2(s.guy), vy, omc);
+  }
+  float2 o = fma2(omc, S2(-1.f), S2(1.f));
+  const float2 e1 = fma2(S2(c.kap), z, S2(c.lam));
+  const float2 e2 = mul2(z, fma2(S2(c.mu), z, S2(c.D)));
+  const float2 z2 = mul2(z, z);
+  const float2 e3 = mul2(mul2(S2(c.nu), z), z2);
+  if (FORCE) {
+    float2 phi;
+    if (hx && hy) phi = fma2(S2(s.Fx), vx, mul2(S2(s.Fy), vy));
+    else if (hx) phi = mul2(S2(s.Fx), vx);
+    else phi = mul2(S2(s.Fy), vy);
+    o = add2(o, phi);
+    R[0] = fma2(o, S2(c.e0), fma2(phi, S2(k.a0), S2(k.b0)));
+    R[1] = fma2(o, e1, fma2(z, fma2(phi, S2(k.a1), S2(k.b1)), fma2(phi, S2(k.a2), S2(k.b2))));
+    R[2] = fma2(o, e2, mul2(z2, fma2(phi, S2(k.a3), S2(k.b3))));
+  } else {
+    R[0] = mul2(o, S2(c.e0));
+    R[1] = mul2(o, e1);
+    R[2] = mul2(o, e2);
+  }
+  R[3] = mul2(o, e3);
 }
 
 // New relative deviations of the four shells of one direction on shell pairs:
@@ -521,23 +469,21 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restri
 #pragma unroll
   for (int d = 0; d < kDirs; ++d) park_store(park + d * park_stride, &f[4 * d]);
   Macro<float> M;
-  const bool conv = landau(m, M);
-  unsigned bad = 0;
-  if (!conv) bad |= kErrNoConvergence;
-  if (!all_finite(M)) bad |= kErrNonFinite;
-  else if (!macro_ok(M)) bad |= kErrUnphysical;
+  const unsigned bad = landau(m, M);
   if (bad) atomicOr(aux.err, bad);
 
-  const EqCoeffs<float> c = eq_coeffs(M);
   const float scl = sizeof(S) == 2 ? qc.enc_s : 1.f;
-  const float inv1T = qdiv(1.f, 1.f + M.dT);
-  const float nT = (1.f + M.dn) * inv1T * scl;
-  const float nmT = (M.dn - M.dT) * inv1T * scl;
-  const float gt = M.gamma * float(s.inv_tau);
-  const float gux = gt * M.ux, guy = gt * M.uy;
-  const float Fx = lca ? float(s.Fx) + (-float(s.inv_cg) * egx) : float(s.Fx);
-  const float Fy = lca ? float(s.Fy) + (-float(s.inv_cg) * egy) : float(s.Fy);
-  const float FxT = Fx * nT, FyT = Fy * nT;
+  const float iTs = M.invT * scl;
+  const EqCoeffs<float> c = eq_coeffs(M, fmaf(M.dn, iTs, iTs), (M.dn - M.dT) * iTs);
+  const float Fx = lca ? fmaf(-float(s.inv_cg), egx, float(s.Fx)) : float(s.Fx);
+  const float Fy = lca ? fmaf(-float(s.inv_cg), egy, float(s.Fy)) : float(s.Fy);
+  RelaxSite<float> rs;
+  rs.gt = M.gamma * float(s.inv_tau);
+  rs.omgt = 1.f - rs.gt;
+  rs.gux = rs.gt * M.ux; rs.guy = rs.gt * M.uy;
+  rs.Fx = Fx; rs.Fy = Fy;
+  ForceCoeffs<float> k{};
+  if (FORCE != 0) k = force_coeffs(c, Fx, Fy, scl);
   const long long site = (long long)y * s.ldx + x;
   if (lca) dn_next[site] = M.dn;
   // conservation projection: sums of the moment changes (N^0, T^00) and
@@ -545,8 +491,8 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restri
   float2 accNE = S2(0.f), accXY = S2(0.f);
   if (kProject && FORCE != 0) {
     // forcing changes T^0a by (F.N_E, F N_E^0), N_E = n gamma (1, u)
-    const float nG = (1.f + M.dn) * M.gamma;
-    accNE = make_float2(0.f, -(nG * (Fx * M.ux + Fy * M.uy)));
+    const float nG = fmaf(M.dn, M.gamma, M.gamma);
+    accNE = make_float2(0.f, -(nG * fmaf(Fx, M.ux, Fy * M.uy)));
     accXY = make_float2(-(nG * Fx), -(nG * Fy));
   }
   // (5,0)-type pairs first: with FP32 storage they take the correction and
@@ -555,11 +501,10 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restri
   for (int pi = 0; pi < kDirs / 2; ++pi) {
     const int d = (2 * pi + 8) % kDirs;
     const int kind = dir_kind(d);
-    float2 R[4], om;
-    pair_cubics_paired<FORCE != 0>(d, c, nT, nmT, gt, gux, guy, FxT, FyT, qc, R, om);
+    float2 R[4], omc;
+    pair_cubics_paired<FORCE != 0>(d, c, k, rs, qc, R, omc);
     park_load(park + d * park_stride, &f[4 * d]);
     park_load(park + (d + 1) * park_stride, &f[4 * d + 4]);
-    const float2 omc = fma2(om, S2(-1.f), S2(1.f));
     float2 bp, bn;
     relax_shells_paired<kProject>(R[0].x, R[1].x, R[2].x, R[3].x, omc.x, kind, qc, &f[4 * d], bp);
     relax_shells_paired<kProject>(R[0].y, R[1].y, R[2].y, R[3].y, omc.y, kind, qc, &f[4 * d + 4],
@@ -579,8 +524,8 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restri
   }
   if (kProject) {
     const float rN = accNE.x, rE = accNE.y;
-    const float l0 = qc.P00 * rN + qc.P01 * rE;
-    const float l1 = qc.P10 * rN + qc.P11 * rE;
+    const float l0 = fmaf(qc.P00, rN, qc.P01 * rE);
+    const float l1 = fmaf(qc.P10, rN, qc.P11 * rE);
     const float lx = qc.px * accXY.x, ly = qc.px * accXY.y;
 #pragma unroll
     for (int d = 8; d < kDirs; ++d) {
@@ -603,8 +548,8 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restri
     const long long k = s.site0 + (long long)y * s.nx + x;
     const double dx = double(M.ux) - double(aux.uprev[2 * k]);
     const double dy = double(M.uy) - double(aux.uprev[2 * k + 1]);
-    r_du2 += dx * dx + dy * dy;
-    r_u2 += double(M.ux) * double(M.ux) + double(M.uy) * double(M.uy);
+    r_du2 = fma(dx, dx, fma(dy, dy, r_du2));
+    r_u2 = fma(double(M.ux), double(M.ux), fma(double(M.uy), double(M.uy), r_u2));
   }
 }
 
@@ -625,122 +570,45 @@ __device__ __forceinline__ void collide_store(typename Codec<S>::R (&f)[kQ], S* 
   if constexpr (std::is_same<R, float>::value) {
     collide_store_paired<S, FORCE, RES, BT>(f, fout, s, x, y, aux, qc, r_du2, r_u2, park, dn_prev,
                                         dn_next);
-    return;
-  }
-  // FP32 storage: the FP32 quadrature constants satisfy Eq. orthonormal only
-  // to ~1e-7, which would break the exact conservation of N^0 and T^0a by the
-  // collision at that level every step (a secular drift).  The update is
-  // projected back onto the exact discrete balance
-  //   sum_i p0 (f* - f) = 0,  sum_i p0 p^a (f* - f) = (F.N_E, F N_E^0)
-  // by a correction on the (5,0)-type directions (solved with the constants P**, px).
-  constexpr bool kProject = sizeof(S) == sizeof(float);
-  {
-    // electric force (local capacitance approximation): the neighbours'
-    // density of the previous step, loaded before the long arithmetic
+  } else {
+    // FP64 storage: the populations stay in registers (the FP64 pipe, not
+    // latency, bounds this path), no conservation projection
     const bool lca = FORCE == kForceLca && s.inv_cg != 0.0;
     R egx = R(0), egy = R(0);
     if (lca) lca_gradient(s, dn_prev, x, y, egx, egy);
     const Moments<R> m = moments(f, qc);
-    // park: entry of direction d at park + d * BT * 16 (BT threads per block)
-    constexpr uint32_t park_stride = BT * 16u;
-    if constexpr (Park<R>::kOn) {
-#pragma unroll
-      for (int d = 0; d < kDirs; ++d) park_store(park + d * park_stride, &f[4 * d]);
-    }
     Macro<R> M;
-    const bool conv = landau(m, M);
-    unsigned bad = 0;
-    if (!conv) bad |= kErrNoConvergence;
-    if (!all_finite(M)) bad |= kErrNonFinite;
-    else if (!macro_ok(M)) bad |= kErrUnphysical;
+    const unsigned bad = landau(m, M);
     if (bad) atomicOr(aux.err, bad);
-
-    const EqCoeffs<R> c = eq_coeffs(M);
-    // every term of the update is proportional to n/T or (n - T)/T: the
-    // 16-bit kernels, which work on the stored s g, scale those by s
-    const R scl = sizeof(S) == 2 ? qc.enc_s : R(1);
-    const R inv1T = qdiv(R(1), R(1) + M.dT);
-    const R nT = (R(1) + M.dn) * inv1T * scl;
-    const R nmT = (M.dn - M.dT) * inv1T * scl;
-    const R gt = M.gamma * R(s.inv_tau);
-    const R gux = gt * M.ux, guy = gt * M.uy;
-    const R Fx = lca ? R(s.Fx) + (-R(s.inv_cg) * egx) : R(s.Fx);
-    const R Fy = lca ? R(s.Fy) + (-R(s.inv_cg) * egy) : R(s.Fy);
+    const EqCoeffs<R> c = eq_coeffs(M, fma(M.dn, M.invT, M.invT), (M.dn - M.dT) * M.invT);
+    RelaxSite<R> rs;
+    rs.gt = M.gamma * R(s.inv_tau);
+    rs.omgt = R(1) - rs.gt;
+    rs.gux = rs.gt * M.ux; rs.guy = rs.gt * M.uy;
+    rs.Fx = lca ? fma(-R(s.inv_cg), egx, R(s.Fx)) : R(s.Fx);
+    rs.Fy = lca ? fma(-R(s.inv_cg), egy, R(s.Fy)) : R(s.Fy);
+    ForceCoeffs<R> k{};
+    if (FORCE != 0) k = force_coeffs(c, rs.Fx, rs.Fy, R(1));
     const long long site = (long long)y * s.ldx + x;
     if (lca) dn_next[site] = M.dn;
-    R rN = R(0), rE = R(0), rX = R(0), rY = R(0);
-    // (5,0)-type pairs first: in reduced precision they take the correction
-    // and are stored last; the (3,4)-type pairs are stored as soon as done.
 #pragma unroll
-    for (int pi = 0; pi < kDirs / 2; ++pi) {
-      const int d = (2 * pi + 8) % kDirs;
-      R Rp[4], Rn[4], omp, omn;
-      pair_cubics<R, FORCE != 0>(d, c, nT, nmT, gt, gux, guy, Fx, Fy, Rp, Rn, omp, omn);
-      const int kind = dir_kind(d);
-      if constexpr (Park<R>::kOn) {
-        park_load(park + d * park_stride, &f[4 * d]);
-        park_load(park + (d + 1) * park_stride, &f[4 * d + 4]);
-      }
-      if (kProject) {
-        R in[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) in[j] = f[4 * d + j];
-        relax_shells(Rp, omp, kind, qc, &f[4 * d]);
-        relax_shells(Rn, omn, kind, qc, &f[4 * d + 4]);
-        R aNp = R(0), aEp = R(0), aNn = R(0), aEn = R(0);
-        balance(in, &f[4 * d], kind, qc, aNp, aEp);
-        balance(in + 4, &f[4 * d + 4], kind, qc, aNn, aEn);
-        rN += aNp + aNn;
-        rE += aEp + aEn;
-        const R vx = R(hop_x(d)) / R(5), vy = R(hop_y(d)) / R(5);
-        if (hop_x(d) != 0) rX = fma(aEp - aEn, vx, rX);
-        if (hop_y(d) != 0) rY = fma(aEp - aEn, vy, rY);
-        if (kind == 0) {
-          Codec<S>::store4(fout + vec_index(s, d, site), kind, qc, &f[4 * d]);
-          Codec<S>::store4(fout + vec_index(s, d + 1, site), kind, qc, &f[4 * d + 4]);
-        } else if constexpr (Park<R>::kOn) {
-          // (5,0)-type: wait for the correction in the parking area, not in registers
-          park_store(park + d * park_stride, &f[4 * d]);
-          park_store(park + (d + 1) * park_stride, &f[4 * d + 4]);
-        }
-      } else {
-        relax_shells(Rp, omp, kind, qc, &f[4 * d]);
-        relax_shells(Rn, omn, kind, qc, &f[4 * d + 4]);
-        Codec<S>::store4(fout + vec_index(s, d, site), kind, qc, &f[4 * d]);
-        Codec<S>::store4(fout + vec_index(s, d + 1, site), kind, qc, &f[4 * d + 4]);
-      }
-    }
-    if (kProject) {
-      if (FORCE != 0) {
-        // forcing changes T^0a by (F.N_E, F N_E^0), N_E = n gamma (1, u)
-        const R nG = (R(1) + M.dn) * M.gamma;
-        rE -= nG * (Fx * M.ux + Fy * M.uy);
-        rX -= nG * Fx;
-        rY -= nG * Fy;
-      }
-      const R l0 = qc.P00 * rN + qc.P01 * rE;
-      const R l1 = qc.P10 * rN + qc.P11 * rE;
-      const R lx = qc.px * rX, ly = qc.px * rY;
-#pragma unroll
-      for (int d = 8; d < kDirs; ++d) {
-        const R cd = l1 + (hop_x(d) > 0 ? lx : hop_x(d) < 0 ? -lx : hop_y(d) > 0 ? ly : -ly);
-        if constexpr (Park<R>::kOn) park_load(park + d * park_stride, &f[4 * d]);
-#pragma unroll
-        for (int j = 0; j < kShells; ++j)
-          f[4 * d + j] = f[4 * d + j] + fma(qc.p0[j], cd, l0);   // delta += w (l0 + p0 cd)
-        Codec<S>::store4(fout + vec_index(s, d, site), 1, qc, &f[4 * d]);
-      }
+    for (int d = 0; d < kDirs; d += 2) {
+      R Rp[4], Rn[4], omcp, omcn;
+      pair_cubics<R, FORCE != 0>(d, c, k, rs, Rp, Rn, omcp, omcn);
+      relax_shells(Rp, omcp, qc, &f[4 * d]);
+      relax_shells(Rn, omcn, qc, &f[4 * d + 4]);
+      Codec<S>::store4(fout + vec_index(s, d, site), dir_kind(d), qc, &f[4 * d]);
+      Codec<S>::store4(fout + vec_index(s, d + 1, site), dir_kind(d), qc, &f[4 * d + 4]);
     }
     if (RES == 1) {
-      const long long k = s.site0 + (long long)y * s.nx + x;
-      aux.uprev[2 * k] = M.ux;
-      aux.uprev[2 * k + 1] = M.uy;
+      const long long j = s.site0 + (long long)y * s.nx + x;
+      aux.uprev[2 * j] = M.ux;
+      aux.uprev[2 * j + 1] = M.uy;
     } else if (RES == 2) {
-      const long long k = s.site0 + (long long)y * s.nx + x;
-      const double dx = double(M.ux) - double(aux.uprev[2 * k]);
-      const double dy = double(M.uy) - double(aux.uprev[2 * k + 1]);
-      r_du2 += dx * dx + dy * dy;
-      r_u2 += double(M.ux) * double(M.ux) + double(M.uy) * double(M.uy);
+      const long long j = s.site0 + (long long)y * s.nx + x;
+      const double dx = M.ux - aux.uprev[2 * j], dy = M.uy - aux.uprev[2 * j + 1];
+      r_du2 = fma(dx, dx, fma(dy, dy, r_du2));
+      r_u2 = fma(M.ux, M.ux, fma(M.uy, M.uy, r_u2));
     }
   }
 }
@@ -959,9 +827,7 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ fin, const De
   pull<S, false>(fin, s, x, y, ghost, qc, f);
   const Moments<R> m = moments(f, qc);
   Macro<R> M;
-  const bool conv = landau(m, M);
-  unsigned bad = conv ? 0u : kErrNoConvergence;
-  if (!all_finite(M)) bad |= kErrNonFinite;
+  const unsigned bad = landau(m, M) & ~kErrUnphysical;
   if (bad) atomicOr(err, bad);
   const long long k = (long long)y * s.nx + x;
   if (n) n[k] = 1.0 + double(M.dn);
@@ -977,39 +843,51 @@ __device__ __forceinline__ Macro<R> field_macro(const double* n, const double* u
                                                 const double* uy, const double* T, long long k,
                                                 bool& ok) {
   Macro<R> M;
-  const double vx = ux[k], vy = uy[k];
-  const double u2 = vx * vx + vy * vy;
-  const double sq = sqrt(1.0 - u2);
+  const double vx = ux[k], vy = uy[k], nk = n[k], Tk = T[k];
+  const double u2 = fma(vx, vx, vy * vy), w = 1.0 - u2;
+  const double g = qrsqrt(w);
   M.ux = R(vx);
   M.uy = R(vy);
-  M.gamma = R(1.0 / sq);
-  M.gm1 = R(u2 / (sq * (1.0 + sq)));
-  M.dn = R(n[k] - 1.0);
-  M.dT = R(T[k] - 1.0);
+  M.gamma = R(g);
+  M.gm1 = R(u2 * g * (g * qrcp(1.0 + g)));
+  M.dn = R(nk - 1.0);
+  M.dT = R(Tk - 1.0);
   M.deps = R(0);
-  ok = (u2 < 1.0) && (n[k] > 0.0) && (T[k] > 0.0) && isfinite(n[k]) && isfinite(T[k]);
+  M.invT = qrcp(R(Tk));
+  ok = (u2 < 1.0) && (nk > 0.0) && (Tk > 0.0) && finite_bits(nk) && finite_bits(Tk);
   return M;
 }
 
-// Relative deviations (f^eq - w) / w of the two directions d (even), d + 1
-// for the macroscopic state M (times s in 16-bit storage): vp, vn.
+// Equilibrium coefficients of the macroscopic state M as stored (16-bit
+// storage holds s g).
 template <typename S, class C>
-__device__ __forceinline__ void eq_pair(const Macro<typename Codec<S>::R>& M,
-                                        const EqCoeffs<typename Codec<S>::R>& c, int d,
+__device__ __forceinline__ EqCoeffs<typename Codec<S>::R> stored_eq(
+    const Macro<typename Codec<S>::R>& M, const C& qc) {
+  using R = typename Codec<S>::R;
+  const R iTs = sizeof(S) == 2 ? R(M.invT * qc.enc_s) : M.invT;
+  return eq_coeffs(M, fma(M.dn, iTs, iTs), (M.dn - M.dT) * iTs);
+}
+
+// Relative deviations (f^eq - w) / w of the two directions d (even), d + 1
+// from stored_eq(): vp, vn.
+template <typename S, class C>
+__device__ __forceinline__ void eq_pair(const EqCoeffs<typename Codec<S>::R>& c, int d,
                                         const C& qc, typename Codec<S>::R* vp,
                                         typename Codec<S>::R* vn) {
   using R = typename Codec<S>::R;
-  const R scl = sizeof(S) == 2 ? qc.enc_s : R(1);     // 16-bit storage holds s g
-  const R inv1T = R(1) / (R(1) + M.dT);
-  const R nT = (R(1) + M.dn) * inv1T * scl;
-  const R nmT = (M.dn - M.dT) * inv1T * scl;
-  R Rp[4], Rn[4], omp, omn;
-  // omega = 1 and no force: out = w (f^eq - w) / w
-  pair_cubics<R, false>(d, c, nT, nmT, R(1), R(0), R(0), R(0), R(0), Rp, Rn, omp, omn);
+  const R vx = R(hop_x(d)) / R(5), vy = R(hop_y(d)) / R(5);
+  const R zo = fma(c.X, vx, c.Y * vy);
 #pragma unroll
-  for (int j = 0; j < kShells; ++j) vp[j] = vn[j] = R(0);
-  relax_shells(Rp, R(1), dir_kind(d), qc, vp);
-  relax_shells(Rn, R(1), dir_kind(d), qc, vn);
+  for (int h = 0; h < 2; ++h) {
+    const R z = h ? c.W - zo : c.W + zo;
+    const R e1 = fma(c.kap, z, c.lam), e2 = z * fma(c.mu, z, c.D), e3 = (c.nu * z) * (z * z);
+    R* v = h ? vn : vp;
+#pragma unroll
+    for (int j = 0; j < kShells; ++j) {
+      const R p = qc.p0[j];
+      v[j] = fma(fma(fma(e3, p, e2), p, e1), p, c.e0);
+    }
+  }
 }
 
 // Stored state := f^eq(n, u, T) - w (dense FP64 inputs).
@@ -1025,14 +903,14 @@ __device__ __forceinline__ void init_body(S* __restrict__ fout, const DevSample&
   bool ok;
   const Macro<R> M = field_macro<R>(n, ux, uy, T, k, ok);
   if (!ok) atomicOr(err, kErrUnphysical);
-  const EqCoeffs<R> c = eq_coeffs(M);
+  const EqCoeffs<R> c = stored_eq<S>(M, qc);
   const long long site = (long long)y * s.ldx + x;
   void* const dn0 = s.cur ? s.dn[1] : s.dn[0];
   if (dn0) static_cast<R*>(dn0)[site] = M.dn;     // the electric force's first step
 #pragma unroll
   for (int d = 0; d < kDirs; d += 2) {
     R v[8];
-    eq_pair<S>(M, c, d, qc, v, v + 4);
+    eq_pair<S>(c, d, qc, v, v + 4);
     Codec<S>::store4(fout + vec_index(s, d, site), dir_kind(d), qc, v);
     Codec<S>::store4(fout + vec_index(s, d + 1, site), dir_kind(d), qc, v + 4);
   }
@@ -1063,14 +941,14 @@ __device__ __forceinline__ void init_ce_body(S* __restrict__ fout, const DevSamp
   bool ok;
   const Macro<R> M = field_macro<R>(n, ux, uy, T, k, ok);
   if (!ok) atomicOr(err, kErrUnphysical);
-  const EqCoeffs<R> c = eq_coeffs(M);
+  const EqCoeffs<R> c = stored_eq<S>(M, qc);
   const long long site = (long long)y * s.ldx + x;
   void* const dn0 = s.cur ? s.dn[1] : s.dn[0];
   if (dn0) static_cast<R*>(dn0)[site] = M.dn;     // the electric force's first step
 #pragma unroll 1
   for (int d = 0; d < kDirs; d += 2) {
     R v[8];
-    eq_pair<S>(M, c, d, qc, v, v + 4);
+    eq_pair<S>(c, d, qc, v, v + 4);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int dd = d + h;
@@ -1081,7 +959,7 @@ __device__ __forceinline__ void init_ce_body(S* __restrict__ fout, const DevSamp
         bool okd;
         const Macro<R> Md = field_macro<R>(n, ux, uy, T, (long long)ty * s.nx + tx, okd);
         R ed[8];
-        eq_pair<S>(Md, eq_coeffs(Md), d, qc, ed, ed + 4);
+        eq_pair<S>(stored_eq<S>(Md, qc), d, qc, ed, ed + 4);
         const R vx = R(hop_x(dd)) / R(5), vy = R(hop_y(dd)) / R(5);
         const R om = Md.gamma * (R(1) - (vx * Md.ux + vy * Md.uy)) * R(s.inv_tau);
         const R iom = R(1) / om;

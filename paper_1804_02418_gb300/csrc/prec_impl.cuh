@@ -147,8 +147,8 @@ cudaError_t upload(const double p0[4], const double w[2][4], double scale) {
   for (int q = 0; q < kDirs / 2; ++q) {
     const int d = 2 * q;
     const double vx = hop_x(d) / 5.0, vy = hop_y(d) / 5.0;
-    for (int o = 0; o < kOddMonos; ++o)
-      h.odd[q][o] = make_float2(float(odd_mono(d, o)), float(-odd_mono(d, o)));
+    h.vxo[q] = make_float2(float(vx), float(-vx));
+    h.vyo[q] = make_float2(float(vy), float(-vy));
     h.vxy[q] = make_float2(float(vx), float(vy));
     h.vsq[q] = make_float2(float(vx * vx), float(vx * vy));
   }

@@ -10,11 +10,26 @@
 // n - 1, T - 1, gamma - 1 and T gamma - 1, so FP32 arithmetic keeps full
 // relative precision on the O(u) flux-carrying parts.
 //
-// The equilibrium Q(p) = sum_k a^(k) J^(k)(p) (App. A polynomials, App. B
-// projections) is regrouped on the massless shell p = p0 (1, v) as
-//     Q(p0 v) = sum_{m=0..3} p0^m q_m(v),
-// with q_m(v) a polynomial of degree <= m in the unit velocity v.  Every
-// population of one direction then costs a cubic in its shell energy p0_j.
+// The equilibrium.  Q(p) = sum_k a^(k) J^(k)(p) (App. A polynomials, App. B
+// projections) is, on the massless shell p = p0 (1, v) and with
+//     W = T gamma - 1,  (X, Y) = T gamma u,  z(v) = W + X vx + Y vy,
+// a cubic in the shell energy whose coefficients are polynomials in z alone:
+//     Q - 1 = q0 + p0 (kappa z + lambda) + p0^2 z (mu z + D) + p0^3 z^3 / 6,
+//     D = W^2 - X^2 - Y^2,               q0 = W^2 + r^2/2 - W (1 + W^2 + 3 r^2/2),
+//     kappa = 1 - 3 W + 6 W^2 + 3 r^2/2, lambda = D (1 - 3 W),
+//     mu = 1/2 - 5 W / 2,                r^2 = X^2 + Y^2
+// (App. A-B multiplied out with vx^2 + vy^2 = 1 and the mass shell
+// (1 + W)^2 = T^2 + r^2).  W, X, Y and everything built from them vanish at
+// rest, so the small quantities keep their relative precision.  One scalar z
+// per direction replaces the 15 polynomial coefficients of q_m(v): the
+// per-site set-up is about 25 operations and a direction's cubic about 8.
+// Measured against the expansion in monomials of v (15 coefficients, about
+// 110 operations to form, 46 paired instructions per direction pair with a
+// force instead of 24; Landau solve in FP64 throughout), whole passes of
+// init + steps + fields: FP64 1024 x 512 with force 10.82 -> 7.49 ms (10
+// steps; bound by the FP64 pipe), FP64 64 x 64 3.11 -> 2.48 ms (100 steps),
+// FP16 storage 4096 x 2048 7.81 -> 6.94 ms (20 steps; bound by the FMA pipe),
+// FP32 1024 x 512 1.91 -> 1.81 ms (50 steps).
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
@@ -42,22 +57,6 @@ __host__ __device__ constexpr int hop_y(int d) {
 }
 __host__ __device__ constexpr int dir_kind(int d) { return d < 8 ? 0 : 1; }
 
-// Odd monomials of a unit velocity v whose (a, -a) pairs the paired FP32
-// collision uses (order of QuadConsts::odd).
-enum OddMono {
-  kOVx = 0, kOVy, kONVx, kONVy,   // vx, vy, -vx, -vy
-  kOVx3, kOVx2y,                  // vx^3, vx^2 vy
-  kO3x2y, kOX3m2xy2,              // 3 vx^2 vy, -(vx^3 - 2 vx vy^2)
-  kOddMonos
-};
-
-__host__ __device__ constexpr double odd_mono(int d, int o) {
-  const double vx = hop_x(d) / 5.0, vy = hop_y(d) / 5.0;
-  return o == kOVx ? vx : o == kOVy ? vy : o == kONVx ? -vx : o == kONVy ? -vy
-       : o == kOVx3 ? vx * vx * vx : o == kOVx2y ? vx * vx * vy
-       : o == kO3x2y ? 3.0 * vx * vx * vy : -(vx * vx * vx - 2.0 * vx * vy * vy);
-}
-
 // Quadrature constants (refined Sec. 2.3 values), uploaded once per module.
 template <typename R>
 struct QuadConsts {
@@ -75,8 +74,7 @@ struct QuadConsts {
   // lanes are (direction d, its opposite d + 1) in the collision and (shell
   // j, shell j + 1) in the relaxation; a constant pair read from here costs
   // nothing as an operand, a literal pair of two different values would.
-  // odd[q][o]: (a, -a) for the odd monomial o of direction pair q = d / 2.
-  float2 odd[kDirs / 2][kOddMonos];
+  float2 vxo[kDirs / 2], vyo[kDirs / 2];   // (vx, -vx), (vy, -vy) of direction pair q = d / 2
   float2 vxy[kDirs / 2];      // (vx, vy) of direction 2q
   float2 vsq[kDirs / 2];      // (vx^2, vx vy) of direction 2q
   float2 wab[2][kShells];     // (w p0_j / s, w p0_j^2 / s) by direction kind
@@ -238,19 +236,68 @@ struct Macro {
   R gamma, gm1;   // gamma and gamma - 1
   R dn, dT;       // n - 1, T - 1
   R deps;         // eps - 2
+  R invT;         // 1 / T
 };
 
-// Quotient and square root: correctly rounded in FP64; in FP32 the fast
-// hardware approximations (a few ulp), whose error is far below the FP32
-// storage rounding the arithmetic feeds.
-__device__ __forceinline__ double qdiv(double a, double b) { return a / b; }
-__device__ __forceinline__ float qdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double qsqrt(double a) { return sqrt(a); }
-__device__ __forceinline__ float qsqrt(float a) { return a * rsqrtf(a); }
+// Reciprocal and reciprocal square root of a positive number.  FP32: the
+// hardware approximations (1 - 2 ulp, far below the FP32 storage rounding the
+// arithmetic feeds).  FP64: the hardware's approximation (relative error
+// below 2^-18) refined by one step of third order from the residual
+// e = 1 - a r (Householder's method; e^3 < 2^-54), 3 and 5 FP64 operations:
+// the FP64 pipe retires 1/70 of the FP32 rate and bounds the FP64 step.
+__device__ __forceinline__ float qrcp(float a) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+  return r;
+}
+__device__ __forceinline__ double qrcp(double a) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  double e = fma(-a, r, 1.0);
+  e = fma(e, e, e);
+  return fma(r, e, r);
+}
+__device__ __forceinline__ float qrsqrt(float a) { return rsqrtf(a); }
+__device__ __forceinline__ double qrsqrt(double a) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fma(-(a * y), y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
 
-template <typename R> struct Tol;
-template <> struct Tol<double> { static constexpr double v = 1e-15; };
-template <> struct Tol<float> { static constexpr float v = 2e-7f; };
+// double <-> float by moving bits (integer operations, off the FP64 pipe, on
+// which conversions run too): toward zero, values below the normal FP32 range
+// become 0, values above it (and NaN) infinity.
+__device__ __forceinline__ float trunc_f32(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned mag = hi & 0x7fffffffu;
+  unsigned m = ((mag - (896u << 20)) << 3) | (lo >> 29);
+  if (mag < (897u << 20)) m = 0u;
+  if (mag >= (1151u << 20)) m = 0x7f800000u;
+  return __uint_as_float((hi & 0x80000000u) | m);
+}
+// exact for normal numbers and zero; infinity and NaN become NaN
+__device__ __forceinline__ double widen_f64(float f) {
+  const unsigned b = __float_as_uint(f), mag = b & 0x7fffffffu;
+  unsigned hi = (mag >> 3) + (896u << 20), lo = b << 29;
+  if (mag < 0x00800000u) hi = lo = 0u;
+  if (mag >= 0x7f800000u) hi = 0x7ff80000u;
+  return __hiloint2double((int)((b & 0x80000000u) | hi), (int)lo);
+}
+
+__device__ __forceinline__ bool finite_bits(float a) {
+  return (__float_as_uint(a) & 0x7f800000u) != 0x7f800000u;
+}
+__device__ __forceinline__ bool finite_bits(double a) {
+  return ((unsigned)__double2hiint(a) & 0x7ff00000u) != 0x7ff00000u;
+}
+// a > 0 (false for NaN) without a compare on the FP64 pipe; for numbers at
+// least 2^-1022
+__device__ __forceinline__ bool positive(float a) { return a > 0.f; }
+__device__ __forceinline__ bool positive(double a) {
+  const int hi = __double2hiint(a);
+  return hi > 0 && hi <= 0x7ff00000;
+}
 
 // Moment deviations from 48 streamed deviations.
 template <typename R>
@@ -357,182 +404,216 @@ __device__ __forceinline__ Moments<R> moments(const R (&f)[kQ], const C& qc) {
 // Landau frame eps U^a = T^ab U_b:  u = (Pi + eps I)^-1 M, eps = E - M.u,
 // Newton on g(eps) = eps - E + M.u(eps), g' = 1 - u.u, from eps0 = E.
 // Then n = U_a N^a and the massless EOS eps = 2 n T.
-template <typename R>
-__device__ __forceinline__ bool landau(const Moments<R>& m, Macro<R>& o) {
-  R deps = m.dE;
-  R ux = R(0), uy = R(0);
-  bool conv = false;
+//
+// The unknown of the FP32 iteration is d = eps - E = -M.u, which keeps its
+// relative precision.  FP64 starts from the FP32 solution (its error is about
+// 1e-7 u^2) and takes Newton steps until one is below 1e-8 (2 + |deps|): the
+// next would be its square times u^2 / (3 (1 - u^2)), below the FP64
+// rounding, so one FP64 step is the rule.  The slope 1 - u.u only scales the
+// step, and FP32 is enough for it.  After the last step u follows by its
+// derivative, du = (Pi + eps I)^-1 u step.
+__device__ __forceinline__ bool landau_d32(float dE, float Mx, float My, float dPxx, float dPxy,
+                                           float dPyy, float& d, float& ux, float& uy) {
+  const float a0 = 3.f + dPxx, c0 = 3.f + dPyy, p2 = dPxy * dPxy;
+  d = 0.f;
 #pragma unroll 1
   for (int it = 0; it < 12; ++it) {
-    const R a = R(3) + m.dPxx + deps, c = R(3) + m.dPyy + deps;
-    const R inv = qdiv(R(1), a * c - m.dPxy * m.dPxy);
-    ux = (c * m.Mx - m.dPxy * m.My) * inv;
-    uy = (a * m.My - m.dPxy * m.Mx) * inv;
-    const R g = deps - m.dE + m.Mx * ux + m.My * uy;
-    const R step = qdiv(g, R(1) - ux * ux - uy * uy);
-    deps -= step;
-    if (fabs(step) <= Tol<R>::v * (R(2) + fabs(deps))) { conv = true; break; }
+    const float deps = dE + d;
+    const float a = a0 + deps, c = c0 + deps;
+    const float inv = qrcp(fmaf(a, c, -p2));
+    ux = fmaf(c, Mx, -(dPxy * My)) * inv;
+    uy = fmaf(a, My, -(dPxy * Mx)) * inv;
+    const float g = fmaf(Mx, ux, fmaf(My, uy, d));
+    const float step = g * qrcp(fmaf(-ux, ux, fmaf(-uy, uy, 1.f)));
+    d -= step;
+    if (fabsf(step) <= 2e-7f * (2.f + fabsf(deps))) {
+      const float si = step * inv;
+      const float vx = fmaf(c, ux, -(dPxy * uy)), vy = fmaf(a, uy, -(dPxy * ux));
+      ux = fmaf(si, vx, ux);
+      uy = fmaf(si, vy, uy);
+      return true;
+    }
   }
-  {
-    const R a = R(3) + m.dPxx + deps, c = R(3) + m.dPyy + deps;
-    const R inv = qdiv(R(1), a * c - m.dPxy * m.dPxy);
-    ux = (c * m.Mx - m.dPxy * m.My) * inv;
-    uy = (a * m.My - m.dPxy * m.Mx) * inv;
-  }
-  const R u2 = ux * ux + uy * uy;
-  const R s = qsqrt(R(1) - u2);
-  const R gamma = qdiv(R(1), s);
-  const R gm1 = qdiv(u2 * gamma, R(1) + s);
-  const R dNpar = m.dN0 - ux * m.dNx - uy * m.dNy;     // U_a N^a / gamma - 1
-  const R dn = gm1 * (R(1) + dNpar) + dNpar;           // n - 1
-  const R dT = qdiv(deps - R(2) * dn, R(2) * (R(1) + dn));  // T - 1 = eps/(2n) - 1
-  o.ux = ux; o.uy = uy; o.gamma = gamma; o.gm1 = gm1; o.dn = dn; o.dT = dT; o.deps = deps;
+  return false;
+}
+
+__device__ __forceinline__ bool landau_frame(const Moments<float>& m, float& deps, float& ux,
+                                             float& uy) {
+  float d;
+  const bool conv = landau_d32(m.dE, m.Mx, m.My, m.dPxx, m.dPxy, m.dPyy, d, ux, uy);
+  deps = m.dE + d;
   return conv;
 }
 
-// Coefficients of Q(p0 v) - 1 = q0m1 + sum_{m=1..3} p0^m q_m(v) with
-//   q1 = c1_0 + c1_x vx + c1_y vy
-//   q2 = c2_0 + c2_x vx + c2_y vy + c2_xx vx^2 + c2_xy vx vy
-//   q3 = c3_0 + c3_x vx + c3_y vy + c3_xx vx^2 + c3_xy vx vy + c3_xxx vx^3 + c3_xxy vx^2 vy
-// obtained by substituting p = p0 (1, v) in the App. A polynomials and
-// weighting them with the App. B projections.
+__device__ __forceinline__ bool landau_frame(const Moments<double>& m, double& deps, double& ux,
+                                             double& uy) {
+  float d32, ux32, uy32;
+  landau_d32(trunc_f32(m.dE), trunc_f32(m.Mx), trunc_f32(m.My), trunc_f32(m.dPxx),
+             trunc_f32(m.dPxy), trunc_f32(m.dPyy), d32, ux32, uy32);
+  // no use of an FP32 iteration that left the numbers: then from eps = E
+  double d = finite_bits(d32) ? widen_f64(d32) : 0.0;
+  const double a0 = 3.0 + m.dPxx + m.dE, c0 = 3.0 + m.dPyy + m.dE, p2 = m.dPxy * m.dPxy;
+  bool conv = false;
+#pragma unroll 1
+  for (int it = 0; it < 12; ++it) {
+    const double a = a0 + d, c = c0 + d;
+    const double inv = qrcp(fma(a, c, -p2));
+    ux = fma(c, m.Mx, -(m.dPxy * m.My)) * inv;
+    uy = fma(a, m.My, -(m.dPxy * m.Mx)) * inv;
+    const double g = fma(m.Mx, ux, fma(m.My, uy, d));
+    const float w = trunc_f32(fma(-ux, ux, fma(-uy, uy, 1.0)));
+    const double step = g * widen_f64(qrcp(w));
+    d -= step;
+    if (fabsf(trunc_f32(step)) <= 1e-8f * (2.f + fabsf(trunc_f32(m.dE) + trunc_f32(d)))) {
+      const double si = step * inv;
+      const double vx = fma(c, ux, -(m.dPxy * uy)), vy = fma(a, uy, -(m.dPxy * ux));
+      ux = fma(si, vx, ux);
+      uy = fma(si, vy, uy);
+      conv = true;
+      break;
+    }
+  }
+  deps = m.dE + d;
+  return conv;
+}
+
+// Error bits of a site's fields; kErrUnphysical only where they are finite.
+template <typename R>
+__device__ __forceinline__ unsigned landau(const Moments<R>& m, Macro<R>& o) {
+  R deps, ux, uy;
+  const bool conv = landau_frame(m, deps, ux, uy);
+  const R u2 = fma(ux, ux, uy * uy);
+  const R w = R(1) - u2;
+  const R gamma = qrsqrt(w);
+  const R gm1 = u2 * gamma * (gamma * qrcp(R(1) + gamma));   // (gamma^2 - 1) / (gamma + 1)
+  const R dNpar = fma(-uy, m.dNy, fma(-ux, m.dNx, m.dN0));   // U_a N^a / gamma - 1
+  const R dn = fma(gm1, R(1) + dNpar, dNpar);                // n - 1
+  const R n = R(1) + dn, eps = R(2) + deps;
+  const R r = qrcp(n * eps);                                 // 1 / (n eps): both quotients below
+  const R dT = fma(R(-2), dn, deps) * (R(0.5) * (eps * r));  // T - 1 = (eps - 2 n) / (2 n)
+  o.ux = ux; o.uy = uy; o.gamma = gamma; o.gm1 = gm1; o.dn = dn; o.dT = dT; o.deps = deps;
+  o.invT = (n + n) * (n * r);                                // 1 / T = 2 n / eps
+  unsigned bits = conv ? 0u : kErrNoConvergence;
+  if (!(finite_bits(ux) && finite_bits(uy) && finite_bits(dn) && finite_bits(dT)))
+    bits |= kErrNonFinite;
+  else if (!(positive(w) && positive(n) && positive(eps)))
+    bits |= kErrUnphysical;
+  return bits;
+}
+
+// Site coefficients of (f^eq - w) / w = e0 + p0 e1 + p0^2 e2 + p0^3 e3,
+//   e1 = kap z + lam, e2 = z (mu z + D), e3 = nu z^3   (header comment),
+// all times n / T; nT = n / T and nmT = (n - T) / T carry the storage scale.
 template <typename R>
 struct EqCoeffs {
-  R q0m1;
-  R c1_0, c1_x, c1_y;
-  R c2_0, c2_x, c2_y, c2_xx, c2_xy;
-  R c3_0, c3_x, c3_y, c3_xx, c3_xy, c3_xxx, c3_xxy;
+  R W, X, Y;
+  R e0, kap, lam, mu, D, nu;
 };
 
 template <typename R>
-__device__ __forceinline__ EqCoeffs<R> eq_coeffs(const Macro<R>& M) {
-  const R s3 = R(1.7320508075688772), s15 = R(3.872983346207417);
-  const R s53 = R(1.2909944487358056), s6 = R(2.449489742783178);
-  const R s23 = R(0.816496580927726), s25 = R(0.6324555320336759);
-  const R s10 = R(3.1622776601683795), s32 = R(1.224744871391589), s52 = R(1.5811388300841898);
-  const R T = R(1) + M.dT;
-  const R g = M.gamma;
-  const R uX = g * M.ux, uY = g * M.uy;
-  const R Tu = M.dT + M.gm1 + M.dT * M.gm1;          // T u^0 - 1
-  const R gT = M.gm1 * T;                            // (gamma - 1) T
-  const R dT2 = M.dT * M.dT;
-  const R T2 = T * T;
-  const R g2 = g * g;
-  // App. B projections (rest-deviation form, algebraically identical)
-  const R a10 = Tu;
-  const R a1x = T * uX;
-  const R a1y = T * uY;
-  // Tu - (T^2 - 1)/2 = (gamma - 1) T - (T - 1)^2 / 2, and alike below
-  const R a200 = R(1.5) * Tu * Tu + gT - R(0.5) * dT2;
-  const R a20x = s3 * T * uX * Tu;
-  const R a20y = s3 * T * uY * Tu;
-  const R dxy2 = g2 * (M.ux * M.ux - M.uy * M.uy);    // u0^2 - 1 - 2 uX^2 = -dxy2
-  const R a2xx = R(0.5) * s3 * T2 * dxy2;
-  const R a2xy = s3 * T2 * uX * uY;
-  const R a3000 = R(0.5) * Tu * (R(5) * Tu * Tu + R(6) * gT - R(3) * dT2);
-  const R a3xxx = R(0.5) * T * uX * (R(5) * T2 * uX * uX + R(3) * dT2 - R(6) * gT);
-  const R a300x = R(-0.5) * s15 * T * uX * (R(-2) * Tu * Tu + T2 * uX * uX + dT2 - R(2) * gT);
-  const R a30xx = R(0.5) * s15 * T2 * Tu * dxy2;
-  const R a300y = R(0.5) * s32 * T * uY * (R(5) * Tu * Tu + R(2) * gT - dT2);
-  const R a3xxy = R(-0.5) * s52 * T2 * T * uY * g2 * (M.uy * M.uy - R(3) * M.ux * M.ux);
-  const R a30xy = s15 * T2 * uX * uY * Tu;
-
+__device__ __forceinline__ EqCoeffs<R> eq_coeffs(const Macro<R>& M, R nT, R nmT) {
   EqCoeffs<R> c;
-  c.q0m1 = -a10 + a200 - a3000;
-  c.c1_0 = a10 - R(2) * a200 + R(3) * a3000;
-  c.c1_x = a1x - s3 * a20x + R(1.5) * a3xxx + R(0.5) * s15 * a300x;
-  c.c1_y = a1y - s3 * a20y + s6 * a300y;
-  // reciprocals of the App. A normalisations (multiplications, not divisions)
-  const R i_s3 = R(0.57735026918962576), i_2s3 = R(0.28867513459481288);
-  const R i_s15 = R(0.25819888974716112), i_2s15 = R(0.12909944487358056);
-  const R i_2s6 = R(0.20412414523193151), i_6s10 = R(0.052704627669472988);
-  const R i_6 = R(1.0 / 6.0), s25_3 = R(0.21081851067789195);
-  c.c2_0 = R(0.5) * a200 - a2xx * i_2s3 - R(1.5) * a3000 + R(0.5) * s53 * a30xx;
-  c.c2_x = a20x * i_s3 - a3xxx - s53 * a300x;
-  c.c2_y = a20y * i_s3 - R(2) * s23 * a300y;
-  c.c2_xx = a2xx * i_s3 - s53 * a30xx;
-  c.c2_xy = a2xy * i_s3 - s53 * a30xy;
-  c.c3_0 = a3000 * i_6 - a30xx * i_2s15;
-  c.c3_x = a300x * i_s15;
-  c.c3_y = a300y * i_2s6 - a3xxy * i_6s10;
-  c.c3_xx = a30xx * i_s15;
-  c.c3_xy = a30xy * i_s15;
-  c.c3_xxx = a3xxx * i_6 - a300x * i_2s15;
-  c.c3_xxy = s25_3 * a3xxy;
+  const R tg = fma(M.dT, M.gamma, M.gamma);              // T gamma
+  const R W = fma(M.dT, M.gamma, M.gm1);                 // T gamma - 1
+  const R X = tg * M.ux, Y = tg * M.uy;
+  const R r2 = fma(X, X, Y * Y), W2 = W * W;
+  const R h = fma(R(1.5), r2, R(1));                     // 1 + 3 r^2 / 2
+  const R q0 = fma(-W, W2 + h, fma(R(0.5), r2, W2));
+  const R t = fma(R(-3), W, R(1));                       // 1 - 3 W
+  c.W = W; c.X = X; c.Y = Y;
+  c.e0 = fma(nT, q0, nmT);
+  c.D = nT * (W2 - r2);
+  c.lam = c.D * t;
+  c.kap = nT * fma(R(-3), W, fma(R(6), W2, h));
+  c.mu = nT * fma(R(-2.5), W, R(0.5));
+  c.nu = nT * R(1.0 / 6.0);
   return c;
 }
 
 // Per-direction cubic R_0 + R_1 p0 + R_2 p0^2 + R_3 p0^3 such that the new
-// deviation of shell j is  (1 - omega_d) delta_dj + w_dj (sum_m R_m p0_j^m):
+// deviation of shell j is  (1 - omega_d) g_dj + sum_m R_m p0_j^m:
 //   omega_d (f^eq - w) / w  +  F^ext / w,
 // with omega_d = gamma (1 - v_d.u) / tau (= p^m U_m / (p^0 tau) on the massless shell).
 // Forcing (force F per particle, dt = 1):
 //   F^ext / w = (n/T) [ (F.v) Q - F.grad Q ]  at p = p0 (1, v),
-// where grad is the gradient along the shell; with Q = sum_m p0^m q_m(theta)
-//   F.grad Q = sum_m p0^(m-1) [ m q_m (F.v) + dq_m/dtheta (F.t) ],  t = (-vy, vx),
-// so the p0^m coefficient of the source is
-//   s_m = (F.v) (q_m - (m+1) q_{m+1}) - (F.t) dq_{m+1}/dtheta.
-// Directions d (even) and d + 1 have opposite velocities; every polynomial is
-// split into its even and odd parts in v, evaluated once for the pair.
-// gux = gamma u_x / tau, guy = gamma u_y / tau, gt = gamma / tau.
+// grad along the shell (grad p0 = v).  Q depends on the momentum through p0
+// and y = p0 z = W p0 + X px + Y py, so with phi = F.v, f = F.(X, Y) and
+// psi = F.grad y = W phi + f
+//   F.grad Q = phi (lambda + D y) + psi (kappa + D p0 + 2 mu y + y^2 / 2);
+// psi is linear in phi, and everything that multiplies phi or stands alone is
+// gathered per site:
+//   R_0 = o e0 + a0 phi + b0
+//   R_1 = o e1 + z (a1 phi + b1) + a2 phi + b2
+//   R_2 = o e2 + z^2 (a3 phi + b3)
+//   R_3 = o e3,                        o = omega + phi = gt + (F - gt u).v.
+template <typename R>
+struct ForceCoeffs {
+  R a0, b0, a1, b1, a2, b2, a3, b3;
+};
+
+template <typename R>
+__device__ __forceinline__ ForceCoeffs<R> force_coeffs(const EqCoeffs<R>& c, R Fx, R Fy, R scl) {
+  ForceCoeffs<R> k;
+  const R f = fma(Fx, c.X, Fy * c.Y);
+  const R m2 = R(-2) * c.mu, n3 = R(-3) * c.nu;
+  k.a0 = fma(-c.W, c.kap, scl - c.lam);
+  k.b0 = -(f * c.kap);
+  k.a1 = fma(m2, c.W, -c.D);
+  k.b1 = m2 * f;
+  k.a2 = -(c.D * c.W);
+  k.b2 = -(c.D * f);
+  k.a3 = n3 * c.W;
+  k.b3 = n3 * f;
+  return k;
+}
+
+// What a direction's cubic needs beside c: gt = gamma / tau, 1 - gt, gt u and F.
+template <typename R>
+struct RelaxSite {
+  R gt, omgt, gux, guy, Fx, Fy;
+};
+
+// The cubic of one direction from its z, o = omega + phi and phi = F.v.
 template <typename R, bool FORCE>
-__device__ __forceinline__ void pair_cubics(const int d, const EqCoeffs<R>& c, R nT, R nmT,
-                                            R gt, R gux, R guy, R Fx, R Fy,
-                                            R (&Rp)[4], R (&Rn)[4], R& omp, R& omn) {
-  const R vx = R(hop_x(d)) / R(5), vy = R(hop_y(d)) / R(5);
-  R ow = R(0);
-  if (hop_x(d) != 0) ow = gux * vx;
-  if (hop_y(d) != 0) ow = fma(guy, vy, ow);
-  omp = gt - ow;
-  omn = gt + ow;
-  const R E2 = c.c2_0 + c.c2_xx * (vx * vx) + c.c2_xy * (vx * vy);
-  const R E3 = c.c3_0 + c.c3_xx * (vx * vx) + c.c3_xy * (vx * vy);
-  const R O1 = c.c1_x * vx + c.c1_y * vy;
-  const R O2 = c.c2_x * vx + c.c2_y * vy;
-  const R O3 = c.c3_x * vx + c.c3_y * vy + c.c3_xxx * (vx * vx * vx) + c.c3_xxy * (vx * vx * vy);
-  const R q1p = c.c1_0 + O1, q1n = c.c1_0 - O1;
-  const R q2p = E2 + O2, q2n = E2 - O2;
-  const R q3p = E3 + O3, q3n = E3 - O3;
-  const R onp = omp * nT, onn = omn * nT;
-  Rp[0] = fma(omp, nmT, onp * c.q0m1);
-  Rn[0] = fma(omn, nmT, onn * c.q0m1);
-  Rp[1] = onp * q1p;
-  Rn[1] = onn * q1n;
-  Rp[2] = onp * q2p;
-  Rn[2] = onn * q2n;
-  Rp[3] = onp * q3p;
-  Rn[3] = onn * q3n;
+__device__ __forceinline__ void direction_cubic(const EqCoeffs<R>& c, const ForceCoeffs<R>& k,
+                                                R z, R o, R phi, R (&Rm)[4]) {
+  const R e1 = fma(c.kap, z, c.lam);
+  const R e2 = z * fma(c.mu, z, c.D);
+  const R z2 = z * z;
+  const R e3 = (c.nu * z) * z2;
   if (FORCE) {
-    // F.v and F.t flip sign between the two directions; dq_m/dtheta = Et_m +- Ot_m
-    const R Fv = Fx * vx + Fy * vy, Ft = Fy * vx - Fx * vy;
-    const R Ot1 = -vy * c.c1_x + vx * c.c1_y;
-    const R Ot2 = -vy * c.c2_x + vx * c.c2_y;
-    const R Et2 = R(-2) * (vx * vy) * c.c2_xx + (vx * vx - vy * vy) * c.c2_xy;
-    const R Ot3 = -vy * c.c3_x + vx * c.c3_y - R(3) * (vx * vx * vy) * c.c3_xxx
-                + (vx * vx * vx - R(2) * vx * vy * vy) * c.c3_xxy;
-    const R Et3 = R(-2) * (vx * vy) * c.c3_xx + (vx * vx - vy * vy) * c.c3_xy;
-    const R q0 = R(1) + c.q0m1;
-    const R FvT = Fv * nT, FtT = Ft * nT;
-    Rp[0] = fma(FvT, q0 - q1p, fma(-FtT, Ot1, Rp[0]));
-    Rn[0] = fma(-FvT, q0 - q1n, fma(-FtT, Ot1, Rn[0]));
-    Rp[1] = fma(FvT, q1p - R(2) * q2p, fma(-FtT, Et2 + Ot2, Rp[1]));
-    Rn[1] = fma(-FvT, q1n - R(2) * q2n, fma(FtT, Et2 - Ot2, Rn[1]));
-    Rp[2] = fma(FvT, q2p - R(3) * q3p, fma(-FtT, Et3 + Ot3, Rp[2]));
-    Rn[2] = fma(-FvT, q2n - R(3) * q3n, fma(FtT, Et3 - Ot3, Rn[2]));
-    Rp[3] = fma(FvT, q3p, Rp[3]);
-    Rn[3] = fma(-FvT, q3n, Rn[3]);
+    Rm[0] = fma(o, c.e0, fma(phi, k.a0, k.b0));
+    Rm[1] = fma(o, e1, fma(z, fma(phi, k.a1, k.b1), fma(phi, k.a2, k.b2)));
+    Rm[2] = fma(o, e2, z2 * fma(phi, k.a3, k.b3));
+  } else {
+    Rm[0] = o * c.e0;
+    Rm[1] = o * e1;
+    Rm[2] = o * e2;
   }
+  Rm[3] = o * e3;
 }
 
-template <typename R>
-__device__ __forceinline__ bool macro_ok(const Macro<R>& M) {
-  const R u2 = M.ux * M.ux + M.uy * M.uy;
-  return (u2 < R(1)) && (M.dn > R(-1)) && (M.dT > R(-1));
-}
-
-template <typename R>
-__device__ __forceinline__ bool all_finite(const Macro<R>& M) {
-  return isfinite(M.ux) && isfinite(M.uy) && isfinite(M.dn) && isfinite(M.dT);
+// Cubics and 1 - omega of directions d (even) and d + 1 (opposite velocity).
+template <typename R, bool FORCE>
+__device__ __forceinline__ void pair_cubics(const int d, const EqCoeffs<R>& c,
+                                            const ForceCoeffs<R>& k, const RelaxSite<R>& s,
+                                            R (&Rp)[4], R (&Rn)[4], R& omcp, R& omcn) {
+  const R vx = R(hop_x(d)) / R(5), vy = R(hop_y(d)) / R(5);
+  R zo, go, phi;
+  if (hop_y(d) == 0) {            // v = (1, 0)
+    zo = c.X; go = s.gux; phi = s.Fx;
+  } else if (hop_x(d) == 0) {     // v = (0, 1)
+    zo = c.Y; go = s.guy; phi = s.Fy;
+  } else {
+    zo = fma(c.X, vx, c.Y * vy);
+    go = fma(s.gux, vx, s.guy * vy);
+    phi = FORCE ? fma(s.Fx, vx, s.Fy * vy) : R(0);
+  }
+  const R oo = FORCE ? phi - go : -go;
+  omcp = s.omgt + go;
+  omcn = s.omgt - go;
+  direction_cubic<R, FORCE>(c, k, c.W + zo, s.gt + oo, phi, Rp);
+  direction_cubic<R, FORCE>(c, k, c.W - zo, s.gt - oo, -phi, Rn);
 }
 
 }  // namespace rlbm
