@@ -195,6 +195,9 @@ size_t plan(const rlbm_config* cfg, const PrecOps* ops, rlbm_ctx* out) {
     d.inv_tau = 1.0 / s.tau;
     d.Fx = s.Fx; d.Fy = s.Fy;
     d.inv_cg = s.inv_cg;
+    d.inv_tau_f = (float)d.inv_tau;
+    d.Fx_f = (float)s.Fx; d.Fy_f = (float)s.Fy;
+    d.inv_cg_f = (float)s.inv_cg;
     d.dn[0] = d.dn[1] = nullptr;     // bound to the workspace by rlbm_create
     d.cur = 0;
     for (int k = 0; k < s.ncontacts; ++k) {

@@ -55,26 +55,76 @@ __device__ __forceinline__ int contact_of(const DevSample& s, int sx, int sy) {
   return -1;
 }
 
+// A thread's site vector in direction plane 0 of the two buffers, and the
+// byte offsets from there to the 12 vectors it pulls (interior sites) and to
+// the 12 direction planes it stores.  The single-sample kernel takes the
+// offsets from its parameters (constant memory: two additions per access);
+// formed from the descriptor by each thread they cost about 100 integer
+// instructions per site, most of them on the pipe that bounds the 16-bit step.
+template <typename S>
+struct Tile {
+  const S* in;
+  S* out;
+  uint64_t policy;     // L2 policy of the pulled vectors
+};
+
+template <typename S>
+__host__ __device__ constexpr long long pull_offset(int d, long long plane, long long ldx) {
+  return ((long long)d * plane - ((long long)hop_y(d) * ldx + hop_x(d))) * (long long)(4 * sizeof(S));
+}
+template <typename S>
+__host__ __device__ constexpr long long plane_offset(int d, long long plane) {
+  return (long long)d * plane * (long long)(4 * sizeof(S));
+}
+
+struct StepOffsets {        // prepared on the host
+  long long pull_[kDirs], plane_[kDirs];
+  __device__ __forceinline__ long long pull(int d) const { return pull_[d]; }
+  __device__ __forceinline__ long long plane(int d) const { return plane_[d]; }
+};
+template <typename S>
+struct SampleOffsets {      // from the descriptor
+  long long p;
+  int ldx;
+  __device__ __forceinline__ long long pull(int d) const { return pull_offset<S>(d, p, ldx); }
+  __device__ __forceinline__ long long plane(int d) const { return plane_offset<S>(d, p); }
+};
+
+template <typename T>
+__device__ __forceinline__ T* byte_ptr(T* base, long long bytes) {
+  using B = typename std::conditional<std::is_const<T>::value, const char, char>::type;
+  return reinterpret_cast<T*>(reinterpret_cast<B*>(base) + bytes);
+}
+
+// L2 policy of the pulls.  Each stored value is read once per step and its
+// line is next written a step later, so when a buffer is not much larger than
+// the L2 the lines just read should leave first and the ones just written
+// (the next step's input) stay; see launch_single for the rule.
+__device__ __forceinline__ uint64_t pull_policy(bool evict_first) {
+  uint64_t a, b;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(a));
+  asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(b));
+  return evict_first ? a : b;
+}
+
 // Gathers the 48 streamed deviations arriving at (x, y).
-template <typename S, bool INTERIOR, class C>
-__device__ __forceinline__ void pull(const S* __restrict__ fin, const DevSample& s, int x, int y,
+template <typename S, bool INTERIOR, class C, class O>
+__device__ __forceinline__ void pull(const S* __restrict__ fin, const Tile<S>& tl, const O& of,
+                                     const DevSample& s, int x, int y,
                                      const typename Codec<S>::R* __restrict__ ghost, const C& qc,
                                      typename Codec<S>::R (&f)[kQ]) {
-  const long long site = (long long)y * s.ldx + x;
 #pragma unroll
   for (int d = 0; d < kDirs; ++d) {
     const int dx = hop_x(d), dy = hop_y(d);
     if (INTERIOR) {
-      Codec<S>::load4(fin + vec_index(s, d, site - ((long long)dy * s.ldx + dx)), dir_kind(d),
-                      qc, &f[4 * d]);
+      Codec<S>::load4(byte_ptr(tl.in, of.pull(d)), tl.policy, &f[4 * d]);
     } else {
       int sx = x - dx, sy = y - dy;
       if (s.periodic_x) sx = sx < 0 ? sx + s.nx : (sx >= s.nx ? sx - s.nx : sx);
       if (s.periodic_y) sy = sy < 0 ? sy + s.ny : (sy >= s.ny ? sy - s.ny : sy);
       const bool inside = (unsigned)sx < (unsigned)s.nx && (unsigned)sy < (unsigned)s.ny;
       if (inside) {
-        Codec<S>::load4(fin + vec_index(s, d, (long long)sy * s.ldx + sx), dir_kind(d), qc,
-                        &f[4 * d]);
+        Codec<S>::load4(fin + vec_index(s, d, (long long)sy * s.ldx + sx), tl.policy, &f[4 * d]);
       } else {
         const int owner = contact_of(s, sx, sy);
         if (owner >= 0) {
@@ -82,7 +132,7 @@ __device__ __forceinline__ void pull(const S* __restrict__ fin, const DevSample&
           for (int j = 0; j < kShells; ++j) f[4 * d + j] = ghost[owner * kQ + 4 * d + j];
         } else {
           // bounce-back: post-collision population of the opposite direction, same shell
-          Codec<S>::load4(fin + vec_index(s, d ^ 1, site), dir_kind(d), qc, &f[4 * d]);
+          Codec<S>::load4(byte_ptr(tl.in, of.plane(d ^ 1)), tl.policy, &f[4 * d]);
         }
       }
     }
@@ -231,9 +281,7 @@ __device__ __forceinline__ void stage_issue(const S* __restrict__ fin, const Dev
         :: "r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-// Where the 48 arriving deviations of a site come from: straight from HBM, or
-// from the staged slot rows of its tile.
-struct DirectSrc {};
+// The staged slot rows of a tile.
 template <typename S, int BX>
 struct StagedSrc {
   uint32_t buf;     // shared-window address of the tile's slot rows
@@ -251,12 +299,13 @@ __device__ __forceinline__ void pull_staged(const S* __restrict__ fin, const Dev
   constexpr int G = Stage<S>::kG, SL = Stage<S>::template slots<BX>();
   constexpr int VB = Stage<S>::kVecBytes;
   const long long site = (long long)y * s.ldx + x;
+  const uint64_t pol = pull_policy(false);
   const int i = x - st.x0;
   if (INTERIOR && __builtin_expect(st.mask == (1u << kDirs) - 1u, 1)) {
 #pragma unroll
     for (int d = 0; d < kDirs; ++d)
       Codec<S>::load4s(st.buf + (uint32_t)((d * SL + i + ((st.x0 - hop_x(d)) & (G - 1))) * VB),
-                       dir_kind(d), qc, &f[4 * d]);
+                        &f[4 * d]);
     return;
   }
 #pragma unroll
@@ -265,25 +314,24 @@ __device__ __forceinline__ void pull_staged(const S* __restrict__ fin, const Dev
     const bool staged = (st.mask >> d) & 1u;
     const uint32_t sp = st.buf + (uint32_t)((d * SL + i + ((st.x0 - dx) & (G - 1))) * VB);
     if (INTERIOR) {
-      if (staged) Codec<S>::load4s(sp, dir_kind(d), qc, &f[4 * d]);
-      else Codec<S>::load4(fin + vec_index(s, d, site - ((long long)dy * s.ldx + dx)), dir_kind(d),
-                           qc, &f[4 * d]);
+      if (staged) Codec<S>::load4s(sp, &f[4 * d]);
+      else Codec<S>::load4(fin + vec_index(s, d, site - ((long long)dy * s.ldx + dx)), pol,
+                           &f[4 * d]);
     } else {
       int sx = x - dx, sy = y - dy;
       if (s.periodic_x) sx = sx < 0 ? sx + s.nx : (sx >= s.nx ? sx - s.nx : sx);
       if (s.periodic_y) sy = sy < 0 ? sy + s.ny : (sy >= s.ny ? sy - s.ny : sy);
       const bool inside = (unsigned)sx < (unsigned)s.nx && (unsigned)sy < (unsigned)s.ny;
       if (inside) {
-        if (staged) Codec<S>::load4s(sp, dir_kind(d), qc, &f[4 * d]);
-        else Codec<S>::load4(fin + vec_index(s, d, (long long)sy * s.ldx + sx), dir_kind(d), qc,
-                             &f[4 * d]);
+        if (staged) Codec<S>::load4s(sp, &f[4 * d]);
+        else Codec<S>::load4(fin + vec_index(s, d, (long long)sy * s.ldx + sx), pol, &f[4 * d]);
       } else {
         const int owner = contact_of(s, sx, sy);
         if (owner >= 0) {
 #pragma unroll
           for (int j = 0; j < kShells; ++j) f[4 * d + j] = ghost[owner * kQ + 4 * d + j];
         } else {
-          Codec<S>::load4(fin + vec_index(s, d ^ 1, site), dir_kind(d), qc, &f[4 * d]);
+          Codec<S>::load4(fin + vec_index(s, d ^ 1, site), pol, &f[4 * d]);
         }
       }
     }
@@ -365,24 +413,21 @@ __device__ __forceinline__ void lca_gradient(const DevSample& s, const R* __rest
   gy = (p[(long long)yp * s.ldx + x] - p[(long long)ym * s.ldx + x]) * hy;
 }
 
-// Gathers the 48 deviations streamed into site (x < nx, y): from HBM or from
-// the staged slot rows.  All 32 threads of a warp must hold consecutive x of
-// the same row (the interior test is per warp).
-template <typename S, class C, class SRC>
-__device__ __forceinline__ void gather(const S* __restrict__ fin, const DevSample& s, int x, int y,
-                                       const typename Codec<S>::R* __restrict__ ghost, const C& qc,
-                                       const SRC& src, typename Codec<S>::R (&f)[kQ]) {
-  // warp-uniform: the 32 sites of this warp pull only from inside the rectangle
+// Whether the 32 sites of a warp (consecutive x of row y) pull only from
+// inside the rectangle.
+__device__ __forceinline__ bool warp_interior(const DevSample& s, int x, int y) {
   const int wx0 = x & ~31;
-  const bool interior = wx0 >= kRadius && wx0 + 32 + kRadius <= s.nx &&
-                        y >= kRadius && y + kRadius < s.ny;
-  if constexpr (std::is_same<SRC, DirectSrc>::value) {
-    if (interior) pull<S, true>(fin, s, x, y, ghost, qc, f);
-    else          pull<S, false>(fin, s, x, y, ghost, qc, f);
-  } else {
-    if (interior) pull_staged<S, true>(fin, s, x, y, ghost, qc, src, f);
-    else          pull_staged<S, false>(fin, s, x, y, ghost, qc, src, f);
-  }
+  return wx0 >= kRadius && wx0 + 32 + kRadius <= s.nx && y >= kRadius && y + kRadius < s.ny;
+}
+
+// Gathers the 48 deviations streamed into site (x < nx, y) from HBM.
+template <typename S, class C, class O>
+__device__ __forceinline__ void gather(const S* __restrict__ fin, const Tile<S>& tl, const O& of,
+                                       const DevSample& s, int x, int y,
+                                       const typename Codec<S>::R* __restrict__ ghost, const C& qc,
+                                       typename Codec<S>::R (&f)[kQ]) {
+  if (warp_interior(s, x, y)) pull<S, true>(fin, tl, of, s, x, y, ghost, qc, f);
+  else pull<S, false>(fin, tl, of, s, x, y, ghost, qc, f);
 }
 
 // pair_cubics() on register pairs, lanes (d, d + 1): the two lanes differ only
@@ -454,20 +499,22 @@ __device__ __forceinline__ void relax_shells_paired(float R0, float R1, float R2
 // collide_store() with FP32 arithmetic (FP32 and 16-bit storage) on register
 // pairs: the same quantities in the same order of operations per population,
 // with each instruction serving two directions or two shells.
-template <typename S, int FORCE, int RES, int BT, class C>
-__device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restrict__ fout,
-                                                     const DevSample& s, int x, int y,
+template <typename S, int FORCE, int RES, int BT, class C, class O>
+__device__ __forceinline__ void collide_store_paired(float (&f)[kQ], const Tile<S>& tl,
+                                                     const O& of, const DevSample& s, int x, int y,
                                                      const StepAux<float>& aux, const C& qc,
                                                      double& r_du2, double& r_u2, uint32_t park,
                                                      const float* dn_prev, float* dn_next) {
   constexpr bool kProject = sizeof(S) == sizeof(float);
-  const bool lca = FORCE == kForceLca && s.inv_cg != 0.0;
+  const bool lca = FORCE == kForceLca && s.dn[0] != nullptr;
   float egx = 0.f, egy = 0.f;
   if (lca) lca_gradient(s, dn_prev, x, y, egx, egy);
   const Moments<float> m = moments(f, qc);
   constexpr uint32_t park_stride = BT * 16u;
+  if constexpr (Park<float>::kOn) {
 #pragma unroll
-  for (int d = 0; d < kDirs; ++d) park_store(park + d * park_stride, &f[4 * d]);
+    for (int d = 0; d < kDirs; ++d) park_store(park + d * park_stride, &f[4 * d]);
+  }
   Macro<float> M;
   const unsigned bad = landau(m, M);
   if (bad) atomicOr(aux.err, bad);
@@ -475,17 +522,16 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restri
   const float scl = sizeof(S) == 2 ? qc.enc_s : 1.f;
   const float iTs = M.invT * scl;
   const EqCoeffs<float> c = eq_coeffs(M, fmaf(M.dn, iTs, iTs), (M.dn - M.dT) * iTs);
-  const float Fx = lca ? fmaf(-float(s.inv_cg), egx, float(s.Fx)) : float(s.Fx);
-  const float Fy = lca ? fmaf(-float(s.inv_cg), egy, float(s.Fy)) : float(s.Fy);
+  const float Fx = lca ? fmaf(-s.inv_cg_f, egx, s.Fx_f) : s.Fx_f;
+  const float Fy = lca ? fmaf(-s.inv_cg_f, egy, s.Fy_f) : s.Fy_f;
   RelaxSite<float> rs;
-  rs.gt = M.gamma * float(s.inv_tau);
+  rs.gt = M.gamma * s.inv_tau_f;
   rs.omgt = 1.f - rs.gt;
   rs.gux = rs.gt * M.ux; rs.guy = rs.gt * M.uy;
   rs.Fx = Fx; rs.Fy = Fy;
   ForceCoeffs<float> k{};
   if (FORCE != 0) k = force_coeffs(c, Fx, Fy, scl);
-  const long long site = (long long)y * s.ldx + x;
-  if (lca) dn_next[site] = M.dn;
+  if (lca) dn_next[(long long)y * s.ldx + x] = M.dn;
   // conservation projection: sums of the moment changes (N^0, T^00) and
   // (T^0x, T^0y), started with minus the forcing's target
   float2 accNE = S2(0.f), accXY = S2(0.f);
@@ -503,8 +549,10 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restri
     const int kind = dir_kind(d);
     float2 R[4], omc;
     pair_cubics_paired<FORCE != 0>(d, c, k, rs, qc, R, omc);
-    park_load(park + d * park_stride, &f[4 * d]);
-    park_load(park + (d + 1) * park_stride, &f[4 * d + 4]);
+    if constexpr (Park<float>::kOn) {
+      park_load(park + d * park_stride, &f[4 * d]);
+      park_load(park + (d + 1) * park_stride, &f[4 * d + 4]);
+    }
     float2 bp, bn;
     relax_shells_paired<kProject>(R[0].x, R[1].x, R[2].x, R[3].x, omc.x, kind, qc, &f[4 * d], bp);
     relax_shells_paired<kProject>(R[0].y, R[1].y, R[2].y, R[3].y, omc.y, kind, qc, &f[4 * d + 4],
@@ -514,9 +562,9 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restri
       accXY = fma2(S2(bp.y - bn.y), qc.vxy[d / 2], accXY);
     }
     if (!kProject || kind == 0) {
-      Codec<S>::store4(fout + vec_index(s, d, site), kind, qc, &f[4 * d]);
-      Codec<S>::store4(fout + vec_index(s, d + 1, site), kind, qc, &f[4 * d + 4]);
-    } else {
+      Codec<S>::store4(byte_ptr(tl.out, of.plane(d)), &f[4 * d]);
+      Codec<S>::store4(byte_ptr(tl.out, of.plane(d + 1)), &f[4 * d + 4]);
+    } else if constexpr (Park<float>::kOn) {
       // (5,0)-type: wait for the correction in the parking area, not in registers
       park_store(park + d * park_stride, &f[4 * d]);
       park_store(park + (d + 1) * park_stride, &f[4 * d + 4]);
@@ -530,14 +578,14 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restri
 #pragma unroll
     for (int d = 8; d < kDirs; ++d) {
       const float cd = l1 + (hop_x(d) > 0 ? lx : hop_x(d) < 0 ? -lx : hop_y(d) > 0 ? ly : -ly);
-      park_load(park + d * park_stride, &f[4 * d]);
+      if constexpr (Park<float>::kOn) park_load(park + d * park_stride, &f[4 * d]);
       // delta += w (l0 + p0 cd)
       const float2 t01 = fma2(S2(cd), qc.p01, S2(l0));
       const float2 t23 = fma2(S2(cd), qc.p23, S2(l0));
       const float2 o01 = add2(make_float2(f[4 * d], f[4 * d + 1]), t01);
       const float2 o23 = add2(make_float2(f[4 * d + 2], f[4 * d + 3]), t23);
       f[4 * d] = o01.x; f[4 * d + 1] = o01.y; f[4 * d + 2] = o23.x; f[4 * d + 3] = o23.y;
-      Codec<S>::store4(fout + vec_index(s, d, site), 1, qc, &f[4 * d]);
+      Codec<S>::store4(byte_ptr(tl.out, of.plane(d)), &f[4 * d]);
     }
   }
   if (RES == 1) {
@@ -558,9 +606,9 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], S* __restri
 // residual; 2 add |u - u_prev|^2 and |u|^2 to r_du2, r_u2 (the caller
 // reduces them).  dn_prev / dn_next: the electric force's density planes of
 // the previous and of this step (used when s.inv_cg != 0).
-template <typename S, int FORCE, int RES, int BT, class C>
-__device__ __forceinline__ void collide_store(typename Codec<S>::R (&f)[kQ], S* __restrict__ fout,
-                                              const DevSample& s, int x, int y,
+template <typename S, int FORCE, int RES, int BT, class C, class O>
+__device__ __forceinline__ void collide_store(typename Codec<S>::R (&f)[kQ], const Tile<S>& tl,
+                                              const O& of, const DevSample& s, int x, int y,
                                               const StepAux<typename Codec<S>::R>& aux,
                                               const C& qc, double& r_du2, double& r_u2,
                                               uint32_t park,
@@ -568,12 +616,12 @@ __device__ __forceinline__ void collide_store(typename Codec<S>::R (&f)[kQ], S* 
                                               typename Codec<S>::R* dn_next) {
   using R = typename Codec<S>::R;
   if constexpr (std::is_same<R, float>::value) {
-    collide_store_paired<S, FORCE, RES, BT>(f, fout, s, x, y, aux, qc, r_du2, r_u2, park, dn_prev,
+    collide_store_paired<S, FORCE, RES, BT>(f, tl, of, s, x, y, aux, qc, r_du2, r_u2, park, dn_prev,
                                         dn_next);
   } else {
     // FP64 storage: the populations stay in registers (the FP64 pipe, not
     // latency, bounds this path), no conservation projection
-    const bool lca = FORCE == kForceLca && s.inv_cg != 0.0;
+    const bool lca = FORCE == kForceLca && s.dn[0] != nullptr;
     R egx = R(0), egy = R(0);
     if (lca) lca_gradient(s, dn_prev, x, y, egx, egy);
     const Moments<R> m = moments(f, qc);
@@ -589,16 +637,15 @@ __device__ __forceinline__ void collide_store(typename Codec<S>::R (&f)[kQ], S* 
     rs.Fy = lca ? fma(-R(s.inv_cg), egy, R(s.Fy)) : R(s.Fy);
     ForceCoeffs<R> k{};
     if (FORCE != 0) k = force_coeffs(c, rs.Fx, rs.Fy, R(1));
-    const long long site = (long long)y * s.ldx + x;
-    if (lca) dn_next[site] = M.dn;
+    if (lca) dn_next[(long long)y * s.ldx + x] = M.dn;
 #pragma unroll
     for (int d = 0; d < kDirs; d += 2) {
       R Rp[4], Rn[4], omcp, omcn;
       pair_cubics<R, FORCE != 0>(d, c, k, rs, Rp, Rn, omcp, omcn);
       relax_shells(Rp, omcp, qc, &f[4 * d]);
       relax_shells(Rn, omcn, qc, &f[4 * d + 4]);
-      Codec<S>::store4(fout + vec_index(s, d, site), dir_kind(d), qc, &f[4 * d]);
-      Codec<S>::store4(fout + vec_index(s, d + 1, site), dir_kind(d), qc, &f[4 * d + 4]);
+      Codec<S>::store4(byte_ptr(tl.out, of.plane(d)), &f[4 * d]);
+      Codec<S>::store4(byte_ptr(tl.out, of.plane(d + 1)), &f[4 * d + 4]);
     }
     if (RES == 1) {
       const long long j = s.site0 + (long long)y * s.nx + x;
@@ -614,34 +661,70 @@ __device__ __forceinline__ void collide_store(typename Codec<S>::R (&f)[kQ], S* 
 }
 
 // Fused stream + collide of site (x, y) (nothing if x >= nx).
-template <typename S, int FORCE, int RES, int BT, class C>
-__device__ __forceinline__ void site_step(const S* __restrict__ fin, S* __restrict__ fout,
-                                          const DevSample& s, int x, int y,
+template <typename S, int FORCE, int RES, int BT, class C, class O>
+__device__ __forceinline__ void site_step(const S* __restrict__ fin, const Tile<S>& tl,
+                                          const O& of, const DevSample& s, int x, int y,
                                           const typename Codec<S>::R* __restrict__ ghost,
                                           const StepAux<typename Codec<S>::R>& aux, const C& qc,
                                           double& r_du2, double& r_u2, uint32_t park, int cur) {
   using R = typename Codec<S>::R;
   if (x < s.nx) {
     R f[kQ];
-    gather(fin, s, x, y, ghost, qc, DirectSrc(), f);
+    gather(fin, tl, of, s, x, y, ghost, qc, f);
     // select, not s.dn[cur]: a runtime index would move the descriptor to local memory
     void* const prev = cur ? s.dn[1] : s.dn[0];
     void* const next = cur ? s.dn[0] : s.dn[1];
-    collide_store<S, FORCE, RES, BT>(f, fout, s, x, y, aux, qc, r_du2, r_u2, park,
-                                 static_cast<const R*>(prev), static_cast<R*>(next));
+    collide_store<S, FORCE, RES, BT>(f, tl, of, s, x, y, aux, qc, r_du2, r_u2, park,
+                                     static_cast<const R*>(prev), static_cast<R*>(next));
   }
 }
 
-// One sample, one block row of kBX sites.
-template <typename S, int FORCE, int RES, class C>
+// Row segments of 32 sites ("warp tiles") of one sample, numbered row by row.
+struct WarpTiles {
+  unsigned per_row, magic, count;   // magic = floor(2^32 / per_row)
+  int evict_first;                  // L2 policy of the pulls (pull_policy)
+  int reverse;                      // walk the tiles from the last to the first
+  __device__ __forceinline__ void row_of(unsigned t, unsigned& y, unsigned& r) const {
+    // the product's high word is the quotient t / per_row or one below it
+    y = __umulhi(t, magic);
+    r = t - y * per_row;
+    if (r >= per_row) { r -= per_row; ++y; }
+  }
+};
+
+// Chained launches: a step kernel lets its successor start as soon as all of
+// its own blocks run, and waits for its predecessor's results only before
+// its first access to them.
+__device__ __forceinline__ void chain_release() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+
+// One sample: each warp of a block of BT threads updates one warp tile.
+template <typename S, int FORCE, int RES, int BT, class C>
 __device__ __forceinline__ void step_body(const S* __restrict__ fin, S* __restrict__ fout,
-                                          const DevSample& s,
+                                          const DevSample& s, const WarpTiles& wt,
+                                          const StepOffsets& of,
                                           const typename Codec<S>::R* __restrict__ ghost,
                                           const StepAux<typename Codec<S>::R>& aux, const C& qc,
                                           unsigned char* park) {
+  chain_release();
   double r_du2 = 0.0, r_u2 = 0.0;
-  site_step<S, FORCE, RES, kBX>(fin, fout, s, blockIdx.x * kBX + threadIdx.x, blockIdx.y, ghost, aux,
-                           qc, r_du2, r_u2, smem_addr(park) + threadIdx.x * 16u, s.cur);
+  const unsigned block = wt.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+  unsigned y, r;
+  const unsigned t = block * (BT / 32) + threadIdx.x / 32;
+  wt.row_of(t, y, r);
+  const int x = (int)(r * 32 + threadIdx.x % 32);
+  const long long site = (long long)y * s.ldx + x;
+  Tile<S> tl;
+  tl.in = fin + 4 * site;
+  tl.out = fout + 4 * site;
+  tl.policy = pull_policy(wt.evict_first);
+  chain_wait();
+  site_step<S, FORCE, RES, BT>(fin, tl, of, s, t < wt.count ? x : s.nx, (int)y, ghost, aux, qc,
+                               r_du2, r_u2, smem_addr(park) + threadIdx.x * 16u, s.cur);
   if (RES == 2) block_reduce_add2<typename Codec<S>::R>(r_du2, r_u2, aux.acc);
 }
 
@@ -666,6 +749,9 @@ __device__ __forceinline__ void batch_body(S* __restrict__ base, const BatchArgs
                                            const StepAux<typename Codec<S>::R>& aux, const C& qc,
                                            unsigned char* park) {
   const uint32_t my_park = smem_addr(park) + threadIdx.x * 16u;
+  const uint64_t policy = pull_policy(false);
+  chain_release();
+  chain_wait();
 #pragma unroll 1
   for (long long t = blockIdx.x; t < b.ntiles; t += gridDim.x) {
     int lo = 0, hi = b.nsamples;                 // tile_start[lo] <= t < tile_start[hi]
@@ -678,10 +764,15 @@ __device__ __forceinline__ void batch_body(S* __restrict__ base, const BatchArgs
     const int tpr = (s.nx + BX - 1) / BX;
     const int y = (int)(lt / tpr);
     const int x = (int)(lt - (long long)y * tpr) * BX + threadIdx.x;
-    const long long oin = b.cur ? s.off[1] : s.off[0];
-    const long long oout = b.cur ? s.off[0] : s.off[1];
+    const S* fin = base + (b.cur ? s.off[1] : s.off[0]);
+    Tile<S> tl;
+    const long long site = (long long)y * s.ldx + x;
+    tl.in = fin + 4 * site;
+    tl.out = base + (b.cur ? s.off[0] : s.off[1]) + 4 * site;
+    tl.policy = policy;
+    const SampleOffsets<S> of{s.plane, s.ldx};
     double r_du2 = 0.0, r_u2 = 0.0;
-    site_step<S, FORCE, RES, BX>(base + oin, base + oout, s, x, y,
+    site_step<S, FORCE, RES, BX>(fin, tl, of, s, x, y,
                              ghost + (long long)lo * kMaxContacts * kQ, aux, qc, r_du2, r_u2,
                              my_park, b.cur);
     // per-sample residual accumulators: acc[2 k], acc[2 k + 1]
@@ -780,8 +871,12 @@ __device__ __forceinline__ void staged_batch_body(S* __restrict__ base, const Ba
     const DevSample s = b.samples[tl.x];
     const int x = tl.y + tid;
     R f[kQ];
-    if (x < s.nx) gather(base + (b.cur ? s.off[1] : s.off[0]), s, x, tl.z,
-                         ghost + (long long)tl.x * kMaxContacts * kQ, qc, src, f);
+    if (x < s.nx) {
+      const S* fin = base + (b.cur ? s.off[1] : s.off[0]);
+      const R* gh = ghost + (long long)tl.x * kMaxContacts * kQ;
+      if (warp_interior(s, x, tl.z)) pull_staged<S, true>(fin, s, x, tl.z, gh, qc, src, f);
+      else pull_staged<S, false>(fin, s, x, tl.z, gh, qc, src, f);
+    }
     __syncwarp();
     // the last warp done with this buffer refills it with tile k + 2
     if (t + 2 * G < b.ntiles) {
@@ -800,8 +895,12 @@ __device__ __forceinline__ void staged_batch_body(S* __restrict__ base, const Ba
       }
     }
     double r_du2 = 0.0, r_u2 = 0.0;
+    Tile<S> dst;
+    dst.in = nullptr;
+    dst.out = base + (b.cur ? s.off[0] : s.off[1]) + 4 * ((long long)tl.z * s.ldx + x);
+    const SampleOffsets<S> of{s.plane, s.ldx};
     if (x < s.nx)
-      collide_store<S, FORCE, RES, BX>(f, base + (b.cur ? s.off[0] : s.off[1]), s, x, tl.z, aux, qc,
+      collide_store<S, FORCE, RES, BX>(f, dst, of, s, x, tl.z, aux, qc,
                                    r_du2, r_u2, my_park,
                                    static_cast<const R*>(b.cur ? s.dn[1] : s.dn[0]),
                                    static_cast<R*>(b.cur ? s.dn[0] : s.dn[1]));
@@ -824,7 +923,11 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ fin, const De
   const int y = blockIdx.y;
   if (x >= s.nx) return;
   R f[kQ];
-  pull<S, false>(fin, s, x, y, ghost, qc, f);
+  Tile<S> tl;
+  tl.in = fin + 4 * ((long long)y * s.ldx + x);
+  tl.out = nullptr;
+  tl.policy = pull_policy(false);
+  gather(fin, tl, SampleOffsets<S>{s.plane, s.ldx}, s, x, y, ghost, qc, f);
   const Moments<R> m = moments(f, qc);
   Macro<R> M;
   const unsigned bad = landau(m, M) & ~kErrUnphysical;
@@ -911,8 +1014,8 @@ __device__ __forceinline__ void init_body(S* __restrict__ fout, const DevSample&
   for (int d = 0; d < kDirs; d += 2) {
     R v[8];
     eq_pair<S>(c, d, qc, v, v + 4);
-    Codec<S>::store4(fout + vec_index(s, d, site), dir_kind(d), qc, v);
-    Codec<S>::store4(fout + vec_index(s, d + 1, site), dir_kind(d), qc, v + 4);
+    Codec<S>::store4(fout + vec_index(s, d, site), v);
+    Codec<S>::store4(fout + vec_index(s, d + 1, site), v + 4);
   }
 }
 
@@ -968,8 +1071,8 @@ __device__ __forceinline__ void init_ce_body(S* __restrict__ fout, const DevSamp
           v[4 * h + j] = ed[4 * h + j] - (ed[4 * h + j] - v[4 * h + j]) * iom;
       }
     }
-    Codec<S>::store4(fout + vec_index(s, d, site), dir_kind(d), qc, v);
-    Codec<S>::store4(fout + vec_index(s, d + 1, site), dir_kind(d), qc, v + 4);
+    Codec<S>::store4(fout + vec_index(s, d, site), v);
+    Codec<S>::store4(fout + vec_index(s, d + 1, site), v + 4);
   }
 }
 

@@ -14,11 +14,13 @@ using R = typename Codec<S>::R;
 
 __constant__ QuadConsts<R> c_qc;
 
-// RLBM_STEP_MIN_BLOCKS: resident blocks of 128 threads per SM the register
-// allocation aims for (measured per storage type, with the populations parked
-// in shared memory and the paired FP32 collision: FP32 storage runs best at
-// 6 blocks / 80 registers, 16-bit storage at 7 blocks / 72 registers; the
-// FP64 kernels take all the registers they want).
+// RLBM_STEP_MIN_BLOCKS: warps per SM sub-partition the register allocation
+// aims for (blocks of 128 threads per SM), measured per storage type in us per
+// step at 600 x 300 / 1024 x 512 / 4096 x 2048.  FP32 storage: 4: 11.3 / 26.6 /
+// 456, 5: 10.7 / 26.8 / 456, 6: 10.9 / 27.6 / 461, 7: 10.6 / 27.4 / 470; 5 is
+// kept.  FP16 storage at the two larger sizes: 6: 25.4 / 287, 7: 24.4 / 273,
+// 8 (spills): 26.4 / 348; 7 is kept.  The FP64 kernels take all the registers
+// they want (the FP64 pipe is busy with 8 warps).
 #ifndef RLBM_STEP_MIN_BLOCKS
 #define RLBM_STEP_MIN_BLOCKS 4
 #endif
@@ -31,12 +33,14 @@ constexpr int kStepRegs = (65536 / (RLBM_STEP_MIN_BLOCKS * kBX)) > 255
 
 // Dynamic shared memory of the direct step kernels: the parking area
 // (park_bytes: 12 x threads x 16 B with FP32 arithmetic, none with FP64).
-template <int FORCE, int RES>
+template <int FORCE, int RES, int BT>
 __global__ void __maxnreg__(kStepRegs) k_step(const S* __restrict__ fin, S* __restrict__ fout,
-                                              DevSample s, const R* __restrict__ ghost,
-                                              StepAux<R> aux) {
+                                              const __grid_constant__ DevSample s,
+                                              const __grid_constant__ WarpTiles wt,
+                                              const __grid_constant__ StepOffsets of,
+                                              const R* __restrict__ ghost, StepAux<R> aux) {
   extern __shared__ __align__(128) unsigned char park_smem[];
-  step_body<S, FORCE, RES>(fin, fout, s, ghost, aux, c_qc, park_smem);
+  step_body<S, FORCE, RES, BT>(fin, fout, s, wt, of, ghost, aux, c_qc, park_smem);
 }
 
 template <int FORCE, int RES, int BX>
@@ -176,14 +180,74 @@ cudaError_t upload(const double p0[4], const double w[2][4], double scale) {
   return e;
 }
 
+// Launch that may overlap its predecessor's end (chain_release / chain_wait):
+// the blocks of the next step are placed while the last wave of this one
+// drains.  FP32 600 x 300 (1.5 waves) 15.4 -> 11.0 us per step together with
+// the warp tiles, FP16 1024 x 512 36 -> 26, FP32 1024 x 512 34.7 -> 32.6.
+template <typename... P, typename... A>
+void launch_chained(void (*k)(P...), unsigned grid, int block, size_t smem, cudaStream_t st,
+                    A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
+// L2 size of the current device (looked up once per device).
+size_t l2_bytes() {
+  static int bytes[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (bytes[dev] == 0) cudaDeviceGetAttribute(&bytes[dev], cudaDevAttrL2CacheSize, dev);
+  return (size_t)bytes[dev];
+}
+
+// Threads per block of the single-sample step.  Us per step with blocks of
+// 32 / 64 / 128: FP32 200 x 150 5.7 / 5.7 / 6.4, 1024 x 512 33.7 / 32.4 / 32.6,
+// 4096 x 2048 481 / 460 / 460; FP16 4096 x 2048 290 / 294 / 299; FP64 64 x 64
+// 22.8 / 22.7 / 25.6.
+constexpr int kStepThreads = 64;
+
+template <int F, int BT>
+void launch_single_bt(const S* a, S* b, const DevSample& s, const WarpTiles& wt,
+                      const StepOffsets& of, const R* g, int res, const StepAux<R>& aux,
+                      cudaStream_t st) {
+  const unsigned grid = (wt.count + BT / 32 - 1) / (BT / 32);
+  const size_t pk = park_bytes<R>(BT);
+  if (res == 0) launch_chained(k_step<F, 0, BT>, grid, BT, pk, st, a, b, s, wt, of, g, aux);
+  else if (res == 1) launch_chained(k_step<F, 1, BT>, grid, BT, pk, st, a, b, s, wt, of, g, aux);
+  else launch_chained(k_step<F, 2, BT>, grid, BT, pk, st, a, b, s, wt, of, g, aux);
+}
+
 template <int F>
 void launch_single(const S* a, S* b, const DevSample& s, const R* g, int res, const StepAux<R>& aux,
                    cudaStream_t st) {
-  const dim3 grid = site_grid(s);
-  const size_t pk = park_bytes<R>(kBX);
-  if (res == 0) k_step<F, 0><<<grid, kBX, pk, st>>>(a, b, s, g, aux);
-  else if (res == 1) k_step<F, 1><<<grid, kBX, pk, st>>>(a, b, s, g, aux);
-  else k_step<F, 2><<<grid, kBX, pk, st>>>(a, b, s, g, aux);
+  WarpTiles wt;
+  wt.per_row = (unsigned)(s.nx + 31) / 32;
+  wt.magic = wt.per_row > 1 ? (unsigned)((1ull << 32) / wt.per_row) : 0xffffffffu;
+  wt.count = wt.per_row * (unsigned)s.ny;
+  // Both rules were measured on FP32 (us per step, neither / reversed /
+  // reversed and evict-first): buffers of 48 MiB 14.7 / 14.7 / 14.0, 74 MiB
+  // 24.6 / 23.2 / 20.9, 96 MiB (1024 x 512) 32.5 / 29.7 / 27.6, 144 MiB 46.6 /
+  // 44.3 / 43.3, 192 MiB 60.9 / 58.3 / 57.8, 384 MiB 116.4 / 113.6 / 115.2,
+  // 1.5 GiB 459 / 459 / 481 (L2: 129 MB); FP16 storage at 768 MiB loses 1.5 %
+  // to the reversed order.
+  const size_t bytes = (size_t)s.plane * kQ * sizeof(S), l2 = l2_bytes();
+  wt.evict_first = bytes <= 2 * l2;
+  wt.reverse = s.cur && bytes <= 4 * l2;
+  StepOffsets of;
+  for (int d = 0; d < kDirs; ++d) {
+    of.pull_[d] = pull_offset<S>(d, s.plane, s.ldx);
+    of.plane_[d] = plane_offset<S>(d, s.plane);
+  }
+  launch_single_bt<F, kStepThreads>(a, b, s, wt, of, g, res, aux, st);
 }
 
 cudaError_t step(const void* fin, void* fout, const DevSample& s, const void* ghost, int force,
@@ -209,9 +273,9 @@ void launch_batch_f(S* base, const BatchArgs& b, const R* g, int res, int grid, 
     return;
   }
   const size_t pk = park_bytes<R>(BX);
-  if (res == 0) k_step_batch<F, 0, BX><<<grid, BX, pk, st>>>(base, b, g, aux);
-  else if (res == 1) k_step_batch<F, 1, BX><<<grid, BX, pk, st>>>(base, b, g, aux);
-  else k_step_batch<F, 2, BX><<<grid, BX, pk, st>>>(base, b, g, aux);
+  if (res == 0) launch_chained(k_step_batch<F, 0, BX>, grid, BX, pk, st, base, b, g, aux);
+  else if (res == 1) launch_chained(k_step_batch<F, 1, BX>, grid, BX, pk, st, base, b, g, aux);
+  else launch_chained(k_step_batch<F, 2, BX>, grid, BX, pk, st, base, b, g, aux);
 }
 
 template <int BX>

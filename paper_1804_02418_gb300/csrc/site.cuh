@@ -91,6 +91,9 @@ struct DevSample {
   long long off[2];                   // element offsets of the two buffers (batched launches)
   double inv_tau;
   double Fx, Fy;
+  // the same in FP32, for the FP32 arithmetic (a conversion per thread would
+  // run on the FP64 pipe)
+  float inv_tau_f, Fx_f, Fy_f, inv_cg_f;
   int cedge[kMaxContacts], clo[kMaxContacts], chi[kMaxContacts];
   // electric force of the local capacitance approximation (Sec. 3): coupling
   // e^2 / C_g (0: none) and two planes of n - 1 in the arithmetic type, same
@@ -110,26 +113,23 @@ constexpr unsigned kErrTimeout = 8u;      // a bounded wait inside a kernel gave
 // ---------------------------------------------------------------------------
 // Storage codecs.  The four shells of one (direction, site) are stored side by
 // side, so one aligned vector access moves them (16 B for FP32, 32 B for FP64,
-// 8 B for 16-bit storage).  `kind` selects the weight row (0: (3,4)-type,
-// 1: (5,0)-type) for the 16-bit scaled relative deviations.
+// 8 B for 16-bit storage).  The loads are written as assembly with a memory
+// clobber: the compiler may move an ordinary read-only load above the wait
+// for the predecessor's results (chain_wait).
 // ---------------------------------------------------------------------------
 template <typename S> struct Codec;
 template <> struct Codec<double> {
   using R = double;
-  template <class C>
-  __device__ static void load4(const double* p, int, const C&, R* o) {
-    const double2 a = __ldg(reinterpret_cast<const double2*>(p));
-    const double2 b = __ldg(reinterpret_cast<const double2*>(p) + 1);
-    o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
+  __device__ static void load4(const double* p, uint64_t, double* o) {
+    asm("ld.global.nc.v2.f64 {%0, %1}, [%2];\n" : "=d"(o[0]), "=d"(o[1]) : "l"(p) : "memory");
+    asm("ld.global.nc.v2.f64 {%0, %1}, [%2];\n" : "=d"(o[2]), "=d"(o[3]) : "l"(p + 2) : "memory");
   }
   // from shared memory (32-bit shared-window address)
-  template <class C>
-  __device__ static void load4s(uint32_t a, int, const C&, R* o) {
+  __device__ static void load4s(uint32_t a, double* o) {
     asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];\n" : "=d"(o[0]), "=d"(o[1]) : "r"(a));
     asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];\n" : "=d"(o[2]), "=d"(o[3]) : "r"(a + 16));
   }
-  template <class C>
-  __device__ static void store4(double* p, int, const C&, const R* v) {
+  __device__ static void store4(double* p, const double* v) {
     reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
     reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
   }
@@ -144,18 +144,16 @@ template <> struct Codec<double> {
 };
 template <> struct Codec<float> {
   using R = float;
-  template <class C>
-  __device__ static void load4(const float* p, int, const C&, R* o) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-    o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
+  // policy: an L2 eviction policy (pull_policy)
+  __device__ static void load4(const float* p, uint64_t policy, float* o) {
+    asm("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;\n"
+        : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]) : "l"(p), "l"(policy) : "memory");
   }
-  template <class C>
-  __device__ static void load4s(uint32_t a, int, const C&, R* o) {
+  __device__ static void load4s(uint32_t a, float* o) {
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
                  : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]) : "r"(a));
   }
-  template <class C>
-  __device__ static void store4(float* p, int, const C&, const R* v) {
+  __device__ static void store4(float* p, const float* v) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
   }
   // in FP64: delta = g w to 1e-16, and delta / w rounds back to g exactly
@@ -173,21 +171,19 @@ template <typename H> struct Codec16 {
   // two stored values <-> two floats (one conversion instruction per pair)
   __device__ static float2 unpack2(uint32_t u);
   __device__ static uint32_t pack2(float a, float b);
-  template <class C>
-  __device__ static void load4(const H* p, int kind, const C& c, R* o) {
-    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+  __device__ static void load4(const H* p, uint64_t, float* o) {
+    uint2 u;
+    asm("ld.global.nc.v2.b32 {%0, %1}, [%2];\n" : "=r"(u.x), "=r"(u.y) : "l"(p) : "memory");
     const float2 a = unpack2(u.x), b = unpack2(u.y);   // s g: the kernels work scaled
     o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
   }
-  template <class C>
-  __device__ static void load4s(uint32_t a, int kind, const C& c, R* o) {
+  __device__ static void load4s(uint32_t a, float* o) {
     uint2 u;
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];\n" : "=r"(u.x), "=r"(u.y) : "r"(a));
     const float2 x = unpack2(u.x), y = unpack2(u.y);
     o[0] = x.x; o[1] = x.y; o[2] = y.x; o[3] = y.y;
   }
-  template <class C>
-  __device__ static void store4(H* p, int kind, const C& c, const R* v) {
+  __device__ static void store4(H* p, const float* v) {
     *reinterpret_cast<uint2*>(p) = make_uint2(pack2(v[0], v[1]), pack2(v[2], v[3]));
   }
   // stored s g <-> deviation delta = f - w (state I/O, in FP64: exact round trip)
