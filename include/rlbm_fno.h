@@ -105,6 +105,50 @@ int rlbm_fno_colsum(const float* X, float* out, long long rows, int cols, void* 
 int rlbm_fno_adam(float* P, const float* G, float* M, float* V, void* P16, long long n,
                   float lr, float beta1, float beta2, float eps, int t, void* stream);
 
+/* The whole operator in fused kernels, for the shapes rlbm_fno_fused_supported
+ * names: width C = 32, projection width Cq = 128, m1 = m2 = 16 kept modes,
+ * cout = 4 outputs, 1 to 16 inputs, canvas N a multiple of 8 from 32 to 512.
+ * All pointers are device pointers, 16-byte aligned, dense; rows = batch N N.
+ *   weights   P [cin][C], W [layers][C][C], Q1 [C][Cq], Q2 [Cq][cout] bf16;
+ *             bp, b, bq1, bq2 and R [layers][2 m1][m2][C][C][2] f32
+ *   matrices  F1 [2 m2][N], D [4 m1][2 N], Dinv [2 N][4 m1], G [N][2 m2] bf16
+ *             (truncated real DFTs) and their transposes F1T, DT, DinvT, GT
+ *   kept      x [rows][cin] bf16, h[0 .. layers] [rows][C] bf16, z[l] [rows][C]
+ *             f32, S2[l] [batch][4 m1][m2 C] f32, y [rows][cout] f32: written by
+ *             rlbm_fno_forward, read by rlbm_fno_backward
+ *   scratch   S1, Wm, dWm, dS1 [batch N][2 m2][C] bf16, dz [rows][C] bf16,
+ *             dU as S2[l]
+ *   gradients gP .. gbq2 f32, shaped as the weights; added to.
+ * The backward pass reads dy [rows][cout] f32.  The results are those of the
+ * same operator as a sequence of rlbm_gemm_bf16_tc calls: bit for bit, but for
+ * the order of the FP32 sums of the weight and bias gradients. */
+#define RLBM_FNO_MAX_LAYERS 16
+typedef struct {
+  int N, batch, layers, cin;
+  const void *P, *W, *Q1, *Q2;
+  const float *bp, *b, *R, *bq1, *bq2;
+  const void *F1, *D, *Dinv, *G, *F1T, *DT, *DinvT, *GT;
+  void *x, *S1, *Wm;
+  void* h[RLBM_FNO_MAX_LAYERS + 1];
+  float* z[RLBM_FNO_MAX_LAYERS];
+  float* S2[RLBM_FNO_MAX_LAYERS];
+  float* y;
+  const float* dy;
+  void *dz, *dWm, *dS1;
+  float* dU;
+  float *gP, *gW, *gQ1, *gQ2, *gbp, *gb, *gR, *gbq1, *gbq2;
+} rlbm_fno_net;
+
+/* 1 if the fused kernels take this shape, else 0 (host only). */
+int rlbm_fno_fused_supported(int N, int C, int Cq, int m1, int m2, int cin, int cout, int layers);
+
+/* y of the inputs x_in [rows][cin] bf16 (16-byte aligned), which are copied to
+ * net->x (x_in may be net->x). */
+int rlbm_fno_forward(const rlbm_fno_net* net, const void* x_in, void* stream);
+
+/* Gradients of the last rlbm_fno_forward for net->dy, added to net->g*. */
+int rlbm_fno_backward(const rlbm_fno_net* net, void* stream);
+
 /* Bilinear resampling of nch f32 planes: src [nch][sh][sw] (row-major) onto
  * dst [nch][dh][dw]; destination pixel (i, j) samples source point
  * ((i + 0.5) * sh / dh - 0.5, (j + 0.5) * sw / dw - 0.5) clamped to the edges. */

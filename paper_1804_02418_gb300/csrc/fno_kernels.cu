@@ -754,6 +754,8 @@ __global__ void k_resample(const float* __restrict__ src, int nch, int sh, int s
   dst[t] = v;
 }
 
+#include "fno_fused.cuh"
+
 inline int grid1(long long n, int bs) { return (int)((n + bs - 1) / bs); }
 
 int status() { return cudaGetLastError() == cudaSuccess ? RLBM_OK : RLBM_ECUDA; }
@@ -762,6 +764,53 @@ int status() { return cudaGetLastError() == cudaSuccess ? RLBM_OK : RLBM_ECUDA; 
 }  // namespace rlbm
 
 using namespace rlbm;
+
+namespace {
+
+struct FusedLaunch {
+  cudaStream_t st;
+  int sms;
+  cudaError_t e;
+  // CTAs that fit an SM by shared memory and tensor memory
+  int slots(size_t smem, int cols) const {
+    const int by_smem = (int)(228 * 1024 / (smem + 2048)), by_tmem = 512 / cols;
+    const int n = by_smem < by_tmem ? by_smem : by_tmem;
+    return sms * (n > 0 ? n : 1);
+  }
+  template <typename P>
+  void run(void (*k)(P), const P& p, dim3 grid, int threads, size_t smem) {
+    if (e != cudaSuccess) return;
+    if (smem > 48 * 1024)
+      e = cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return;
+    k<<<grid, threads, smem, st>>>(p);
+    e = cudaGetLastError();
+  }
+  template <typename P>
+  void rows(void (*k)(P), const P& p, int items, size_t smem, int cols) {
+    const int s = slots(smem, cols);
+    run(k, p, dim3((unsigned)(items < s ? items : s)), 128, smem);
+  }
+};
+
+int fused_start(const rlbm_fno_net* n, void* stream, FusedLaunch& f) {
+  if (!n || n->batch < 1 || n->batch > 65535 ||
+      !rlbm_fno_fused_supported(n->N, fused::kC, fused::kQ, 16, 16, n->cin, 4, n->layers) ||
+      (long long)n->batch * n->N > 0x7fffffffLL)
+    return RLBM_EINVAL;
+  f.st = static_cast<cudaStream_t>(stream);
+  f.e = cudaSuccess;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return RLBM_ECUDA;
+  return RLBM_OK;
+}
+
+const __nv_bfloat16* b16(const void* p) { return static_cast<const __nv_bfloat16*>(p); }
+__nv_bfloat16* b16(void* p) { return static_cast<__nv_bfloat16*>(p); }
+
+}  // namespace
 
 extern "C" {
 
@@ -934,6 +983,88 @@ int rlbm_resample_bilinear(const float* src, int nch, int sh, int sw, float* dst
   k_resample<<<grid1(n, 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(src, nch, sh, sw, dst,
                                                                           dh, dw);
   return status();
+}
+
+int rlbm_fno_fused_supported(int N, int C, int Cq, int m1, int m2, int cin, int cout, int layers) {
+  return N >= 32 && N <= 512 && N % 8 == 0 && C == fused::kC && Cq == fused::kQ && m1 == 16 &&
+         m2 == fused::kKy && cin >= 1 && cin <= 16 && cout == 4 && layers >= 1 &&
+         layers <= RLBM_FNO_MAX_LAYERS;
+}
+
+int rlbm_fno_forward(const rlbm_fno_net* n, const void* x, void* stream) {
+  FusedLaunch f;
+  const int r = fused_start(n, stream, f);
+  if (r != RLBM_OK) return r;
+  if (!x || (reinterpret_cast<uintptr_t>(x) & 15)) return RLBM_EINVAL;
+  const int C = fused::kC, items = n->batch * n->N, T = (n->N + 127) / 128, L = n->layers;
+  fused::FwdRows in{};
+  in.in = b16(x); in.F1 = b16(n->F1); in.W = b16(n->P); in.bias = n->bp;
+  in.h = b16(n->h[0]); in.S1 = b16(n->S1); in.xcopy = b16(n->x);
+  in.N = n->N; in.items = items; in.cin = n->cin;
+  f.rows(fused::k_fwd_rows<0>, in, items, fused::fwd_smem<0>(T), 128);
+  for (int l = 0; l < L; ++l) {
+    fused::Spectral s{};
+    s.A1 = b16(n->D); s.X = b16(n->S1); s.A2 = b16(n->Dinv);
+    s.R = n->R + (long long)l * (fused::kModes / 2) * fused::kKy * C * C * 2;
+    s.S2 = n->S2[l]; s.out = b16(n->Wm); s.N = n->N;
+    f.run(fused::k_spectral<false>, s, dim3(fused::kKy, (unsigned)n->batch), 256, fused::kSpectralSmem);
+    fused::FwdRows w{};
+    w.in = b16(n->h[l]); w.Wm = b16(n->Wm); w.G = b16(n->G); w.F1 = b16(n->F1);
+    w.W = b16(n->W) + (long long)l * C * C; w.bias = n->b + (long long)l * C;
+    w.z = n->z[l]; w.h = b16(n->h[l + 1]); w.S1 = b16(n->S1);
+    w.N = n->N; w.items = items;
+    if (l < L - 1) f.rows(fused::k_fwd_rows<1>, w, items, fused::fwd_smem<1>(T), 128);
+    else f.rows(fused::k_fwd_rows<2>, w, items, fused::fwd_smem<2>(T), 128);
+  }
+  fused::Head h{};
+  h.h = b16(n->h[L]); h.Q1 = b16(n->Q1); h.Q2 = b16(n->Q2); h.bq1 = n->bq1; h.bq2 = n->bq2;
+  h.y = n->y; h.rows = (long long)items * n->N;
+  const long long tiles = (h.rows + 127) / 128;
+  f.rows(fused::k_head_fwd, h, (int)(tiles < 0x7fffffff ? tiles : 0x7fffffff), fused::kHeadFwdSmem, 128);
+  return f.e == cudaSuccess ? RLBM_OK : RLBM_ECUDA;
+}
+
+int rlbm_fno_backward(const rlbm_fno_net* n, void* stream) {
+  FusedLaunch f;
+  const int r = fused_start(n, stream, f);
+  if (r != RLBM_OK) return r;
+  const int C = fused::kC, items = n->batch * n->N, T = (n->N + 127) / 128, L = n->layers;
+  const long long nr = (long long)(fused::kModes / 2) * fused::kKy * C * C * 2;
+  fused::Head h{};
+  h.h = b16(n->h[L]); h.Q1 = b16(n->Q1); h.Q2 = b16(n->Q2); h.bq1 = n->bq1; h.bq2 = n->bq2;
+  h.dy = n->dy; h.dz = b16(n->dz);
+  h.gQ1 = n->gQ1; h.gb1 = n->gbq1; h.gQ2 = n->gQ2; h.gb2 = n->gbq2;
+  h.gb = n->gb + (long long)(L - 1) * C;
+  h.rows = (long long)items * n->N;
+  const long long tiles = (h.rows + 127) / 128;
+  f.rows(fused::k_head_bwd, h, (int)(tiles < 0x7fffffff ? tiles : 0x7fffffff), fused::kHeadBwdSmem, 256);
+  for (int l = L - 1; l >= -1; --l) {
+    fused::BwdRows w{};
+    w.dz = b16(n->dz); w.N = n->N; w.items = items; w.cin = n->cin;
+    w.dWm = b16(n->dWm); w.GT = b16(n->GT); w.F1T = b16(n->F1T); w.dS1 = b16(n->dS1);
+    if (l < L - 1) w.W = b16(n->W) + (long long)(l + 1) * C * C;
+    if (l >= 0) {
+      w.left = b16(n->h[l]);
+      w.z = n->z[l];
+      w.gW = n->gW + (long long)l * C * C;
+      w.gb = n->gb + (long long)l * C;
+      if (l == L - 1) f.rows(fused::k_bwd_rows<0>, w, items, fused::bwd_smem<0>(T), 128);
+      else f.rows(fused::k_bwd_rows<1>, w, items, fused::bwd_smem<1>(T), 128);
+      fused::Spectral s{};
+      s.A1 = b16(n->DinvT); s.X = b16(n->dWm); s.A2 = b16(n->DT);
+      s.R = n->R + l * nr; s.S2 = n->dU; s.out = b16(n->dS1); s.N = n->N;
+      f.run(fused::k_spectral<true>, s, dim3(fused::kKy, (unsigned)n->batch), 256, fused::kSpectralSmem);
+      if (f.e == cudaSuccess) {
+        fused::k_mix_grad<<<(fused::kModes / 2) * fused::kKy, 256, 0, f.st>>>(
+            n->S2[l], n->dU, reinterpret_cast<float2*>(n->gR + l * nr), n->batch);
+        f.e = cudaGetLastError();
+      }
+    } else {
+      w.left = b16(n->x); w.gW = n->gP; w.gb = n->gbp;
+      f.rows(fused::k_bwd_rows<2>, w, items, fused::bwd_smem<2>(T), 128);
+    }
+  }
+  return f.e == cudaSuccess ? RLBM_OK : RLBM_ECUDA;
 }
 
 }  // extern "C"

@@ -53,6 +53,25 @@ _FNO_EXPORTS = {
     "rlbm_resample_bilinear": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                               ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_void_p]),
 }
+MAX_LAYERS = 16
+
+
+class _Net(ctypes.Structure):
+    """rlbm_fno_net of include/rlbm_fno.h."""
+    _fields_ = ([(k, ctypes.c_int) for k in ("N", "batch", "layers", "cin")]
+                + [(k, ctypes.c_void_p) for k in (
+                    "P", "W", "Q1", "Q2", "bp", "b", "R", "bq1", "bq2", "F1", "D", "Dinv", "G",
+                    "F1T", "DT", "DinvT", "GT", "x", "S1", "Wm")]
+                + [("h", ctypes.c_void_p * (MAX_LAYERS + 1)), ("z", ctypes.c_void_p * MAX_LAYERS),
+                   ("S2", ctypes.c_void_p * MAX_LAYERS)]
+                + [(k, ctypes.c_void_p) for k in (
+                    "y", "dy", "dz", "dWm", "dS1", "dU", "gP", "gW", "gQ1", "gQ2", "gbp", "gb", "gR",
+                    "gbq1", "gbq2")])
+
+
+_FNO_EXPORTS["rlbm_fno_fused_supported"] = (ctypes.c_int, [ctypes.c_int] * 8)
+_FNO_EXPORTS["rlbm_fno_forward"] = (ctypes.c_int, [ctypes.POINTER(_Net), ctypes.c_void_p, ctypes.c_void_p])
+_FNO_EXPORTS["rlbm_fno_backward"] = (ctypes.c_int, [ctypes.POINTER(_Net), ctypes.c_void_p])
 _FNO_EXPORTS["rlbm_gemm_bf16_tc"] = _FNO_EXPORTS["rlbm_gemm_bf16"]
 _FNO_EXPORTS["rlbm_gemm_f32"] = _FNO_EXPORTS["rlbm_gemm_bf16"]
 rlbm.EXPORTS.update(_FNO_EXPORTS)
@@ -112,6 +131,11 @@ class FNOConfig:
     cout: int = 4
 
 
+def _fused_shape(lib, cfg) -> bool:
+    return bool(lib.rlbm_fno_fused_supported(cfg.N, cfg.C, cfg.Cq, cfg.m1, cfg.m2, cfg.cin, cfg.cout,
+                                             cfg.L))
+
+
 class FNO:
     """Parameters live in one flat FP32 vector (Adam state alongside) with a
     BF16 shadow used by the GEMMs.
@@ -120,7 +144,10 @@ class FNO:
     the tensor cores (gemm_impl "tc" or "mma"), FP32 accumulation and FP32
     spectral mixing.  act = "f32": everything in FP32 on the FP32 units
     (rlbm_gemm_f32), the same sequence of kernels; the "16" buffers are then
-    the FP32 buffers themselves.  Inputs to forward() are of the act type."""
+    the FP32 buffers themselves.  Inputs to forward() are of the act type.
+    With act = "bf16" and gemm_impl = "tc" the default shape (C 32, Cq 128,
+    m1 = m2 = 16, N a multiple of 8 from 32 to 512) runs in the fused kernels
+    of rlbm_fno_forward / rlbm_fno_backward, which give the same results."""
 
     def __init__(self, cfg: FNOConfig, batch: int, seed: int = 0, device="cuda",
                  gemm_impl: str = "tc", act: str = "bf16"):
@@ -168,6 +195,26 @@ class FNO:
         self.rows = rows
         e16 = lambda *s: torch.empty(*s, **b16)
         e32 = lambda *s: torch.empty(*s, **f32)
+        self.loss_buf = torch.zeros(4, **f32)
+        # the default shape runs in fused kernels, which keep less per site and
+        # move it less often; every other shape as a sequence of GEMMs
+        self.fused = act == "bf16" and gemm_impl == "tc" and _fused_shape(self.lib, cfg)
+        if self.fused:
+            self.F1T, self.DT, self.DinvT, self.GT = (
+                a.t().contiguous() for a in (self.F1, self.D, self.Dinv, self.G))
+            self.x16 = e16(rows, cin)
+            self.h16 = [e16(rows, C) for _ in range(L + 1)]
+            self.z = [e32(rows, C) for _ in range(L)]
+            self.S1 = e16(batch * N, 2 * m2, C)
+            self.S2 = [e32(batch, 2 * KX, m2 * C) for _ in range(L)]
+            self.Wm16 = e16(batch * N, 2 * m2, C)
+            self.y = e32(rows, cfg.cout)
+            self.dy = e32(rows, cfg.cout)
+            self.dz16 = e16(rows, C)
+            self.dWm16 = e16(batch * N, 2 * m2, C)
+            self.dS116 = e16(batch * N, 2 * m2, C)
+            self.dU = e32(batch, 2 * KX, m2 * C)
+            return
         self.x16 = e16(rows, cin)
         self.h16 = [e16(rows, C) for _ in range(L + 1)]
         self.z = [e32(rows, C) for _ in range(L)]
@@ -194,7 +241,6 @@ class FNO:
         self.dS216 = self.dS2 if f32mode else e16(batch, 2 * KX, m2 * C)
         self.dS116 = e16(batch * N, 2 * m2, C)
         self.dh16 = self.dh if f32mode else e16(rows, C)
-        self.loss_buf = torch.zeros(4, **f32)
 
     # -- parameters ---------------------------------------------------------
     def init_params(self, rng):
@@ -259,6 +305,27 @@ class FNO:
             return
         _ok(self.lib.rlbm_fno_to_bf16(_p(x), _p(y), x.numel(), self._stream()), "to_bf16")
 
+    def _net(self):
+        """The pointers of this object's buffers, as they are now."""
+        c = self.cfg
+        n = _Net(c.N, self.B, c.L, c.cin)
+        t16, t32, g = self.theta16.data_ptr(), self.theta.data_ptr(), self.grad.data_ptr()
+        for k in ("P", "W", "Q1", "Q2"):
+            setattr(n, k, t16 + 2 * self.offsets[k][0])
+        for k in ("bp", "b", "R", "bq1", "bq2"):
+            setattr(n, k, t32 + 4 * self.offsets[k][0])
+        for k, (off, _) in self.offsets.items():
+            setattr(n, "g" + k, g + 4 * off)
+        for k in ("F1", "D", "Dinv", "G", "F1T", "DT", "DinvT", "GT", "S1", "y", "dy", "dU"):
+            setattr(n, k, getattr(self, k).data_ptr())
+        n.x, n.Wm, n.dz = self.x16.data_ptr(), self.Wm16.data_ptr(), self.dz16.data_ptr()
+        n.dWm, n.dS1 = self.dWm16.data_ptr(), self.dS116.data_ptr()
+        for l in range(c.L):
+            n.h[l], n.z[l], n.S2[l] = (self.h16[l].data_ptr(), self.z[l].data_ptr(),
+                                       self.S2[l].data_ptr())
+        n.h[c.L] = self.h16[c.L].data_ptr()
+        return n
+
     # -- forward ------------------------------------------------------------
     def forward(self, x16):
         """x16: [B N N, cin] of the act type (already on the device).  Returns
@@ -267,6 +334,15 @@ class FNO:
         N, C, Cq, L, m2, KX = c.N, c.C, c.Cq, c.L, c.m2, self.KX
         B, rows = self.B, self.rows
         t16 = self.theta16
+        if self.fused:
+            if not (x16.is_cuda and x16.dtype == self.x16.dtype and x16.shape == self.x16.shape
+                    and x16.device == self.x16.device and x16.is_contiguous()
+                    and x16.data_ptr() % 16 == 0):
+                self.x16.copy_(x16)
+                x16 = self.x16
+            _ok(self.lib.rlbm_fno_forward(ctypes.byref(self._net()), ctypes.c_void_p(x16.data_ptr()),
+                                          self._stream()), "forward")
+            return self.y
         self.x16.copy_(x16)
         self.gemm(self.x16, self.get("P", "theta16"), rows, C, c.cin, lda=c.cin, ldb=C,
                   bias=self.get("bp"), D=self.h16[0])
@@ -312,6 +388,9 @@ class FNO:
         B, rows = self.B, self.rows
         st = self._stream()
         self.grad.zero_()
+        if self.fused:
+            _ok(self.lib.rlbm_fno_backward(ctypes.byref(self._net()), st), "backward")
+            return self.grad
         self.to16(self.dy, self.dy16)
         self.gemm_tn_sum(self.y116, self.dy16, Cq, c.cout, rows, self.get("Q2", "grad"))
         _ok(self.lib.rlbm_fno_colsum(_p(self.dy), _p(self.get("bq2", "grad")), rows, c.cout, st), "colsum")
