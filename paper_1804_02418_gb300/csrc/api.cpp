@@ -608,8 +608,10 @@ int init_sample(rlbm_ctx* c, int sample, const double* n, const double* ux, cons
     }
     DevSample d = L.dev;
     d.cur = c->cur;      // the electric force's first step reads this density plane
-    e = (ce ? c->ops->init_ce : c->ops->init)(dst, d, dp[0], dp[1], dp[2], dp[3],
-                                              at<unsigned>(c, c->err_off), c->stream);
+    unsigned* err = at<unsigned>(c, c->err_off);
+    e = ce ? c->ops->init_ce(dst, buf(c, sample, c->cur ^ 1), d, dp[0], dp[1], dp[2], dp[3], err,
+                             c->stream)
+           : c->ops->init(dst, d, dp[0], dp[1], dp[2], dp[3], err, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "init kernel");
     c->launches++;
   }

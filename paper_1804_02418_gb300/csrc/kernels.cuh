@@ -933,31 +933,38 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ fin, const De
   const unsigned bad = landau(m, M) & ~kErrUnphysical;
   if (bad) atomicOr(err, bad);
   const long long k = (long long)y * s.nx + x;
-  if (n) n[k] = 1.0 + double(M.dn);
-  if (ux) ux[k] = double(M.ux);
-  if (uy) uy[k] = double(M.uy);
-  if (T) T[k] = 1.0 + double(M.dT);
+  if (n) n[k] = 1.0 + as_f64(M.dn);
+  if (ux) ux[k] = as_f64(M.ux);
+  if (uy) uy[k] = as_f64(M.uy);
+  if (T) T[k] = 1.0 + as_f64(M.dT);
   if (dn_out) dn_out[(long long)y * s.ldx + x] = M.dn;
 }
 
-// Macroscopic state of site k of dense FP64 fields (n, u, T).
+// Macroscopic state of site k of dense FP64 fields (n, u, T).  FP32
+// arithmetic takes n - 1 and T - 1 from the FP64 fields and forms gamma - 1
+// (relative error 2e-7 of a second-order quantity) itself: 8 operations on
+// the FP64 pipe instead of 26, which bounded k_init (FP16 storage
+// 4096 x 2048: 608 -> 159 us,
+// 268 MB in and 805 MB out).
 template <typename R>
 __device__ __forceinline__ Macro<R> field_macro(const double* n, const double* ux,
                                                 const double* uy, const double* T, long long k,
                                                 bool& ok) {
   Macro<R> M;
   const double vx = ux[k], vy = uy[k], nk = n[k], Tk = T[k];
-  const double u2 = fma(vx, vx, vy * vy), w = 1.0 - u2;
-  const double g = qrsqrt(w);
   M.ux = R(vx);
   M.uy = R(vy);
-  M.gamma = R(g);
-  M.gm1 = R(u2 * g * (g * qrcp(1.0 + g)));
   M.dn = R(nk - 1.0);
   M.dT = R(Tk - 1.0);
   M.deps = R(0);
-  M.invT = qrcp(R(Tk));
-  ok = (u2 < 1.0) && (nk > 0.0) && (Tk > 0.0) && finite_bits(nk) && finite_bits(Tk);
+  const R u2 = fma(M.ux, M.ux, M.uy * M.uy);
+  M.gamma = qrsqrt(R(1) - u2);
+  M.gm1 = u2 * M.gamma * (M.gamma * qrcp(R(1) + M.gamma));
+  M.invT = qrcp(R(1) + M.dT);
+  // |u| < 1 in FP64 where FP32 rounding could decide it
+  const bool slow = sizeof(R) == 8 || !(u2 < R(0.99));
+  ok = (slow ? fma(vx, vx, vy * vy) < 1.0 : true) && positive(nk) && positive(Tk) &&
+       finite_bits(nk) && finite_bits(Tk);
   return M;
 }
 
@@ -1076,32 +1083,86 @@ __device__ __forceinline__ void init_ce_body(S* __restrict__ fout, const DevSamp
   }
 }
 
-// Dense FP64 deviations [48][ny][nx]  <->  stored vectors.
-// Populations q0 .. q0 + gridDim.z - 1; `out` / `in` point at population q0
-// of the dense array.
+// The seed in two passes: `eq` holds the stored f^eq of every site (init_body
+// into the other buffer), and each site d sends, for every direction,
+//   f*_i(d - n_i) = f^eq_i(d) - (f^eq_i(d) - f^eq_i(d - n_i)) / omega_i(d)
+// to the site it came from, and keeps f^eq_i(d) where its own arrival site
+// d + n_i lies outside.  For FP64 and FP32 storage, where `eq` holds the
+// values init_ce_body forms in registers (16-bit storage would round them
+// twice).  init_ce_body evaluates the equilibrium coefficients at 13 sites per
+// site, about 1,300 FP64 operations more than the two passes: FP64 1024 x 512
+// about 1.7 ms -> 0.44 ms (0.28 + 0.16).
 template <typename S, class C>
-__device__ __forceinline__ void get_state_body(const S* __restrict__ fin, const DevSample& s,
-                                               int q0, double* out, const C& qc) {
-  const int x = blockIdx.x * kBX + threadIdx.x;
-  const int y = blockIdx.y;
-  const int dq = blockIdx.z, q = q0 + dq;
-  if (x >= s.nx) return;
-  const int d = q >> 2, j = q & 3;
-  const S v = fin[vec_index(s, d, (long long)y * s.ldx + x) + j];
-  out[((long long)dq * s.ny + y) * s.nx + x] = Codec<S>::decode(v, dir_kind(d), j, qc);
-}
-
-template <typename S, class C>
-__device__ __forceinline__ void set_state_body(S* __restrict__ fout, const DevSample& s, int q0,
-                                               const double* in, const C& qc) {
+__device__ __forceinline__ void ce_from_eq_body(const S* __restrict__ eq, S* __restrict__ fout,
+                                                const DevSample& s, const double* ux,
+                                                const double* uy, const C& qc) {
   using R = typename Codec<S>::R;
   const int x = blockIdx.x * kBX + threadIdx.x;
   const int y = blockIdx.y;
-  const int dq = blockIdx.z, q = q0 + dq;
   if (x >= s.nx) return;
-  const int d = q >> 2, j = q & 3;
-  const double v = in[((long long)dq * s.ny + y) * s.nx + x];
-  fout[vec_index(s, d, (long long)y * s.ldx + x) + j] = Codec<S>::encode(v, dir_kind(d), j, qc);
+  const long long k = (long long)y * s.nx + x, site = (long long)y * s.ldx + x;
+  const double vx = ux[k], vy = uy[k];
+  const double g = qrsqrt(1.0 - fma(vx, vx, vy * vy));
+  const R gt = R(g) * R(s.inv_tau), gx = gt * R(vx), gy = gt * R(vy);
+#pragma unroll
+  for (int d = 0; d < kDirs; ++d) {
+    const int dx = hop_x(d), dy = hop_y(d);
+    R own[4];
+    Codec<S>::load4(eq + vec_index(s, d, site), pull_policy(false), own);
+    int sx = x - dx, sy = y - dy;
+    if (s.periodic_x) sx = sx < 0 ? sx + s.nx : (sx >= s.nx ? sx - s.nx : sx);
+    if (s.periodic_y) sy = sy < 0 ? sy + s.ny : (sy >= s.ny ? sy - s.ny : sy);
+    if ((unsigned)sx < (unsigned)s.nx && (unsigned)sy < (unsigned)s.ny) {
+      const long long from = vec_index(s, d, (long long)sy * s.ldx + sx);
+      R src[4];
+      Codec<S>::load4(eq + from, pull_policy(false), src);
+      const R om = fma(-gy, R(dy) / R(5), fma(-gx, R(dx) / R(5), gt));
+      R iom;
+      if constexpr (sizeof(R) == 8) iom = qrcp(om);
+      else iom = R(1) / om;
+#pragma unroll
+      for (int j = 0; j < kShells; ++j) src[j] = fma(src[j] - own[j], iom, own[j]);
+      Codec<S>::store4(fout + from, src);
+    }
+    int tx = x + dx, ty = y + dy;
+    if (s.periodic_x) tx = tx < 0 ? tx + s.nx : (tx >= s.nx ? tx - s.nx : tx);
+    if (s.periodic_y) ty = ty < 0 ? ty + s.ny : (ty >= s.ny ? ty - s.ny : ty);
+    if (!((unsigned)tx < (unsigned)s.nx && (unsigned)ty < (unsigned)s.ny))
+      Codec<S>::store4(fout + vec_index(s, d, site), own);
+  }
+}
+
+// Dense FP64 deviations [48][ny][nx]  <->  stored vectors.
+// Directions d0 .. d0 + gridDim.z - 1, one thread per site and direction (one
+// vector access against four plane accesses, all coalesced); `out` / `in`
+// point at population 4 d0 of the dense array.
+template <typename S, class C>
+__device__ __forceinline__ void get_state_body(const S* __restrict__ fin, const DevSample& s,
+                                               int d0, double* out, const C& qc) {
+  const int x = blockIdx.x * kBX + threadIdx.x;
+  const int y = blockIdx.y;
+  const int dd = blockIdx.z, d = d0 + dd;
+  if (x >= s.nx) return;
+  struct alignas(4 * sizeof(S) < 16 ? 4 * sizeof(S) : 16) Vec { S v[4]; };
+  const Vec v = *reinterpret_cast<const Vec*>(fin + vec_index(s, d, (long long)y * s.ldx + x));
+#pragma unroll
+  for (int j = 0; j < kShells; ++j)
+    out[((long long)(4 * dd + j) * s.ny + y) * s.nx + x] = Codec<S>::decode(v.v[j], dir_kind(d), j, qc);
+}
+
+template <typename S, class C>
+__device__ __forceinline__ void set_state_body(S* __restrict__ fout, const DevSample& s, int d0,
+                                               const double* in, const C& qc) {
+  const int x = blockIdx.x * kBX + threadIdx.x;
+  const int y = blockIdx.y;
+  const int dd = blockIdx.z, d = d0 + dd;
+  if (x >= s.nx) return;
+  struct alignas(4 * sizeof(S) < 16 ? 4 * sizeof(S) : 16) Vec { S v[4]; };
+  Vec v;
+#pragma unroll
+  for (int j = 0; j < kShells; ++j)
+    v.v[j] = Codec<S>::encode(in[((long long)(4 * dd + j) * s.ny + y) * s.nx + x], dir_kind(d), j, qc);
+  *reinterpret_cast<Vec*>(fout + vec_index(s, d, (long long)y * s.ldx + x)) = v;
 }
 
 }  // namespace rlbm

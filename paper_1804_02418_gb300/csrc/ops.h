@@ -30,10 +30,11 @@ struct PrecOps {
                          cudaStream_t st);
   cudaError_t (*init)(void* fout, const DevSample& s, const double* n, const double* ux,
                       const double* uy, const double* T, unsigned* err, cudaStream_t st);
-  // the Chapman-Enskog seed of the fields (kernels.cuh: init_ce_body)
-  cudaError_t (*init_ce)(void* fout, const DevSample& s, const double* n, const double* ux,
+  // the Chapman-Enskog seed of the fields (kernels.cuh: init_ce_body);
+  // scratch: the other population buffer, overwritten
+  cudaError_t (*init_ce)(void* fout, void* scratch, const DevSample& s, const double* n, const double* ux,
                          const double* uy, const double* T, unsigned* err, cudaStream_t st);
-  // planes q0 .. q0+nq-1 <-> dense FP64 [nq][ny][nx]
+  // planes q0 .. q0+nq-1 (both multiples of 4) <-> dense FP64 [nq][ny][nx]
   cudaError_t (*get_state)(const void* fin, const DevSample& s, int q0, int nq, double* out,
                            cudaStream_t st);
   cudaError_t (*set_state)(void* fout, const DevSample& s, int q0, int nq, const double* in,

@@ -120,14 +120,20 @@ __global__ void __launch_bounds__(kBX) k_init_ce(S* __restrict__ fout, DevSample
   init_ce_body<S>(fout, s, n, ux, uy, T, err, c_qc);
 }
 
-__global__ void __launch_bounds__(kBX) k_get(const S* __restrict__ fin, DevSample s, int q0,
-                                             double* out) {
-  get_state_body<S>(fin, s, q0, out, c_qc);
+__global__ void __launch_bounds__(kBX) k_ce_from_eq(const S* __restrict__ eq, S* __restrict__ fout,
+                                                    DevSample s, const double* ux,
+                                                    const double* uy) {
+  ce_from_eq_body<S>(eq, fout, s, ux, uy, c_qc);
 }
 
-__global__ void __launch_bounds__(kBX) k_set(S* __restrict__ fout, DevSample s, int q0,
+__global__ void __launch_bounds__(kBX) k_get(const S* __restrict__ fin, DevSample s, int d0,
+                                             double* out) {
+  get_state_body<S>(fin, s, d0, out, c_qc);
+}
+
+__global__ void __launch_bounds__(kBX) k_set(S* __restrict__ fout, DevSample s, int d0,
                                              const double* in) {
-  set_state_body<S>(fout, s, q0, in, c_qc);
+  set_state_body<S>(fout, s, d0, in, c_qc);
 }
 
 dim3 site_grid(const DevSample& s) { return dim3((s.nx + kBX - 1) / kBX, s.ny, 1); }
@@ -142,6 +148,8 @@ cudaError_t upload(const double p0[4], const double w[2][4], double scale) {
     for (int k = 0; k < 2; ++k) {
       h.w[k][j] = R(w[k][j]);
       h.wd[k][j] = w[k][j];
+      h.iwd[k][j] = 1.0 / w[k][j];
+      h.iwl[k][j] = std::fma(-w[k][j], h.iwd[k][j], 1.0) / w[k][j];
       h.wp0[k][j] = R(w[k][j] * p0[j] / scale);
       h.wp0sq[k][j] = R(w[k][j] * p0[j] * p0[j] / scale);
     }
@@ -313,25 +321,32 @@ cudaError_t init(void* fout, const DevSample& s, const double* n, const double* 
   return cudaGetLastError();
 }
 
-cudaError_t init_ce(void* fout, const DevSample& s, const double* n, const double* ux,
-                    const double* uy, const double* T, unsigned* err, cudaStream_t st) {
-  k_init_ce<<<site_grid(s), kBX, 0, st>>>(static_cast<S*>(fout), s, n, ux, uy, T, err);
+cudaError_t init_ce(void* fout, void* scratch, const DevSample& s, const double* n,
+                    const double* ux, const double* uy, const double* T, unsigned* err,
+                    cudaStream_t st) {
+  if (sizeof(S) >= sizeof(float)) {
+    k_init<<<site_grid(s), kBX, 0, st>>>(static_cast<S*>(scratch), s, n, ux, uy, T, err);
+    k_ce_from_eq<<<site_grid(s), kBX, 0, st>>>(static_cast<const S*>(scratch),
+                                               static_cast<S*>(fout), s, ux, uy);
+  } else {
+    k_init_ce<<<site_grid(s), kBX, 0, st>>>(static_cast<S*>(fout), s, n, ux, uy, T, err);
+  }
   return cudaGetLastError();
 }
 
 cudaError_t get_state(const void* fin, const DevSample& s, int q0, int nq, double* out,
                       cudaStream_t st) {
   dim3 grid = site_grid(s);
-  grid.z = nq;
-  k_get<<<grid, kBX, 0, st>>>(static_cast<const S*>(fin), s, q0, out);
+  grid.z = nq / kShells;
+  k_get<<<grid, kBX, 0, st>>>(static_cast<const S*>(fin), s, q0 / kShells, out);
   return cudaGetLastError();
 }
 
 cudaError_t set_state(void* fout, const DevSample& s, int q0, int nq, const double* in,
                       cudaStream_t st) {
   dim3 grid = site_grid(s);
-  grid.z = nq;
-  k_set<<<grid, kBX, 0, st>>>(static_cast<S*>(fout), s, q0, in);
+  grid.z = nq / kShells;
+  k_set<<<grid, kBX, 0, st>>>(static_cast<S*>(fout), s, q0 / kShells, in);
   return cudaGetLastError();
 }
 

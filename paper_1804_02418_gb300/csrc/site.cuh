@@ -66,6 +66,7 @@ struct QuadConsts {
   R wp0sq[2][kShells];      // w p0_j^2 / s
   R dec_s, enc_s;           // 16-bit storage scale: 1 / s, s (the 16-bit kernels compute on s g)
   double wd[2][kShells];    // w in FP64: state I/O converts g <-> delta = w g in FP64
+  double iwd[2][kShells], iwl[2][kShells];   // 1 / w = iwd + iwl
   // Conservation projection (reduced precision): correction
   // w_2j (l0 + l1 p0_j + p0_j (lx vx + ly vy)) on the (5,0)-type directions,
   // (l0, l1) = P (rN, rE), (lx, ly) = px (rX, rY).
@@ -110,6 +111,14 @@ constexpr unsigned kErrUnphysical = 2u;
 constexpr unsigned kErrNoConvergence = 4u;
 constexpr unsigned kErrTimeout = 8u;      // a bounded wait inside a kernel gave up
 
+// delta / w for a weight w: the product with 1 / w held as hi + lo, rounded
+// once (error below half an ulp and 2^-50 of one, as the division's, in 2
+// instead of about 10 FP64 operations).
+template <class C>
+__device__ __forceinline__ double over_weight(double v, int kind, int j, const C& c) {
+  return fma(v, c.iwd[kind][j], v * c.iwl[kind][j]);
+}
+
 // ---------------------------------------------------------------------------
 // Storage codecs.  The four shells of one (direction, site) are stored side by
 // side, so one aligned vector access moves them (16 B for FP32, 32 B for FP64,
@@ -139,7 +148,7 @@ template <> struct Codec<double> {
     return v * c.wd[kind][j];
   }
   template <class C> __device__ static double encode(double v, int kind, int j, const C& c) {
-    return v / c.wd[kind][j];
+    return over_weight(v, kind, j, c);
   }
 };
 template <> struct Codec<float> {
@@ -161,7 +170,7 @@ template <> struct Codec<float> {
     return double(v) * c.wd[kind][j];
   }
   template <class C> __device__ static float encode(double v, int kind, int j, const C& c) {
-    return float(v / c.wd[kind][j]);
+    return float(over_weight(v, kind, j, c));
   }
 };
 template <typename H> struct Codec16 {
@@ -191,7 +200,7 @@ template <typename H> struct Codec16 {
     return double(tof(v)) * double(c.dec_s) * c.wd[kind][j];
   }
   template <class C> __device__ static H encode(double v, int kind, int j, const C& c) {
-    return fromf(float(v / c.wd[kind][j] * double(c.enc_s)));
+    return fromf(float(over_weight(v, kind, j, c) * double(c.enc_s)));
   }
 };
 template <> __device__ inline float2 Codec16<__half>::unpack2(uint32_t u) {
@@ -279,6 +288,13 @@ __device__ __forceinline__ double widen_f64(float f) {
   if (mag < 0x00800000u) hi = lo = 0u;
   if (mag >= 0x7f800000u) hi = 0x7ff80000u;
   return __hiloint2double((int)((b & 0x80000000u) | hi), (int)lo);
+}
+
+// double(a), off the FP64 pipe for normal numbers and zero
+__device__ __forceinline__ double as_f64(double a) { return a; }
+__device__ __forceinline__ double as_f64(float a) {
+  const unsigned e = __float_as_uint(a) & 0x7f800000u;
+  return (e - 0x00800000u) < 0x7f000000u || a == 0.f ? widen_f64(a) : double(a);
 }
 
 __device__ __forceinline__ bool finite_bits(float a) {
