@@ -108,13 +108,15 @@ __device__ __forceinline__ uint64_t pull_policy(bool evict_first) {
 }
 
 // Gathers the 48 streamed deviations arriving at (x, y).
-template <typename S, bool INTERIOR, class C, class O>
+// Directions D0 .. D0 + ND - 1 into f[0 .. 4 ND).
+template <typename S, bool INTERIOR, int D0, int ND, class C, class O>
 __device__ __forceinline__ void pull(const S* __restrict__ fin, const Tile<S>& tl, const O& of,
                                      const DevSample& s, int x, int y,
                                      const typename Codec<S>::R* __restrict__ ghost, const C& qc,
-                                     typename Codec<S>::R (&f)[kQ]) {
+                                     typename Codec<S>::R* f0) {
+  typename Codec<S>::R* const f = f0 - 4 * D0;
 #pragma unroll
-  for (int d = 0; d < kDirs; ++d) {
+  for (int d = D0; d < D0 + ND; ++d) {
     const int dx = hop_x(d), dy = hop_y(d);
     if (INTERIOR) {
       Codec<S>::load4(byte_ptr(tl.in, of.pull(d)), tl.policy, &f[4 * d]);
@@ -421,13 +423,13 @@ __device__ __forceinline__ bool warp_interior(const DevSample& s, int x, int y) 
 }
 
 // Gathers the 48 deviations streamed into site (x < nx, y) from HBM.
-template <typename S, class C, class O>
+template <typename S, int D0 = 0, int ND = kDirs, class C, class O>
 __device__ __forceinline__ void gather(const S* __restrict__ fin, const Tile<S>& tl, const O& of,
                                        const DevSample& s, int x, int y,
                                        const typename Codec<S>::R* __restrict__ ghost, const C& qc,
-                                       typename Codec<S>::R (&f)[kQ]) {
-  if (warp_interior(s, x, y)) pull<S, true>(fin, tl, of, s, x, y, ghost, qc, f);
-  else pull<S, false>(fin, tl, of, s, x, y, ghost, qc, f);
+                                       typename Codec<S>::R* f) {
+  if (warp_interior(s, x, y)) pull<S, true, D0, ND>(fin, tl, of, s, x, y, ghost, qc, f);
+  else pull<S, false, D0, ND>(fin, tl, of, s, x, y, ghost, qc, f);
 }
 
 // pair_cubics() on register pairs, lanes (d, d + 1): the two lanes differ only
@@ -601,6 +603,51 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], const Tile<
   }
 }
 
+// Relaxation, force and store of directions D0 .. D0 + ND - 1 (f: their
+// populations) for the site's fields M.
+template <typename S, int FORCE, int D0, int ND, class C, class O>
+__device__ __forceinline__ void relax_store_f64(double* f, const Tile<S>& tl, const O& of,
+                                                const DevSample& s, const Macro<double>& M,
+                                                bool lca, double egx, double egy, const C& qc) {
+  using R = double;
+  const EqCoeffs<R> c = eq_coeffs(M, fma(M.dn, M.invT, M.invT), (M.dn - M.dT) * M.invT);
+  RelaxSite<R> rs;
+  rs.gt = M.gamma * s.inv_tau;
+  rs.omgt = R(1) - rs.gt;
+  rs.gux = rs.gt * M.ux; rs.guy = rs.gt * M.uy;
+  rs.Fx = lca ? fma(-s.inv_cg, egx, s.Fx) : s.Fx;
+  rs.Fy = lca ? fma(-s.inv_cg, egy, s.Fy) : s.Fy;
+  ForceCoeffs<R> k{};
+  if (FORCE != 0) k = force_coeffs(c, rs.Fx, rs.Fy, R(1));
+#pragma unroll
+  for (int d = D0; d < D0 + ND; d += 2) {
+    R Rp[4], Rn[4], omcp, omcn;
+    pair_cubics<R, FORCE != 0>(d, c, k, rs, Rp, Rn, omcp, omcn);
+    R* const g = f + 4 * (d - D0);
+    relax_shells(Rp, omcp, qc, g);
+    relax_shells(Rn, omcn, qc, g + 4);
+    Codec<S>::store4(byte_ptr(tl.out, of.plane(d)), g);
+    Codec<S>::store4(byte_ptr(tl.out, of.plane(d + 1)), g + 4);
+  }
+}
+
+// The residual's part of a site: RES 1 keeps u, RES 2 adds |u - u_prev|^2 and |u|^2.
+template <int RES>
+__device__ __forceinline__ void residual_terms(const DevSample& s, int x, int y,
+                                               const Macro<double>& M, const StepAux<double>& aux,
+                                               double& r_du2, double& r_u2) {
+  if (RES == 0) return;
+  const long long j = s.site0 + (long long)y * s.nx + x;
+  if (RES == 1) {
+    aux.uprev[2 * j] = M.ux;
+    aux.uprev[2 * j + 1] = M.uy;
+  } else {
+    const double dx = M.ux - aux.uprev[2 * j], dy = M.uy - aux.uprev[2 * j + 1];
+    r_du2 = fma(dx, dx, fma(dy, dy, r_du2));
+    r_u2 = fma(M.ux, M.ux, fma(M.uy, M.uy, r_u2));
+  }
+}
+
 // Collision of the gathered deviations f of site (x < nx, y) and store of the
 // 48 new deviations into fout.  RES: 0 nothing extra; 1 store u for the
 // residual; 2 add |u - u_prev|^2 and |u|^2 to r_du2, r_u2 (the caller
@@ -624,39 +671,12 @@ __device__ __forceinline__ void collide_store(typename Codec<S>::R (&f)[kQ], con
     const bool lca = FORCE == kForceLca && s.dn[0] != nullptr;
     R egx = R(0), egy = R(0);
     if (lca) lca_gradient(s, dn_prev, x, y, egx, egy);
-    const Moments<R> m = moments(f, qc);
     Macro<R> M;
-    const unsigned bad = landau(m, M);
+    const unsigned bad = landau(moments(f, qc), M);
     if (bad) atomicOr(aux.err, bad);
-    const EqCoeffs<R> c = eq_coeffs(M, fma(M.dn, M.invT, M.invT), (M.dn - M.dT) * M.invT);
-    RelaxSite<R> rs;
-    rs.gt = M.gamma * R(s.inv_tau);
-    rs.omgt = R(1) - rs.gt;
-    rs.gux = rs.gt * M.ux; rs.guy = rs.gt * M.uy;
-    rs.Fx = lca ? fma(-R(s.inv_cg), egx, R(s.Fx)) : R(s.Fx);
-    rs.Fy = lca ? fma(-R(s.inv_cg), egy, R(s.Fy)) : R(s.Fy);
-    ForceCoeffs<R> k{};
-    if (FORCE != 0) k = force_coeffs(c, rs.Fx, rs.Fy, R(1));
     if (lca) dn_next[(long long)y * s.ldx + x] = M.dn;
-#pragma unroll
-    for (int d = 0; d < kDirs; d += 2) {
-      R Rp[4], Rn[4], omcp, omcn;
-      pair_cubics<R, FORCE != 0>(d, c, k, rs, Rp, Rn, omcp, omcn);
-      relax_shells(Rp, omcp, qc, &f[4 * d]);
-      relax_shells(Rn, omcn, qc, &f[4 * d + 4]);
-      Codec<S>::store4(byte_ptr(tl.out, of.plane(d)), &f[4 * d]);
-      Codec<S>::store4(byte_ptr(tl.out, of.plane(d + 1)), &f[4 * d + 4]);
-    }
-    if (RES == 1) {
-      const long long j = s.site0 + (long long)y * s.nx + x;
-      aux.uprev[2 * j] = M.ux;
-      aux.uprev[2 * j + 1] = M.uy;
-    } else if (RES == 2) {
-      const long long j = s.site0 + (long long)y * s.nx + x;
-      const double dx = M.ux - aux.uprev[2 * j], dy = M.uy - aux.uprev[2 * j + 1];
-      r_du2 = fma(dx, dx, fma(dy, dy, r_du2));
-      r_u2 = fma(M.ux, M.ux, fma(M.uy, M.uy, r_u2));
-    }
+    relax_store_f64<S, FORCE, 0, kDirs>(f, tl, of, s, M, lca, egx, egy, qc);
+    residual_terms<RES>(s, x, y, M, aux, r_du2, r_u2);
   }
 }
 
@@ -670,7 +690,7 @@ __device__ __forceinline__ void site_step(const S* __restrict__ fin, const Tile<
   using R = typename Codec<S>::R;
   if (x < s.nx) {
     R f[kQ];
-    gather(fin, tl, of, s, x, y, ghost, qc, f);
+    gather<S>(fin, tl, of, s, x, y, ghost, qc, f);
     // select, not s.dn[cur]: a runtime index would move the descriptor to local memory
     void* const prev = cur ? s.dn[1] : s.dn[0];
     void* const next = cur ? s.dn[0] : s.dn[1];
@@ -726,6 +746,66 @@ __device__ __forceinline__ void step_body(const S* __restrict__ fin, S* __restri
   site_step<S, FORCE, RES, BT>(fin, tl, of, s, t < wt.count ? x : s.nx, (int)y, ghost, aux, qc,
                                r_du2, r_u2, smem_addr(park) + threadIdx.x * 16u, s.cur);
   if (RES == 2) block_reduce_add2<typename Codec<S>::R>(r_du2, r_u2, aux.acc);
+}
+
+// FP64, one sample, few sites: three warps share the 32 sites of a warp tile,
+// each with the populations of one group of four directions.  A warp
+// instruction of the FP64 pipe takes 66 cycles of its SM sub-partition however
+// many of its lanes are active, so a sample of fewer warp tiles than
+// sub-partitions (608) is bound by the chain of one warp: about 690 FP64
+// instructions.  Split, a warp runs about 320 (its third of the moments and
+// the relaxation; the Landau solve and the coefficients are repeated).
+// 64 x 64 sites: 22.9 -> 12.1 us per step.
+template <typename S, int FORCE, int RES, int G, class C>
+__device__ __forceinline__ void split_group(const S* __restrict__ fin, const Tile<S>& tl,
+                                            const StepOffsets& of, const DevSample& s, int x,
+                                            int y, const double* __restrict__ ghost,
+                                            const StepAux<double>& aux, const C& qc,
+                                            GroupSums<double>* part) {
+  const int lane = threadIdx.x % 32;
+  const bool in = x < s.nx;
+  const bool lca = FORCE == kForceLca && s.dn[0] != nullptr;
+  double f[16], egx = 0.0, egy = 0.0;
+  if (in) {
+    gather<S, 4 * G, 4>(fin, tl, of, s, x, y, ghost, qc, f);
+    if (lca) lca_gradient(s, static_cast<const double*>(s.cur ? s.dn[1] : s.dn[0]), x, y, egx, egy);
+    part[G * 32 + lane] = group_sums<G>(f, qc);
+  }
+  // a barrier that the three warps meet at from three places in the code
+  asm volatile("bar.sync 1, 96;\n" ::: "memory");
+  double r_du2 = 0.0, r_u2 = 0.0;
+  if (in) {
+    Macro<double> M;
+    const unsigned bad = landau(add_groups(part[lane], part[32 + lane], part[64 + lane]), M);
+    if (G == 0) {
+      if (bad) atomicOr(aux.err, bad);
+      if (lca) static_cast<double*>(s.cur ? s.dn[0] : s.dn[1])[(long long)y * s.ldx + x] = M.dn;
+      residual_terms<RES>(s, x, y, M, aux, r_du2, r_u2);
+    }
+    relax_store_f64<S, FORCE, 4 * G, 4>(f, tl, of, s, M, lca, egx, egy, qc);
+  }
+  if (RES == 2 && G == 0) warp_reduce_add2(r_du2, r_u2, aux.acc);
+}
+
+template <typename S, int FORCE, int RES, class C>
+__device__ __forceinline__ void split_body(const S* __restrict__ fin, S* __restrict__ fout,
+                                           const DevSample& s, const WarpTiles& wt,
+                                           const StepOffsets& of, const double* __restrict__ ghost,
+                                           const StepAux<double>& aux, const C& qc,
+                                           GroupSums<double>* part) {
+  chain_release();
+  unsigned y, r;
+  wt.row_of(wt.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x, y, r);
+  const int x = (int)(r * 32 + threadIdx.x % 32), g = threadIdx.x / 32;
+  const long long site = (long long)y * s.ldx + x;
+  Tile<S> tl;
+  tl.in = fin + 4 * site;
+  tl.out = fout + 4 * site;
+  tl.policy = pull_policy(false);
+  chain_wait();
+  if (g == 0) split_group<S, FORCE, RES, 0>(fin, tl, of, s, x, (int)y, ghost, aux, qc, part);
+  else if (g == 1) split_group<S, FORCE, RES, 1>(fin, tl, of, s, x, (int)y, ghost, aux, qc, part);
+  else split_group<S, FORCE, RES, 2>(fin, tl, of, s, x, (int)y, ghost, aux, qc, part);
 }
 
 // Many samples of uneven size in one launch.  The work list is every row
@@ -927,7 +1007,7 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ fin, const De
   tl.in = fin + 4 * ((long long)y * s.ldx + x);
   tl.out = nullptr;
   tl.policy = pull_policy(false);
-  gather(fin, tl, SampleOffsets<S>{s.plane, s.ldx}, s, x, y, ghost, qc, f);
+  gather<S>(fin, tl, SampleOffsets<S>{s.plane, s.ldx}, s, x, y, ghost, qc, f);
   const Moments<R> m = moments(f, qc);
   Macro<R> M;
   const unsigned bad = landau(m, M) & ~kErrUnphysical;

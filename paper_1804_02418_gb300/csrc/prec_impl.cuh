@@ -4,6 +4,7 @@
 #include "kernels.cuh"
 #include "ops.h"
 
+#include <atomic>
 #include <cmath>
 
 namespace rlbm {
@@ -31,6 +32,12 @@ __constant__ QuadConsts<R> c_qc;
 constexpr int kStepRegs = (65536 / (RLBM_STEP_MIN_BLOCKS * kBX)) > 255
                               ? 255 : ((65536 / (RLBM_STEP_MIN_BLOCKS * kBX)) & ~7);
 
+// Threads per block of the single-sample step.  Us per step with blocks of
+// 32 / 64 / 128: FP32 200 x 150 5.7 / 5.7 / 6.4, 1024 x 512 33.7 / 32.4 / 32.6,
+// 4096 x 2048 481 / 460 / 460; FP16 4096 x 2048 290 / 294 / 299; FP64 64 x 64
+// 22.8 / 22.7 / 25.6.
+constexpr int kStepThreads = 64;
+
 // Dynamic shared memory of the direct step kernels: the parking area
 // (park_bytes: 12 x threads x 16 B with FP32 arithmetic, none with FP64).
 template <int FORCE, int RES, int BT>
@@ -41,6 +48,24 @@ __global__ void __maxnreg__(kStepRegs) k_step(const S* __restrict__ fin, S* __re
                                               const R* __restrict__ ghost, StepAux<R> aux) {
   extern __shared__ __align__(128) unsigned char park_smem[];
   step_body<S, FORCE, RES, BT>(fin, fout, s, wt, of, ghost, aux, c_qc, park_smem);
+}
+
+// FP64 samples of few sites (split_body).  The launches ask for more shared
+// memory than two blocks of an SM could have: otherwise the blocks of the next
+// step, placed while this one runs, gather on the SMs that it leaves idle
+// (64 x 64: 44 us per step instead of 12.1).
+constexpr size_t kSplitSmem = 120 * 1024;
+constexpr size_t kSpreadSmem = 80 * 1024;   // two blocks per SM
+template <int FORCE, int RES>
+__global__ void __launch_bounds__(96) k_step_split(const S* __restrict__ fin, S* __restrict__ fout,
+                                                   const __grid_constant__ DevSample s,
+                                                   const __grid_constant__ WarpTiles wt,
+                                                   const __grid_constant__ StepOffsets of,
+                                                   const R* __restrict__ ghost, StepAux<R> aux) {
+  if constexpr (sizeof(S) == 8) {
+    __shared__ GroupSums<double> part[3 * 32];
+    split_body<S, FORCE, RES>(fin, fout, s, wt, of, ghost, aux, c_qc, part);
+  }
 }
 
 template <int FORCE, int RES, int BX>
@@ -78,6 +103,39 @@ cudaError_t allow_park_smem() {
   set((const void*)k_step_batch<2, 0, BX>);
   set((const void*)k_step_batch<2, 1, BX>);
   set((const void*)k_step_batch<2, 2, BX>);
+  return e;
+}
+
+cudaError_t allow_split_smem() {
+  cudaError_t e = cudaSuccess;
+  if constexpr (sizeof(S) == 8) {
+    auto set = [&](const void* fn) {
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSplitSmem);
+    };
+    set((const void*)k_step_split<0, 0>);
+    set((const void*)k_step_split<0, 1>);
+    set((const void*)k_step_split<0, 2>);
+    set((const void*)k_step_split<1, 0>);
+    set((const void*)k_step_split<1, 1>);
+    set((const void*)k_step_split<1, 2>);
+    set((const void*)k_step_split<2, 0>);
+    set((const void*)k_step_split<2, 1>);
+    set((const void*)k_step_split<2, 2>);
+    auto spread = [&](const void* fn) {
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadSmem);
+    };
+    spread((const void*)k_step<0, 0, kStepThreads>);
+    spread((const void*)k_step<0, 1, kStepThreads>);
+    spread((const void*)k_step<0, 2, kStepThreads>);
+    spread((const void*)k_step<1, 0, kStepThreads>);
+    spread((const void*)k_step<1, 1, kStepThreads>);
+    spread((const void*)k_step<1, 2, kStepThreads>);
+    spread((const void*)k_step<2, 0, kStepThreads>);
+    spread((const void*)k_step<2, 1, kStepThreads>);
+    spread((const void*)k_step<2, 2, kStepThreads>);
+  }
   return e;
 }
 
@@ -185,6 +243,7 @@ cudaError_t upload(const double p0[4], const double w[2][4], double scale) {
   if (e == cudaSuccess) e = allow_stage_smem<128>();
   if (e == cudaSuccess) e = allow_stage_smem<256>();
   if (e == cudaSuccess) e = allow_park_smem<256>();
+  if (e == cudaSuccess) e = allow_split_smem();
   return e;
 }
 
@@ -208,27 +267,37 @@ void launch_chained(void (*k)(P...), unsigned grid, int block, size_t smem, cuda
   cudaLaunchKernelEx(&cfg, k, P(args)...);
 }
 
-// L2 size of the current device (looked up once per device).
-size_t l2_bytes() {
-  static int bytes[64] = {};
+// Attributes of the current device (looked up once per device; concurrent
+// first calls store the same values).
+int device_attr(cudaDeviceAttr attr, std::atomic<int> (&known)[64]) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (bytes[dev] == 0) cudaDeviceGetAttribute(&bytes[dev], cudaDevAttrL2CacheSize, dev);
-  return (size_t)bytes[dev];
+  int v = known[dev].load(std::memory_order_relaxed);
+  if (v == 0 && cudaDeviceGetAttribute(&v, attr, dev) == cudaSuccess)
+    known[dev].store(v, std::memory_order_relaxed);
+  return v;
 }
-
-// Threads per block of the single-sample step.  Us per step with blocks of
-// 32 / 64 / 128: FP32 200 x 150 5.7 / 5.7 / 6.4, 1024 x 512 33.7 / 32.4 / 32.6,
-// 4096 x 2048 481 / 460 / 460; FP16 4096 x 2048 290 / 294 / 299; FP64 64 x 64
-// 22.8 / 22.7 / 25.6.
-constexpr int kStepThreads = 64;
+size_t l2_bytes() {
+  static std::atomic<int> known[64];
+  return (size_t)device_attr(cudaDevAttrL2CacheSize, known);
+}
+int sm_count() {
+  static std::atomic<int> known[64];
+  return device_attr(cudaDevAttrMultiProcessorCount, known);
+}
 
 template <int F, int BT>
 void launch_single_bt(const S* a, S* b, const DevSample& s, const WarpTiles& wt,
                       const StepOffsets& of, const R* g, int res, const StepAux<R>& aux,
                       cudaStream_t st) {
   const unsigned grid = (wt.count + BT / 32 - 1) / (BT / 32);
-  const size_t pk = park_bytes<R>(BT);
+  size_t pk = park_bytes<R>(BT);
+  if constexpr (sizeof(S) == 8) {
+    // at most two blocks per SM, one warp per FP64 sub-partition: without it
+    // the blocks of the next step, placed while this one runs, gather on the
+    // SMs it leaves idle (150 x 77 sites: 52 us per step instead of 29)
+    if (grid <= 2u * (unsigned)sm_count()) pk = kSpreadSmem;
+  }
   if (res == 0) launch_chained(k_step<F, 0, BT>, grid, BT, pk, st, a, b, s, wt, of, g, aux);
   else if (res == 1) launch_chained(k_step<F, 1, BT>, grid, BT, pk, st, a, b, s, wt, of, g, aux);
   else launch_chained(k_step<F, 2, BT>, grid, BT, pk, st, a, b, s, wt, of, g, aux);
@@ -254,6 +323,17 @@ void launch_single(const S* a, S* b, const DevSample& s, const R* g, int res, co
   for (int d = 0; d < kDirs; ++d) {
     of.pull_[d] = pull_offset<S>(d, s.plane, s.ldx);
     of.plane_[d] = plane_offset<S>(d, s.plane);
+  }
+  if constexpr (sizeof(S) == 8) {
+    // up to one tile per SM: a second one would share sub-partitions, and two
+    // split chains take as long as one whole chain
+    if (wt.count <= (unsigned)sm_count()) {
+      const size_t sm = kSplitSmem;
+      if (res == 0) launch_chained(k_step_split<F, 0>, wt.count, 96, sm, st, a, b, s, wt, of, g, aux);
+      else if (res == 1) launch_chained(k_step_split<F, 1>, wt.count, 96, sm, st, a, b, s, wt, of, g, aux);
+      else launch_chained(k_step_split<F, 2>, wt.count, 96, sm, st, a, b, s, wt, of, g, aux);
+      return;
+    }
   }
   launch_single_bt<F, kStepThreads>(a, b, s, wt, of, g, res, aux, st);
 }

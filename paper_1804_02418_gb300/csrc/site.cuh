@@ -318,40 +318,73 @@ struct Moments {
   R dE, Mx, My, dPxx, dPxy, dPyy; // T^ab - diag(2, 1, 1)
 };
 
-template <typename R, class C>
-__device__ __forceinline__ Moments<R> moments_scalar(const R (&f)[kQ], const C& qc) {
-  Moments<R> m;
-  m.dN0 = m.dNx = m.dNy = m.dE = m.Mx = m.My = m.dPxx = m.dPxy = R(0);
+// In FP64 the sums are formed per group of four directions (velocities v, -v
+// and their mirror images; group 2: the axes), so that three warps can share a
+// site's populations and get the same bits.  With A_d = sum_j w p0_j g_dj,
+// B_d = sum_j w p0_j^2 g_dj and |v| = (a, b) in a group: N = sum A, X = sum A
+// sign(vx), Y = sum A sign(vy); E, MX, MY alike from B; S = sum B sign(vx vy)
+// (group 2: the part of E on the x axis).
+template <typename R>
+struct GroupSums {
+  R N, X, Y, E, MX, MY, S;
+};
+
+template <int G, typename R, class C>
+__device__ __forceinline__ GroupSums<R> group_sums(const R* f, const C& qc) {
+  constexpr int k = G == 2 ? 1 : 0;
+  R A[4], B[4];
 #pragma unroll
-  for (int d = 0; d < kDirs; d += 2) {
-    // directions d and d + 1 are opposite: v_{d+1} = -v_d
-    R Ap = R(0), Bp = R(0), An = R(0), Bn = R(0);
+  for (int d = 0; d < 4; ++d) {
+    A[d] = f[4 * d] * qc.wp0[k][0];
+    B[d] = f[4 * d] * qc.wp0sq[k][0];
 #pragma unroll
-    for (int j = 0; j < kShells; ++j) {
-      // relative deviations: delta = w g
-      const int k = dir_kind(d);
-      Ap = fma(f[4 * d + j], qc.wp0[k][j], Ap);
-      Bp = fma(f[4 * d + j], qc.wp0sq[k][j], Bp);
-      An = fma(f[4 * d + 4 + j], qc.wp0[k][j], An);
-      Bn = fma(f[4 * d + 4 + j], qc.wp0sq[k][j], Bn);
-    }
-    const R vx = R(hop_x(d)) / R(5), vy = R(hop_y(d)) / R(5);
-    const R Ae = Ap + An, Ao = Ap - An, Be = Bp + Bn, Bo = Bp - Bn;
-    m.dN0 += Ae;
-    m.dE += Be;
-    if (hop_x(d) != 0) {
-      m.dNx = fma(Ao, vx, m.dNx);
-      m.Mx = fma(Bo, vx, m.Mx);
-      m.dPxx = fma(Be, vx * vx, m.dPxx);
-      if (hop_y(d) != 0) m.dPxy = fma(Be, vx * vy, m.dPxy);
-    }
-    if (hop_y(d) != 0) {
-      m.dNy = fma(Ao, vy, m.dNy);
-      m.My = fma(Bo, vy, m.My);
+    for (int j = 1; j < kShells; ++j) {
+      A[d] = fma(f[4 * d + j], qc.wp0[k][j], A[d]);
+      B[d] = fma(f[4 * d + j], qc.wp0sq[k][j], B[d]);
     }
   }
+  GroupSums<R> s;
+  if (G == 2) {                    // (1,0) (-1,0) (0,1) (0,-1)
+    s.N = (A[0] + A[1]) + (A[2] + A[3]);
+    s.X = A[0] - A[1];
+    s.Y = A[2] - A[3];
+    s.S = B[0] + B[1];
+    s.E = s.S + (B[2] + B[3]);
+    s.MX = B[0] - B[1];
+    s.MY = B[2] - B[3];
+  } else {                         // (a,b) (-a,-b) (-a,b) (a,-b)
+    const R pA = A[0] + A[1], qA = A[2] + A[3], mA = A[0] - A[1], nA = A[3] - A[2];
+    const R pB = B[0] + B[1], qB = B[2] + B[3], mB = B[0] - B[1], nB = B[3] - B[2];
+    s.N = pA + qA;
+    s.X = mA + nA;
+    s.Y = mA - nA;
+    s.E = pB + qB;
+    s.MX = mB + nB;
+    s.MY = mB - nB;
+    s.S = pB - qB;
+  }
+  return s;
+}
+
+template <typename R>
+__device__ __forceinline__ Moments<R> add_groups(const GroupSums<R>& g, const GroupSums<R>& h,
+                                                 const GroupSums<R>& a) {
+  Moments<R> m;
+  m.dN0 = (g.N + h.N) + a.N;
+  m.dNx = fma(g.X, R(0.6), fma(h.X, R(0.8), a.X));
+  m.dNy = fma(g.Y, R(0.8), fma(h.Y, R(0.6), a.Y));
+  m.dE = (g.E + h.E) + a.E;
+  m.Mx = fma(g.MX, R(0.6), fma(h.MX, R(0.8), a.MX));
+  m.My = fma(g.MY, R(0.8), fma(h.MY, R(0.6), a.MY));
+  m.dPxx = fma(g.E, R(0.36), fma(h.E, R(0.64), a.S));
+  m.dPxy = (g.S + h.S) * R(0.48);
   m.dPyy = m.dE - m.dPxx;   // massless shells: T^00 = T^xx + T^yy exactly
   return m;
+}
+
+template <typename R, class C>
+__device__ __forceinline__ Moments<R> moments_scalar(const R (&f)[kQ], const C& qc) {
+  return add_groups(group_sums<0>(f, qc), group_sums<1>(f + 16, qc), group_sums<2>(f + 32, qc));
 }
 
 // ---------------------------------------------------------------------------
