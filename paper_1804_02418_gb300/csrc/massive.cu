@@ -40,6 +40,7 @@
 #include <string>
 
 #include "massive_tables.h"
+#include "site.cuh"
 
 namespace rlbm {
 namespace massive {
@@ -55,20 +56,45 @@ constexpr double kA0 = (kM * kM * kM + 6 * kM * kM + 15 * kM + 15) / kM1;   // a
 constexpr double kC2 = kM * kM / (kM1 * kM1 * kM1);             // 25/216
 constexpr double kSD0 = 2 * kM + 4 - kE0;                        // sqrt of the EOS discriminant at rest
 
-constexpr unsigned kErrNonFinite = 1u, kErrUnphysical = 2u, kErrNoConvergence = 4u;
+// Tables of the step.  A class holds the vectors of one energy: axis (a, 0),
+// diagonal (a, a), or eight (a, b) with a > b > 0.  By the square's symmetry a
+// class needs one row for the radial part of g^eq, one for its (px^2 - py^2)
+// part, one for its px py part and, per component magnitude, one for the part
+// odd in that component; the pairs of the class follow by additions:
+//   g^eq(a, b) even = A + C1 + C2, (-a, b): A + C1 - C2, (b, a): A - C1 + C2, ..
+//   odd(a, b) = X_a + Y_b, (-a, b): -X_a + Y_b, (b, a): X_b + Y_a, ..
+// 117 paired + 75 scalar operations per site in FP32 where 22 separate rows
+// of 28 took 275 paired ones.
+template <typename R> struct V2 { using T = double2; };
+template <> struct V2<float> { using T = float2; };
+
+// component functions: axis and diagonal classes one, classes of eight two
+constexpr int kOddFns = 11;
+__host__ __device__ constexpr int class_kind(int c) {      // 0 axis, 1 diagonal, 2 eight
+  return c == 3 || c == 6 ? 2 : c == 1 || c == 4 || c == 7 ? 1 : 0;
+}
+__host__ __device__ constexpr int class_pair(int c) {      // first pair of class c
+  return c == 0 ? 0 : c == 1 ? 2 : c == 2 ? 4 : c == 3 ? 6 : c == 4 ? 10 : c == 5 ? 12 : c == 6 ? 14
+       : c == 7 ? 18 : 20;
+}
+__host__ __device__ constexpr int class_fn(int c) {        // first component function of class c
+  return c <= 3 ? c : c <= 6 ? c + 1 : c + 2;
+}
 
 template <typename R>
 struct MConsts {
-  R vx[kPairs], vy[kPairs];
+  using V = typename V2<R>::T;
   R mN0[kPairs], mE[kPairs], mPxx[kPairs], mPxy[kPairs], mPyy[kPairs];
   R mNx[kPairs], mNy[kPairs], mMx[kPairs], mMy[kPairs];
-  R LT[kPairs], LX[kPairs], LY[kPairs];
-  R WE[kPairs][5], WO[kPairs][4];
-  R BE[kPairs][8], BO[kPairs][8];
-  R mvE[kPairs][8], mvO[kPairs][8];
+  R A[kClasses][8];      // dT, dn dT, dT^2, ux^2 + uy^2, E0, E1, E2 + E4, E5 + E7 (9: rest)
+  R C1[kClasses][3];     // ux^2 - uy^2, E2 - E4, E5 - E7
+  R C2[kClasses][3];     // ux uy, E3, E6
+  V O[kOddFns][7];       // (x, y) lanes alike: u, dn u, dT u, O0/O1, O2/O3, O4/O7, O6/O5
+  V va[kOddFns], pa[kOddFns];   // v and p of the component, both lanes alike
+  R p0[kClasses], rr[kClasses], dd[kClasses], pp[kClasses];   // (px^2 +- py^2) / 2, |px py|
   R gi[16][16];
-  R restN0, restE, restLT, restWE[5], restBE[8];
-  double f0[kQm];
+  R restN0, restE;
+  double f0[kQm], if0[kQm], ifl[kQm];      // 1 / f0 = if0 + ifl
 };
 
 __constant__ MConsts<float> c_f;
@@ -77,13 +103,6 @@ __constant__ MConsts<double> c_d;
 template <typename R> __device__ __forceinline__ const MConsts<R>& mc();
 template <> __device__ __forceinline__ const MConsts<float>& mc<float>() { return c_f; }
 template <> __device__ __forceinline__ const MConsts<double>& mc<double>() { return c_d; }
-
-__device__ __forceinline__ double mdiv(double a, double b) { return a / b; }
-__device__ __forceinline__ float mdiv(float a, float b) { return __fdividef(a, b); }
-
-template <typename R> struct MTol;
-template <> struct MTol<double> { static constexpr double v = 1e-15; };
-template <> struct MTol<float> { static constexpr float v = 2e-7f; };
 
 // library monomial order (massive_tables.h): exponents of p0, px, py
 __host__ __device__ constexpr int mon_b(int k) {
@@ -107,7 +126,7 @@ struct MGeom {
 
 template <typename R>
 struct MMacro {
-  R ux, uy, gamma, gm1, s;   // s = sqrt(1 - u^2), gm1 = gamma - 1
+  R ux, uy, gamma, gm1, r1;  // gm1 = gamma - 1, r1 = 1 / (1 + sqrt(1 - u^2))
   R dn, dT;                  // n - 1, T - 1
 };
 
@@ -118,21 +137,64 @@ struct MMom {
   R dPxx, dPxy, dPyy;        // T^ij - delta_ij
 };
 
+// Byte offsets, prepared on the host: from a site to the source of each pull
+// (interior sites) and to each population plane.
+struct MOffsets {
+  long long pull[kQm], plane[kQm];
+};
+
+template <typename S>
+__device__ __forceinline__ const S* at_bytes(const S* p, long long b) {
+  return reinterpret_cast<const S*>(reinterpret_cast<const char*>(p) + b);
+}
+template <typename S>
+__device__ __forceinline__ S* at_bytes(S* p, long long b) {
+  return reinterpret_cast<S*>(reinterpret_cast<char*>(p) + b);
+}
+
+// A read-only load that stays behind the wait for the predecessor's results
+// (an ordinary one may be moved above it).
+__device__ __forceinline__ float ld_pull(const float* p, uint64_t policy) {
+  float v;
+  asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;\n" : "=f"(v) : "l"(p), "l"(policy) : "memory");
+  return v;
+}
+__device__ __forceinline__ double ld_pull(const double* p, uint64_t) {
+  double v;
+  asm("ld.global.nc.f64 %0, [%1];\n" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// Which group of an NS-way split holds class c (the rest vector: class 9).
+// The groups hold about the same number of pairs.
+__host__ __device__ constexpr int class_group(int ns, int c) {
+  return ns == 1 ? 0
+       : ns == 2 ? (c <= 3 || c == 9 ? 0 : 1)
+       : (c == 2 || c == 3 ? 0 : c == 6 || c == 0 ? 1 : c == 1 || c == 4 || c == 5 ? 2 : 3);
+}
+__host__ __device__ constexpr bool mine(int ns, int g, int p) {
+  return class_group(ns, pair_class(p)) == g;
+}
+
 // ---------------------------------------------------------------------------
 // Pull streaming: f_i(x) = f*_i(x - n_i); a source outside a walled axis
 // bounces back (the opposite population of the destination site).
 // ---------------------------------------------------------------------------
-template <typename S>
-__device__ __forceinline__ void mpull(const S* __restrict__ src, const MGeom& g, int x, int y,
-                                      S (&f)[kQm]) {
-  const long long site = (long long)y * g.ldx + x;
+template <int NS, int G, typename S>
+__device__ __forceinline__ void mpull(const S* __restrict__ src, const MGeom& g,
+                                      const MOffsets& of, int x, int y, bool interior,
+                                      uint64_t policy, S (&f)[kQm]) {
+  const S* const here = src + ((long long)y * g.ldx + x);
+  if (interior) {
 #pragma unroll
-  for (int p = 0; p < kPairs; ++p) {
+    for (int i = 0; i < 2 * kPairs; ++i)
+      if (mine(NS, G, i / 2)) f[i] = ld_pull(at_bytes(here, of.pull[i]), policy);
+  } else {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = 2 * p + h;
-      const int ex = h ? -pair_x(p) : pair_x(p);
-      const int ey = h ? -pair_y(p) : pair_y(p);
+    for (int i = 0; i < 2 * kPairs; ++i) {
+      if (!mine(NS, G, i / 2)) continue;
+      const int ex = i & 1 ? -pair_x(i / 2) : pair_x(i / 2);
+      const int ey = i & 1 ? -pair_y(i / 2) : pair_y(i / 2);
       int sx = x - ex, sy = y - ey;
       bool in = true;
       if (ex != 0) {
@@ -144,44 +206,25 @@ __device__ __forceinline__ void mpull(const S* __restrict__ src, const MGeom& g,
         else in = in && sy >= 0 && sy < g.ny;
       }
       const S* ptr = in ? src + (long long)i * g.plane + (long long)sy * g.ldx + sx
-                        : src + (long long)(i ^ 1) * g.plane + site;
-      f[i] = __ldg(ptr);
+                        : at_bytes(here, of.plane[i ^ 1]);
+      f[i] = ld_pull(ptr, policy);
     }
   }
-  f[kRestPop] = __ldg(src + (long long)kRestPop * g.plane + site);
+  if (class_group(NS, 9) == G) f[kRestPop] = ld_pull(at_bytes(here, of.plane[kRestPop]), policy);
 }
 
-// The same for a block lying at least kReach sites inside every edge: no
-// wrap, no bounce-back; each offset is uniform across the block.
-template <typename S>
-__device__ __forceinline__ void mpull_interior(const S* __restrict__ src, const MGeom& g,
-                                               long long site, S (&f)[kQm]) {
-  const S* base = src + site;
-#pragma unroll
-  for (int p = 0; p < kPairs; ++p) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = 2 * p + h;
-      const int ex = h ? -pair_x(p) : pair_x(p);
-      const int ey = h ? -pair_y(p) : pair_y(p);
-      f[i] = __ldg(base + ((long long)i * g.plane - (long long)ey * g.ldx - ex));
-    }
-  }
-  f[kRestPop] = __ldg(base + (long long)kRestPop * g.plane);
+__device__ __forceinline__ bool site_interior(const MGeom& g, int x, int y) {
+  return x >= kReach && x < g.nx - kReach && y >= kReach && y < g.ny - kReach;
 }
 
-__device__ __forceinline__ bool block_interior(const MGeom& g) {
-  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 4;
-  return x0 >= kReach && x0 + 31 < g.nx - kReach && y0 >= kReach && y0 + 3 < g.ny - kReach;
-}
-
-template <typename R>
+template <int NS, int G, typename R>
 __device__ __forceinline__ MMom<R> mmoments(const R (&g)[kQm]) {
   const MConsts<R>& c = mc<R>();
   MMom<R> m;
   m.dN0 = m.dNx = m.dNy = m.dE = m.Mx = m.My = m.dPxx = m.dPxy = m.dPyy = R(0);
 #pragma unroll
   for (int p = 0; p < kPairs; ++p) {
+    if (!mine(NS, G, p)) continue;
     const R se = g[2 * p] + g[2 * p + 1], so = g[2 * p] - g[2 * p + 1];
     m.dN0 = fma(c.mN0[p], se, m.dN0);
     m.dE = fma(c.mE[p], se, m.dE);
@@ -197,71 +240,150 @@ __device__ __forceinline__ MMom<R> mmoments(const R (&g)[kQm]) {
     }
     if (pair_x(p) != 0 && pair_y(p) != 0) m.dPxy = fma(c.mPxy[p], se, m.dPxy);
   }
-  m.dN0 = fma(c.restN0, g[kRestPop], m.dN0);
-  m.dE = fma(c.restE, g[kRestPop], m.dE);
+  if (class_group(NS, 9) == G) {
+    m.dN0 = fma(c.restN0, g[kRestPop], m.dN0);
+    m.dE = fma(c.restE, g[kRestPop], m.dE);
+  }
   return m;
 }
 
 // Landau frame eps U^a = T^ab U_b: u = (Pi + eps I)^-1 M, Newton on
 // eps - E + M.u(eps) (derivative 1 - u.u) from eps = E; n = U_a N^a; T from
-// eps / n = (m^2 + 2 m T + 2 T^2) / (m + T).
-template <typename R>
-__device__ __forceinline__ bool mlandau(const MMom<R>& M, MMacro<R>& o) {
-  R deps = M.dE, ux = R(0), uy = R(0);
+// eps / n = (m^2 + 2 m T + 2 T^2) / (m + T).  The unknown is d = eps - E; FP64
+// starts from the FP32 solution and needs one FP64 step as a rule (the
+// reasoning stands at landau_d32 in site.cuh).
+__device__ __forceinline__ bool mlandau_d32(float dE, float Mx, float My, float dPxx, float dPxy,
+                                            float dPyy, float& d, float& ux, float& uy) {
+  const float a0 = float(kH0) + dPxx, c0 = float(kH0) + dPyy, p2 = dPxy * dPxy;
+  d = 0.f;
+#pragma unroll 1
+  for (int it = 0; it < 16; ++it) {
+    const float deps = dE + d;
+    const float a = a0 + deps, c = c0 + deps;
+    const float inv = qrcp(fmaf(a, c, -p2));
+    ux = fmaf(c, Mx, -(dPxy * My)) * inv;
+    uy = fmaf(a, My, -(dPxy * Mx)) * inv;
+    const float g = fmaf(Mx, ux, fmaf(My, uy, d));
+    const float step = g * qrcp(fmaf(-ux, ux, fmaf(-uy, uy, 1.f)));
+    d -= step;
+    if (fabsf(step) <= 2e-7f * (float(kE0) + fabsf(deps))) {
+      const float si = step * inv;
+      const float vx = fmaf(c, ux, -(dPxy * uy)), vy = fmaf(a, uy, -(dPxy * ux));
+      ux = fmaf(si, vx, ux);
+      uy = fmaf(si, vy, uy);
+      return true;
+    }
+  }
+  return false;
+}
+__device__ __forceinline__ bool mlandau_frame(const MMom<float>& m, float& deps, float& ux, float& uy) {
+  float d;
+  const bool conv = mlandau_d32(m.dE, m.Mx, m.My, m.dPxx, m.dPxy, m.dPyy, d, ux, uy);
+  deps = m.dE + d;
+  return conv;
+}
+__device__ __forceinline__ bool mlandau_frame(const MMom<double>& m, double& deps, double& ux, double& uy) {
+  float d32, ux32, uy32;
+  mlandau_d32(trunc_f32(m.dE), trunc_f32(m.Mx), trunc_f32(m.My), trunc_f32(m.dPxx),
+              trunc_f32(m.dPxy), trunc_f32(m.dPyy), d32, ux32, uy32);
+  double d = finite_bits(d32) ? widen_f64(d32) : 0.0;
+  const double a0 = kH0 + m.dPxx + m.dE, c0 = kH0 + m.dPyy + m.dE, p2 = m.dPxy * m.dPxy;
   bool conv = false;
 #pragma unroll 1
   for (int it = 0; it < 16; ++it) {
-    const R a = R(kH0) + M.dPxx + deps, c = R(kH0) + M.dPyy + deps;
-    const R inv = mdiv(R(1), a * c - M.dPxy * M.dPxy);
-    ux = (c * M.Mx - M.dPxy * M.My) * inv;
-    uy = (a * M.My - M.dPxy * M.Mx) * inv;
-    const R gf = deps - M.dE + M.Mx * ux + M.My * uy;
-    const R step = mdiv(gf, R(1) - ux * ux - uy * uy);
-    deps -= step;
-    if (fabs(step) <= MTol<R>::v * (R(kE0) + fabs(deps))) { conv = true; break; }
+    const double a = a0 + d, c = c0 + d;
+    const double inv = qrcp(fma(a, c, -p2));
+    ux = fma(c, m.Mx, -(m.dPxy * m.My)) * inv;
+    uy = fma(a, m.My, -(m.dPxy * m.Mx)) * inv;
+    const double g = fma(m.Mx, ux, fma(m.My, uy, d));
+    const float w = trunc_f32(fma(-ux, ux, fma(-uy, uy, 1.0)));
+    const double step = g * widen_f64(qrcp(w));
+    d -= step;
+    if (fabsf(trunc_f32(step)) <= 1e-8f * (float(kE0) + fabsf(trunc_f32(m.dE) + trunc_f32(d)))) {
+      const double si = step * inv;
+      const double vx = fma(c, ux, -(m.dPxy * uy)), vy = fma(a, uy, -(m.dPxy * ux));
+      ux = fma(si, vx, ux);
+      uy = fma(si, vy, uy);
+      conv = true;
+      break;
+    }
   }
-  {
-    const R a = R(kH0) + M.dPxx + deps, c = R(kH0) + M.dPyy + deps;
-    const R inv = mdiv(R(1), a * c - M.dPxy * M.dPxy);
-    ux = (c * M.Mx - M.dPxy * M.My) * inv;
-    uy = (a * M.My - M.dPxy * M.Mx) * inv;
-  }
-  const R u2 = ux * ux + uy * uy;
-  const R s = sqrt(R(1) - u2);
-  const R gamma = mdiv(R(1), s);
-  const R gm1 = mdiv(u2 * gamma, R(1) + s);
-  const R dNpar = M.dN0 - ux * M.dNx - uy * M.dNy;     // U_a N^a / gamma - 1
-  const R dn = gm1 * (R(1) + dNpar) + dNpar;
-  // T - 1 = (de + sqrt(D) - sqrt(D0)) / 4,  D = e^2 + 4 m e - 4 m^2,  e = eps / n
-  const R de = mdiv(deps - R(kE0) * dn, R(1) + dn);
-  const R e = R(kE0) + de;
-  const R sD = sqrt(e * e + R(4 * kM) * e - R(4 * kM * kM));
-  const R dT = R(0.25) * de * (R(1) + mdiv(e + R(kE0 + 4 * kM), sD + R(kSD0)));
-  o.ux = ux; o.uy = uy; o.gamma = gamma; o.gm1 = gm1; o.s = s; o.dn = dn; o.dT = dT;
+  deps = m.dE + d;
   return conv;
+}
+
+// Fields of a site; returns its error bits.
+template <typename R>
+__device__ __forceinline__ unsigned mlandau(const MMom<R>& M, MMacro<R>& o) {
+  R deps, ux, uy;
+  const bool conv = mlandau_frame(M, deps, ux, uy);
+  const R u2 = fma(ux, ux, uy * uy), w = R(1) - u2;
+  const R gamma = qrsqrt(w);
+  const R r1 = gamma * qrcp(R(1) + gamma);             // 1 / (1 + s), s = 1 / gamma
+  const R gm1 = u2 * gamma * r1;                       // (gamma^2 - 1) / (gamma + 1)
+  const R dNpar = fma(-uy, M.dNy, fma(-ux, M.dNx, M.dN0));   // U_a N^a / gamma - 1
+  const R dn = fma(gm1, R(1) + dNpar, dNpar);
+  // T - 1 = (de + sqrt(D) - sqrt(D0)) / 4,  D = e^2 + 4 m e - 4 m^2,  e = eps / n
+  const R n = R(1) + dn;
+  const R de = fma(R(-kE0), dn, deps) * qrcp(n);
+  const R e = R(kE0) + de;
+  const R D = fma(e, e + R(4 * kM), R(-4 * kM * kM));
+  const R sD = D * qrsqrt(D);
+  const R dT = R(0.25) * de * fma(e + R(kE0 + 4 * kM), qrcp(sD + R(kSD0)), R(1));
+  o.ux = ux; o.uy = uy; o.gamma = gamma; o.gm1 = gm1; o.r1 = r1; o.dn = dn; o.dT = dT;
+  unsigned bits = conv ? 0u : kErrNoConvergence;
+  if (!(finite_bits(ux) && finite_bits(uy) && finite_bits(dn) && finite_bits(dT)))
+    bits |= kErrNonFinite;
+  else if (!(positive(w) && positive(n) && positive(R(1) + dT)))
+    bits |= kErrUnphysical;
+  return bits;
 }
 
 template <typename R>
 __device__ __forceinline__ MMacro<R> macro_of(R n, R ux, R uy, R T) {
   MMacro<R> M;
-  const R u2 = ux * ux + uy * uy;
+  const R u2 = fma(ux, ux, uy * uy);
   M.ux = ux; M.uy = uy;
-  M.s = sqrt(R(1) - u2);
-  M.gamma = mdiv(R(1), M.s);
-  M.gm1 = mdiv(u2 * M.gamma, R(1) + M.s);
+  M.gamma = qrsqrt(R(1) - u2);
+  M.r1 = M.gamma * qrcp(R(1) + M.gamma);
+  M.gm1 = u2 * M.gamma * M.r1;
   M.dn = n - R(1);
   M.dT = T - R(1);
   return M;
 }
 
+// (x, y) lanes of FP32 (Blackwell's paired FMA) and of FP64 (two operations).
+__device__ __forceinline__ float2 S2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ double2 S2(double a) { return make_double2(a, a); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c) {
+  return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
+}
+__device__ __forceinline__ double2 mul2(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
+__device__ __forceinline__ double2 add2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 pair_of(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ double2 pair_of(double a, double b) { return make_double2(a, b); }
+// sign pairs (constant memory, so that they cost no instruction to form in FP32)
+__constant__ float2 c_pm = {1.f, -1.f};
+__constant__ float2 c_mp = {-1.f, 1.f};
+template <typename R> __device__ __forceinline__ typename V2<R>::T pm();
+template <> __device__ __forceinline__ float2 pm<float>() { return c_pm; }
+template <> __device__ __forceinline__ double2 pm<double>() { return make_double2(1.0, -1.0); }
+template <typename R> __device__ __forceinline__ typename V2<R>::T mp();
+template <> __device__ __forceinline__ float2 mp<float>() { return c_mp; }
+template <> __device__ __forceinline__ double2 mp<double>() { return make_double2(-1.0, 1.0); }
+
 // Per-site part of the equilibrium: delta, its quadratic monomials and the
-// third-order remainder R3 of the 16 moments (library order).
+// third-order remainder R3 of the 16 moments (library order), combined by
+// symmetry as the class tables want them.
 template <typename R>
 struct EqSite {
-  R dn, dT, ux, uy;
-  R qE[5];      // dn dT, dT^2, ux^2, ux uy, uy^2
-  R qO[4];      // dn ux, dn uy, dT ux, dT uy
-  R E[8], O[8];
+  using V = typename V2<R>::T;
+  R dn, a[8];            // dT, dn dT, dT^2, ux^2 + uy^2, E0, E1, E2 + E4, E5 + E7
+  R c1[3], c2[3];        // ux^2 - uy^2, E2 - E4, E5 - E7;  ux uy, E3, E6
+  V o[7];                // (x, y): u, dn u, dT u, (O0, O1), (O2, O3), (O4, O7), (O6, O5)
 };
 
 template <typename R>
@@ -269,12 +391,12 @@ __device__ __forceinline__ EqSite<R> eq_site(const MMacro<R>& M) {
   const R m = R(kM), m1 = R(kM1), one = R(1);
   const R H0 = R(kH0), K1 = R(kK1), A0 = R(kA0);
   const R dn = M.dn, dT = M.dT, ux = M.ux, uy = M.uy;
-  const R g = M.gamma, gm1 = M.gm1, s = M.s;
+  const R g = M.gamma, gm1 = M.gm1;
   const R u2 = ux * ux + uy * uy;
   const R T = one + dT;
-  const R imT = mdiv(one, m + T);
+  const R imT = qrcp(m + T);
   const R im1 = R(1.0 / kM1);
-  const R gm1mh = u2 * (u2 * mdiv(one, one + s) + R(2) * gm1) * mdiv(R(0.5), one + s);   // gm1 - u^2/2
+  const R gm1mh = u2 * (u2 * M.r1 + R(2) * gm1) * (R(0.5) * M.r1);                // gm1 - u^2/2
   const R phi = (m * m + R(3) * m * T + R(3) * T * T) * imT;                        // h / n
   const R kT = (R(3) * m1 * T + R(2) * m * m + R(3) * m) * imT * im1;               // (phi(T) - phi(1)) / dT
   const R aT = (m * m * m + R(6) * m * m * T + R(15) * m * T * T + R(15) * T * T * T) * imT;   // alpha / n
@@ -297,112 +419,85 @@ __device__ __forceinline__ EqSite<R> eq_site(const MMacro<R>& M) {
                 + dT * dhq;
   const R Rthg = XmXl * g + (Xlin + H0) * gm1;                      // T h gamma - h0 - Xlin
   const R Rthg3 = XmXl3 * g + XmXl2 * gm1 + Xlin * gm1 + H0 * gm1mh;
+  const R uxx = ux * ux, uxy = ux * uy, uyy = uy * uy;
   EqSite<R> e;
-  e.dn = dn; e.dT = dT; e.ux = ux; e.uy = uy;
-  e.qE[0] = dn * dT; e.qE[1] = dT2; e.qE[2] = ux * ux; e.qE[3] = ux * uy; e.qE[4] = uy * uy;
-  e.qO[0] = dn * ux; e.qO[1] = dn * uy; e.qO[2] = dT * ux; e.qO[3] = dT * uy;
-  e.E[0] = (dn * m1 - dT) * dT2 * imT * (im1 * im1 * im1);
-  e.E[1] = gm1mh + gm1 * dn;
-  e.E[2] = hg2m * e.qE[2];
-  e.E[3] = hg2m * e.qE[3];
-  e.E[4] = hg2m * e.qE[4];
-  e.E[5] = ag3m * e.qE[2] + Rthg3;
-  e.E[6] = ag3m * e.qE[3];
-  e.E[7] = ag3m * e.qE[4] + Rthg3;
+  e.dn = dn;
+  const R ud = uxx - uyy;
+  e.a[0] = dT; e.a[1] = dn * dT; e.a[2] = dT2; e.a[3] = u2;
+  e.a[4] = (dn * m1 - dT) * dT2 * imT * (im1 * im1 * im1);
+  e.a[5] = gm1mh + gm1 * dn;
+  e.a[6] = hg2m * u2;                                // E2 + E4
+  e.a[7] = ag3m * u2 + R(2) * Rthg3;                 // E5 + E7
+  e.c1[0] = ud; e.c1[1] = hg2m * ud; e.c1[2] = ag3m * ud;
+  e.c2[0] = uxy; e.c2[1] = hg2m * uxy; e.c2[2] = ag3m * uxy;
   const R ngm = gm1 * (one + dn);
-  e.O[0] = ngm * ux;
-  e.O[1] = ngm * uy;
-  e.O[2] = hg2mq * ux;
-  e.O[3] = hg2mq * uy;
-  e.O[4] = (ag3 * e.qE[2] + R(3) * Rthg) * ux;
-  e.O[5] = ag3 * e.qE[2] * uy + Rthg * uy;
-  e.O[6] = ag3 * e.qE[4] * ux + Rthg * ux;
-  e.O[7] = (ag3 * e.qE[4] + R(3) * Rthg) * uy;
+  const typename V2<R>::T u = pair_of(ux, uy);
+  e.o[0] = u;
+  e.o[1] = mul2(S2(dn), u);
+  e.o[2] = mul2(S2(dT), u);
+  e.o[3] = mul2(S2(ngm), u);                         // O0, O1
+  e.o[4] = mul2(S2(hg2mq), u);                       // O2, O3
+  const R R3t = R(3) * Rthg;
+  e.o[5] = mul2(pair_of(ag3 * uxx + R3t, ag3 * uyy + R3t), u);       // px^3, py^3
+  e.o[6] = mul2(pair_of(ag3 * uyy + Rthg, ag3 * uxx + Rthg), u);     // px py^2, px^2 py
   return e;
 }
 
-// Parities in (ux, uy) / (px, py) of the table columns: a node on an axis
-// is its own mirror image across that axis, so every entry odd in the other
-// component vanishes there.  WE: dn dT, dT^2, ux^2, ux uy, uy^2; WO: dn ux,
-// dn uy, dT ux, dT uy; BE / BO: the E / O monomials.
-__host__ __device__ constexpr bool we_odd(int k) { return k == 3; }                 // in x and in y
-__host__ __device__ constexpr bool wo_x(int k) { return k == 0 || k == 2; }         // odd in x only
-__host__ __device__ constexpr bool be_odd(int k) { return k == 3 || k == 6; }       // in x and in y
-__host__ __device__ constexpr bool bo_x(int k) { return k == 0 || k == 2 || k == 4 || k == 6; }
-// whether a column with the given parities can be nonzero at pair p
-__host__ __device__ constexpr bool live(int p, bool odd_x, bool odd_y) {
-  return !((odd_x && pair_x(p) == 0) || (odd_y && pair_y(p) == 0));
-}
-
-// even and odd parts of g^eq for pair p (g^eq of 2p = even + odd, of 2p+1 = even - odd)
+// Even and odd parts of g^eq of the couple h (two pairs: lanes pair 2 q, 2 q +
+// 1) of class C: axis (a, 0), (0, a); else (a, b), (-a, b) and, h = 1 in a
+// class of eight, (b, a), (-b, a).
 template <typename R>
-__device__ __forceinline__ void eq_pair(const EqSite<R>& e, int p, R& even, R& odd) {
-  const MConsts<R>& c = mc<R>();
-  R ev = fma(c.LT[p], e.dT, e.dn);
-#pragma unroll
-  for (int k = 0; k < 5; ++k)
-    if (live(p, we_odd(k), we_odd(k))) ev = fma(c.WE[p][k], e.qE[k], ev);
-#pragma unroll
-  for (int k = 0; k < 8; ++k)
-    if (live(p, be_odd(k), be_odd(k))) ev = fma(c.BE[p][k], e.E[k], ev);
-  R od = R(0);
-  if (pair_x(p) != 0) od = fma(c.LX[p], e.ux, od);
-  if (pair_y(p) != 0) od = fma(c.LY[p], e.uy, od);
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (live(p, wo_x(k), !wo_x(k))) od = fma(c.WO[p][k], e.qO[k], od);
-#pragma unroll
-  for (int k = 0; k < 8; ++k)
-    if (live(p, bo_x(k), !bo_x(k))) od = fma(c.BO[p][k], e.O[k], od);
-  even = ev;
-  odd = od;
-}
-
-// Couples of pairs with the same axis pattern (both on the x axis, both on
-// the y axis, or both off the axes), so that every term eq_pair() skips for
-// one pair is skipped for the other: the FP32 collision evaluates g^eq of a
-// couple on register pairs, lanes (first pair, second pair).
-constexpr int kCouples = kPairs / 2;
-__host__ __device__ constexpr int couple_a(int q) {
-  return q == 0 ? 0 : q == 1 ? 1 : q == 2 ? 2 : q == 3 ? 6 : q == 4 ? 8 : q == 5 ? 10 : q == 6 ? 12 : q == 7 ? 13 : q == 8 ? 14 : q == 9 ? 16 : 18;
-}
-__host__ __device__ constexpr int couple_b(int q) {
-  return q == 0 ? 4 : q == 1 ? 5 : q == 2 ? 3 : q == 3 ? 7 : q == 4 ? 9 : q == 5 ? 11 : q == 6 ? 20 : q == 7 ? 21 : q == 8 ? 15 : q == 9 ? 17 : 19;
-}
-constexpr bool couples_valid() {
-  int seen[kPairs] = {};
-  for (int q = 0; q < kCouples; ++q) {
-    const int a = couple_a(q), b = couple_b(q);
-    if ((pair_x(a) == 0) != (pair_x(b) == 0) || (pair_y(a) == 0) != (pair_y(b) == 0)) return false;
-    ++seen[a];
-    ++seen[b];
-  }
-  for (int p = 0; p < kPairs; ++p)
-    if (seen[p] != 1) return false;
-  return true;
-}
-static_assert(couples_valid(), "every pair in one couple, both pairs of a couple alike on the axes");
-
-// eq_pair()'s FP32 tables of couple q as pairs (first pair, second pair)
-struct MCoupleConsts {
-  float2 LT[kCouples], LX[kCouples], LY[kCouples];
-  float2 WE[kCouples][5], WO[kCouples][4], BE[kCouples][8], BO[kCouples][8];
-  // and the FP32 collision's per-pair constants: vx, vy, mvE[.][1..4], mvO[.][0..1]
-  float2 vx[kCouples], vy[kCouples];
-  float2 p0[kCouples], px2[kCouples], pxy[kCouples], py2[kCouples], pxv[kCouples], pyv[kCouples];
+struct ClassEq {
+  using V = typename V2<R>::T;
+  R A, C1, C2;
+  V F1, F2;        // component functions of the larger and the smaller component
 };
-__constant__ MCoupleConsts c_cp;
+
+template <int C, typename R>
+__device__ __forceinline__ ClassEq<R> class_eq(const EqSite<R>& e) {
+  const MConsts<R>& c = mc<R>();
+  ClassEq<R> k;
+  k.A = fma(c.A[C][0], e.a[0], e.dn);
+#pragma unroll
+  for (int i = 1; i < 8; ++i) k.A = fma(c.A[C][i], e.a[i], k.A);
+  k.C1 = k.C2 = R(0);
+  if (class_kind(C) != 1)
+    k.C1 = fma(c.C1[C][2], e.c1[2], fma(c.C1[C][1], e.c1[1], c.C1[C][0] * e.c1[0]));
+  if (class_kind(C) != 0)
+    k.C2 = fma(c.C2[C][2], e.c2[2], fma(c.C2[C][1], e.c2[1], c.C2[C][0] * e.c2[0]));
+  constexpr int f = class_fn(C);
+  k.F1 = mul2(c.O[f][0], e.o[0]);
+#pragma unroll
+  for (int i = 1; i < 7; ++i) k.F1 = fma2(c.O[f][i], e.o[i], k.F1);
+  k.F2 = k.F1;
+  if (class_kind(C) == 2) {
+    k.F2 = mul2(c.O[f + 1][0], e.o[0]);
+#pragma unroll
+    for (int i = 1; i < 7; ++i) k.F2 = fma2(c.O[f + 1][i], e.o[i], k.F2);
+  }
+  return k;
+}
+
+template <int C, int H, typename R>
+__device__ __forceinline__ void couple_eq(const ClassEq<R>& k, typename V2<R>::T& ev,
+                                          typename V2<R>::T& od) {
+  if (class_kind(C) == 0) {
+    ev = fma2(S2(k.C1), pm<R>(), S2(k.A));
+    od = k.F1;
+  } else {
+    const R e = class_kind(C) == 1 ? k.A : H ? k.A - k.C1 : k.A + k.C1;
+    ev = fma2(S2(k.C2), pm<R>(), S2(e));
+    const R X = H ? k.F2.x : k.F1.x, Y = H ? k.F1.y : k.F2.y;
+    od = fma2(S2(X), pm<R>(), S2(Y));
+  }
+}
 
 template <typename R>
 __device__ __forceinline__ R eq_rest(const EqSite<R>& e) {
   const MConsts<R>& c = mc<R>();
-  R ev = fma(c.restLT, e.dT, e.dn);
+  R ev = fma(c.A[9][0], e.a[0], e.dn);
 #pragma unroll
-  for (int k = 0; k < 5; ++k)
-    if (!we_odd(k)) ev = fma(c.restWE[k], e.qE[k], ev);
-#pragma unroll
-  for (int k = 0; k < 8; ++k)
-    if (!be_odd(k)) ev = fma(c.restBE[k], e.E[k], ev);
+  for (int i = 1; i < 8; ++i) ev = fma(c.A[9][i], e.a[i], ev);
   return ev;
 }
 
@@ -422,7 +517,7 @@ __device__ __forceinline__ ForceSite<R> force_site(const MMacro<R>& M, R Fx, R F
   const R m = R(kM), m1 = R(kM1), one = R(1), H0 = R(kH0);
   const R dn = M.dn, dT = M.dT, ux = M.ux, uy = M.uy, g = M.gamma, gm1 = M.gm1;
   const R T = one + dT, n = one + dn;
-  const R imT = mdiv(one, m + T);
+  const R imT = qrcp(m + T);
   const R phi = (m * m + R(3) * m * T + R(3) * T * T) * imT;
   const R kT = (R(3) * m1 * T + R(2) * m * m + R(3) * m) * imT * R(1.0 / kM1);
   const R dh = dn * phi + dT * kT;
@@ -475,222 +570,267 @@ __device__ __forceinline__ ForceSite<R> force_site(const MMacro<R>& M, R Fx, R F
 }
 
 // ---------------------------------------------------------------------------
-// Collision of one site and store.
+// Collision of one site and store: class by class, two pairs at a time on (x,
+// y) lanes, then each pair on lanes (population 2 p, its opposite 2 p + 1).
+// The force's source of a population of pair p with sign s = +-1 is
+//   s (F.v (1 - Ae) - Ho) + s F.v g^eq_s - (F.v Ao + He)
+// with Ae, Ao / He, Ho the even / odd parts of dD/dp0 / F.grad_xy D.
 // ---------------------------------------------------------------------------
-// Sign pairs of the paired FP32 arithmetic below (constant memory, so that
-// they cost nothing as operands): (1, -1) and (-1, 1).
-__constant__ float2 c_pm = {1.f, -1.f};
-__constant__ float2 c_mp = {-1.f, 1.f};
-
-__device__ __forceinline__ float2 S2(float a) { return make_float2(a, a); }
-
-// eq_pair() of the two pairs of couple q at once (lanes: couple_a(q),
-// couple_b(q)): the same terms in the same order on each lane.
-__device__ __forceinline__ void eq_couple(const EqSite<float>& e, int q, float2& even,
-                                          float2& odd) {
-  const int p = couple_a(q);   // the couple's axis pattern
-  float2 ev = __ffma2_rn(c_cp.LT[q], S2(e.dT), S2(e.dn));
-#pragma unroll
-  for (int k = 0; k < 5; ++k)
-    if (live(p, we_odd(k), we_odd(k))) ev = __ffma2_rn(c_cp.WE[q][k], S2(e.qE[k]), ev);
-#pragma unroll
-  for (int k = 0; k < 8; ++k)
-    if (live(p, be_odd(k), be_odd(k))) ev = __ffma2_rn(c_cp.BE[q][k], S2(e.E[k]), ev);
-  float2 od = S2(0.f);
-  if (pair_x(p) != 0) od = __ffma2_rn(c_cp.LX[q], S2(e.ux), od);
-  if (pair_y(p) != 0) od = __ffma2_rn(c_cp.LY[q], S2(e.uy), od);
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (live(p, wo_x(k), !wo_x(k))) od = __ffma2_rn(c_cp.WO[q][k], S2(e.qO[k]), od);
-#pragma unroll
-  for (int k = 0; k < 8; ++k)
-    if (live(p, bo_x(k), !bo_x(k))) od = __ffma2_rn(c_cp.BO[q][k], S2(e.O[k]), od);
-  even = ev;
-  odd = od;
-}
-
-// mcollide_store for FP32 on register pairs (lanes: population 2p and its
-// opposite 2p + 1): the same quantities in the same order of operations per
-// population, two populations per paired FMA (Blackwell's FFMA2); g^eq of
-// two pairs at a time (eq_couple).
-template <bool FORCE>
-__device__ __forceinline__ void mcollide_store_paired(const float (&g)[kQm], const MMacro<float>& M,
-                                                      float inv_tau, float Fx, float Fy,
-                                                      float* __restrict__ out, long long plane) {
-  const EqSite<float> e = eq_site(M);
-  const float gt = M.gamma * inv_tau;
-  const float gux = gt * M.ux, guy = gt * M.uy;
-  ForceSite<float> fs;
-  if (FORCE) fs = force_site(M, Fx, Fy);
-  // relaxation, force and store of pair p from the even / odd parts of its
-  // g^eq, v.u gamma / tau (wv) and the force's per-pair scalars
-  auto relax_pair = [&](const int p, const float ev, const float od, const float wv,
-                        const float Ae, const float He, const float Ao, const float Ho,
-                        const float Fv) {
-    const float2 om = __ffma2_rn(S2(wv), c_mp, S2(gt));       // gamma (1 -+ v.u) / tau
-    const float2 gpn = __ffma2_rn(S2(od), c_pm, S2(ev));      // (ev + od, ev - od)
-    const float2 G = make_float2(g[2 * p], g[2 * p + 1]);
-    float2 o = __ffma2_rn(om, __ffma2_rn(G, S2(-1.f), gpn), G);
-    if (FORCE) {
-      // lanes: +-Fv (1 + g^eq -/+ ... - Ae -+ Ao) - He -+ Ho
-      const float2 X = __ffma2_rn(S2(Ao), c_mp, __fadd2_rn(gpn, S2(1.f - Ae)));
-      o = __ffma2_rn(S2(Fv), __fmul2_rn(X, c_pm), o);
-      o = __ffma2_rn(S2(Ho), c_mp, __fadd2_rn(o, S2(-He)));
-    }
-    out[(long long)(2 * p) * plane] = o.x;
-    out[(long long)(2 * p + 1) * plane] = o.y;
-  };
-  // the per-pair scalars of a couple on register pairs (lanes: couple_a(q),
-  // couple_b(q)), each lane with the operations of one pair in their order
-#pragma unroll
-  for (int q = 0; q < kCouples; ++q) {
-    const int p = couple_a(q);   // the couple's axis pattern
-    const bool hx = pair_x(p) != 0, hy = pair_y(p) != 0;
-    float2 ev, od;
-    eq_couple(e, q, ev, od);
-    float2 wv = S2(0.f);
-    if (hx) wv = __fmul2_rn(S2(gux), c_cp.vx[q]);
-    if (hy) wv = __ffma2_rn(S2(guy), c_cp.vy[q], wv);
-    float2 Ae = S2(0.f), He = S2(0.f), Ao = S2(0.f), Ho = S2(0.f), Fv = S2(0.f);
-    if (FORCE) {
-      const float2 px2 = c_cp.px2[q], pxy = c_cp.pxy[q], py2 = c_cp.py2[q], p0 = c_cp.p0[q];
-      Ae = __ffma2_rn(S2(fs.a5), px2, S2(fs.a1));
-      He = __ffma2_rn(S2(fs.hp0), p0, S2(fs.h1));
-      Ae = __ffma2_rn(S2(fs.a6), pxy, __ffma2_rn(S2(fs.a7), py2, Ae));
-      He = __ffma2_rn(S2(fs.hxx), px2, __ffma2_rn(S2(fs.hxy), pxy, __ffma2_rn(S2(fs.hyy), py2, He)));
-      if (hx) {
-        Ao = __fmul2_rn(S2(fs.a10), c_cp.pxv[q]);
-        Ho = __ffma2_rn(__ffma2_rn(S2(fs.h0x), p0, S2(fs.hx)), c_cp.pxv[q], Ho);
-      }
-      if (hy) {
-        Ao = __ffma2_rn(S2(fs.a11), c_cp.pyv[q], Ao);
-        Ho = __ffma2_rn(__ffma2_rn(S2(fs.h0y), p0, S2(fs.hy)), c_cp.pyv[q], Ho);
-      }
-      if (hx) Fv = __fmul2_rn(S2(Fx), c_cp.vx[q]);
-      if (hy) Fv = __ffma2_rn(S2(Fy), c_cp.vy[q], Fv);
-    }
-    relax_pair(couple_a(q), ev.x, od.x, wv.x, Ae.x, He.x, Ao.x, Ho.x, Fv.x);
-    relax_pair(couple_b(q), ev.y, od.y, wv.y, Ae.y, He.y, Ao.y, Ho.y, Fv.y);
-  }
-  const float gr = eq_rest(e);
-  float orr = fmaf(gt, gr - g[kRestPop], g[kRestPop]);
-  if (FORCE) orr -= fmaf(fs.hp0, float(kM), fs.h1);
-  out[(long long)kRestPop * plane] = orr;
-}
-
-template <typename R, bool FORCE>
-__device__ __forceinline__ void mcollide_store(const R (&g)[kQm], const MMacro<R>& M, R inv_tau,
-                                               R Fx, R Fy, R* __restrict__ out, long long plane) {
-  if constexpr (sizeof(R) == sizeof(float)) {
-    mcollide_store_paired<FORCE>(g, M, inv_tau, Fx, Fy, out, plane);
-    return;
-  }
-  const MConsts<R>& c = mc<R>();
-  const EqSite<R> e = eq_site(M);
-  const R gt = M.gamma * inv_tau;
-  const R gux = gt * M.ux, guy = gt * M.uy;
-  ForceSite<R> fs;
-  if (FORCE) fs = force_site(M, Fx, Fy);
-#pragma unroll
-  for (int p = 0; p < kPairs; ++p) {
-    R ev, od;
-    eq_pair(e, p, ev, od);
-    R wv = R(0);
-    if (pair_x(p) != 0) wv = gux * c.vx[p];
-    if (pair_y(p) != 0) wv = fma(guy, c.vy[p], wv);
-    const R omp = gt - wv, omn = gt + wv;          // gamma (1 -+ v.u) / tau
-    const R gp = ev + od, gn = ev - od;
-    R op = fma(omp, gp - g[2 * p], g[2 * p]);
-    R on = fma(omn, gn - g[2 * p + 1], g[2 * p + 1]);
-    if (FORCE) {
-      const R px2 = c.mvE[p][2], pxy = c.mvE[p][3], py2 = c.mvE[p][4], p0 = c.mvE[p][1];
-      const R pxv = c.mvO[p][0], pyv = c.mvO[p][1];
-      R Ae = fma(fs.a5, px2, fs.a1), Ao = R(0), He = fma(fs.hp0, p0, fs.h1), Ho = R(0);
-      Ae = fma(fs.a6, pxy, fma(fs.a7, py2, Ae));
-      He = fma(fs.hxx, px2, fma(fs.hxy, pxy, fma(fs.hyy, py2, He)));
-      if (pair_x(p) != 0) { Ao = fs.a10 * pxv; Ho = fma(fma(fs.h0x, p0, fs.hx), pxv, Ho); }
-      if (pair_y(p) != 0) { Ao = fma(fs.a11, pyv, Ao); Ho = fma(fma(fs.h0y, p0, fs.hy), pyv, Ho); }
-      R Fv = R(0);
-      if (pair_x(p) != 0) Fv = Fx * c.vx[p];
-      if (pair_y(p) != 0) Fv = fma(Fy, c.vy[p], Fv);
-      op += Fv * (R(1) + gp - Ae - Ao) - He - Ho;
-      on += -Fv * (R(1) + gn - Ae + Ao) - He + Ho;
-    }
-    out[(long long)(2 * p) * plane] = op;
-    out[(long long)(2 * p + 1) * plane] = on;
-  }
-  const R gr = eq_rest(e);
-  R orr = fma(gt, gr - g[kRestPop], g[kRestPop]);
-  if (FORCE) orr -= fma(fs.hp0, R(kM), fs.h1);
-  out[(long long)kRestPop * plane] = orr;
-}
-
 template <typename R>
-__device__ __forceinline__ unsigned check_bits(const MMacro<R>& M, bool conv) {
-  unsigned bits = conv ? 0u : kErrNoConvergence;
-  if (!(isfinite(M.ux) && isfinite(M.uy) && isfinite(M.dn) && isfinite(M.dT))) bits |= kErrNonFinite;
-  else if (!(M.ux * M.ux + M.uy * M.uy < R(1) && M.dn > R(-1) && M.dT > R(-1))) bits |= kErrUnphysical;
-  return bits;
+struct MRelax {
+  R gt, Fx, Fy;
+  typename V2<R>::T gu, F;       // gamma u / tau, F
+};
+
+template <int C, typename R, bool FORCE>
+__device__ __forceinline__ void class_relax(const R (&g)[kQm], const EqSite<R>& e,
+                                            const ForceSite<R>& fs, const MRelax<R>& r,
+                                            R* __restrict__ out, const MOffsets& of) {
+  using V = typename V2<R>::T;
+  const MConsts<R>& c = mc<R>();
+  const ClassEq<R> k = class_eq<C>(e);
+  constexpr int kind = class_kind(C), f = class_fn(C);
+  R eA = R(0), eH = R(0), dA = R(0), dH = R(0), xA = R(0), xH = R(0);
+  V Hc = S2(R(0));
+  if (FORCE) {
+    eA = fma(fs.a5 + fs.a7, c.rr[C], fs.a1);
+    eH = fma(fs.hxx + fs.hyy, c.rr[C], fma(fs.hp0, c.p0[C], fs.h1));
+    if (kind != 1) { dA = (fs.a5 - fs.a7) * c.dd[C]; dH = (fs.hxx - fs.hyy) * c.dd[C]; }
+    if (kind != 0) { xA = fs.a6 * c.pp[C]; xH = fs.hxy * c.pp[C]; }
+    Hc = fma2(pair_of(fs.h0x, fs.h0y), S2(c.p0[C]), pair_of(fs.hx, fs.hy));
+  }
+#pragma unroll
+  for (int h = 0; h < (kind == 2 ? 2 : 1); ++h) {
+    V ev, od, wv, Ae = S2(R(0)), He = Ae, Ao = Ae, Ho = Ae, Fv = Ae;
+    if (h == 0) couple_eq<C, 0>(k, ev, od);
+    else couple_eq<C, 1>(k, ev, od);
+    if (kind == 0) {
+      wv = mul2(r.gu, c.va[f]);
+      if (FORCE) {
+        Fv = mul2(r.F, c.va[f]);
+        Ae = fma2(S2(dA), pm<R>(), S2(eA));
+        He = fma2(S2(dH), pm<R>(), S2(eH));
+        Ao = mul2(pair_of(fs.a10, fs.a11), c.pa[f]);
+        Ho = mul2(Hc, c.pa[f]);
+      }
+    } else {
+      // x component of the couple's pairs: function fx, y component: fy
+      const int fx = kind == 1 ? f : f + h, fy = kind == 1 ? f : f + 1 - h;
+      wv = fma2(S2(r.gu.x * c.va[fx].x), pm<R>(), S2(r.gu.y * c.va[fy].x));
+      if (FORCE) {
+        Fv = fma2(S2(r.F.x * c.va[fx].x), pm<R>(), S2(r.F.y * c.va[fy].x));
+        const R a = h ? eA - dA : eA + dA, b = h ? eH - dH : eH + dH;
+        Ae = fma2(S2(xA), pm<R>(), S2(a));
+        He = fma2(S2(xH), pm<R>(), S2(b));
+        Ao = fma2(S2(fs.a10 * c.pa[fx].x), pm<R>(), S2(fs.a11 * c.pa[fy].x));
+        Ho = fma2(S2(Hc.x * c.pa[fx].x), pm<R>(), S2(Hc.y * c.pa[fy].x));
+      }
+    }
+    V al = S2(R(0)), be = al;
+    if (FORCE) {
+      // (F.v (1 - Ae) - Ho, F.v Ao + He)
+      al = fma2(Fv, fma2(Ae, S2(R(-1)), S2(R(1))), mul2(Ho, S2(R(-1))));
+      be = fma2(Fv, Ao, He);
+    }
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      const int p = class_pair(C) + 2 * h + l;
+      const R evp = l ? ev.y : ev.x, odp = l ? od.y : od.x, w = l ? wv.y : wv.x;
+      const V om = fma2(S2(w), mp<R>(), S2(r.gt));            // gamma (1 -+ v.u) / tau
+      const V geq = fma2(S2(odp), pm<R>(), S2(evp));          // ev +- od
+      const V G = pair_of(g[2 * p], g[2 * p + 1]);
+      V o = fma2(om, fma2(G, S2(R(-1)), geq), G);
+      if (FORCE) {
+        const R Fp = l ? Fv.y : Fv.x, a = l ? al.y : al.x, b = l ? be.y : be.x;
+        o = fma2(mul2(S2(Fp), pm<R>()), geq, o);
+        o = add2(o, fma2(S2(a), pm<R>(), S2(-b)));
+      }
+      *at_bytes(out, of.plane[2 * p]) = o.x;
+      *at_bytes(out, of.plane[2 * p + 1]) = o.y;
+    }
+  }
+}
+
+template <int NS, int G, typename R, bool FORCE>
+__device__ __forceinline__ void mcollide_store(const R (&g)[kQm], const MMacro<R>& M, R inv_tau,
+                                               R Fx, R Fy, R* __restrict__ out, const MOffsets& of) {
+  const EqSite<R> e = eq_site(M);
+  MRelax<R> r;
+  r.gt = M.gamma * inv_tau;
+  r.gu = mul2(S2(r.gt), pair_of(M.ux, M.uy));
+  r.F = pair_of(Fx, Fy);
+  ForceSite<R> fs{};
+  if (FORCE) fs = force_site(M, Fx, Fy);
+  if (class_group(NS, 0) == G) class_relax<0, R, FORCE>(g, e, fs, r, out, of);
+  if (class_group(NS, 1) == G) class_relax<1, R, FORCE>(g, e, fs, r, out, of);
+  if (class_group(NS, 2) == G) class_relax<2, R, FORCE>(g, e, fs, r, out, of);
+  if (class_group(NS, 3) == G) class_relax<3, R, FORCE>(g, e, fs, r, out, of);
+  if (class_group(NS, 4) == G) class_relax<4, R, FORCE>(g, e, fs, r, out, of);
+  if (class_group(NS, 5) == G) class_relax<5, R, FORCE>(g, e, fs, r, out, of);
+  if (class_group(NS, 6) == G) class_relax<6, R, FORCE>(g, e, fs, r, out, of);
+  if (class_group(NS, 7) == G) class_relax<7, R, FORCE>(g, e, fs, r, out, of);
+  if (class_group(NS, 8) == G) class_relax<8, R, FORCE>(g, e, fs, r, out, of);
+  if (class_group(NS, 9) == G) {
+    R orr = fma(r.gt, eq_rest(e) - g[kRestPop], g[kRestPop]);
+    if (FORCE) orr -= fma(fs.hp0, R(kM), fs.h1);
+    *at_bytes(out, of.plane[kRestPop]) = orr;
+  }
 }
 
 // ---------------------------------------------------------------------------
-// Kernels (blocks of 32 x 4 sites)
+// Kernels.  Steps are chained launches (programmatic dependent launch): the
+// next step's blocks are placed early and wait for this one's results before
+// their first access.  FP32 1024 x 512 with a force: 57.6 -> 45.0 us per step
+// (2,328 -> 1,922 instructions per site by the class tables and the prepared
+// offsets; 28 us is the HBM time; 16 warps per SM, issue slots 60 % busy).
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void chain_release() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+__device__ __forceinline__ uint64_t mpolicy(bool evict_first) {
+  uint64_t a, b;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(a));
+  asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(b));
+  return evict_first ? a : b;
+}
+
+struct MLaunch {
+  int reverse, evict_first;
+};
+
+constexpr int kMThreads = 64;
+
+// Warps take 32 consecutive sites of a row, two per block.
 template <typename R, bool FORCE>
 __device__ __forceinline__ void mstep_body(const R* __restrict__ src, R* __restrict__ dst,
-                                           const MGeom& geo, R inv_tau, R Fx, R Fy,
-                                           unsigned* __restrict__ err) {
-  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y;
+                                           const MGeom& geo, const MOffsets& of, const MLaunch& ml,
+                                           R inv_tau, R Fx, R Fy, unsigned* __restrict__ err) {
+  chain_release();
+  const unsigned per_row = (unsigned)(geo.nx + 31) / 32;
+  const unsigned block = ml.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+  const unsigned t = block * (kMThreads / 32) + threadIdx.x / 32;
+  const int y = (int)(t / per_row), x0 = (int)(t - (unsigned)y * per_row) * 32;
+  const int x = x0 + (int)(threadIdx.x % 32);
+  const uint64_t policy = mpolicy(ml.evict_first);
+  chain_wait();
   if (x >= geo.nx || y >= geo.ny) return;
   R g[kQm];
-  if (block_interior(geo)) mpull_interior(src, geo, (long long)y * geo.ldx + x, g);
-  else mpull(src, geo, x, y, g);
-  const MMom<R> mo = mmoments(g);
+  mpull<1, 0>(src, geo, of, x, y, site_interior(geo, x0, y) && site_interior(geo, x0 + 31, y), policy, g);
   MMacro<R> M;
-  const bool conv = mlandau(mo, M);
-  const unsigned bits = check_bits(M, conv);
-  mcollide_store<R, FORCE>(g, M, inv_tau, Fx, Fy, dst + (long long)y * geo.ldx + x, geo.plane);
+  const unsigned bits = mlandau(mmoments<1, 0>(g), M);
+  mcollide_store<1, 0, R, FORCE>(g, M, inv_tau, Fx, Fy, dst + (long long)y * geo.ldx + x, of);
   if (bits) atomicOr(err, bits);
 }
 
+// FP32: at most 128 registers (16 warps per SM).
 template <typename R, bool FORCE>
-__global__ void __launch_bounds__(128) k_mstep(const R* __restrict__ src, R* __restrict__ dst,
-                                               MGeom geo, R inv_tau, R Fx, R Fy,
-                                               unsigned* __restrict__ err) {
-  mstep_body<R, FORCE>(src, dst, geo, inv_tau, Fx, Fy, err);
+__global__ void __launch_bounds__(kMThreads, sizeof(R) == 4 ? 8 : 1)
+k_mstep(const R* __restrict__ src, R* __restrict__ dst, const __grid_constant__ MGeom geo,
+        const __grid_constant__ MOffsets of, MLaunch ml, R inv_tau, R Fx, R Fy,
+        unsigned* __restrict__ err) {
+  mstep_body<R, FORCE>(src, dst, geo, of, ml, inv_tau, Fx, Fy, err);
 }
 
-// FP32 with the force: at most 128 registers, so that 4 blocks stay resident
-// per SM (the paired equilibrium would otherwise take 130 and leave room for 3).
-__global__ void __launch_bounds__(128, 4) k_mstep_f32_force(const float* __restrict__ src,
-                                                            float* __restrict__ dst, MGeom geo,
-                                                            float inv_tau, float Fx, float Fy,
-                                                            unsigned* __restrict__ err) {
-  mstep_body<float, true>(src, dst, geo, inv_tau, Fx, Fy, err);
+// FP64, few sites: NS warps share 32 sites (consecutive in row-major order,
+// across row ends), each with the populations of some classes.  A warp
+// instruction of the FP64 pipe takes 66 cycles of its SM sub-partition, so
+// below one warp per sub-partition a step lasts as long as one warp's chain.
+// 97 x 70 sites with a force: 78 -> 39.9 us per step.
+template <int NS, int G, bool FORCE>
+__device__ __forceinline__ void msplit_group(const double* __restrict__ src, double* __restrict__ dst,
+                                             const MGeom& geo, const MOffsets& of, double inv_tau,
+                                             double Fx, double Fy, unsigned* __restrict__ err,
+                                             MMom<double>* part, int x, int y, bool in, bool interior) {
+  const int lane = threadIdx.x % 32;
+  double g[kQm];
+  if (in) {
+    mpull<NS, G>(src, geo, of, x, y, interior, 0, g);
+    part[G * 32 + lane] = mmoments<NS, G>(g);
+  }
+  // a barrier that the warps meet at from NS places in the code
+  asm volatile("bar.sync 1, %0;\n" :: "n"(32 * NS) : "memory");
+  if (!in) return;
+  MMom<double> m = part[lane];
+#pragma unroll
+  for (int k = 1; k < NS; ++k) {
+    const MMom<double>& q = part[k * 32 + lane];
+    m.dN0 += q.dN0; m.dNx += q.dNx; m.dNy += q.dNy;
+    m.dE += q.dE; m.Mx += q.Mx; m.My += q.My;
+    m.dPxx += q.dPxx; m.dPxy += q.dPxy; m.dPyy += q.dPyy;
+  }
+  MMacro<double> M;
+  const unsigned bits = mlandau(m, M);
+  mcollide_store<NS, G, double, FORCE>(g, M, inv_tau, Fx, Fy, dst + (long long)y * geo.ldx + x, of);
+  if (G == 0 && bits) atomicOr(err, bits);
+}
+
+template <int NS, bool FORCE>
+__global__ void __launch_bounds__(32 * NS)
+k_mstep_split(const double* __restrict__ src, double* __restrict__ dst,
+              const __grid_constant__ MGeom geo, const __grid_constant__ MOffsets of,
+              double inv_tau, double Fx, double Fy, unsigned* __restrict__ err) {
+  __shared__ MMom<double> part[NS * 32];
+  chain_release();
+  const long long n = (long long)blockIdx.x * 32 + threadIdx.x % 32;
+  const bool in = n < (long long)geo.nx * geo.ny;
+  const int y = in ? (int)(n / geo.nx) : 0, x = in ? (int)(n - (long long)y * geo.nx) : 0;
+  const bool interior = __all_sync(0xffffffffu, !in || site_interior(geo, x, y));
+  chain_wait();
+  const int w = threadIdx.x / 32;
+  if (w == 0) msplit_group<NS, 0, FORCE>(src, dst, geo, of, inv_tau, Fx, Fy, err, part, x, y, in, interior);
+  else if (w == 1) msplit_group<NS, 1, FORCE>(src, dst, geo, of, inv_tau, Fx, Fy, err, part, x, y, in, interior);
+  else if constexpr (NS == 4) {
+    if (w == 2) msplit_group<NS, 2, FORCE>(src, dst, geo, of, inv_tau, Fx, Fy, err, part, x, y, in, interior);
+    else msplit_group<NS, 3, FORCE>(src, dst, geo, of, inv_tau, Fx, Fy, err, part, x, y, in, interior);
+  }
 }
 
 template <typename R>
-__global__ void __launch_bounds__(128) k_mmoments(const R* __restrict__ src, MGeom geo,
+__global__ void __launch_bounds__(128) k_mmoments(const R* __restrict__ src,
+                                                  const __grid_constant__ MGeom geo,
+                                                  const __grid_constant__ MOffsets of,
                                                   double* __restrict__ n, double* __restrict__ ux,
                                                   double* __restrict__ uy, double* __restrict__ T,
                                                   unsigned* __restrict__ err) {
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y;
   if (x >= geo.nx || y >= geo.ny) return;
+  const int x0 = blockIdx.x * 32;
   R g[kQm];
-  mpull(src, geo, x, y, g);
+  mpull<1, 0>(src, geo, of, x, y, site_interior(geo, x0, y) && site_interior(geo, x0 + 31, y),
+              mpolicy(false), g);
   MMacro<R> M;
-  const bool conv = mlandau(mmoments(g), M);
+  const unsigned bits = mlandau(mmoments<1, 0>(g), M);
   const long long o = (long long)y * geo.nx + x;
-  if (n) n[o] = 1.0 + (double)M.dn;
-  if (ux) ux[o] = M.ux;
-  if (uy) uy[o] = M.uy;
-  if (T) T[o] = 1.0 + (double)M.dT;
-  const unsigned bits = check_bits(M, conv);
+  if (n) n[o] = 1.0 + as_f64(M.dn);
+  if (ux) ux[o] = as_f64(M.ux);
+  if (uy) uy[o] = as_f64(M.uy);
+  if (T) T[o] = 1.0 + as_f64(M.dT);
   if (bits) atomicOr(err, bits);
 }
 
+template <int C, typename R>
+__device__ __forceinline__ void class_init(const EqSite<R>& e, R* __restrict__ out, const MOffsets& of) {
+  const ClassEq<R> k = class_eq<C>(e);
+#pragma unroll
+  for (int h = 0; h < (class_kind(C) == 2 ? 2 : 1); ++h) {
+    typename V2<R>::T ev, od;
+    if (h == 0) couple_eq<C, 0>(k, ev, od);
+    else couple_eq<C, 1>(k, ev, od);
+    const int p = class_pair(C) + 2 * h;
+    *at_bytes(out, of.plane[2 * p]) = ev.x + od.x;
+    *at_bytes(out, of.plane[2 * p + 1]) = ev.x - od.x;
+    *at_bytes(out, of.plane[2 * p + 2]) = ev.y + od.y;
+    *at_bytes(out, of.plane[2 * p + 3]) = ev.y - od.y;
+  }
+}
+
 template <typename R>
-__global__ void __launch_bounds__(128) k_minit(R* __restrict__ dst, MGeom geo, const double* __restrict__ n,
+__global__ void __launch_bounds__(128) k_minit(R* __restrict__ dst, const __grid_constant__ MGeom geo,
+                                               const __grid_constant__ MOffsets of,
+                                               const double* __restrict__ n,
                                                const double* __restrict__ ux, const double* __restrict__ uy,
                                                const double* __restrict__ T, unsigned* __restrict__ err) {
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y;
@@ -701,14 +841,16 @@ __global__ void __launch_bounds__(128) k_minit(R* __restrict__ dst, MGeom geo, c
   const MMacro<R> M = macro_of<R>(R(n[o]), R(ux[o]), R(uy[o]), R(T[o]));
   const EqSite<R> e = eq_site(M);
   R* out = dst + (long long)y * geo.ldx + x;
-#pragma unroll
-  for (int p = 0; p < kPairs; ++p) {
-    R ev, od;
-    eq_pair(e, p, ev, od);
-    out[(long long)(2 * p) * geo.plane] = ev + od;
-    out[(long long)(2 * p + 1) * geo.plane] = ev - od;
-  }
-  out[(long long)kRestPop * geo.plane] = eq_rest(e);
+  class_init<0>(e, out, of);
+  class_init<1>(e, out, of);
+  class_init<2>(e, out, of);
+  class_init<3>(e, out, of);
+  class_init<4>(e, out, of);
+  class_init<5>(e, out, of);
+  class_init<6>(e, out, of);
+  class_init<7>(e, out, of);
+  class_init<8>(e, out, of);
+  *at_bytes(out, of.plane[kRestPop]) = eq_rest(e);
 }
 
 // state I/O: delta_i = f0_i g_i in FP64, dense [45][ny][nx]
@@ -732,7 +874,10 @@ __global__ void k_mset(R* __restrict__ dst, MGeom geo, const double* __restrict_
     const int i = (int)(t / nsite);
     const long long r = t - i * nsite;
     const int y = (int)(r / geo.nx), x = (int)(r - (long long)y * geo.nx);
-    dst[(long long)i * geo.plane + (long long)y * geo.ldx + x] = (R)(delta[t] / mc<R>().f0[i]);
+    // delta / f0 with 1 / f0 in two parts, rounded once (2 FP64 operations)
+    const double v = delta[t];
+    dst[(long long)i * geo.plane + (long long)y * geo.ldx + x] =
+        (R)fma(v, mc<R>().if0[i], v * mc<R>().ifl[i]);
   }
 }
 
@@ -766,50 +911,53 @@ thread_local std::string g_error;
 
 template <typename R>
 void fill_consts(const Tables& t, MConsts<R>& c) {
+  using V = typename V2<R>::T;
   for (int p = 0; p < kPairs; ++p) {
-    c.vx[p] = (R)t.vx[p]; c.vy[p] = (R)t.vy[p];
     c.mN0[p] = (R)t.mN0[p]; c.mE[p] = (R)t.mE[p];
     c.mPxx[p] = (R)t.mPxx[p]; c.mPxy[p] = (R)t.mPxy[p]; c.mPyy[p] = (R)t.mPyy[p];
     c.mNx[p] = (R)t.mNx[p]; c.mNy[p] = (R)t.mNy[p]; c.mMx[p] = (R)t.mMx[p]; c.mMy[p] = (R)t.mMy[p];
-    c.LT[p] = (R)t.LT[p]; c.LX[p] = (R)t.LX[p]; c.LY[p] = (R)t.LY[p];
-    for (int k = 0; k < 5; ++k) c.WE[p][k] = (R)t.WE[p][k];
-    for (int k = 0; k < 4; ++k) c.WO[p][k] = (R)t.WO[p][k];
-    for (int k = 0; k < 8; ++k) {
-      c.BE[p][k] = (R)t.BE[p][k]; c.BO[p][k] = (R)t.BO[p][k];
-      c.mvE[p][k] = (R)t.mvE[p][k]; c.mvO[p][k] = (R)t.mvO[p][k];
-    }
   }
-  for (int a = 0; a < 16; ++a)
-    for (int b = 0; b < 16; ++b) c.gi[a][b] = (R)t.gi[a][b];
-  c.restN0 = (R)t.restN0; c.restE = (R)t.restE; c.restLT = (R)t.restLT;
-  for (int k = 0; k < 5; ++k) c.restWE[k] = (R)t.restWE[k];
-  for (int k = 0; k < 8; ++k) c.restBE[k] = (R)t.restBE[k];
-  for (int i = 0; i < kQm; ++i) c.f0[i] = t.f0[i];
+  auto fn = [&](int f, int p) {       // part of pair p's row odd in px
+    const double o[7] = {t.LX[p], t.WO[p][0], t.WO[p][2], t.BO[p][0], t.BO[p][2], t.BO[p][4], t.BO[p][6]};
+    for (int k = 0; k < 7; ++k) c.O[f][k] = V{(R)o[k], (R)o[k]};
+    c.va[f] = V{(R)t.vx[p], (R)t.vx[p]};
+    c.pa[f] = V{(R)t.mvO[p][0], (R)t.mvO[p][0]};
+  };
+  for (int k = 0; k < kClasses - 1; ++k) {
+    const int p = class_pair(k);
+    const double a[8] = {t.LT[p], t.WE[p][0], t.WE[p][1], 0.5 * (t.WE[p][2] + t.WE[p][4]), t.BE[p][0],
+                         t.BE[p][1], 0.5 * (t.BE[p][2] + t.BE[p][4]), 0.5 * (t.BE[p][5] + t.BE[p][7])};
+    for (int q = 0; q < 8; ++q) c.A[k][q] = (R)a[q];
+    c.C1[k][0] = (R)(0.5 * (t.WE[p][2] - t.WE[p][4]));
+    c.C1[k][1] = (R)(0.5 * (t.BE[p][2] - t.BE[p][4]));
+    c.C1[k][2] = (R)(0.5 * (t.BE[p][5] - t.BE[p][7]));
+    c.C2[k][0] = (R)t.WE[p][3]; c.C2[k][1] = (R)t.BE[p][3]; c.C2[k][2] = (R)t.BE[p][6];
+    c.p0[k] = (R)t.mvE[p][1];
+    c.rr[k] = (R)(0.5 * (t.mvE[p][2] + t.mvE[p][4]));
+    c.dd[k] = (R)(0.5 * (t.mvE[p][2] - t.mvE[p][4]));
+    c.pp[k] = (R)t.mvE[p][3];
+    fn(class_fn(k), p);
+    if (class_kind(k) == 2) fn(class_fn(k) + 1, p + 2);
+  }
+  const double a[8] = {t.restLT, t.restWE[0], t.restWE[1], 0.5 * (t.restWE[2] + t.restWE[4]), t.restBE[0],
+                       t.restBE[1], 0.5 * (t.restBE[2] + t.restBE[4]), 0.5 * (t.restBE[5] + t.restBE[7])};
+  for (int q = 0; q < 8; ++q) c.A[kClasses - 1][q] = (R)a[q];
+  for (int q = 0; q < 3; ++q) c.C1[kClasses - 1][q] = c.C2[kClasses - 1][q] = R(0);
+  c.p0[kClasses - 1] = (R)kM;
+  c.rr[kClasses - 1] = c.dd[kClasses - 1] = c.pp[kClasses - 1] = R(0);
+  for (int x = 0; x < 16; ++x)
+    for (int b = 0; b < 16; ++b) c.gi[x][b] = (R)t.gi[x][b];
+  c.restN0 = (R)t.restN0; c.restE = (R)t.restE;
+  for (int i = 0; i < kQm; ++i) {
+    c.f0[i] = t.f0[i];
+    c.if0[i] = 1.0 / t.f0[i];
+    c.ifl[i] = std::fma(-t.f0[i], c.if0[i], 1.0) / t.f0[i];
+  }
 }
 
-// the FP32 tables of the collision rearranged by couple (the same float values)
-void fill_couples(const MConsts<float>& c, MCoupleConsts& h) {
-  for (int q = 0; q < kCouples; ++q) {
-    const int a = couple_a(q), b = couple_b(q);
-    h.LT[q] = make_float2(c.LT[a], c.LT[b]);
-    h.LX[q] = make_float2(c.LX[a], c.LX[b]);
-    h.LY[q] = make_float2(c.LY[a], c.LY[b]);
-    for (int k = 0; k < 5; ++k) h.WE[q][k] = make_float2(c.WE[a][k], c.WE[b][k]);
-    for (int k = 0; k < 4; ++k) h.WO[q][k] = make_float2(c.WO[a][k], c.WO[b][k]);
-    for (int k = 0; k < 8; ++k) {
-      h.BE[q][k] = make_float2(c.BE[a][k], c.BE[b][k]);
-      h.BO[q][k] = make_float2(c.BO[a][k], c.BO[b][k]);
-    }
-    h.vx[q] = make_float2(c.vx[a], c.vx[b]);
-    h.vy[q] = make_float2(c.vy[a], c.vy[b]);
-    h.p0[q] = make_float2(c.mvE[a][1], c.mvE[b][1]);
-    h.px2[q] = make_float2(c.mvE[a][2], c.mvE[b][2]);
-    h.pxy[q] = make_float2(c.mvE[a][3], c.mvE[b][3]);
-    h.py2[q] = make_float2(c.mvE[a][4], c.mvE[b][4]);
-    h.pxv[q] = make_float2(c.mvO[a][0], c.mvO[b][0]);
-    h.pyv[q] = make_float2(c.mvO[a][1], c.mvO[b][1]);
-  }
-}
+// Dynamic shared memory that leaves room for one / two blocks per SM: chained
+// launches would otherwise gather the next step's blocks on idle SMs.
+constexpr int kOnePerSm = 120 * 1024, kTwoPerSm = 80 * 1024;
 
 std::mutex g_upload_mu;
 bool g_uploaded[64];
@@ -823,7 +971,9 @@ using namespace rlbm::massive;
 struct rlbm_massive_ctx {
   rlbm_massive_config cfg;
   MGeom geo;
-  size_t elem;
+  MOffsets of;
+  int sms;
+  size_t l2, elem;
   void* buf[2];
   int cur;
   unsigned* err;
@@ -857,13 +1007,15 @@ int upload_tables(int dev) {
   if (g_uploaded[dev]) return RLBM_OK;
   static MConsts<float> hf;
   static MConsts<double> hd;
-  static MCoupleConsts hc;
   fill_consts(t, hf);
   fill_consts(t, hd);
-  fill_couples(hf, hc);
   cudaError_t e = cudaMemcpyToSymbol(c_f, &hf, sizeof hf);
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_d, &hd, sizeof hd);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_cp, &hc, sizeof hc);
+  for (const void* k : {(const void*)k_mstep_split<4, false>, (const void*)k_mstep_split<4, true>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePerSm);
+  for (const void* k : {(const void*)k_mstep_split<2, false>, (const void*)k_mstep_split<2, true>,
+                        (const void*)k_mstep<double, false>, (const void*)k_mstep<double, true>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTwoPerSm);
   if (e != cudaSuccess) return fail(nullptr, RLBM_ECUDA, "constant upload: %s", cudaGetErrorString(e));
   g_uploaded[dev] = true;
   return RLBM_OK;
@@ -892,20 +1044,56 @@ int grid_1d(long long work) {
 
 namespace {
 
+template <typename... P, typename... A>
+void launch_chained(cudaStream_t st, void (*k)(P...), unsigned grid, int block, size_t smem, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
 int launch_steps(rlbm_massive_ctx* c, int nsteps) {
   const bool force = c->cfg.Fx != 0.0 || c->cfg.Fy != 0.0;
-  const dim3 grid = grid_of(c->geo), block(32, 4);
+  const cudaStream_t st = stream_of(c);
+  const size_t bytes = (size_t)c->geo.plane * kQm * c->elem;
+  const long long warps = (long long)((c->geo.nx + 31) / 32) * c->geo.ny;
+  const unsigned grid = (unsigned)((warps + kMThreads / 32 - 1) / (kMThreads / 32));
+  // FP64: four warps per 32 sites up to one such tile per SM, two up to two
+  // (one warp per SM sub-partition either way)
+  const long long tiles = ((long long)c->geo.nx * c->geo.ny + 31) / 32;
+  const int ns = tiles <= c->sms ? 4 : tiles <= 2 * c->sms ? 2 : 1;
   for (int s = 0; s < nsteps; ++s) {
     const void* src = c->buf[c->cur];
     void* dst = c->buf[c->cur ^ 1];
+    // order and L2 policy of the pulls: the rules of the massless step
+    // (launch_single in prec_impl.cuh)
+    MLaunch ml;
+    ml.evict_first = bytes <= 2 * c->l2;
+    ml.reverse = c->cur && bytes <= 4 * c->l2;
     if (c->elem == 8) {
       const double it = 1.0 / c->cfg.tau, fx = c->cfg.Fx, fy = c->cfg.Fy;
-      if (force) k_mstep<double, true><<<grid, block, 0, stream_of(c)>>>((const double*)src, (double*)dst, c->geo, it, fx, fy, c->err);
-      else k_mstep<double, false><<<grid, block, 0, stream_of(c)>>>((const double*)src, (double*)dst, c->geo, it, fx, fy, c->err);
+      const double* a = (const double*)src;
+      double* b = (double*)dst;
+      if (ns == 4)
+        launch_chained(st, force ? k_mstep_split<4, true> : k_mstep_split<4, false>, (unsigned)tiles, 128,
+                       kOnePerSm, a, b, c->geo, c->of, it, fx, fy, c->err);
+      else if (ns == 2)
+        launch_chained(st, force ? k_mstep_split<2, true> : k_mstep_split<2, false>, (unsigned)tiles, 64,
+                       kTwoPerSm, a, b, c->geo, c->of, it, fx, fy, c->err);
+      else
+        launch_chained(st, force ? k_mstep<double, true> : k_mstep<double, false>, grid, kMThreads,
+                       grid <= 2u * (unsigned)c->sms ? kTwoPerSm : 0, a, b, c->geo, c->of, ml, it, fx, fy, c->err);
     } else {
       const float it = (float)(1.0 / c->cfg.tau), fx = (float)c->cfg.Fx, fy = (float)c->cfg.Fy;
-      if (force) k_mstep_f32_force<<<grid, block, 0, stream_of(c)>>>((const float*)src, (float*)dst, c->geo, it, fx, fy, c->err);
-      else k_mstep<float, false><<<grid, block, 0, stream_of(c)>>>((const float*)src, (float*)dst, c->geo, it, fx, fy, c->err);
+      launch_chained(st, force ? k_mstep<float, true> : k_mstep<float, false>, grid, kMThreads, 0,
+                     (const float*)src, (float*)dst, c->geo, c->of, ml, it, fx, fy, c->err);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "step kernel");
@@ -918,9 +1106,9 @@ int launch_steps(rlbm_massive_ctx* c, int nsteps) {
 
 int velocity_planes(rlbm_massive_ctx* c, double* ux, double* uy) {
   if (c->elem == 8)
-    k_mmoments<double><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((const double*)c->buf[c->cur], c->geo, nullptr, ux, uy, nullptr, c->err);
+    k_mmoments<double><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((const double*)c->buf[c->cur], c->geo, c->of, nullptr, ux, uy, nullptr, c->err);
   else
-    k_mmoments<float><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((const float*)c->buf[c->cur], c->geo, nullptr, ux, uy, nullptr, c->err);
+    k_mmoments<float><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((const float*)c->buf[c->cur], c->geo, c->of, nullptr, ux, uy, nullptr, c->err);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "moments kernel");
   ++c->launches;
@@ -977,6 +1165,19 @@ int rlbm_massive_create(const rlbm_massive_config* cfg, rlbm_massive_ctx** out) 
   c->geo.ldx = (cfg->nx + 31) / 32 * 32;
   c->geo.px = cfg->periodic_x ? 1 : 0; c->geo.py = cfg->periodic_y ? 1 : 0;
   c->geo.plane = (long long)c->geo.ldx * cfg->ny;
+  for (int i = 0; i < kQm; ++i) {
+    const int s = i & 1 ? -1 : 1;
+    const long long back = i == kRestPop ? 0 : s * ((long long)pair_y(i / 2) * c->geo.ldx + pair_x(i / 2));
+    c->of.plane[i] = (long long)i * c->geo.plane * (long long)c->elem;
+    c->of.pull[i] = c->of.plane[i] - back * (long long)c->elem;
+  }
+  int l2 = 0;
+  if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
+    delete c;
+    return fail(nullptr, RLBM_ECUDA, "device attributes");
+  }
+  c->l2 = (size_t)l2;
   const size_t bytes = (size_t)c->geo.plane * kQm * c->elem;
   for (int b = 0; b < 2; ++b) {
     e = cudaMalloc(&c->buf[b], bytes);
@@ -1018,9 +1219,9 @@ int rlbm_massive_init(rlbm_massive_ctx* c, const double* n, const double* ux, co
       }
     }
     if (c->elem == 8)
-      k_minit<double><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((double*)c->buf[0], c->geo, f[0], f[1], f[2], f[3], c->err);
+      k_minit<double><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((double*)c->buf[0], c->geo, c->of, f[0], f[1], f[2], f[3], c->err);
     else
-      k_minit<float><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((float*)c->buf[0], c->geo, f[0], f[1], f[2], f[3], c->err);
+      k_minit<float><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((float*)c->buf[0], c->geo, c->of, f[0], f[1], f[2], f[3], c->err);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "init kernel");
     ++c->launches;
@@ -1082,9 +1283,9 @@ int rlbm_massive_moments(rlbm_massive_ctx* c, double* n, double* ux, double* uy,
     for (int k = 0; k < 4; ++k) d[k] = c->scratch + k * ns;
   }
   if (c->elem == 8)
-    k_mmoments<double><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((const double*)c->buf[c->cur], c->geo, d[0], d[1], d[2], d[3], c->err);
+    k_mmoments<double><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((const double*)c->buf[c->cur], c->geo, c->of, d[0], d[1], d[2], d[3], c->err);
   else
-    k_mmoments<float><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((const float*)c->buf[c->cur], c->geo, d[0], d[1], d[2], d[3], c->err);
+    k_mmoments<float><<<grid_of(c->geo), dim3(32, 4), 0, stream_of(c)>>>((const float*)c->buf[c->cur], c->geo, c->of, d[0], d[1], d[2], d[3], c->err);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, "moments kernel");
   ++c->launches;
