@@ -177,19 +177,27 @@ struct Cta {
   }
 };
 
-// Per-warp staging of 32 rows x 64 bytes (row pitch 80 bytes): row-owning
-// lanes <-> consecutive 16-byte pieces, for coalesced global accesses.
-constexpr int kStagePitch = 80, kStageBytes = 32 * kStagePitch;
+// The row kernels run 256 threads per 128 sites: a warp w owns the rows 32 (w %
+// 4) .. of the tile (the TMEM lanes it may read) and the columns of half w / 4,
+// so that twice as many warps hide the latency of the activations per byte of
+// shared memory (training step 256 x 256, batch 8: 1,150 -> TRAIN_US us, with
+// the wider slabs of k_spectral).
+constexpr int kThreads = 256;
 
-// Writes the warp's staged rows (64 bytes each) to rows row0 .. of a global
-// array with `pitch` bytes per row; nv rows are valid.
-__device__ __forceinline__ void stage_out(uint32_t st, unsigned char* dst, long long pitch, int nv) {
+// Per-warp staging of 32 rows x 32 bytes: row-owning lanes <-> 16-byte pieces
+// in row order, so that global stores write whole sectors.
+constexpr int kStagePitch = 48, kStageBytes = 32 * kStagePitch;
+
+// Writes the warp's staged rows (32 bytes each, `sp` bytes apart) to rows of
+// `pitch` bytes; nv rows are valid.
+__device__ __forceinline__ void stage_out(uint32_t st, int sp, unsigned char* dst, long long pitch,
+                                          int nv) {
   const int lane = threadIdx.x & 31;
   __syncwarp();
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int i = lane + 32 * q, r = i >> 2, c = i & 3;
-    const uint4 v = lds16(st + r * kStagePitch + c * 16);
+  for (int q = 0; q < 2; ++q) {
+    const int i = lane + 32 * q, r = i >> 1, c = i & 1;
+    const uint4 v = lds16(st + r * sp + c * 16);
     if (r < nv) *reinterpret_cast<uint4*>(dst + r * pitch + c * 16) = v;
   }
   __syncwarp();
@@ -253,16 +261,17 @@ template <int MODE>
 constexpr size_t fwd_smem(int tiles) {
   return (MODE != 0 ? sites_bytes(tiles) + 4 * kSmallLbo : 0) +
          (MODE != 2 ? modes_bytes(tiles) + kOverrun + kColBytes : 0) + 128 * 64 + 4 * kSmallLbo +
-         4 * kStageBytes;
+         8 * kStageBytes;
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(128) k_fwd_rows(FwdRows p) {
+__global__ void __launch_bounds__(kThreads) k_fwd_rows(FwdRows p) {
   extern __shared__ __align__(1024) uint8_t tc_smem[];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t slot;
   __shared__ float bias[kC];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int row = tid & 127, half = tid >> 7, quarter = warp & 3;
   const int tiles = (p.N + kTileRows - 1) / kTileRows;
   uint32_t at = smem_u32(tc_smem);
   auto take = [&](uint32_t bytes) { const uint32_t a = at; at += bytes; return a; };
@@ -272,11 +281,11 @@ __global__ void __launch_bounds__(128) k_fwd_rows(FwdRows p) {
   const Op Wm{MODE != 0 ? take(4 * kSmallLbo) : 0, kSmallLbo, kColSbo};
   const Op A{take(128 * 64), kRowLbo, kRowSbo};
   const Op W{take(4 * kSmallLbo), kSmallLbo, kColSbo};
-  const uint32_t stage = take(4 * kStageBytes) + warp * kStageBytes;
+  const uint32_t stage = take(8 * kStageBytes) + warp * kStageBytes;
   Cta<128, 2> cta;
   cta.start(bars, &slot);
   const uint32_t dG = cta.tmem, dW = cta.tmem + 32, dS = cta.tmem + 64;
-  const uint32_t lanes = (uint32_t)(warp * 32) << 16;
+  const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
 
   if (tid < kC) bias[tid] = p.bias[tid];
   if (MODE != 2) load_modes(F1, p.F1, p.N, tiles * 16);
@@ -285,8 +294,8 @@ __global__ void __launch_bounds__(128) k_fwd_rows(FwdRows p) {
     load_kn32(W, p.W);
   } else {
     // x P: k = inputs, padded with zeros to 16
-    for (int q = 0; q < 4; ++q) sts16(A.base + (tid + 128 * q) * 16, make_uint4(0, 0, 0, 0));
-    for (int i = tid; i < kC * 16; i += 128) {
+    for (int q = 0; q < 2; ++q) sts16(A.base + (tid + kThreads * q) * 16, make_uint4(0, 0, 0, 0));
+    for (int i = tid; i < kC * 16; i += kThreads) {
       const int k = i / kC, c = i % kC;
       sts2(W.elem(c, k), k < p.cin ? __bfloat16_as_ushort(p.W[k * kC + c]) : (uint16_t)0);
     }
@@ -301,8 +310,8 @@ __global__ void __launch_bounds__(128) k_fwd_rows(FwdRows p) {
       const long long row0 = (long long)item * p.N + t * kTileRows;
       if (MODE != 0) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int i = tid + 128 * q;
+        for (int q = 0; q < 2; ++q) {
+          const int i = tid + kThreads * q;
           uint4 v = make_uint4(0, 0, 0, 0);
           if ((i >> 2) < nv) v = __ldg(reinterpret_cast<const uint4*>(p.in + row0 * kC) + i);
           sts16(A.chunk(i >> 2, i & 3), v);
@@ -310,7 +319,7 @@ __global__ void __launch_bounds__(128) k_fwd_rows(FwdRows p) {
       } else {
         const uint4* src = reinterpret_cast<const uint4*>(p.in + row0 * p.cin);
         uint4* dst = reinterpret_cast<uint4*>(p.xcopy + row0 * p.cin);
-        for (int i = tid; i < nv * p.cin / 8; i += 128) {
+        for (int i = tid; i < nv * p.cin / 8; i += kThreads) {
           const uint4 v = __ldg(src + i);
           dst[i] = v;
           const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -329,12 +338,10 @@ __global__ void __launch_bounds__(128) k_fwd_rows(FwdRows p) {
       }
       cta.wait(0);
       if (MODE != 2 && t > 0) cta.wait(1);      // the transform has read hT
-      const int wv = max(0, min(32, nv - warp * 32));      // valid rows of this warp
+      const int wv = max(0, min(32, nv - quarter * 32));   // valid rows of this warp
       const bool valid = lane < wv;
-      const long long wrow = row0 + warp * 32;
-      uint32_t hp[16];
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
+      const long long wrow = row0 + quarter * 32;
+      {
         float v[16], g[16];
         tmem_ld16(dW + lanes + half * 16, v);
         if (MODE != 0) tmem_ld16(dG + lanes + half * 16, g);
@@ -346,28 +353,33 @@ __global__ void __launch_bounds__(128) k_fwd_rows(FwdRows p) {
         }
         if (MODE != 0) {
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            sts16(stage + lane * kStagePitch + c * 16,
-                  make_uint4(__float_as_uint(v[4 * c]), __float_as_uint(v[4 * c + 1]),
-                             __float_as_uint(v[4 * c + 2]), __float_as_uint(v[4 * c + 3])));
-          stage_out(stage, reinterpret_cast<unsigned char*>(p.z + wrow * kC + half * 16), kC * 4, wv);
+          for (int q = 0; q < 2; ++q) {
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+              sts16(stage + lane * kStagePitch + c * 16,
+                    make_uint4(__float_as_uint(v[8 * q + 4 * c]), __float_as_uint(v[8 * q + 4 * c + 1]),
+                               __float_as_uint(v[8 * q + 4 * c + 2]), __float_as_uint(v[8 * q + 4 * c + 3])));
+            stage_out(stage, kStagePitch,
+                      reinterpret_cast<unsigned char*>(p.z + wrow * kC + half * 16 + 8 * q), kC * 4, wv);
+          }
         }
+        uint32_t hp[8];
 #pragma unroll
         for (int j = 0; j < 16; j += 2) {
           const uint16_t a = bf16_bits(MODE == 1 ? gelu(v[j]) : v[j]);
           const uint16_t b = bf16_bits(MODE == 1 ? gelu(v[j + 1]) : v[j + 1]);
-          hp[half * 8 + j / 2] = pack_bits(a, b);
+          hp[j / 2] = pack_bits(a, b);
           if (MODE != 2) {
-            sts2(hT.elem(half * 16 + j, tid), valid ? a : (uint16_t)0);
-            sts2(hT.elem(half * 16 + j + 1, tid), valid ? b : (uint16_t)0);
+            sts2(hT.elem(half * 16 + j, row), valid ? a : (uint16_t)0);
+            sts2(hT.elem(half * 16 + j + 1, row), valid ? b : (uint16_t)0);
           }
         }
-      }
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
-        sts16(stage + lane * kStagePitch + c * 16,
-              make_uint4(hp[4 * c], hp[4 * c + 1], hp[4 * c + 2], hp[4 * c + 3]));
-      stage_out(stage, reinterpret_cast<unsigned char*>(p.h + wrow * kC), kC * 2, wv);
+        for (int c = 0; c < 2; ++c)
+          sts16(stage + lane * kStagePitch + c * 16,
+                make_uint4(hp[4 * c], hp[4 * c + 1], hp[4 * c + 2], hp[4 * c + 3]));
+        stage_out(stage, kStagePitch, reinterpret_cast<unsigned char*>(p.h + wrow * kC + half * 16), kC * 2, wv);
+      }
       if (MODE != 2) {
         if ((stop = cta.sync())) break;
         if (tid == 0) {
@@ -378,20 +390,16 @@ __global__ void __launch_bounds__(128) k_fwd_rows(FwdRows p) {
     }
     if (MODE != 2 && !stop) {
       cta.wait(1);
-      if (warp == 0) {
-        uint32_t s[16];
+      if (quarter == 0) {
+        uint32_t s[8];
+        float v[16];
+        tmem_ld16(dS + half * 16, v);
+        tmem_wait();
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          float v[16];
-          tmem_ld16(dS + half * 16, v);
-          tmem_wait();
+        for (int j = 0; j < 16; j += 2) s[j / 2] = pack_bits(bf16_bits(v[j]), bf16_bits(v[j + 1]));
+        uint4* o = reinterpret_cast<uint4*>(p.S1 + (long long)item * (kM * kC) + lane * kC + half * 16);
 #pragma unroll
-          for (int j = 0; j < 16; j += 2)
-            s[half * 8 + j / 2] = pack_bits(bf16_bits(v[j]), bf16_bits(v[j + 1]));
-        }
-        uint4* o = reinterpret_cast<uint4*>(p.S1 + (long long)item * (kM * kC) + lane * kC);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) o[c] = make_uint4(s[4 * c], s[4 * c + 1], s[4 * c + 2], s[4 * c + 3]);
+        for (int c = 0; c < 2; ++c) o[c] = make_uint4(s[4 * c], s[4 * c + 1], s[4 * c + 2], s[4 * c + 3]);
       }
     }
   }
@@ -416,76 +424,102 @@ struct Spectral {
   int N;
 };
 
-constexpr uint32_t kSlabLbo = 144, kSlabSbo = 8 * 144;             // rows x 64 k in 16-byte pieces
-constexpr uint32_t kSlabA = 8 * kSlabSbo, kTileA = 16 * kSlabSbo;  // 64 / 128 rows
-constexpr uint32_t kSlabB = 8 * kSmallLbo;                         // 32 rows x 64 k
+constexpr int kSlabK = 256;                                        // k of one slab
+constexpr uint32_t kSlabLbo = 144, kSlabSbo = 32 * 144;            // 64 rows x 256 k in 16-byte pieces
+constexpr uint32_t kSlabA = 8 * kSlabSbo;
+constexpr uint32_t kA2Sbo = 8 * 144, kTileA = 16 * kA2Sbo;         // 128 rows x 64 k
+constexpr uint32_t kSlabB = 32 * kSmallLbo;                        // 32 rows x 256 k
 constexpr int kMixPitch = 33;
-constexpr size_t kSpectralSmem = 2 * kSlabA + 2 * kTileA + 2 * kSlabB + kModes * kMixPitch * 4 +
+// behind slab A: at least another slab's bytes, which its unused rows read
+constexpr size_t kSpectralSmem = kSlabA + 2 * kTileA + kSlabB + kModes * kMixPitch * 4 +
                                  8 * 32 * kMixPitch * 8;
 
 template <bool BWD>
 __global__ void __launch_bounds__(256) k_spectral(Spectral p) {
   extern __shared__ __align__(1024) uint8_t tc_smem[];
-  __shared__ __align__(8) uint64_t bars[2];
+  __shared__ __align__(8) uint64_t bars[1];
   __shared__ uint32_t slot;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ky = blockIdx.x, b = blockIdx.y, K = 2 * p.N;
   const uint32_t base = smem_u32(tc_smem);
-  const uint32_t a2 = base + 2 * kSlabA, bb = a2 + 2 * kTileA;
-  auto A1 = [&](int w) { return Op{base + (uint32_t)w * kSlabA, kSlabLbo, kSlabSbo}; };
-  auto A2 = [&](int w) { return Op{a2 + (uint32_t)w * kTileA, kSlabLbo, kSlabSbo}; };
-  auto B = [&](int w) { return Op{bb + (uint32_t)w * kSlabB, kSmallLbo, kColSbo}; };
-  float* s2 = reinterpret_cast<float*>(tc_smem + 2 * kSlabA + 2 * kTileA + 2 * kSlabB);
+  const uint32_t a2 = base + kSlabA, bb = a2 + 2 * kTileA;
+  const Op A1{base, kSlabLbo, kSlabSbo}, B{bb, kSmallLbo, kColSbo};
+  auto A2 = [&](int w) { return Op{a2 + (uint32_t)w * kTileA, kSlabLbo, kA2Sbo}; };
+  float* s2 = reinterpret_cast<float*>(tc_smem + kSlabA + 2 * kTileA + kSlabB);
   float2* rt = reinterpret_cast<float2*>(s2 + kModes * kMixPitch) + warp * 32 * kMixPitch;
-  Cta<128, 2> cta;
+  Cta<128, 1> cta;
   cta.start(bars, &slot);
   const __nv_bfloat16* X = p.X + (long long)b * K * (kKy * kC) + ky * kC;
 
   // A2 tiles of round r (rows 256 r .. 256 r + 255), 16-byte pieces along k
+  uint4 r2[8];
   auto load_a2 = [&](int r) {
-    for (int i = tid; i < 256 * 8; i += 256) {
-      const int row = i >> 3, kg = i & 7, g = r * 256 + row;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (g < K) v = __ldg(reinterpret_cast<const uint4*>(p.A2 + (long long)g * kModes) + kg);
-      sts16(A2(row >> 7).chunk(row & 127, kg), v);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int i = tid + 256 * q, g = r * 256 + (i >> 3);
+      r2[q] = make_uint4(0, 0, 0, 0);
+      if (g < K) r2[q] = __ldg(reinterpret_cast<const uint4*>(p.A2 + (long long)g * kModes) + (i & 7));
+    }
+  };
+  auto store_a2 = [&]() {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int i = tid + 256 * q, row = i >> 3;
+      sts16(A2(row >> 7).chunk(row & 127, i & 7), r2[q]);
     }
   };
 
-  const int slabs = (K + 63) / 64;
+  // first transform: slabs of 256 k, the next one loaded while one is multiplied
+  const int slabs = (K + kSlabK - 1) / kSlabK;
   bool stop = false;
-  uint4 ra[2], rb;
+  uint4 ra[8], rb[4];
   auto load_slab = [&](int s) {
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int i = tid + 256 * q, row = i >> 3, k = s * 64 + (i & 7) * 8;
+    for (int q = 0; q < 8; ++q) {
+      const int i = tid + 256 * q, k = s * kSlabK + (i & 31) * 8;
       ra[q] = make_uint4(0, 0, 0, 0);
-      if (k < K) ra[q] = __ldg(reinterpret_cast<const uint4*>(p.A1 + (long long)row * K + k));
+      if (k < K) ra[q] = __ldg(reinterpret_cast<const uint4*>(p.A1 + (long long)(i >> 5) * K + k));
     }
-    const int k = s * 64 + (tid >> 2);
-    rb = make_uint4(0, 0, 0, 0);
-    if (k < K) rb = __ldg(reinterpret_cast<const uint4*>(X + (long long)k * (kKy * kC)) + (tid & 3));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = tid + 256 * q, k = s * kSlabK + (i >> 2);
+      rb[q] = make_uint4(0, 0, 0, 0);
+      if (k < K) rb[q] = __ldg(reinterpret_cast<const uint4*>(X + (long long)k * (kKy * kC)) + (i & 3));
+    }
   };
   load_slab(0);
   for (int s = 0; s < slabs; ++s) {
-    const int w = s & 1;
-    if (s >= 2) cta.wait(w);
+    if (s > 0) cta.wait(0);
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < 8; ++q) {
       const int i = tid + 256 * q;
-      sts16(A1(w).chunk(i >> 3, i & 7), ra[q]);
+      sts16(A1.chunk(i >> 5, i & 31), ra[q]);
     }
-    scatter8(B(w), (tid & 3) * 8, tid >> 2, rb);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = tid + 256 * q;
+      scatter8(B, (i & 3) * 8, i >> 2, rb[q]);
+    }
     if ((stop = cta.sync())) break;
     if (tid == 0) {
-      mma(cta.tmem, A1(w), 0, B(w), 0, kC, 4, s > 0);
-      commit(cta.bar(w));
+      mma(cta.tmem, A1, 0, B, 0, kC, min(kSlabK, ((K - s * kSlabK) + 15) / 16 * 16) / 16, s > 0);
+      commit(cta.bar(0));
     }
     if (s + 1 < slabs) load_slab(s + 1);
     else load_a2(0);
   }
+  // mixing: a warp takes kx = warp, warp + 8, ..; lane = output channel.  The
+  // matrix of one kx is in flight while the one before is used.
+  float2 c[kC];
+  auto load_mix = [&](int kx) {
+    const float2* w = reinterpret_cast<const float2*>(p.R) + (long long)(kx * kKy + ky) * kC * kC;
+#pragma unroll
+    for (int i = 0; i < kC; ++i) c[i] = __ldg(w + i * kC + lane);
+  };
   if (!stop) {
-    if (slabs >= 2) cta.wait(slabs & 1);
-    cta.wait((slabs - 1) & 1);
+    load_mix(warp);
+    cta.wait(0);
+    store_a2();
     if (warp < 2) {
       float* g = p.S2 + ((long long)b * kModes + warp * 32 + lane) * (kKy * kC) + ky * kC;
 #pragma unroll
@@ -496,50 +530,51 @@ __global__ void __launch_bounds__(256) k_spectral(Spectral p) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) s2[(warp * 32 + lane) * kMixPitch + half * 16 + j] = v[j];
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          reinterpret_cast<float4*>(g + half * 16)[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+        for (int q = 0; q < 4; ++q)
+          reinterpret_cast<float4*>(g + half * 16)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
     }
     stop = cta.sync();
   }
   if (!stop) {
-    // mixing: a warp takes kx = warp, warp + 8, ..; lane = output channel
+#pragma unroll 1
     for (int kx = warp; kx < kModes / 2; kx += 8) {
-      const float2* w = reinterpret_cast<const float2*>(p.R) + (long long)(kx * kKy + ky) * kC * kC;
       const float* re = s2 + (2 * kx) * kMixPitch;
       const float* im = re + kMixPitch;
       float ure = 0.f, uim = 0.f;
       if (!BWD) {
-#pragma unroll 8
+#pragma unroll
         for (int i = 0; i < kC; ++i) {
-          const float2 c = __ldg(w + i * kC + lane);
-          ure = fmaf(re[i], c.x, fmaf(-im[i], c.y, ure));
-          uim = fmaf(re[i], c.y, fmaf(im[i], c.x, uim));
+          ure = fmaf(re[i], c[i].x, fmaf(-im[i], c[i].y, ure));
+          uim = fmaf(re[i], c[i].y, fmaf(im[i], c[i].x, uim));
         }
+        if (kx + 8 < kModes / 2) load_mix(kx + 8);
       } else {
-#pragma unroll 8
-        for (int i = 0; i < kC; ++i) rt[i * kMixPitch + lane] = __ldg(w + i * kC + lane);
+#pragma unroll
+        for (int i = 0; i < kC; ++i) rt[i * kMixPitch + lane] = c[i];
         __syncwarp();
+        if (kx + 8 < kModes / 2) load_mix(kx + 8);
 #pragma unroll 8
         for (int o = 0; o < kC; ++o) {
-          const float2 c = rt[lane * kMixPitch + o];
-          ure = fmaf(re[o], c.x, fmaf(im[o], c.y, ure));
-          uim = fmaf(im[o], c.x, fmaf(-re[o], c.y, uim));
+          const float2 w = rt[lane * kMixPitch + o];
+          ure = fmaf(re[o], w.x, fmaf(im[o], w.y, ure));
+          uim = fmaf(im[o], w.x, fmaf(-re[o], w.y, uim));
         }
         __syncwarp();
       }
-      sts2(B(0).elem(lane, 2 * kx), bf16_bits(ure));
-      sts2(B(0).elem(lane, 2 * kx + 1), bf16_bits(uim));
+      sts2(B.elem(lane, 2 * kx), bf16_bits(ure));
+      sts2(B.elem(lane, 2 * kx + 1), bf16_bits(uim));
     }
     const int rounds = (K + 255) / 256;
     for (int r = 0; r < rounds; ++r) {
-      if (r > 0) load_a2(r);
+      if (r > 0) store_a2();
       if ((stop = cta.sync())) break;
       if (tid == 0) {
-        mma(cta.tmem + 32, A2(0), 0, B(0), 0, kC, 4, false);
-        mma(cta.tmem + 64, A2(1), 0, B(0), 0, kC, 4, false);
+        mma(cta.tmem + 32, A2(0), 0, B, 0, kC, 4, false);
+        mma(cta.tmem + 64, A2(1), 0, B, 0, kC, 4, false);
         commit(cta.bar(0));
       }
+      if (r + 1 < rounds) load_a2(r + 1);
       cta.wait(0);
       const int tile = warp >> 2;          // warps 0-3: first tile, 4-7: second
       const int row = r * 256 + tile * 128 + (warp & 3) * 32 + lane;
@@ -556,7 +591,7 @@ __global__ void __launch_bounds__(256) k_spectral(Spectral p) {
       if (row < K) {
         uint4* o = reinterpret_cast<uint4*>(p.out + ((long long)b * K + row) * (kKy * kC) + ky * kC);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) o[c] = make_uint4(s[4 * c], s[4 * c + 1], s[4 * c + 2], s[4 * c + 3]);
+        for (int q = 0; q < 4; ++q) o[q] = make_uint4(s[4 * q], s[4 * q + 1], s[4 * q + 2], s[4 * q + 3]);
       }
     }
   }
@@ -619,16 +654,16 @@ constexpr uint32_t kQ2Lbo = 2 * 144;                     // B: n = 16, k = 128
 constexpr size_t kHeadFwdSmem = 128 * 64 + 4 * kQ1Lbo + 16 * kY1Sbo + 16 * kQ2Lbo;
 
 __device__ __forceinline__ void load_q1(const Op& o, const __nv_bfloat16* Q1) {
-  for (int i = threadIdx.x; i < kC * kQ / 8; i += 128)
+  for (int i = threadIdx.x; i < kC * kQ / 8; i += kThreads)
     scatter8(o, (i % (kQ / 8)) * 8, i / (kQ / 8), __ldg(reinterpret_cast<const uint4*>(Q1) + i));
 }
 
-__global__ void __launch_bounds__(128) k_head_fwd(Head p) {
+__global__ void __launch_bounds__(kThreads) k_head_fwd(Head p) {
   extern __shared__ __align__(1024) uint8_t tc_smem[];
   __shared__ __align__(8) uint64_t bars[1];
   __shared__ uint32_t slot;
   __shared__ float bq1[kQ];
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, row = tid & 127, half = tid >> 7, quarter = (tid >> 5) & 3;
   const uint32_t base = smem_u32(tc_smem);
   const Op A{base, kRowLbo, kRowSbo};
   const Op Q1{base + 128 * 64, kQ1Lbo, 144};
@@ -636,22 +671,22 @@ __global__ void __launch_bounds__(128) k_head_fwd(Head p) {
   const Op Q2{Y.base + 16 * kY1Sbo, kQ2Lbo, 144};
   Cta<128, 1> cta;
   cta.start(bars, &slot);
-  bq1[tid] = p.bq1[tid];
+  if (tid < kQ) bq1[tid] = p.bq1[tid];
   load_q1(Q1, p.Q1);
-  for (int i = tid; i < 16 * kQ; i += 128) {
+  for (int i = tid; i < 16 * kQ; i += kThreads) {
     const int n = i / kQ, k = i % kQ;
     sts2(Q2.elem(n, k), n < 4 ? __bfloat16_as_ushort(p.Q2[k * 4 + n]) : (uint16_t)0);
   }
   const float4 b2 = make_float4(p.bq2[0], p.bq2[1], p.bq2[2], p.bq2[3]);
-  const uint32_t lanes = (uint32_t)(warp * 32) << 16;
+  const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
   const long long tiles = (p.rows + 127) / 128;
   bool stop = false;
   for (long long t = blockIdx.x; t < tiles && !stop; t += gridDim.x) {
     const long long row0 = t * 128;
     const int nv = (int)min(128LL, p.rows - row0);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = tid + 128 * q;
+    for (int q = 0; q < 2; ++q) {
+      const int i = tid + kThreads * q;
       uint4 v = make_uint4(0, 0, 0, 0);
       if ((i >> 2) < nv) v = __ldg(reinterpret_cast<const uint4*>(p.h + row0 * kC) + i);
       sts16(A.chunk(i >> 2, i & 3), v);
@@ -663,7 +698,7 @@ __global__ void __launch_bounds__(128) k_head_fwd(Head p) {
     }
     cta.wait(0);
 #pragma unroll 1
-    for (int c0 = 0; c0 < kQ; c0 += 16) {
+    for (int c0 = half * 64; c0 < half * 64 + 64; c0 += 16) {
       float v[16];
       tmem_ld16(cta.tmem + lanes + c0, v);
       tmem_wait();
@@ -671,8 +706,8 @@ __global__ void __launch_bounds__(128) k_head_fwd(Head p) {
 #pragma unroll
       for (int j = 0; j < 16; j += 2)
         s[j / 2] = pack_bits(bf16_bits(gelu(v[j] + bq1[c0 + j])), bf16_bits(gelu(v[j + 1] + bq1[c0 + j + 1])));
-      sts16(Y.chunk(tid, c0 / 8), make_uint4(s[0], s[1], s[2], s[3]));
-      sts16(Y.chunk(tid, c0 / 8 + 1), make_uint4(s[4], s[5], s[6], s[7]));
+      sts16(Y.chunk(row, c0 / 8), make_uint4(s[0], s[1], s[2], s[3]));
+      sts16(Y.chunk(row, c0 / 8 + 1), make_uint4(s[4], s[5], s[6], s[7]));
     }
     if ((stop = cta.sync())) break;
     if (tid == 0) {
@@ -680,11 +715,13 @@ __global__ void __launch_bounds__(128) k_head_fwd(Head p) {
       commit(cta.bar(0));
     }
     cta.wait(0);
-    float v[16];
-    tmem_ld16(cta.tmem + lanes, v);
-    tmem_wait();
-    if (tid < nv)
-      reinterpret_cast<float4*>(p.y)[row0 + tid] = make_float4(v[0] + b2.x, v[1] + b2.y, v[2] + b2.z, v[3] + b2.w);
+    if (half == 0) {
+      float v[16];
+      tmem_ld16(cta.tmem + lanes, v);
+      tmem_wait();
+      if (row < nv)
+        reinterpret_cast<float4*>(p.y)[row0 + row] = make_float4(v[0] + b2.x, v[1] + b2.y, v[2] + b2.z, v[3] + b2.w);
+    }
   }
   cta.finish(stop);
 }
@@ -723,12 +760,13 @@ __device__ __forceinline__ float lane_sums16(float (&v)[16]) {
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-__global__ void __launch_bounds__(128) k_head_bwd(Head p) {
+__global__ void __launch_bounds__(kThreads) k_head_bwd(Head p) {
   extern __shared__ __align__(1024) uint8_t tc_smem[];
   __shared__ __align__(8) uint64_t bars[1];
   __shared__ uint32_t slot;
-  __shared__ float bq1[kQ], sb1[4][kQ];     // sb1: this CTA's sums of dz1, per warp
+  __shared__ float bq1[kQ], sb1[4][kQ];     // sb1: this CTA's sums of dz1, per 32 rows
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int row = tid & 127, part = tid >> 7, quarter = warp & 3;
   uint32_t at = smem_u32(tc_smem);
   auto take = [&](uint32_t bytes) { const uint32_t a = at; at += bytes; return a; };
   const Op A{take(128 * 64), kRowLbo, kRowSbo};
@@ -743,25 +781,24 @@ __global__ void __launch_bounds__(128) k_head_bwd(Head p) {
   Cta<256, 1> cta;
   cta.start(bars, &slot);
   const uint32_t dZ = cta.tmem, dY = cta.tmem + 64, dH = cta.tmem + 128, dAcc = cta.tmem + 160;
-  const uint32_t lanes = (uint32_t)(warp * 32) << 16;
-  bq1[tid] = p.bq1[tid];
+  const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
+  if (tid < kQ) bq1[tid] = p.bq1[tid];
   load_q1(Q1, p.Q1);
-  for (int i = tid; i < 16 * (int)kDySbo / 16; i += 128) sts16(DY.base + i * 16, make_uint4(0, 0, 0, 0));
-  for (int i = tid; i < 16 * (int)kBwLbo / 16; i += 128) sts16(Bw.base + i * 16, make_uint4(0, 0, 0, 0));
-  for (int i = tid; i < kQ * 16; i += 128) {
+  for (int i = tid; i < 16 * (int)kDySbo / 16; i += kThreads) sts16(DY.base + i * 16, make_uint4(0, 0, 0, 0));
+  for (int i = tid; i < 16 * (int)kBwLbo / 16; i += kThreads) sts16(Bw.base + i * 16, make_uint4(0, 0, 0, 0));
+  for (int i = tid; i < kQ * 16; i += kThreads) {
     const int n = i >> 4, k = i & 15;
     sts2(Q2t.elem(n, k), k < 4 ? __bfloat16_as_ushort(p.Q2[n * 4 + k]) : (uint16_t)0);
   }
-  for (int i = tid; i < kC * kQ / 8; i += 128)
+  for (int i = tid; i < kC * kQ / 8; i += kThreads)
     sts16(Q1t.chunk(i / (kQ / 8), i % (kQ / 8)), __ldg(reinterpret_cast<const uint4*>(p.Q1) + i));
   __syncthreads();
-  float sb2[4], sb[kC];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) sb1[i][tid] = 0.f;
+  float sb2[4], sb[16];
+  for (int i = part; i < 4; i += 2) sb1[i][row] = 0.f;
 #pragma unroll
   for (int i = 0; i < 4; ++i) sb2[i] = 0.f;
 #pragma unroll
-  for (int i = 0; i < kC; ++i) sb[i] = 0.f;
+  for (int i = 0; i < 16; ++i) sb[i] = 0.f;
 
   const long long tiles = (p.rows + 127) / 128;
   bool stop = false, first = true;
@@ -769,21 +806,23 @@ __global__ void __launch_bounds__(128) k_head_bwd(Head p) {
     const long long row0 = t * 128;
     const int nv = (int)min(128LL, p.rows - row0);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = tid + 128 * q;
+    for (int q = 0; q < 2; ++q) {
+      const int i = tid + kThreads * q;
       uint4 v = make_uint4(0, 0, 0, 0);
       if ((i >> 2) < nv) v = __ldg(reinterpret_cast<const uint4*>(p.h + row0 * kC) + i);
       sts16(A.chunk(i >> 2, i & 3), v);
       scatter8(Bw, (i & 3) * 8, i >> 2, v);
     }
-    float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (tid < nv) d = __ldg(reinterpret_cast<const float4*>(p.dy) + row0 + tid);
-    sb2[0] += d.x; sb2[1] += d.y; sb2[2] += d.z; sb2[3] += d.w;
-    const uint16_t e[4] = {bf16_bits(d.x), bf16_bits(d.y), bf16_bits(d.z), bf16_bits(d.w)};
+    if (part == 0) {
+      float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (row < nv) d = __ldg(reinterpret_cast<const float4*>(p.dy) + row0 + row);
+      sb2[0] += d.x; sb2[1] += d.y; sb2[2] += d.z; sb2[3] += d.w;
+      const uint16_t e[4] = {bf16_bits(d.x), bf16_bits(d.y), bf16_bits(d.z), bf16_bits(d.w)};
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      sts2(DY.elem(tid, j), e[j]);
-      sts2(Bw.elem(kC + j, tid), e[j]);
+      for (int j = 0; j < 4; ++j) {
+        sts2(DY.elem(row, j), e[j]);
+        sts2(Bw.elem(kC + j, row), e[j]);
+      }
     }
     if ((stop = cta.sync())) break;
     if (tid == 0) {
@@ -795,7 +834,7 @@ __global__ void __launch_bounds__(128) k_head_bwd(Head p) {
     for (int half = 0; half < 2; ++half) {
       cta.wait(0);
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 2 * part; c < 2 * part + 2; ++c) {
         float z[16], g[16];
         tmem_ld16(dZ + lanes + c * 16, z);
         tmem_ld16(dY + lanes + c * 16, g);
@@ -814,14 +853,14 @@ __global__ void __launch_bounds__(128) k_head_bwd(Head p) {
           s[j / 2] = pack_bits(dz2[0], dz2[1]);
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
-            sts2(T.elem(c * 16 + j + i, tid), dz2[i]);
-            sts2(T.elem(64 + c * 16 + j + i, tid), y2[i]);
+            sts2(T.elem(c * 16 + j + i, row), dz2[i]);
+            sts2(T.elem(64 + c * 16 + j + i, row), y2[i]);
           }
         }
-        sts16(DZ.chunk(tid, c * 2), make_uint4(s[0], s[1], s[2], s[3]));
-        sts16(DZ.chunk(tid, c * 2 + 1), make_uint4(s[4], s[5], s[6], s[7]));
+        sts16(DZ.chunk(row, c * 2), make_uint4(s[0], s[1], s[2], s[3]));
+        sts16(DZ.chunk(row, c * 2 + 1), make_uint4(s[4], s[5], s[6], s[7]));
         const float col = lane_sums16(g);
-        if ((lane & 1) == 0) sb1[warp][half * 64 + c * 16 + (lane >> 1)] += col;
+        if ((lane & 1) == 0) sb1[quarter][half * 64 + c * 16 + (lane >> 1)] += col;
       }
       if ((stop = cta.sync())) break;
       if (tid == 0) {
@@ -836,62 +875,57 @@ __global__ void __launch_bounds__(128) k_head_bwd(Head p) {
     }
     if (stop) break;
     cta.wait(0);
-    const int wv = max(0, min(32, nv - warp * 32));
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
+    const int wv = max(0, min(32, nv - quarter * 32));
+    {
       float v[16];
-      tmem_ld16(dH + lanes + half * 16, v);
+      tmem_ld16(dH + lanes + part * 16, v);
       tmem_wait();
 #pragma unroll
-      for (int j = 0; j < 16; ++j) sb[half * 16 + j] += v[j];
+      for (int j = 0; j < 16; ++j) sb[j] += v[j];
 #pragma unroll
       for (int c = 0; c < 2; ++c)
-        sts16(stage + lane * kStagePitch + half * 32 + c * 16,
+        sts16(stage + lane * kStagePitch + c * 16,
               make_uint4(pack_bits(bf16_bits(v[8 * c]), bf16_bits(v[8 * c + 1])),
                          pack_bits(bf16_bits(v[8 * c + 2]), bf16_bits(v[8 * c + 3])),
                          pack_bits(bf16_bits(v[8 * c + 4]), bf16_bits(v[8 * c + 5])),
                          pack_bits(bf16_bits(v[8 * c + 6]), bf16_bits(v[8 * c + 7]))));
     }
-    stage_out(stage, reinterpret_cast<unsigned char*>(p.dz + (row0 + warp * 32) * kC), kC * 2, wv);
+    stage_out(stage, kStagePitch,
+              reinterpret_cast<unsigned char*>(p.dz + (row0 + quarter * 32) * kC + part * 16), kC * 2, wv);
   }
   if (!stop) stop = cta.sync();
   if (!stop && !first) {
     // accumulators: rows 0 .. 63 dz1 channels (columns: h), 64 .. 127 y1 channels (columns 32 ..: dy)
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const int q = half * 64 + (tid & 63);
-      if (warp < 2) {
+    {
+      const int q = part * 64 + (row & 63);          // part: the half of the projected channels
+      if (quarter < 2) {
 #pragma unroll
         for (int c0 = 0; c0 < kC; c0 += 16) {
           float v[16];
-          tmem_ld16(dAcc + half * 48 + lanes + c0, v);
+          tmem_ld16(dAcc + part * 48 + lanes + c0, v);
           tmem_wait();
 #pragma unroll
           for (int j = 0; j < 16; ++j) atomicAdd(p.gQ1 + (c0 + j) * kQ + q, v[j]);
         }
       } else {
         float v[16];
-        tmem_ld16(dAcc + half * 48 + lanes + kC, v);
+        tmem_ld16(dAcc + part * 48 + lanes + kC, v);
         tmem_wait();
 #pragma unroll
         for (int j = 0; j < 4; ++j) atomicAdd(p.gQ2 + q * 4 + j, v[j]);
       }
     }
-    atomicAdd(p.gb1 + tid, (sb1[0][tid] + sb1[1][tid]) + (sb1[2][tid] + sb1[3][tid]));
+    if (tid < kQ) atomicAdd(p.gb1 + tid, (sb1[0][tid] + sb1[1][tid]) + (sb1[2][tid] + sb1[3][tid]));
+    const float s = lane_sums16(sb);
+    if ((lane & 1) == 0) atomicAdd(p.gb + part * 16 + (lane >> 1), s);
+    if (part == 0) {
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      float v[16];
+      for (int j = 0; j < 4; ++j) {
+        float d = sb2[j];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = sb[c * 16 + j];
-      const float s = lane_sums16(v);
-      if ((lane & 1) == 0) atomicAdd(p.gb + c * 16 + (lane >> 1), s);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      float s = sb2[j];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) atomicAdd(p.gb2 + j, s);
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (lane == 0) atomicAdd(p.gb2 + j, d);
+      }
     }
   }
   cta.finish(stop);
@@ -922,11 +956,12 @@ constexpr size_t bwd_smem(int tiles) {
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(128) k_bwd_rows(BwdRows p) {
+__global__ void __launch_bounds__(kThreads) k_bwd_rows(BwdRows p) {
   extern __shared__ __align__(1024) uint8_t tc_smem[];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t slot;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int row = tid & 127, half = tid >> 7, quarter = warp & 3;
   const int tiles = (p.N + kTileRows - 1) / kTileRows;
   uint32_t at = smem_u32(tc_smem);
   auto take = [&](uint32_t bytes) { const uint32_t a = at; at += bytes; return a; };
@@ -941,19 +976,19 @@ __global__ void __launch_bounds__(128) k_bwd_rows(BwdRows p) {
   Cta<128, 2> cta;
   cta.start(bars, &slot);
   const uint32_t tW = cta.tmem, tF = cta.tmem + 32, tM = cta.tmem + 64, tG = cta.tmem + 96;
-  const uint32_t lanes = (uint32_t)(warp * 32) << 16;
+  const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
   if (MODE != 2) load_modes(GT, p.GT, p.N, tiles * 16);
   if (MODE != 0) {
     load_sites(F1T, p.F1T, p.N, tiles * kTileRows);
-    sts16(W.chunk(tid >> 2, tid & 3), __ldg(reinterpret_cast<const uint4*>(p.W) + tid));
+    if (tid < 128) sts16(W.chunk(tid >> 2, tid & 3), __ldg(reinterpret_cast<const uint4*>(p.W) + tid));
   }
   if (MODE == 2) {      // rows of left^T beyond the inputs stay zero
-    for (int i = tid; i < (int)kColBytes / 16; i += 128) sts16(L.base + i * 16, make_uint4(0, 0, 0, 0));
+    for (int i = tid; i < (int)kColBytes / 16; i += kThreads) sts16(L.base + i * 16, make_uint4(0, 0, 0, 0));
     __syncthreads();
   }
-  float sb[kC];
+  float sb[16];
 #pragma unroll
-  for (int i = 0; i < kC; ++i) sb[i] = 0.f;
+  for (int i = 0; i < 16; ++i) sb[i] = 0.f;
 
   bool stop = false, first = true, pending = false;
   for (int item = blockIdx.x; item < p.items && !stop; item += gridDim.x) {
@@ -961,11 +996,11 @@ __global__ void __launch_bounds__(128) k_bwd_rows(BwdRows p) {
     for (int t = 0; t < tiles && !stop; ++t) {
       const int nv = min(kTileRows, p.N - t * kTileRows);
       const long long row0 = (long long)item * p.N + t * kTileRows;
-      const int wv = max(0, min(32, nv - warp * 32));
+      const int wv = max(0, min(32, nv - quarter * 32));
       if (MODE != 0) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int i = tid + 128 * q;
+        for (int q = 0; q < 2; ++q) {
+          const int i = tid + kThreads * q;
           uint4 v = make_uint4(0, 0, 0, 0);
           if ((i >> 2) < nv) v = *(reinterpret_cast<const uint4*>(p.dz + row0 * kC) + i);
           sts16(A.chunk(i >> 2, i & 3), v);
@@ -981,8 +1016,8 @@ __global__ void __launch_bounds__(128) k_bwd_rows(BwdRows p) {
       if (pending) { cta.wait(1); pending = false; }
       if (MODE != 2) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int i = tid + 128 * q;
+        for (int q = 0; q < 2; ++q) {
+          const int i = tid + kThreads * q;
           uint4 v = make_uint4(0, 0, 0, 0), d = v;
           if ((i >> 2) < nv) {
             v = __ldg(reinterpret_cast<const uint4*>(p.left + row0 * kC) + i);
@@ -993,7 +1028,7 @@ __global__ void __launch_bounds__(128) k_bwd_rows(BwdRows p) {
         }
       } else {
         const uint4* src = reinterpret_cast<const uint4*>(p.left + row0 * p.cin);
-        for (int i = tid; i < kTileRows * p.cin / 8; i += 128) {
+        for (int i = tid; i < kTileRows * p.cin / 8; i += kThreads) {
           uint4 v = make_uint4(0, 0, 0, 0);
           if (i < nv * p.cin / 8) v = __ldg(src + i);
           const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -1004,60 +1039,58 @@ __global__ void __launch_bounds__(128) k_bwd_rows(BwdRows p) {
           }
         }
       }
+      const uint32_t zw = zs + quarter * 32 * kZPitch + half * 64;   // this warp's rows and columns
       if (MODE == 1) {
-        // this warp's rows of z, coalesced into shared memory (row pitch 144 B)
+        // z, coalesced into shared memory
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int i = lane + 32 * q, r = i >> 3, c = i & 7;
+        for (int q = 0; q < 4; ++q) {
+          const int i = lane + 32 * q, r = i >> 2, c = i & 3;
           uint4 v = make_uint4(0, 0, 0, 0);
-          if (r < wv) v = __ldg(reinterpret_cast<const uint4*>(p.z + (row0 + warp * 32) * kC) + i);
-          sts16(zs + (warp * 32 + r) * kZPitch + c * 16, v);
+          if (r < wv) v = __ldg(reinterpret_cast<const uint4*>(p.z + (row0 + quarter * 32 + r) * kC + half * 16) + c);
+          sts16(zw + r * kZPitch + c * 16, v);
         }
         __syncwarp();
       }
       if (MODE != 0) {
         cta.wait(0);
-        uint32_t hp[16];
+        uint32_t hp[8];
+        float v[16], f[16];
+        tmem_ld16(tW + lanes + half * 16, v);
+        tmem_ld16(tF + lanes + half * 16, f);
+        tmem_wait();
+        if (MODE == 1) {
+          float z[16];
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          float v[16], f[16];
-          tmem_ld16(tW + lanes + half * 16, v);
-          tmem_ld16(tF + lanes + half * 16, f);
-          tmem_wait();
-          if (MODE == 1) {
-            float z[16];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              const uint4 u = lds16(zs + tid * kZPitch + half * 64 + c * 16);
-              z[4 * c] = __uint_as_float(u.x); z[4 * c + 1] = __uint_as_float(u.y);
-              z[4 * c + 2] = __uint_as_float(u.z); z[4 * c + 3] = __uint_as_float(u.w);
-            }
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = (f[j] + v[j]) * gelu_grad(z[j]);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = f[j] + v[j];
+          for (int c = 0; c < 4; ++c) {
+            const uint4 u = lds16(zw + lane * kZPitch + c * 16);
+            z[4 * c] = __uint_as_float(u.x); z[4 * c + 1] = __uint_as_float(u.y);
+            z[4 * c + 2] = __uint_as_float(u.z); z[4 * c + 3] = __uint_as_float(u.w);
           }
 #pragma unroll
-          for (int j = 0; j < 16; j += 2) {
-            if (lane >= wv) v[j] = v[j + 1] = 0.f;
-            sb[half * 16 + j] += v[j];
-            sb[half * 16 + j + 1] += v[j + 1];
-            const uint16_t a = bf16_bits(v[j]), b = bf16_bits(v[j + 1]);
-            hp[half * 8 + j / 2] = pack_bits(a, b);
-            sts2(dzT.elem(half * 16 + j, tid), a);
-            sts2(dzT.elem(half * 16 + j + 1, tid), b);
-          }
+          for (int j = 0; j < 16; ++j) v[j] = (f[j] + v[j]) * gelu_grad(z[j]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] = f[j] + v[j];
+        }
+#pragma unroll
+        for (int j = 0; j < 16; j += 2) {
+          if (lane >= wv) v[j] = v[j + 1] = 0.f;
+          sb[j] += v[j];
+          sb[j + 1] += v[j + 1];
+          const uint16_t a = bf16_bits(v[j]), b = bf16_bits(v[j + 1]);
+          hp[j / 2] = pack_bits(a, b);
+          sts2(dzT.elem(half * 16 + j, row), a);
+          sts2(dzT.elem(half * 16 + j + 1, row), b);
         }
         if (MODE == 1) {
-          // staged in this warp's z rows (read above)
+          // staged in this warp's part of z (read above)
           __syncwarp();
-          const uint32_t stage = zs + warp * 32 * kZPitch;
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            sts16(stage + lane * kStagePitch + c * 16,
+          for (int c = 0; c < 2; ++c)
+            sts16(zw + lane * kZPitch + c * 16,
                   make_uint4(hp[4 * c], hp[4 * c + 1], hp[4 * c + 2], hp[4 * c + 3]));
-          stage_out(stage, reinterpret_cast<unsigned char*>(p.dz + (row0 + warp * 32) * kC), kC * 2, wv);
+          stage_out(zw, kZPitch,
+                    reinterpret_cast<unsigned char*>(p.dz + (row0 + quarter * 32) * kC + half * 16), kC * 2, wv);
         }
       }
       if ((stop = cta.sync())) break;
@@ -1072,49 +1105,36 @@ __global__ void __launch_bounds__(128) k_bwd_rows(BwdRows p) {
     if (MODE != 2 && !stop) {
       cta.wait(1);
       pending = false;
-      if (warp == 0) {
-        uint32_t s[16];
+      if (quarter == 0) {
+        uint32_t s[8];
+        float v[16];
+        tmem_ld16(tM + half * 16, v);
+        tmem_wait();
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          float v[16];
-          tmem_ld16(tM + half * 16, v);
-          tmem_wait();
+        for (int j = 0; j < 16; j += 2) s[j / 2] = pack_bits(bf16_bits(v[j]), bf16_bits(v[j + 1]));
+        uint4* o = reinterpret_cast<uint4*>(p.dWm + (long long)item * (kM * kC) + lane * kC + half * 16);
 #pragma unroll
-          for (int j = 0; j < 16; j += 2)
-            s[half * 8 + j / 2] = pack_bits(bf16_bits(v[j]), bf16_bits(v[j + 1]));
-        }
-        uint4* o = reinterpret_cast<uint4*>(p.dWm + (long long)item * (kM * kC) + lane * kC);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) o[c] = make_uint4(s[4 * c], s[4 * c + 1], s[4 * c + 2], s[4 * c + 3]);
+        for (int c = 0; c < 2; ++c) o[c] = make_uint4(s[4 * c], s[4 * c + 1], s[4 * c + 2], s[4 * c + 3]);
       }
     }
   }
   if (pending && !stop) { cta.wait(1); pending = false; }
   if (!first && !stop) {
-    if (warp == 0) {
+    if (quarter == 0) {
       const int rows = MODE == 2 ? p.cin : kC;
+      float v[16];
+      tmem_ld16(tG + half * 16, v);
+      tmem_wait();
+      if (lane < rows) {
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        float v[16];
-        tmem_ld16(tG + half * 16, v);
-        tmem_wait();
-        if (lane < rows) {
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            atomicAdd(reinterpret_cast<float4*>(p.gW + lane * kC + half * 16 + 4 * c),
-                      make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]));
-        }
+        for (int c = 0; c < 4; ++c)
+          atomicAdd(reinterpret_cast<float4*>(p.gW + lane * kC + half * 16 + 4 * c),
+                    make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]));
       }
     }
     if (MODE != 0) {
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        float v[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = sb[c * 16 + j];
-        const float s = lane_sums16(v);
-        if ((lane & 1) == 0) atomicAdd(p.gb + c * 16 + (lane >> 1), s);
-      }
+      const float s = lane_sums16(sb);
+      if ((lane & 1) == 0) atomicAdd(p.gb + half * 16 + (lane >> 1), s);
     }
   }
   cta.finish(stop);

@@ -789,7 +789,7 @@ struct FusedLaunch {
   template <typename P>
   void rows(void (*k)(P), const P& p, int items, size_t smem, int cols) {
     const int s = slots(smem, cols);
-    run(k, p, dim3((unsigned)(items < s ? items : s)), 128, smem);
+    run(k, p, dim3((unsigned)(items < s ? items : s)), fused::kThreads, smem);
   }
 };
 
