@@ -24,8 +24,8 @@
 // then the additions of its epilogues), so outputs agree with it bit for bit;
 // only the order of the FP32 sums of weight and bias gradients differs.
 // Measured, GEMM sequence -> fused: training step 256 x 256, batch 8, 3.84 ->
-// 1.15 ms, 64 x 64, batch 4, 1.70 -> 0.33 ms (105 launches from Python -> 22
-// from one call), inference 256 x 256, batch 1, 0.65 -> 0.185 ms.
+// 0.90 ms, 64 x 64, batch 4, 1.70 -> 0.22 ms (105 launches from Python -> 22
+// from one call), inference 256 x 256, batch 1, 0.65 -> 0.105 ms.
 
 namespace fused {
 
@@ -180,9 +180,29 @@ struct Cta {
 // The row kernels run 256 threads per 128 sites: a warp w owns the rows 32 (w %
 // 4) .. of the tile (the TMEM lanes it may read) and the columns of half w / 4,
 // so that twice as many warps hide the latency of the activations per byte of
-// shared memory (training step 256 x 256, batch 8: 1,150 -> TRAIN_US us, with
-// the wider slabs of k_spectral).
+// shared memory (training step 256 x 256, batch 8: 1,150 -> 972 us, with the
+// wider slabs of k_spectral).
 constexpr int kThreads = 256;
+
+// Chained launches (programmatic dependent launch): a kernel loads its constant
+// operands while its predecessor's last CTAs run, then waits for the
+// predecessor's results, and only then lets its own successor start, so that
+// whatever ran before the predecessor is complete too.  Before the wait a
+// kernel reads nothing but weights and DFT matrices, which no kernel of a pass
+// writes; the first kernel of a pass is launched without overlap.  Together
+// with the prefetch of the next tile's rows: training step 256 x 256, batch 8,
+// 972 -> 902 us, 64 x 64, batch 4, 285 -> 224, inference 139 -> 105.
+__device__ __forceinline__ void chain() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+// Read-only load that stays behind chain().
+__device__ __forceinline__ uint4 ldg16(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];\n"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
 
 // Per-warp staging of 32 rows x 32 bytes: row-owning lanes <-> 16-byte pieces
 // in row order, so that global stores write whole sectors.
@@ -205,10 +225,16 @@ __device__ __forceinline__ void stage_out(uint32_t st, int sp, unsigned char* ds
 
 // B operand (n = 32, k = 32) from a row-major [k][n] BF16 matrix, one 16-byte
 // piece per thread of 128.
-__device__ __forceinline__ void load_kn32(const Op& o, const __nv_bfloat16* p) {
+__device__ __forceinline__ uint4 fetch_kn32(const __nv_bfloat16* p) {
+  return threadIdx.x < 128 ? ldg16(reinterpret_cast<const uint4*>(p) + threadIdx.x) : make_uint4(0, 0, 0, 0);
+}
+__device__ __forceinline__ void store_kn32(const Op& o, uint4 v) {
   const int i = threadIdx.x;
-  if (i < 128)
-    scatter8(o, (i & 3) * 8, i >> 2, __ldg(reinterpret_cast<const uint4*>(p) + i));
+  if (i < 128) scatter8(o, (i & 3) * 8, i >> 2, v);
+}
+// Piece i of rows row0 .. of a [rows][32] BF16 array (nv rows valid).
+__device__ __forceinline__ uint4 fetch_row(const __nv_bfloat16* p, long long row0, int i, int nv) {
+  return (i >> 2) < nv ? ldg16(reinterpret_cast<const uint4*>(p + row0 * kC) + i) : make_uint4(0, 0, 0, 0);
 }
 
 // A operand (32 rows, k = sites) from a row-major [32][N] matrix, zero beyond N.
@@ -265,7 +291,7 @@ constexpr size_t fwd_smem(int tiles) {
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kThreads) k_fwd_rows(FwdRows p) {
+__global__ void __launch_bounds__(kThreads, 3) k_fwd_rows(FwdRows p) {
   extern __shared__ __align__(1024) uint8_t tc_smem[];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t slot;
@@ -291,7 +317,7 @@ __global__ void __launch_bounds__(kThreads) k_fwd_rows(FwdRows p) {
   if (MODE != 2) load_modes(F1, p.F1, p.N, tiles * 16);
   if (MODE != 0) {
     load_sites(G, p.G, p.N, tiles * kTileRows);
-    load_kn32(W, p.W);
+    store_kn32(W, fetch_kn32(p.W));
   } else {
     // x P: k = inputs, padded with zeros to 16
     for (int q = 0; q < 2; ++q) sts16(A.base + (tid + kThreads * q) * 16, make_uint4(0, 0, 0, 0));
@@ -301,10 +327,23 @@ __global__ void __launch_bounds__(kThreads) k_fwd_rows(FwdRows p) {
     }
     __syncthreads();
   }
+  chain();
 
+  // the next tile's rows (and the next canvas row's Wm) are loaded while this
+  // one is computed
+  uint4 nextA[2] = {}, nextW = make_uint4(0, 0, 0, 0);
+  auto prefetch = [&](int item, int t) {
+    if (MODE == 0 || item >= p.items) return;
+    const int nv = min(kTileRows, p.N - t * kTileRows);
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      nextA[q] = fetch_row(p.in, (long long)item * p.N + t * kTileRows, tid + kThreads * q, nv);
+    if (t == 0) nextW = fetch_kn32(p.Wm + (long long)item * (kM * kC));
+  };
+  prefetch(blockIdx.x, 0);
   bool stop = false;
   for (int item = blockIdx.x; item < p.items && !stop; item += gridDim.x) {
-    if (MODE != 0) load_kn32(Wm, p.Wm + (long long)item * (kM * kC));
+    if (MODE != 0) store_kn32(Wm, nextW);
     for (int t = 0; t < tiles && !stop; ++t) {
       const int nv = min(kTileRows, p.N - t * kTileRows);
       const long long row0 = (long long)item * p.N + t * kTileRows;
@@ -312,9 +351,7 @@ __global__ void __launch_bounds__(kThreads) k_fwd_rows(FwdRows p) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const int i = tid + kThreads * q;
-          uint4 v = make_uint4(0, 0, 0, 0);
-          if ((i >> 2) < nv) v = __ldg(reinterpret_cast<const uint4*>(p.in + row0 * kC) + i);
-          sts16(A.chunk(i >> 2, i & 3), v);
+          sts16(A.chunk(i >> 2, i & 3), nextA[q]);
         }
       } else {
         const uint4* src = reinterpret_cast<const uint4*>(p.in + row0 * p.cin);
@@ -336,6 +373,8 @@ __global__ void __launch_bounds__(kThreads) k_fwd_rows(FwdRows p) {
         mma(dW, A, 0, W, 0, kC, MODE != 0 ? 2 : 1, false);
         commit(cta.bar(0));
       }
+      if (t + 1 < tiles) prefetch(item, t + 1);
+      else prefetch(item + (int)gridDim.x, 0);
       cta.wait(0);
       if (MODE != 2 && t > 0) cta.wait(1);      // the transform has read hT
       const int wv = max(0, min(32, nv - quarter * 32));   // valid rows of this warp
@@ -473,21 +512,25 @@ __global__ void __launch_bounds__(256) k_spectral(Spectral p) {
   const int slabs = (K + kSlabK - 1) / kSlabK;
   bool stop = false;
   uint4 ra[8], rb[4];
-  auto load_slab = [&](int s) {
+  auto load_a1 = [&](int s) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int i = tid + 256 * q, k = s * kSlabK + (i & 31) * 8;
       ra[q] = make_uint4(0, 0, 0, 0);
       if (k < K) ra[q] = __ldg(reinterpret_cast<const uint4*>(p.A1 + (long long)(i >> 5) * K + k));
     }
+  };
+  auto load_x = [&](int s) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int i = tid + 256 * q, k = s * kSlabK + (i >> 2);
       rb[q] = make_uint4(0, 0, 0, 0);
-      if (k < K) rb[q] = __ldg(reinterpret_cast<const uint4*>(X + (long long)k * (kKy * kC)) + (i & 3));
+      if (k < K) rb[q] = ldg16(reinterpret_cast<const uint4*>(X + (long long)k * (kKy * kC)) + (i & 3));
     }
   };
-  load_slab(0);
+  load_a1(0);
+  chain();
+  load_x(0);
   for (int s = 0; s < slabs; ++s) {
     if (s > 0) cta.wait(0);
 #pragma unroll
@@ -505,7 +548,7 @@ __global__ void __launch_bounds__(256) k_spectral(Spectral p) {
       mma(cta.tmem, A1, 0, B, 0, kC, min(kSlabK, ((K - s * kSlabK) + 15) / 16 * 16) / 16, s > 0);
       commit(cta.bar(0));
     }
-    if (s + 1 < slabs) load_slab(s + 1);
+    if (s + 1 < slabs) { load_a1(s + 1); load_x(s + 1); }
     else load_a2(0);
   }
   // mixing: a warp takes kx = warp, warp + 8, ..; lane = output channel.  The
@@ -600,11 +643,21 @@ __global__ void __launch_bounds__(256) k_spectral(Spectral p) {
 
 // dR(kx, ky, i, o) += sum_b conj(S(b, kx, ky, i)) dU(b, kx, ky, o); one block
 // per (kx, ky), the batch's modes in shared memory, 8-byte accesses of dR.
-__global__ void __launch_bounds__(256) k_mix_grad(const float* __restrict__ S,
-                                                  const float* __restrict__ dU, float2* dR, int batch) {
+struct MixGrad {
+  const float *S, *dU;
+  float2* dR;
+  int batch;
+};
+
+__global__ void __launch_bounds__(256) k_mix_grad(MixGrad p) {
+  const float* const S = p.S;
+  const float* const dU = p.dU;
+  float2* const dR = p.dR;
+  const int batch = p.batch;
   __shared__ float s[16][2][kC], g[16][2][kC];
   const int kx = blockIdx.x / kKy, ky = blockIdx.x % kKy, o = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float rre[4] = {}, rim[4] = {};
+  chain();
   for (int b0 = 0; b0 < batch; b0 += 16) {
     const int nb = min(16, batch - b0);
     __syncthreads();
@@ -658,7 +711,7 @@ __device__ __forceinline__ void load_q1(const Op& o, const __nv_bfloat16* Q1) {
     scatter8(o, (i % (kQ / 8)) * 8, i / (kQ / 8), __ldg(reinterpret_cast<const uint4*>(Q1) + i));
 }
 
-__global__ void __launch_bounds__(kThreads) k_head_fwd(Head p) {
+__global__ void __launch_bounds__(kThreads, 4) k_head_fwd(Head p) {
   extern __shared__ __align__(1024) uint8_t tc_smem[];
   __shared__ __align__(8) uint64_t bars[1];
   __shared__ uint32_t slot;
@@ -680,6 +733,15 @@ __global__ void __launch_bounds__(kThreads) k_head_fwd(Head p) {
   const float4 b2 = make_float4(p.bq2[0], p.bq2[1], p.bq2[2], p.bq2[3]);
   const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
   const long long tiles = (p.rows + 127) / 128;
+  chain();
+  uint4 next[2];
+  auto prefetch = [&](long long t) {
+    if (t >= tiles) return;
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      next[q] = fetch_row(p.h, t * 128, tid + kThreads * q, (int)min(128LL, p.rows - t * 128));
+  };
+  prefetch(blockIdx.x);
   bool stop = false;
   for (long long t = blockIdx.x; t < tiles && !stop; t += gridDim.x) {
     const long long row0 = t * 128;
@@ -687,15 +749,14 @@ __global__ void __launch_bounds__(kThreads) k_head_fwd(Head p) {
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int i = tid + kThreads * q;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if ((i >> 2) < nv) v = __ldg(reinterpret_cast<const uint4*>(p.h + row0 * kC) + i);
-      sts16(A.chunk(i >> 2, i & 3), v);
+      sts16(A.chunk(i >> 2, i & 3), next[q]);
     }
     if ((stop = cta.sync())) break;
     if (tid == 0) {
       mma(cta.tmem, A, 0, Q1, 0, kQ, 2, false);
       commit(cta.bar(0));
     }
+    prefetch(t + gridDim.x);
     cta.wait(0);
 #pragma unroll 1
     for (int c0 = half * 64; c0 < half * 64 + 64; c0 += 16) {
@@ -760,7 +821,7 @@ __device__ __forceinline__ float lane_sums16(float (&v)[16]) {
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-__global__ void __launch_bounds__(kThreads) k_head_bwd(Head p) {
+__global__ void __launch_bounds__(kThreads, 2) k_head_bwd(Head p) {
   extern __shared__ __align__(1024) uint8_t tc_smem[];
   __shared__ __align__(8) uint64_t bars[1];
   __shared__ uint32_t slot;
@@ -801,6 +862,17 @@ __global__ void __launch_bounds__(kThreads) k_head_bwd(Head p) {
   for (int i = 0; i < 16; ++i) sb[i] = 0.f;
 
   const long long tiles = (p.rows + 127) / 128;
+  chain();
+  uint4 nextA[2], nextD = make_uint4(0, 0, 0, 0);
+  auto prefetch = [&](long long t) {
+    if (t >= tiles) return;
+    const int nv = (int)min(128LL, p.rows - t * 128);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) nextA[q] = fetch_row(p.h, t * 128, tid + kThreads * q, nv);
+    if (part == 0)
+      nextD = row < nv ? ldg16(reinterpret_cast<const uint4*>(p.dy) + t * 128 + row) : make_uint4(0, 0, 0, 0);
+  };
+  prefetch(blockIdx.x);
   bool stop = false, first = true;
   for (long long t = blockIdx.x; t < tiles && !stop; t += gridDim.x, first = false) {
     const long long row0 = t * 128;
@@ -808,14 +880,12 @@ __global__ void __launch_bounds__(kThreads) k_head_bwd(Head p) {
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int i = tid + kThreads * q;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if ((i >> 2) < nv) v = __ldg(reinterpret_cast<const uint4*>(p.h + row0 * kC) + i);
-      sts16(A.chunk(i >> 2, i & 3), v);
-      scatter8(Bw, (i & 3) * 8, i >> 2, v);
+      sts16(A.chunk(i >> 2, i & 3), nextA[q]);
+      scatter8(Bw, (i & 3) * 8, i >> 2, nextA[q]);
     }
     if (part == 0) {
-      float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (row < nv) d = __ldg(reinterpret_cast<const float4*>(p.dy) + row0 + row);
+      const float4 d = make_float4(__uint_as_float(nextD.x), __uint_as_float(nextD.y),
+                                   __uint_as_float(nextD.z), __uint_as_float(nextD.w));
       sb2[0] += d.x; sb2[1] += d.y; sb2[2] += d.z; sb2[3] += d.w;
       const uint16_t e[4] = {bf16_bits(d.x), bf16_bits(d.y), bf16_bits(d.z), bf16_bits(d.w)};
 #pragma unroll
@@ -830,6 +900,7 @@ __global__ void __launch_bounds__(kThreads) k_head_bwd(Head p) {
       mma(dY, DY, 0, Q2t, 0, 64, 1, false);
       commit(cta.bar(0));
     }
+    prefetch(t + gridDim.x);
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
       cta.wait(0);
@@ -956,7 +1027,7 @@ constexpr size_t bwd_smem(int tiles) {
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kThreads) k_bwd_rows(BwdRows p) {
+__global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(BwdRows p) {
   extern __shared__ __align__(1024) uint8_t tc_smem[];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t slot;
@@ -990,9 +1061,25 @@ __global__ void __launch_bounds__(kThreads) k_bwd_rows(BwdRows p) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) sb[i] = 0.f;
 
+  chain();
+  // the next tile's dz and left operand (and the next canvas row's dS1) are
+  // loaded while this one is computed
+  uint4 nextD[2] = {}, nextL[2] = {}, nextS = make_uint4(0, 0, 0, 0);
+  auto prefetch = [&](int item, int t) {
+    if (item >= p.items) return;
+    const int nv = min(kTileRows, p.N - t * kTileRows);
+    const long long row0 = (long long)item * p.N + t * kTileRows;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      nextD[q] = fetch_row(p.dz, row0, tid + kThreads * q, nv);
+      if (MODE != 2) nextL[q] = fetch_row(p.left, row0, tid + kThreads * q, nv);
+    }
+    if (MODE != 0 && t == 0) nextS = fetch_kn32(p.dS1 + (long long)item * (kM * kC));
+  };
+  prefetch(blockIdx.x, 0);
   bool stop = false, first = true, pending = false;
   for (int item = blockIdx.x; item < p.items && !stop; item += gridDim.x) {
-    if (MODE != 0) load_kn32(dS, p.dS1 + (long long)item * (kM * kC));
+    if (MODE != 0) store_kn32(dS, nextS);
     for (int t = 0; t < tiles && !stop; ++t) {
       const int nv = min(kTileRows, p.N - t * kTileRows);
       const long long row0 = (long long)item * p.N + t * kTileRows;
@@ -1001,9 +1088,7 @@ __global__ void __launch_bounds__(kThreads) k_bwd_rows(BwdRows p) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const int i = tid + kThreads * q;
-          uint4 v = make_uint4(0, 0, 0, 0);
-          if ((i >> 2) < nv) v = *(reinterpret_cast<const uint4*>(p.dz + row0 * kC) + i);
-          sts16(A.chunk(i >> 2, i & 3), v);
+          sts16(A.chunk(i >> 2, i & 3), nextD[q]);
         }
         if ((stop = cta.sync())) break;
         if (tid == 0) {
@@ -1018,13 +1103,8 @@ __global__ void __launch_bounds__(kThreads) k_bwd_rows(BwdRows p) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const int i = tid + kThreads * q;
-          uint4 v = make_uint4(0, 0, 0, 0), d = v;
-          if ((i >> 2) < nv) {
-            v = __ldg(reinterpret_cast<const uint4*>(p.left + row0 * kC) + i);
-            if (MODE == 0) d = __ldg(reinterpret_cast<const uint4*>(p.dz + row0 * kC) + i);
-          }
-          scatter8(L, (i & 3) * 8, i >> 2, v);
-          if (MODE == 0) scatter8(dzT, (i & 3) * 8, i >> 2, d);
+          scatter8(L, (i & 3) * 8, i >> 2, nextL[q]);
+          if (MODE == 0) scatter8(dzT, (i & 3) * 8, i >> 2, nextD[q]);
         }
       } else {
         const uint4* src = reinterpret_cast<const uint4*>(p.left + row0 * p.cin);
@@ -1039,6 +1119,8 @@ __global__ void __launch_bounds__(kThreads) k_bwd_rows(BwdRows p) {
           }
         }
       }
+      if (t + 1 < tiles) prefetch(item, t + 1);
+      else prefetch(item + (int)gridDim.x, 0);
       const uint32_t zw = zs + quarter * 32 * kZPitch + half * 64;   // this warp's rows and columns
       if (MODE == 1) {
         // z, coalesced into shared memory

@@ -771,6 +771,7 @@ struct FusedLaunch {
   cudaStream_t st;
   int sms;
   cudaError_t e;
+  bool first;       // the first kernel of a pass starts after everything before it
   // CTAs that fit an SM by shared memory and tensor memory
   int slots(size_t smem, int cols) const {
     const int by_smem = (int)(228 * 1024 / (smem + 2048)), by_tmem = 512 / cols;
@@ -783,8 +784,19 @@ struct FusedLaunch {
     if (smem > 48 * 1024)
       e = cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return;
-    k<<<grid, threads, smem, st>>>(p);
-    e = cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = first ? 0 : 1;
+    first = false;
+    e = cudaLaunchKernelEx(&cfg, k, p);
+    if (e == cudaSuccess) e = cudaGetLastError();
   }
   template <typename P>
   void rows(void (*k)(P), const P& p, int items, size_t smem, int cols) {
@@ -800,6 +812,7 @@ int fused_start(const rlbm_fno_net* n, void* stream, FusedLaunch& f) {
     return RLBM_EINVAL;
   f.st = static_cast<cudaStream_t>(stream);
   f.e = cudaSuccess;
+  f.first = true;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -1054,11 +1067,8 @@ int rlbm_fno_backward(const rlbm_fno_net* n, void* stream) {
       s.A1 = b16(n->DinvT); s.X = b16(n->dWm); s.A2 = b16(n->DT);
       s.R = n->R + l * nr; s.S2 = n->dU; s.out = b16(n->dS1); s.N = n->N;
       f.run(fused::k_spectral<true>, s, dim3(fused::kKy, (unsigned)n->batch), 256, fused::kSpectralSmem);
-      if (f.e == cudaSuccess) {
-        fused::k_mix_grad<<<(fused::kModes / 2) * fused::kKy, 256, 0, f.st>>>(
-            n->S2[l], n->dU, reinterpret_cast<float2*>(n->gR + l * nr), n->batch);
-        f.e = cudaGetLastError();
-      }
+      const fused::MixGrad m{n->S2[l], n->dU, reinterpret_cast<float2*>(n->gR + l * nr), n->batch};
+      f.run(fused::k_mix_grad, m, dim3((fused::kModes / 2) * fused::kKy), 256, 0);
     } else {
       w.left = b16(n->x); w.gW = n->gP; w.gb = n->gbp;
       f.rows(fused::k_bwd_rows<2>, w, items, fused::bwd_smem<2>(T), 128);
