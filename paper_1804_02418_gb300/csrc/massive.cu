@@ -84,16 +84,21 @@ __host__ __device__ constexpr int class_fn(int c) {        // first component fu
 template <typename R>
 struct MConsts {
   using V = typename V2<R>::T;
-  R mN0[kPairs], mE[kPairs], mPxx[kPairs], mPxy[kPairs], mPyy[kPairs];
-  R mNx[kPairs], mNy[kPairs], mMx[kPairs], mMy[kPairs];
+  // moments: f0 times 1, p0, (p^x v^x + p^y v^y) / 2, its difference, p^x v^y
+  R mN0[kClasses], mE[kClasses], mPs[kClasses], mPd[kClasses], mPxy[kClasses];
+  V mN[kOddFns], mM[kOddFns];   // f0 v and f0 p of the component, both lanes alike
   R A[kClasses][8];      // dT, dn dT, dT^2, ux^2 + uy^2, E0, E1, E2 + E4, E5 + E7 (9: rest)
   R C1[kClasses][3];     // ux^2 - uy^2, E2 - E4, E5 - E7
   R C2[kClasses][3];     // ux uy, E3, E6
   V O[kOddFns][7];       // (x, y) lanes alike: u, dn u, dT u, O0/O1, O2/O3, O4/O7, O6/O5
   V va[kOddFns], pa[kOddFns];   // v and p of the component, both lanes alike
   R p0[kClasses], rr[kClasses], dd[kClasses], pp[kClasses];   // (px^2 +- py^2) / 2, |px py|
-  R gi[16][16];
-  R restN0, restE;
+  // (m + 1) G^-1 by symmetry.  Even rows, negated (the source takes them with
+  // that sign): p0; px^2 + py^2 and its difference; px py; the same times p0.
+  // Columns: 1, p0, px^2 + py^2, p0 (px^2 + py^2), or those of one parity.
+  // Odd rows and columns px, p0 px, px^3, px py^2, in lanes with py, p0 py, ..
+  R n1[4], nS[4], n0S[4], nD[2], n0D[2], nX[2], n0X[2];
+  V gO[4][4];
   double f0[kQm], if0[kQm], ifl[kQm];      // 1 / f0 = if0 + ifl
 };
 
@@ -103,20 +108,6 @@ __constant__ MConsts<double> c_d;
 template <typename R> __device__ __forceinline__ const MConsts<R>& mc();
 template <> __device__ __forceinline__ const MConsts<float>& mc<float>() { return c_f; }
 template <> __device__ __forceinline__ const MConsts<double>& mc<double>() { return c_d; }
-
-// library monomial order (massive_tables.h): exponents of p0, px, py
-__host__ __device__ constexpr int mon_b(int k) {
-  return k == 2 ? 2 : k == 3 ? 1 : k == 5 ? 2 : k == 6 ? 1 : k == 8 ? 1 : k == 10 ? 1 : k == 12 ? 3
-       : k == 13 ? 2 : k == 14 ? 1 : 0;
-}
-__host__ __device__ constexpr int mon_c(int k) {
-  return k == 3 ? 1 : k == 4 ? 2 : k == 6 ? 1 : k == 7 ? 2 : k == 9 ? 1 : k == 11 ? 1 : k == 13 ? 1
-       : k == 14 ? 2 : k == 15 ? 3 : 0;
-}
-// G couples two monomials only if their px and py exponents have equal parities
-__host__ __device__ constexpr bool same_block(int a, int b) {
-  return ((mon_b(a) ^ mon_b(b)) & 1) == 0 && ((mon_c(a) ^ mon_c(b)) & 1) == 0;
-}
 
 struct MGeom {
   int nx, ny, ldx;
@@ -217,33 +208,95 @@ __device__ __forceinline__ bool site_interior(const MGeom& g, int x, int y) {
   return x >= kReach && x < g.nx - kReach && y >= kReach && y < g.ny - kReach;
 }
 
+// (x, y) lanes of FP32 (Blackwell's paired FMA) and of FP64 (two operations).
+__device__ __forceinline__ float2 S2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ double2 S2(double a) { return make_double2(a, a); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c) {
+  return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
+}
+__device__ __forceinline__ double2 mul2(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
+__device__ __forceinline__ double2 add2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 pair_of(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ double2 pair_of(double a, double b) { return make_double2(a, b); }
+// sign pairs (constant memory, so that they cost no instruction to form in FP32)
+__constant__ float2 c_pm = {1.f, -1.f};
+__constant__ float2 c_mp = {-1.f, 1.f};
+template <typename R> __device__ __forceinline__ typename V2<R>::T pm();
+template <> __device__ __forceinline__ float2 pm<float>() { return c_pm; }
+template <> __device__ __forceinline__ double2 pm<double>() { return make_double2(1.0, -1.0); }
+template <typename R> __device__ __forceinline__ typename V2<R>::T mp();
+template <> __device__ __forceinline__ float2 mp<float>() { return c_mp; }
+template <> __device__ __forceinline__ double2 mp<double>() { return make_double2(-1.0, 1.0); }
+
+// Moments class by class: the sums of a class that its symmetry leaves, once
+// per monomial (171 operations per site, where pair by pair took 235).
+template <typename R>
+struct MomSums {
+  using V = typename V2<R>::T;
+  R n0, e, ps, pd, xy;       // N^0, T^00, (T^xx + T^yy) / 2, (T^xx - T^yy) / 2, T^xy
+  V n, m;                    // N^a, T^0a
+};
+
+template <int C, typename R>
+__device__ __forceinline__ void class_moments(const R (&g)[kQm], MomSums<R>& s) {
+  const MConsts<R>& c = mc<R>();
+  constexpr int q = 2 * class_pair(C), kind = class_kind(C), f = class_fn(C);
+  const R s0 = g[q] + g[q + 1], s1 = g[q + 2] + g[q + 3];
+  const R o0 = g[q] - g[q + 1], o1 = g[q + 2] - g[q + 3];
+  R S = s0 + s1;
+  const R D = s0 - s1;
+  if constexpr (kind == 0) {                   // (a, 0), (0, a)
+    s.pd = fma(c.mPd[C], D, s.pd);
+    const auto o = pair_of(o0, o1);
+    s.n = fma2(c.mN[f], o, s.n);
+    s.m = fma2(c.mM[f], o, s.m);
+  } else if constexpr (kind == 1) {            // (a, a), (-a, a)
+    s.xy = fma(c.mPxy[C], D, s.xy);
+    const auto o = pair_of(o0 - o1, o0 + o1);
+    s.n = fma2(c.mN[f], o, s.n);
+    s.m = fma2(c.mM[f], o, s.m);
+  } else {                                     // (a, b), (-a, b), (b, a), (-b, a)
+    const R s2 = g[q + 4] + g[q + 5], s3 = g[q + 6] + g[q + 7];
+    const R o2 = g[q + 4] - g[q + 5], o3 = g[q + 6] - g[q + 7];
+    const R S1 = s2 + s3;
+    s.pd = fma(c.mPd[C], S - S1, s.pd);
+    s.xy = fma(c.mPxy[C], D + (s2 - s3), s.xy);
+    S += S1;
+    const auto oa = pair_of(o0 - o1, o2 + o3), ob = pair_of(o2 - o3, o0 + o1);
+    s.n = fma2(c.mN[f + 1], ob, fma2(c.mN[f], oa, s.n));
+    s.m = fma2(c.mM[f + 1], ob, fma2(c.mM[f], oa, s.m));
+  }
+  s.n0 = fma(c.mN0[C], S, s.n0);
+  s.e = fma(c.mE[C], S, s.e);
+  s.ps = fma(c.mPs[C], S, s.ps);
+}
+
 template <int NS, int G, typename R>
 __device__ __forceinline__ MMom<R> mmoments(const R (&g)[kQm]) {
   const MConsts<R>& c = mc<R>();
-  MMom<R> m;
-  m.dN0 = m.dNx = m.dNy = m.dE = m.Mx = m.My = m.dPxx = m.dPxy = m.dPyy = R(0);
-#pragma unroll
-  for (int p = 0; p < kPairs; ++p) {
-    if (!mine(NS, G, p)) continue;
-    const R se = g[2 * p] + g[2 * p + 1], so = g[2 * p] - g[2 * p + 1];
-    m.dN0 = fma(c.mN0[p], se, m.dN0);
-    m.dE = fma(c.mE[p], se, m.dE);
-    if (pair_x(p) != 0) {
-      m.dPxx = fma(c.mPxx[p], se, m.dPxx);
-      m.dNx = fma(c.mNx[p], so, m.dNx);
-      m.Mx = fma(c.mMx[p], so, m.Mx);
-    }
-    if (pair_y(p) != 0) {
-      m.dPyy = fma(c.mPyy[p], se, m.dPyy);
-      m.dNy = fma(c.mNy[p], so, m.dNy);
-      m.My = fma(c.mMy[p], so, m.My);
-    }
-    if (pair_x(p) != 0 && pair_y(p) != 0) m.dPxy = fma(c.mPxy[p], se, m.dPxy);
-  }
+  MomSums<R> s;
+  s.n0 = s.e = s.ps = s.pd = s.xy = R(0);
+  s.n = s.m = S2(R(0));
+  if (class_group(NS, 0) == G) class_moments<0>(g, s);
+  if (class_group(NS, 1) == G) class_moments<1>(g, s);
+  if (class_group(NS, 2) == G) class_moments<2>(g, s);
+  if (class_group(NS, 3) == G) class_moments<3>(g, s);
+  if (class_group(NS, 4) == G) class_moments<4>(g, s);
+  if (class_group(NS, 5) == G) class_moments<5>(g, s);
+  if (class_group(NS, 6) == G) class_moments<6>(g, s);
+  if (class_group(NS, 7) == G) class_moments<7>(g, s);
+  if (class_group(NS, 8) == G) class_moments<8>(g, s);
   if (class_group(NS, 9) == G) {
-    m.dN0 = fma(c.restN0, g[kRestPop], m.dN0);
-    m.dE = fma(c.restE, g[kRestPop], m.dE);
+    s.n0 = fma(c.mN0[9], g[kRestPop], s.n0);
+    s.e = fma(c.mE[9], g[kRestPop], s.e);
   }
+  MMom<R> m;
+  m.dN0 = s.n0; m.dNx = s.n.x; m.dNy = s.n.y;
+  m.dE = s.e; m.Mx = s.m.x; m.My = s.m.y;
+  m.dPxx = s.ps + s.pd; m.dPxy = s.xy; m.dPyy = s.ps - s.pd;
   return m;
 }
 
@@ -352,29 +405,6 @@ __device__ __forceinline__ MMacro<R> macro_of(R n, R ux, R uy, R T) {
   return M;
 }
 
-// (x, y) lanes of FP32 (Blackwell's paired FMA) and of FP64 (two operations).
-__device__ __forceinline__ float2 S2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ double2 S2(double a) { return make_double2(a, a); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c) {
-  return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
-}
-__device__ __forceinline__ double2 mul2(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
-__device__ __forceinline__ double2 add2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 pair_of(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ double2 pair_of(double a, double b) { return make_double2(a, b); }
-// sign pairs (constant memory, so that they cost no instruction to form in FP32)
-__constant__ float2 c_pm = {1.f, -1.f};
-__constant__ float2 c_mp = {-1.f, 1.f};
-template <typename R> __device__ __forceinline__ typename V2<R>::T pm();
-template <> __device__ __forceinline__ float2 pm<float>() { return c_pm; }
-template <> __device__ __forceinline__ double2 pm<double>() { return make_double2(1.0, -1.0); }
-template <typename R> __device__ __forceinline__ typename V2<R>::T mp();
-template <> __device__ __forceinline__ float2 mp<float>() { return c_mp; }
-template <> __device__ __forceinline__ double2 mp<double>() { return make_double2(-1.0, 1.0); }
-
 // Per-site part of the equilibrium: delta, its quadratic monomials and the
 // third-order remainder R3 of the 16 moments (library order), combined by
 // symmetry as the class tables want them.
@@ -384,6 +414,9 @@ struct EqSite {
   R dn, a[8];            // dT, dn dT, dT^2, ux^2 + uy^2, E0, E1, E2 + E4, E5 + E7
   R c1[3], c2[3];        // ux^2 - uy^2, E2 - E4, E5 - E7;  ux uy, E3, E6
   V o[7];                // (x, y): u, dn u, dT u, (O0, O1), (O2, O3), (O4, O7), (O6, O5)
+  // for the source: alpha gamma^3, h gamma^2, T h at linear order, T h gamma -
+  // h0, n gamma, M[1] - 1 / (m + 1)
+  R ag3, hg2, Xl, Thgm, ng, d0;
 };
 
 template <typename R>
@@ -424,7 +457,8 @@ __device__ __forceinline__ EqSite<R> eq_site(const MMacro<R>& M) {
   e.dn = dn;
   const R ud = uxx - uyy;
   e.a[0] = dT; e.a[1] = dn * dT; e.a[2] = dT2; e.a[3] = u2;
-  e.a[4] = (dn * m1 - dT) * dT2 * imT * (im1 * im1 * im1);
+  e.d0 = (dn * m1 - dT) * imT * im1;
+  e.a[4] = e.d0 * dT2 * (im1 * im1);
   e.a[5] = gm1mh + gm1 * dn;
   e.a[6] = hg2m * u2;                                // E2 + E4
   e.a[7] = ag3m * u2 + R(2) * Rthg3;                 // E5 + E7
@@ -440,6 +474,7 @@ __device__ __forceinline__ EqSite<R> eq_site(const MMacro<R>& M) {
   const R R3t = R(3) * Rthg;
   e.o[5] = mul2(pair_of(ag3 * uxx + R3t, ag3 * uyy + R3t), u);       // px^3, py^3
   e.o[6] = mul2(pair_of(ag3 * uyy + Rthg, ag3 * uxx + Rthg), u);     // px py^2, px^2 py
+  e.ag3 = ag3; e.hg2 = H0 + hg2m; e.Xl = Xlin + H0; e.Thgm = Rthg + Xlin; e.ng = ngm + dn;
   return e;
 }
 
@@ -506,66 +541,48 @@ __device__ __forceinline__ R eq_rest(const EqSite<R>& e) {
 //   F^ext_i / f0_i = (F.v_i)(1 + g^eq_i) - (F.v_i) dD/dp0(p_i) - F.grad_xy D(p_i).
 template <typename R>
 struct ForceSite {
-  R a1, a5, a6, a7, a10, a11;               // dD/dp0 = a1 + a5 px^2 + a6 px py + a7 py^2 + a10 px + a11 py
-  R h1, hp0, hxx, hxy, hyy;                 // F.grad_xy D, even part
-  R hx, hy, h0x, h0y;                       //              odd part
+  using V = typename V2<R>::T;
+  R b1, bS, bD, bX;      // 1 - dD/dp0, even part: b1 + bS rr + bD (px^2 - py^2) / 2 + bX px py
+  V a;                   // dD/dp0, odd part: a.x px + a.y py
+  R h1, hp0, hS, hD, hX; // F.grad_xy D, even part, alike (h1 + hp0 p0 + ..)
+  V nh, nh0;             // -F.grad_xy D, odd part: (nh + nh0 p0) . p
 };
 
+// The rows of (m + 1) G^-1 in the combinations that x <-> y leaves uncoupled:
+// 20 even products and 16 on (x, y) lanes (66 without).
 template <typename R>
-__device__ __forceinline__ ForceSite<R> force_site(const MMacro<R>& M, R Fx, R Fy) {
+__device__ __forceinline__ ForceSite<R> force_site(const EqSite<R>& e, R Fx, R Fy) {
+  using V = typename V2<R>::T;
   const MConsts<R>& c = mc<R>();
-  const R m = R(kM), m1 = R(kM1), one = R(1), H0 = R(kH0);
-  const R dn = M.dn, dT = M.dT, ux = M.ux, uy = M.uy, g = M.gamma, gm1 = M.gm1;
-  const R T = one + dT, n = one + dn;
-  const R imT = qrcp(m + T);
-  const R phi = (m * m + R(3) * m * T + R(3) * T * T) * imT;
-  const R kT = (R(3) * m1 * T + R(2) * m * m + R(3) * m) * imT * R(1.0 / kM1);
-  const R dh = dn * phi + dT * kT;
-  const R alpha = n * (m * m * m + R(6) * m * m * T + R(15) * m * T * T + R(15) * T * T * T) * imT;
-  const R hg2 = (H0 + dh) * g * g;
-  const R ag3 = alpha * g * g * g;
-  const R X = T * dh + H0 * dT;                       // T h - h0
-  const R Thgm = X * g + H0 * gm1;                    // T h gamma - h0
-  const R Thg = H0 + Thgm;
-  const R P1 = dn + dT + dn * dT;                     // P - 1
-  const R ngam = dn + gm1 + dn * gm1;                 // n gamma - 1
-  R dM[16];
-  dM[0] = (dn * m1 - dT) * imT * R(1.0 / kM1);
-  dM[1] = ngam;
-  dM[2] = hg2 * ux * ux + P1;
-  dM[3] = hg2 * ux * uy;
-  dM[4] = hg2 * uy * uy + P1;
-  dM[5] = ag3 * ux * ux + Thgm;
-  dM[6] = ag3 * ux * uy;
-  dM[7] = ag3 * uy * uy + Thgm;
-  dM[8] = (one + ngam) * ux;
-  dM[9] = (one + ngam) * uy;
-  dM[10] = hg2 * ux;
-  dM[11] = hg2 * uy;
-  dM[12] = (ag3 * ux * ux + R(3) * Thg) * ux;
-  dM[13] = (ag3 * ux * ux + Thg) * uy;
-  dM[14] = (ag3 * uy * uy + Thg) * ux;
-  dM[15] = (ag3 * uy * uy + R(3) * Thg) * uy;
-  R d[16];
+  const R dn = e.dn, dT = e.a[0], u2 = e.a[3], ud = e.c1[0], uxy = e.c2[0];
+  const R P1 = dn + dT + e.a[1];                      // P - 1
+  // deviations of the moments: 1, p0, px^2 + py^2, p0 (px^2 + py^2) ..
+  const R M[4] = {e.d0, e.ng, fma(e.hg2, u2, P1 + P1), fma(e.ag3, u2, e.Thgm + e.Thgm)};
+  const R MD[2] = {e.hg2 * ud, e.ag3 * ud}, MX[2] = {e.hg2 * uxy, e.ag3 * uxy};
+  const V u = e.o[0];
+  // .. and px, p0 px, px^3, px py^2 with their y partners
+  const V MO[4] = {mul2(S2(R(1) + e.ng), u), mul2(S2(e.hg2), u), fma2(S2(R(3) * e.Xl), u, e.o[5]),
+                   fma2(S2(e.Xl), u, e.o[6])};
+  auto row4 = [&](const R (&t)[4]) { return fma(t[3], M[3], fma(t[2], M[2], fma(t[1], M[1], t[0] * M[0]))); };
+  const R n1 = row4(c.n1), nS = row4(c.nS), n0S = row4(c.n0S);
+  const R nD = fma(c.nD[1], MD[1], c.nD[0] * MD[0]), n0D = fma(c.n0D[1], MD[1], c.n0D[0] * MD[0]);
+  const R nX = fma(c.nX[1], MX[1], c.nX[0] * MX[0]), n0X = fma(c.n0X[1], MX[1], c.n0X[0] * MX[0]);
+  V d[4];
 #pragma unroll
-  for (int a = 0; a < 16; ++a) {
-    R s = R(0);
-#pragma unroll
-    for (int b = 0; b < 16; ++b)
-      if (same_block(a, b)) s = fma(c.gi[a][b], dM[b], s);
-    d[a] = s;
-  }
+  for (int k = 0; k < 4; ++k)
+    d[k] = fma2(c.gO[k][3], MO[3], fma2(c.gO[k][2], MO[2], fma2(c.gO[k][1], MO[1], mul2(c.gO[k][0], MO[0]))));
   ForceSite<R> f;
-  f.a1 = d[1]; f.a5 = d[5]; f.a6 = d[6]; f.a7 = d[7]; f.a10 = d[10]; f.a11 = d[11];
-  f.h1 = Fx * d[8] + Fy * d[9];
-  f.hp0 = Fx * d[10] + Fy * d[11];
-  f.hxx = R(3) * Fx * d[12] + Fy * d[13];
-  f.hxy = R(2) * Fx * d[13] + R(2) * Fy * d[14];
-  f.hyy = Fx * d[14] + R(3) * Fy * d[15];
-  f.hx = R(2) * Fx * d[2] + Fy * d[3];
-  f.hy = Fx * d[3] + R(2) * Fy * d[4];
-  f.h0x = R(2) * Fx * d[5] + Fy * d[6];
-  f.h0y = Fx * d[6] + R(2) * Fy * d[7];
+  f.b1 = R(1) + n1; f.bS = n0S; f.bD = n0D; f.bX = n0X;
+  f.a = d[1];
+  f.h1 = fma(Fx, d[0].x, Fy * d[0].y);
+  f.hp0 = fma(Fx, d[1].x, Fy * d[1].y);
+  // d[2] = (px^3, py^3), d[3] = (px py^2, px^2 py)
+  const R cx = R(3) * Fx * d[2].x, cy = R(3) * Fy * d[2].y, qx = Fx * d[3].x, qy = Fy * d[3].y;
+  const R xx = cx + qy, yy = cy + qx;
+  f.hS = xx + yy; f.hD = xx - yy;
+  f.hX = R(2) * fma(Fx, d[3].y, Fy * d[3].x);
+  f.nh = pair_of(fma(Fx, nS + nD, Fy * nX), fma(Fy, nS - nD, Fx * nX));
+  f.nh0 = pair_of(fma(Fx, n0S + n0D, Fy * n0X), fma(Fy, n0S - n0D, Fx * n0X));
   return f;
 }
 
@@ -573,8 +590,9 @@ __device__ __forceinline__ ForceSite<R> force_site(const MMacro<R>& M, R Fx, R F
 // Collision of one site and store: class by class, two pairs at a time on (x,
 // y) lanes, then each pair on lanes (population 2 p, its opposite 2 p + 1).
 // The force's source of a population of pair p with sign s = +-1 is
-//   s (F.v (1 - Ae) - Ho) + s F.v g^eq_s - (F.v Ao + He)
-// with Ae, Ao / He, Ho the even / odd parts of dD/dp0 / F.grad_xy D.
+//   s (F.v (1 - Ae) - Ho + F.v g^eq_s) - (F.v Ao + He)
+// with Ae, Ao / He, Ho the even / odd parts of dD/dp0 / F.grad_xy D; B = 1 - Ae
+// and N = -Ho are what force_site prepares.
 // ---------------------------------------------------------------------------
 template <typename R>
 struct MRelax {
@@ -590,28 +608,28 @@ __device__ __forceinline__ void class_relax(const R (&g)[kQm], const EqSite<R>& 
   const MConsts<R>& c = mc<R>();
   const ClassEq<R> k = class_eq<C>(e);
   constexpr int kind = class_kind(C), f = class_fn(C);
-  R eA = R(0), eH = R(0), dA = R(0), dH = R(0), xA = R(0), xH = R(0);
-  V Hc = S2(R(0));
+  R eB = R(0), eH = R(0), dB = R(0), dH = R(0), xB = R(0), xH = R(0);
+  V Nc = S2(R(0));
   if (FORCE) {
-    eA = fma(fs.a5 + fs.a7, c.rr[C], fs.a1);
-    eH = fma(fs.hxx + fs.hyy, c.rr[C], fma(fs.hp0, c.p0[C], fs.h1));
-    if (kind != 1) { dA = (fs.a5 - fs.a7) * c.dd[C]; dH = (fs.hxx - fs.hyy) * c.dd[C]; }
-    if (kind != 0) { xA = fs.a6 * c.pp[C]; xH = fs.hxy * c.pp[C]; }
-    Hc = fma2(pair_of(fs.h0x, fs.h0y), S2(c.p0[C]), pair_of(fs.hx, fs.hy));
+    eB = fma(fs.bS, c.rr[C], fs.b1);
+    eH = fma(fs.hS, c.rr[C], fma(fs.hp0, c.p0[C], fs.h1));
+    if (kind != 1) { dB = fs.bD * c.dd[C]; dH = fs.hD * c.dd[C]; }
+    if (kind != 0) { xB = fs.bX * c.pp[C]; xH = fs.hX * c.pp[C]; }
+    Nc = fma2(fs.nh0, S2(c.p0[C]), fs.nh);
   }
 #pragma unroll
   for (int h = 0; h < (kind == 2 ? 2 : 1); ++h) {
-    V ev, od, wv, Ae = S2(R(0)), He = Ae, Ao = Ae, Ho = Ae, Fv = Ae;
+    V ev, od, wv, B = S2(R(0)), He = B, Ao = B, N = B, Fv = B;
     if (h == 0) couple_eq<C, 0>(k, ev, od);
     else couple_eq<C, 1>(k, ev, od);
     if (kind == 0) {
       wv = mul2(r.gu, c.va[f]);
       if (FORCE) {
         Fv = mul2(r.F, c.va[f]);
-        Ae = fma2(S2(dA), pm<R>(), S2(eA));
+        B = fma2(S2(dB), pm<R>(), S2(eB));
         He = fma2(S2(dH), pm<R>(), S2(eH));
-        Ao = mul2(pair_of(fs.a10, fs.a11), c.pa[f]);
-        Ho = mul2(Hc, c.pa[f]);
+        Ao = mul2(fs.a, c.pa[f]);
+        N = mul2(Nc, c.pa[f]);
       }
     } else {
       // x component of the couple's pairs: function fx, y component: fy
@@ -619,17 +637,16 @@ __device__ __forceinline__ void class_relax(const R (&g)[kQm], const EqSite<R>& 
       wv = fma2(S2(r.gu.x * c.va[fx].x), pm<R>(), S2(r.gu.y * c.va[fy].x));
       if (FORCE) {
         Fv = fma2(S2(r.F.x * c.va[fx].x), pm<R>(), S2(r.F.y * c.va[fy].x));
-        const R a = h ? eA - dA : eA + dA, b = h ? eH - dH : eH + dH;
-        Ae = fma2(S2(xA), pm<R>(), S2(a));
+        const R a = h ? eB - dB : eB + dB, b = h ? eH - dH : eH + dH;
+        B = fma2(S2(xB), pm<R>(), S2(a));
         He = fma2(S2(xH), pm<R>(), S2(b));
-        Ao = fma2(S2(fs.a10 * c.pa[fx].x), pm<R>(), S2(fs.a11 * c.pa[fy].x));
-        Ho = fma2(S2(Hc.x * c.pa[fx].x), pm<R>(), S2(Hc.y * c.pa[fy].x));
+        Ao = fma2(S2(fs.a.x * c.pa[fx].x), pm<R>(), S2(fs.a.y * c.pa[fy].x));
+        N = fma2(S2(Nc.x * c.pa[fx].x), pm<R>(), S2(Nc.y * c.pa[fy].x));
       }
     }
     V al = S2(R(0)), be = al;
     if (FORCE) {
-      // (F.v (1 - Ae) - Ho, F.v Ao + He)
-      al = fma2(Fv, fma2(Ae, S2(R(-1)), S2(R(1))), mul2(Ho, S2(R(-1))));
+      al = fma2(Fv, B, N);
       be = fma2(Fv, Ao, He);
     }
 #pragma unroll
@@ -642,8 +659,7 @@ __device__ __forceinline__ void class_relax(const R (&g)[kQm], const EqSite<R>& 
       V o = fma2(om, fma2(G, S2(R(-1)), geq), G);
       if (FORCE) {
         const R Fp = l ? Fv.y : Fv.x, a = l ? al.y : al.x, b = l ? be.y : be.x;
-        o = fma2(mul2(S2(Fp), pm<R>()), geq, o);
-        o = add2(o, fma2(S2(a), pm<R>(), S2(-b)));
+        o = fma2(fma2(S2(Fp), geq, S2(a)), pm<R>(), add2(o, S2(-b)));
       }
       *at_bytes(out, of.plane[2 * p]) = o.x;
       *at_bytes(out, of.plane[2 * p + 1]) = o.y;
@@ -660,7 +676,7 @@ __device__ __forceinline__ void mcollide_store(const R (&g)[kQm], const MMacro<R
   r.gu = mul2(S2(r.gt), pair_of(M.ux, M.uy));
   r.F = pair_of(Fx, Fy);
   ForceSite<R> fs{};
-  if (FORCE) fs = force_site(M, Fx, Fy);
+  if (FORCE) fs = force_site(e, Fx, Fy);
   if (class_group(NS, 0) == G) class_relax<0, R, FORCE>(g, e, fs, r, out, of);
   if (class_group(NS, 1) == G) class_relax<1, R, FORCE>(g, e, fs, r, out, of);
   if (class_group(NS, 2) == G) class_relax<2, R, FORCE>(g, e, fs, r, out, of);
@@ -681,8 +697,9 @@ __device__ __forceinline__ void mcollide_store(const R (&g)[kQm], const MMacro<R
 // Kernels.  Steps are chained launches (programmatic dependent launch): the
 // next step's blocks are placed early and wait for this one's results before
 // their first access.  FP32 1024 x 512 with a force: 57.6 -> 45.0 us per step
-// (2,328 -> 1,922 instructions per site by the class tables and the prepared
-// offsets; 28 us is the HBM time; 16 warps per SM, issue slots 60 % busy).
+// by the class tables and the prepared offsets, -> 41 us by moments per class
+// and the source's symmetric rows (28 us is the HBM time; 16 warps per SM,
+// instruction issue bounds it).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void chain_release() {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
@@ -738,7 +755,7 @@ k_mstep(const R* __restrict__ src, R* __restrict__ dst, const __grid_constant__ 
 // across row ends), each with the populations of some classes.  A warp
 // instruction of the FP64 pipe takes 66 cycles of its SM sub-partition, so
 // below one warp per sub-partition a step lasts as long as one warp's chain.
-// 97 x 70 sites with a force: 78 -> 39.9 us per step.
+// 97 x 70 sites with a force: 78 -> 38 us per step.
 template <int NS, int G, bool FORCE>
 __device__ __forceinline__ void msplit_group(const double* __restrict__ src, double* __restrict__ dst,
                                              const MGeom& geo, const MOffsets& of, double inv_tau,
@@ -912,16 +929,13 @@ thread_local std::string g_error;
 template <typename R>
 void fill_consts(const Tables& t, MConsts<R>& c) {
   using V = typename V2<R>::T;
-  for (int p = 0; p < kPairs; ++p) {
-    c.mN0[p] = (R)t.mN0[p]; c.mE[p] = (R)t.mE[p];
-    c.mPxx[p] = (R)t.mPxx[p]; c.mPxy[p] = (R)t.mPxy[p]; c.mPyy[p] = (R)t.mPyy[p];
-    c.mNx[p] = (R)t.mNx[p]; c.mNy[p] = (R)t.mNy[p]; c.mMx[p] = (R)t.mMx[p]; c.mMy[p] = (R)t.mMy[p];
-  }
   auto fn = [&](int f, int p) {       // part of pair p's row odd in px
     const double o[7] = {t.LX[p], t.WO[p][0], t.WO[p][2], t.BO[p][0], t.BO[p][2], t.BO[p][4], t.BO[p][6]};
     for (int k = 0; k < 7; ++k) c.O[f][k] = V{(R)o[k], (R)o[k]};
     c.va[f] = V{(R)t.vx[p], (R)t.vx[p]};
     c.pa[f] = V{(R)t.mvO[p][0], (R)t.mvO[p][0]};
+    c.mN[f] = V{(R)t.mNx[p], (R)t.mNx[p]};
+    c.mM[f] = V{(R)t.mMx[p], (R)t.mMx[p]};
   };
   for (int k = 0; k < kClasses - 1; ++k) {
     const int p = class_pair(k);
@@ -932,6 +946,9 @@ void fill_consts(const Tables& t, MConsts<R>& c) {
     c.C1[k][1] = (R)(0.5 * (t.BE[p][2] - t.BE[p][4]));
     c.C1[k][2] = (R)(0.5 * (t.BE[p][5] - t.BE[p][7]));
     c.C2[k][0] = (R)t.WE[p][3]; c.C2[k][1] = (R)t.BE[p][3]; c.C2[k][2] = (R)t.BE[p][6];
+    c.mN0[k] = (R)t.mN0[p]; c.mE[k] = (R)t.mE[p]; c.mPxy[k] = (R)t.mPxy[p];
+    c.mPs[k] = (R)(0.5 * (t.mPxx[p] + t.mPyy[p]));
+    c.mPd[k] = (R)(0.5 * (t.mPxx[p] - t.mPyy[p]));
     c.p0[k] = (R)t.mvE[p][1];
     c.rr[k] = (R)(0.5 * (t.mvE[p][2] + t.mvE[p][4]));
     c.dd[k] = (R)(0.5 * (t.mvE[p][2] - t.mvE[p][4]));
@@ -945,9 +962,25 @@ void fill_consts(const Tables& t, MConsts<R>& c) {
   for (int q = 0; q < 3; ++q) c.C1[kClasses - 1][q] = c.C2[kClasses - 1][q] = R(0);
   c.p0[kClasses - 1] = (R)kM;
   c.rr[kClasses - 1] = c.dd[kClasses - 1] = c.pp[kClasses - 1] = R(0);
-  for (int x = 0; x < 16; ++x)
-    for (int b = 0; b < 16; ++b) c.gi[x][b] = (R)t.gi[x][b];
-  c.restN0 = (R)t.restN0; c.restE = (R)t.restE;
+  c.mN0[kClasses - 1] = (R)t.restN0; c.mE[kClasses - 1] = (R)t.restE;
+  c.mPs[kClasses - 1] = c.mPd[kClasses - 1] = c.mPxy[kClasses - 1] = R(0);
+  const auto& gi = t.gi;
+  const int col[4] = {0, 1, 2, 5};     // monomials 1, p0, px^2, p0 px^2 (py^2: 4, 7)
+  for (int k = 0; k < 4; ++k) {
+    c.n1[k] = (R)-gi[1][col[k]];
+    c.nS[k] = (R)-(gi[2][col[k]] + gi[4][col[k]]);
+    c.n0S[k] = (R)-(gi[5][col[k]] + gi[7][col[k]]);
+  }
+  for (int k = 0; k < 2; ++k) {
+    const int b = k ? 5 : 2, x = k ? 6 : 3;
+    c.nD[k] = (R)-(gi[2][b] - gi[4][b]);
+    c.n0D[k] = (R)-(gi[5][b] - gi[7][b]);
+    c.nX[k] = (R)-gi[3][x];
+    c.n0X[k] = (R)-gi[6][x];
+  }
+  const int odd[4] = {8, 10, 12, 14};  // px, p0 px, px^3, px py^2
+  for (int k = 0; k < 4; ++k)
+    for (int b = 0; b < 4; ++b) c.gO[k][b] = V{(R)gi[odd[k]][odd[b]], (R)gi[odd[k]][odd[b]]};
   for (int i = 0; i < kQm; ++i) {
     c.f0[i] = t.f0[i];
     c.if0[i] = 1.0 / t.f0[i];
