@@ -39,7 +39,7 @@ constexpr int kStepRegs = (65536 / (RLBM_STEP_MIN_BLOCKS * kBX)) > 255
 constexpr int kStepThreads = 64;
 
 // Dynamic shared memory of the direct step kernels: the parking area
-// (park_bytes: 12 x threads x 16 B with FP32 arithmetic, none with FP64).
+// (park_bytes: 12 x threads x 16 B with 16-bit storage, else none).
 template <int FORCE, int RES, int BT>
 __global__ void __maxnreg__(kStepRegs) k_step(const S* __restrict__ fin, S* __restrict__ fout,
                                               const __grid_constant__ DevSample s,
@@ -84,11 +84,11 @@ k_step_staged(S* __restrict__ base, BatchArgs b, const R* __restrict__ ghost, St
 }
 
 // Shared-memory opt-in of the direct batched kernels: the parking area of a
-// 256-thread block (12 x 256 x 16 B = 48 KiB with FP32 arithmetic) plus the
+// 256-thread block (12 x 256 x 16 B = 48 KiB with 16-bit storage) plus the
 // residual reduction's static scratch exceed the default 48 KiB.
 template <int BX>
 cudaError_t allow_park_smem() {
-  const int bytes = (int)park_bytes<R>(BX);
+  const int bytes = (int)park_bytes<S>(BX);
   cudaError_t e = cudaSuccess;
   if (bytes == 0) return e;
   auto set = [&](const void* fn) {
@@ -291,7 +291,7 @@ void launch_single_bt(const S* a, S* b, const DevSample& s, const WarpTiles& wt,
                       const StepOffsets& of, const R* g, int res, const StepAux<R>& aux,
                       cudaStream_t st) {
   const unsigned grid = (wt.count + BT / 32 - 1) / (BT / 32);
-  size_t pk = park_bytes<R>(BT);
+  size_t pk = park_bytes<S>(BT);
   if constexpr (sizeof(S) == 8) {
     // at most two blocks per SM, one warp per FP64 sub-partition: without it
     // the blocks of the next step, placed while this one runs, gather on the
@@ -360,7 +360,7 @@ void launch_batch_f(S* base, const BatchArgs& b, const R* g, int res, int grid, 
     else k_step_staged<F, 2, BX><<<grid, BX, sm, st>>>(base, b, g, aux);
     return;
   }
-  const size_t pk = park_bytes<R>(BX);
+  const size_t pk = park_bytes<S>(BX);
   if (res == 0) launch_chained(k_step_batch<F, 0, BX>, grid, BX, pk, st, base, b, g, aux);
   else if (res == 1) launch_chained(k_step_batch<F, 1, BX>, grid, BX, pk, st, base, b, g, aux);
   else launch_chained(k_step_batch<F, 2, BX>, grid, BX, pk, st, base, b, g, aux);
