@@ -109,6 +109,8 @@ template <typename R> __device__ __forceinline__ const MConsts<R>& mc();
 template <> __device__ __forceinline__ const MConsts<float>& mc<float>() { return c_f; }
 template <> __device__ __forceinline__ const MConsts<double>& mc<double>() { return c_d; }
 
+constexpr int kMThreads = 64;
+
 struct MGeom {
   int nx, ny, ldx;
   int px, py;            // periodic axes
@@ -667,9 +669,48 @@ __device__ __forceinline__ void class_relax(const R (&g)[kQm], const EqSite<R>& 
   }
 }
 
+// Parking of the gathered populations (FP32): between the moments and the
+// relaxation they wait in shared memory, [4 populations][thread], 16 bytes an
+// entry, and come back class by class.  128 -> 80 registers, 16 -> 24 warps per
+// SM: 2048 x 2048 sites with a force 280 -> 262 us per step, 1024 x 512 41.2 ->
+// 40.4 (20 warps 264 and 40.7, 28 warps spill: 292 and 42.8; 200 x 150, less
+// than a wave, 9.1 us both ways).  The accesses are volatile so that the
+// compiler cannot keep the register copies alive instead.
+template <typename R> struct MPark { static constexpr bool kOn = sizeof(R) == 4; };
+constexpr int kParkStride = kMThreads * 16;
+
+__device__ __forceinline__ void park_all(uint32_t a, const float (&g)[kQm]) {
+#pragma unroll
+  for (int v = 0; v < kQm / 4; ++v)
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n"
+                 :: "r"(a + v * kParkStride), "f"(g[4 * v]), "f"(g[4 * v + 1]), "f"(g[4 * v + 2]), "f"(g[4 * v + 3])
+                 : "memory");
+  asm volatile("st.shared.f32 [%0], %1;\n" :: "r"(a + kQm / 4 * kParkStride), "f"(g[kRestPop]) : "memory");
+}
+template <int C>
+__device__ __forceinline__ void unpark(uint32_t a, float (&g)[kQm]) {
+  constexpr int v0 = class_pair(C) / 2, n = class_kind(C) == 2 ? 2 : 1;
+#pragma unroll
+  for (int v = v0; v < v0 + n; ++v)
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=f"(g[4 * v]), "=f"(g[4 * v + 1]), "=f"(g[4 * v + 2]), "=f"(g[4 * v + 3])
+                 : "r"(a + v * kParkStride) : "memory");
+}
+
+template <int C, int NS, int G, typename R, bool FORCE>
+__device__ __forceinline__ void class_step(R (&g)[kQm], const EqSite<R>& e, const ForceSite<R>& fs,
+                                           const MRelax<R>& r, R* __restrict__ out, const MOffsets& of,
+                                           uint32_t park) {
+  if constexpr (class_group(NS, C) == G) {
+    if constexpr (MPark<R>::kOn) unpark<C>(park, g);
+    class_relax<C, R, FORCE>(g, e, fs, r, out, of);
+  }
+}
+
 template <int NS, int G, typename R, bool FORCE>
-__device__ __forceinline__ void mcollide_store(const R (&g)[kQm], const MMacro<R>& M, R inv_tau,
-                                               R Fx, R Fy, R* __restrict__ out, const MOffsets& of) {
+__device__ __forceinline__ void mcollide_store(R (&g)[kQm], const MMacro<R>& M, R inv_tau,
+                                               R Fx, R Fy, R* __restrict__ out, const MOffsets& of,
+                                               uint32_t park) {
   const EqSite<R> e = eq_site(M);
   MRelax<R> r;
   r.gt = M.gamma * inv_tau;
@@ -677,16 +718,18 @@ __device__ __forceinline__ void mcollide_store(const R (&g)[kQm], const MMacro<R
   r.F = pair_of(Fx, Fy);
   ForceSite<R> fs{};
   if (FORCE) fs = force_site(e, Fx, Fy);
-  if (class_group(NS, 0) == G) class_relax<0, R, FORCE>(g, e, fs, r, out, of);
-  if (class_group(NS, 1) == G) class_relax<1, R, FORCE>(g, e, fs, r, out, of);
-  if (class_group(NS, 2) == G) class_relax<2, R, FORCE>(g, e, fs, r, out, of);
-  if (class_group(NS, 3) == G) class_relax<3, R, FORCE>(g, e, fs, r, out, of);
-  if (class_group(NS, 4) == G) class_relax<4, R, FORCE>(g, e, fs, r, out, of);
-  if (class_group(NS, 5) == G) class_relax<5, R, FORCE>(g, e, fs, r, out, of);
-  if (class_group(NS, 6) == G) class_relax<6, R, FORCE>(g, e, fs, r, out, of);
-  if (class_group(NS, 7) == G) class_relax<7, R, FORCE>(g, e, fs, r, out, of);
-  if (class_group(NS, 8) == G) class_relax<8, R, FORCE>(g, e, fs, r, out, of);
+  class_step<0, NS, G, R, FORCE>(g, e, fs, r, out, of, park);
+  class_step<1, NS, G, R, FORCE>(g, e, fs, r, out, of, park);
+  class_step<2, NS, G, R, FORCE>(g, e, fs, r, out, of, park);
+  class_step<3, NS, G, R, FORCE>(g, e, fs, r, out, of, park);
+  class_step<4, NS, G, R, FORCE>(g, e, fs, r, out, of, park);
+  class_step<5, NS, G, R, FORCE>(g, e, fs, r, out, of, park);
+  class_step<6, NS, G, R, FORCE>(g, e, fs, r, out, of, park);
+  class_step<7, NS, G, R, FORCE>(g, e, fs, r, out, of, park);
+  class_step<8, NS, G, R, FORCE>(g, e, fs, r, out, of, park);
   if (class_group(NS, 9) == G) {
+    if constexpr (MPark<R>::kOn)
+      asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(g[kRestPop]) : "r"(park + kQm / 4 * kParkStride) : "memory");
     R orr = fma(r.gt, eq_rest(e) - g[kRestPop], g[kRestPop]);
     if (FORCE) orr -= fma(fs.hp0, R(kM), fs.h1);
     *at_bytes(out, of.plane[kRestPop]) = orr;
@@ -698,8 +741,8 @@ __device__ __forceinline__ void mcollide_store(const R (&g)[kQm], const MMacro<R
 // next step's blocks are placed early and wait for this one's results before
 // their first access.  FP32 1024 x 512 with a force: 57.6 -> 45.0 us per step
 // by the class tables and the prepared offsets, -> 41 us by moments per class
-// and the source's symmetric rows (28 us is the HBM time; 16 warps per SM,
-// instruction issue bounds it).
+// and the source's symmetric rows, -> 40.4 with 24 instead of 16 warps per SM
+// (28 us is the HBM time; instruction issue bounds it).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void chain_release() {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
@@ -718,7 +761,6 @@ struct MLaunch {
   int reverse, evict_first;
 };
 
-constexpr int kMThreads = 64;
 
 // Warps take 32 consecutive sites of a row, two per block.
 template <typename R, bool FORCE>
@@ -737,14 +779,21 @@ __device__ __forceinline__ void mstep_body(const R* __restrict__ src, R* __restr
   R g[kQm];
   mpull<1, 0>(src, geo, of, x, y, site_interior(geo, x0, y) && site_interior(geo, x0 + 31, y), policy, g);
   MMacro<R> M;
-  const unsigned bits = mlandau(mmoments<1, 0>(g), M);
-  mcollide_store<1, 0, R, FORCE>(g, M, inv_tau, Fx, Fy, dst + (long long)y * geo.ldx + x, of);
+  const MMom<R> mom = mmoments<1, 0>(g);
+  uint32_t park = 0;
+  if constexpr (MPark<R>::kOn) {
+    __shared__ __align__(16) unsigned char area[(kQm / 4 + 1) * kParkStride];
+    park = (uint32_t)__cvta_generic_to_shared(area) + threadIdx.x * 16u;
+    park_all(park, g);
+  }
+  const unsigned bits = mlandau(mom, M);
+  mcollide_store<1, 0, R, FORCE>(g, M, inv_tau, Fx, Fy, dst + (long long)y * geo.ldx + x, of, park);
   if (bits) atomicOr(err, bits);
 }
 
-// FP32: at most 128 registers (16 warps per SM).
+// FP32: at most 80 registers (24 warps per SM; MPark).
 template <typename R, bool FORCE>
-__global__ void __launch_bounds__(kMThreads, sizeof(R) == 4 ? 8 : 1)
+__global__ void __launch_bounds__(kMThreads, sizeof(R) == 4 ? 12 : 1)
 k_mstep(const R* __restrict__ src, R* __restrict__ dst, const __grid_constant__ MGeom geo,
         const __grid_constant__ MOffsets of, MLaunch ml, R inv_tau, R Fx, R Fy,
         unsigned* __restrict__ err) {
@@ -780,7 +829,7 @@ __device__ __forceinline__ void msplit_group(const double* __restrict__ src, dou
   }
   MMacro<double> M;
   const unsigned bits = mlandau(m, M);
-  mcollide_store<NS, G, double, FORCE>(g, M, inv_tau, Fx, Fy, dst + (long long)y * geo.ldx + x, of);
+  mcollide_store<NS, G, double, FORCE>(g, M, inv_tau, Fx, Fy, dst + (long long)y * geo.ldx + x, of, 0);
   if (G == 0 && bits) atomicOr(err, bits);
 }
 
