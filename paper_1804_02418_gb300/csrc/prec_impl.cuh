@@ -17,18 +17,19 @@ __constant__ QuadConsts<R> c_qc;
 
 // RLBM_STEP_MIN_BLOCKS: warps per SM sub-partition the register allocation
 // aims for (blocks of 128 threads per SM), measured per storage type in us per
-// step at 600 x 300 / 1024 x 512 / 4096 x 2048.  FP32 storage: 4: 11.3 / 26.6 /
-// 456, 5: 10.7 / 26.8 / 456, 6: 10.9 / 27.6 / 461, 7: 10.6 / 27.4 / 470; 5 is
-// kept.  FP16 storage at the two larger sizes: 6: 25.4 / 287, 7: 24.4 / 273,
-// 8 (spills): 26.4 / 348; 7 is kept.  The FP64 kernels take all the registers
-// they want (the FP64 pipe is busy with 8 warps).
+// step at 600 x 300 / 1024 x 512 / 4096 x 2048.  FP32 storage: 4: 11.0 / 27.5 /
+// 458, 5: 10.5 / 26.5 / 458 (with the values parked in shared memory 5: 10.7 /
+// 26.8 / 456, 6: 10.9 / 27.6 / 461, 7: 10.6 / 27.4 / 470); 5 is kept.  FP16
+// storage at the two larger sizes: 6: 25.4 / 287, 7: 24.4 / 273, 8 (spills):
+// 26.4 / 348; 7 is kept.  The FP64 kernels take all the registers they want
+// (the FP64 pipe is busy with 8 warps).
 #ifndef RLBM_STEP_MIN_BLOCKS
 #define RLBM_STEP_MIN_BLOCKS 4
 #endif
 // Registers per thread of every step kernel of the module: one cap for all
-// block widths (64 / 128 / 256 sites), so that every launch shape compiles the
-// per-site arithmetic alike (the code generator's multiply-add contraction
-// depends on the register budget) and all shapes give bit-identical states.
+// block widths (64 / 128 / 256 sites).  All launch shapes give bit-identical
+// states: the module is compiled without contraction, every fused multiply-add
+// of the per-site arithmetic is written out.
 constexpr int kStepRegs = (65536 / (RLBM_STEP_MIN_BLOCKS * kBX)) > 255
                               ? 255 : ((65536 / (RLBM_STEP_MIN_BLOCKS * kBX)) & ~7);
 
@@ -204,7 +205,6 @@ cudaError_t upload(const double p0[4], const double w[2][4], double scale) {
   for (int j = 0; j < kShells; ++j) {
     h.p0[j] = R(p0[j]);
     for (int k = 0; k < 2; ++k) {
-      h.w[k][j] = R(w[k][j]);
       h.wd[k][j] = w[k][j];
       h.iwd[k][j] = 1.0 / w[k][j];
       h.iwl[k][j] = std::fma(-w[k][j], h.iwd[k][j], 1.0) / w[k][j];

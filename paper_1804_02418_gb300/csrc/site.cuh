@@ -61,7 +61,6 @@ __host__ __device__ constexpr int dir_kind(int d) { return d < 8 ? 0 : 1; }
 template <typename R>
 struct QuadConsts {
   R p0[kShells];            // shell energies p0_j
-  R w[2][kShells];          // weights by direction kind and shell
   R wp0[2][kShells];        // w p0_j / s   (moments of the stored s g; s = 1 above 16 bits)
   R wp0sq[2][kShells];      // w p0_j^2 / s
   R dec_s, enc_s;           // 16-bit storage scale: 1 / s, s (the 16-bit kernels compute on s g)
