@@ -173,7 +173,9 @@ int rlbm_sample_residuals(const rlbm_ctx* ctx, double* out);
  * the number of blocks walking the work list of all samples (one per tile, or
  * 1..16 per SM, persistent) and whether the pulls are staged in shared memory
  * (0 none; 1 bulk asynchronous copies of the 12 shifted row segments of a
- * tile, the next tile in flight while the current one is computed).  With
+ * tile, the next tile in flight while the current one is computed).  A single
+ * sample with FP32 arithmetic and buffers of at most four times the L2 takes
+ * its own kernel without timing.  With
  * rlbm_config.tune_cache the choice is read from / added to that file
  * (a JSON object {"<key>": {"bx": B, "grid": G, "staged": S}, ...}, the key
  * naming the GPU, the precision and the batch's geometry).  Needs an initialised state.  Writes the

@@ -811,10 +811,22 @@ int rlbm_autotune(rlbm_ctx* c, int* bx_out, int* grid_out, int* staged_out) {
     }
   }
   if (!found) {
+    // A single sample with FP32 arithmetic whose buffers are within reach of
+    // the L2 runs its own kernel, untimed: consecutive steps overlap and start
+    // on the lines the last one wrote, which steps repeated from one buffer do
+    // not show.  Us per step, own kernel / best batched shape: FP32 200 x 150
+    // 5.87 / 5.93, 600 x 300 9.8 / 10.5, 1024 x 512 27.4 / 32.3 (the batched
+    // one won the timing here), 1600 x 1000 86.8 / 90.5; FP16 storage 8.1 / 8.3,
+    // 11.9 / 12.6, 24.7 / 26.3, 61 / 68.  FP64 (bound by its pipe) is timed:
+    // 200 x 150 54.0 / 47.4, 1024 x 512 680 / 677.
+    int l2 = 0;
+    cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device);
+    const bool own = c->samples.size() == 1 && c->ops->real_bytes == 4 &&
+                     (size_t)c->samples[0].dev.plane * kQ * c->ops->elem_bytes <= 4 * (size_t)l2;
     struct Cand { int bx, grid, staged; };
     std::vector<Cand> cands;
     if (c->samples.size() == 1) cands.push_back({0, 0, 0});
-    for (int b = 0; b < 3; ++b) {
+    for (int b = 0; b < 3 && !own; ++b) {
       const int bx = kBxChoices[b];
       cands.push_back({bx, 0, 0});                    // one block per tile
       for (int m : {1, 2, 4, 8, 16}) {

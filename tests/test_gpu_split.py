@@ -52,3 +52,16 @@ def test_split_step_equals_one_thread_per_site(rl, name):
             got.append((sv.get_state(), r))
     assert np.array_equal(got[0][0], got[1][0])
     assert abs(got[0][1] - got[1][1]) <= 1e-12 * got[1][1]
+
+
+@pytest.mark.parametrize("prec,own", [("f32", True), ("f16dev", True), ("f64", False)])
+def test_tuning_of_a_single_sample(rl, prec, own):
+    """FP32 arithmetic and buffers within reach of the L2: the sample's own
+    kernel, untimed; FP64 is timed and may take any shape."""
+    s = SAMPLES["electric_force"]()
+    with rl.Solver(s, prec=prec) as sv:
+        sv.init(0)
+        shape = sv.autotune()
+        sv.step(2)
+        sv.check()
+    assert shape == (0, 0, 0) if own else shape[0] in (0, 64, 128, 256)
