@@ -196,10 +196,13 @@ __device__ __forceinline__ void chain() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
-// Read-only load that stays behind chain().
+// Load that stays behind chain(): coherent, because a predecessor may still
+// write the data when this kernel starts (and k_bwd_rows replaces dz in place).
+// Weights and DFT matrices, which no kernel of a pass writes, and what an
+// earlier pass has left are read with __ldg.
 __device__ __forceinline__ uint4 ldg16(const void* p) {
   uint4 v;
-  asm volatile("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];\n"
+  asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];\n"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
   return v;
 }
@@ -357,7 +360,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_fwd_rows(FwdRows p) {
         const uint4* src = reinterpret_cast<const uint4*>(p.in + row0 * p.cin);
         uint4* dst = reinterpret_cast<uint4*>(p.xcopy + row0 * p.cin);
         for (int i = tid; i < nv * p.cin / 8; i += kThreads) {
-          const uint4 v = __ldg(src + i);
+          const uint4 v = ldg16(src + i);      // src may be dst
           dst[i] = v;
           const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -1110,7 +1113,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(BwdRows p) {
         const uint4* src = reinterpret_cast<const uint4*>(p.left + row0 * p.cin);
         for (int i = tid; i < kTileRows * p.cin / 8; i += kThreads) {
           uint4 v = make_uint4(0, 0, 0, 0);
-          if (i < nv * p.cin / 8) v = __ldg(src + i);
+          if (i < nv * p.cin / 8) v = ldg16(src + i);
           const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
           for (int j = 0; j < 8; ++j) {

@@ -400,9 +400,21 @@ __device__ __forceinline__ void relax_shells(const R (&Rm)[4], R omc, const C& q
 // forward or backward difference over 5 sites next to a walled edge, wrapped
 // on periodic axes (Sec. 3, local capacitance approximation; a difference over
 // neighbouring sites would drive density structure finer than a hop).
+// The previous step may still write the plane when this kernel starts:
+// coherent loads behind the wait, as the pulls (Codec::load4).
+__device__ __forceinline__ float ld_plane(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];\n" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double ld_plane(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];\n" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
 template <typename R>
-__device__ __forceinline__ void lca_gradient(const DevSample& s, const R* __restrict__ p, int x,
-                                             int y, R& gx, R& gy) {
+__device__ __forceinline__ void lca_gradient(const DevSample& s, const R* p, int x, int y, R& gx,
+                                             R& gy) {
   constexpr int h = kRadius;
   int xm = x - h, xp = x + h, ym = y - h, yp = y + h;
   R hx = R(0.5), hy = R(0.5);
@@ -413,8 +425,8 @@ __device__ __forceinline__ void lca_gradient(const DevSample& s, const R* __rest
   else if (ym < 0) { ym = y; hy = R(1); }
   else if (yp >= s.ny) { yp = y; hy = R(1); }
   const long long row = (long long)y * s.ldx;
-  gx = (p[row + xp] - p[row + xm]) * hx;
-  gy = (p[(long long)yp * s.ldx + x] - p[(long long)ym * s.ldx + x]) * hy;
+  gx = (ld_plane(p + row + xp) - ld_plane(p + row + xm)) * hx;
+  gy = (ld_plane(p + (long long)yp * s.ldx + x) - ld_plane(p + (long long)ym * s.ldx + x)) * hy;
 }
 
 // Whether the 32 sites of a warp (consecutive x of row y) pull only from

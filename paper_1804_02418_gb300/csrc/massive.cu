@@ -145,16 +145,17 @@ __device__ __forceinline__ S* at_bytes(S* p, long long b) {
   return reinterpret_cast<S*>(reinterpret_cast<char*>(p) + b);
 }
 
-// A read-only load that stays behind the wait for the predecessor's results
-// (an ordinary one may be moved above it).
+// A load that stays behind the wait for the predecessor's results (an ordinary
+// read-only one may be moved above it), coherent because the predecessor may
+// still write the buffer when this kernel starts.
 __device__ __forceinline__ float ld_pull(const float* p, uint64_t policy) {
   float v;
-  asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;\n" : "=f"(v) : "l"(p), "l"(policy) : "memory");
+  asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;\n" : "=f"(v) : "l"(p), "l"(policy) : "memory");
   return v;
 }
 __device__ __forceinline__ double ld_pull(const double* p, uint64_t) {
   double v;
-  asm("ld.global.nc.f64 %0, [%1];\n" : "=d"(v) : "l"(p) : "memory");
+  asm volatile("ld.global.f64 %0, [%1];\n" : "=d"(v) : "l"(p) : "memory");
   return v;
 }
 

@@ -123,14 +123,17 @@ __device__ __forceinline__ double over_weight(double v, int kind, int j, const C
 // side, so one aligned vector access moves them (16 B for FP32, 32 B for FP64,
 // 8 B for 16-bit storage).  The loads are written as assembly with a memory
 // clobber: the compiler may move an ordinary read-only load above the wait
-// for the predecessor's results (chain_wait).
+// for the predecessor's results (chain_wait).  They are coherent loads, not
+// ld.global.nc: a chained step is resident while its predecessor still writes
+// the buffer it will read, and .nc is defined only for memory that nothing
+// writes during the whole kernel.
 // ---------------------------------------------------------------------------
 template <typename S> struct Codec;
 template <> struct Codec<double> {
   using R = double;
   __device__ static void load4(const double* p, uint64_t, double* o) {
-    asm("ld.global.nc.v2.f64 {%0, %1}, [%2];\n" : "=d"(o[0]), "=d"(o[1]) : "l"(p) : "memory");
-    asm("ld.global.nc.v2.f64 {%0, %1}, [%2];\n" : "=d"(o[2]), "=d"(o[3]) : "l"(p + 2) : "memory");
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];\n" : "=d"(o[0]), "=d"(o[1]) : "l"(p) : "memory");
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];\n" : "=d"(o[2]), "=d"(o[3]) : "l"(p + 2) : "memory");
   }
   // from shared memory (32-bit shared-window address)
   __device__ static void load4s(uint32_t a, double* o) {
@@ -154,8 +157,8 @@ template <> struct Codec<float> {
   using R = float;
   // policy: an L2 eviction policy (pull_policy)
   __device__ static void load4(const float* p, uint64_t policy, float* o) {
-    asm("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;\n"
-        : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]) : "l"(p), "l"(policy) : "memory");
+    asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;\n"
+                 : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]) : "l"(p), "l"(policy) : "memory");
   }
   __device__ static void load4s(uint32_t a, float* o) {
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
@@ -181,7 +184,7 @@ template <typename H> struct Codec16 {
   __device__ static uint32_t pack2(float a, float b);
   __device__ static void load4(const H* p, uint64_t, float* o) {
     uint2 u;
-    asm("ld.global.nc.v2.b32 {%0, %1}, [%2];\n" : "=r"(u.x), "=r"(u.y) : "l"(p) : "memory");
+    asm volatile("ld.global.v2.b32 {%0, %1}, [%2];\n" : "=r"(u.x), "=r"(u.y) : "l"(p) : "memory");
     const float2 a = unpack2(u.x), b = unpack2(u.y);   // s g: the kernels work scaled
     o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
   }
