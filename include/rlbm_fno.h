@@ -66,7 +66,8 @@ int rlbm_gemm_f32(int transA, int transB, int M, int N, int K, float alpha,
                   float beta, float* C, long long ldc, long long strideC,
                   const float* bias, float* D, int epilogue, int batch, void* stream);
 
-/* Reads (and clears) the timeout flag of rlbm_gemm_bf16_tc on the current
+/* Reads (and clears) the timeout flag of rlbm_gemm_bf16_tc and of the fused
+ * operator kernels (rlbm_fno_forward, rlbm_fno_backward) on the current
  * device: *flag = 0 if no CTA gave up since the last call.  Synchronous with
  * respect to the device (the read waits for prior work). */
 int rlbm_gemm_tc_error(int* flag);
@@ -119,6 +120,9 @@ int rlbm_fno_adam(float* P, const float* G, float* M, float* V, void* P16, long 
  *   scratch   S1, Wm, dWm, dS1 [batch N][2 m2][C] bf16, dz [rows][C] bf16,
  *             dU as S2[l]
  *   gradients gP .. gbq2 f32, shaped as the weights; added to.
+ * Every wait inside the kernels is bounded (wait_limit): a block whose wait
+ * gives up leaves its remaining outputs unwritten and sets the device flag
+ * that rlbm_gemm_tc_error reports.
  * The backward pass reads dy [rows][cout] f32.  The results are those of the
  * same operator as a sequence of rlbm_gemm_bf16_tc calls: bit for bit, but for
  * the order of the FP32 sums of the weight and bias gradients. */
@@ -137,6 +141,7 @@ typedef struct {
   void *dz, *dWm, *dS1;
   float* dU;
   float *gP, *gW, *gQ1, *gQ2, *gbp, *gb, *gR, *gbq1, *gbq2;
+  long long wait_limit;   /* clock cycles a wait may take before it gives up; 0: about 2 s */
 } rlbm_fno_net;
 
 /* 1 if the fused kernels take this shape, else 0 (host only). */

@@ -122,13 +122,20 @@ __device__ __forceinline__ void tmem_wait() {
   // uses of the loaded registers stay behind the wait
 }
 
-// TMEM columns and mbarriers of a CTA; warp 0 allocates.
+// TMEM columns and mbarriers of a CTA; warp 0 allocates.  Every wait is bounded:
+// a warp whose wait gives up leaves out what depends on it, the CTA stops at its
+// next sync() (at the latest in finish()), raises the error flag, waits
+// (bounded by the default limit) for the MMAs it has committed and frees its
+// TMEM.
 template <int COLS, int BARS>
 struct Cta {
-  uint32_t tmem, bar0, phases;      // bit i of phases: parity of barrier i's next completion
-  bool bad;
+  uint32_t tmem, bar0;
+  uint32_t phases;      // bit i: parity of barrier i's next completion
+  uint32_t open;        // bit i: committed to barrier i and not yet waited for
+  long long limit;      // cycles a wait may take
+  bool bad;             // a wait of this warp gave up
   __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * (uint32_t)i; }
-  __device__ __forceinline__ void start(uint64_t* bars, uint32_t* slot) {
+  __device__ __forceinline__ void start(uint64_t* bars, uint32_t* slot, long long cycles) {
     const int tid = threadIdx.x;
     if (tid < 32) {
       asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
@@ -145,15 +152,29 @@ struct Cta {
     tc_after();
     tmem = *slot;
     bar0 = smem_u32(bars);
-    phases = 0;
+    phases = open = 0;
+    limit = cycles;
     bad = false;
   }
-  // waits for the next completion of barrier i (bounded)
-  __device__ __forceinline__ void wait(int i) {
-    if (!mbar_wait(bar(i), (phases >> i) & 1u)) bad = true;
-    phases ^= 1u << i;
-    tc_after();
+  // all threads, where thread 0 commits the MMAs it has issued to barrier i
+  __device__ __forceinline__ void commit(int i) {
+    if (threadIdx.x == 0) fused::commit(bar(i));
+    open |= 1u << i;
   }
+  // Waits (a warp) for the next completion of barrier i; false if any lane gave
+  // up: the barrier's phase is then still the one to wait for.
+  __device__ __forceinline__ bool wait(int i) {
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(bar(i), (phases >> i) & 1u, limit));
+    tc_after();
+    if (ok) {
+      phases ^= 1u << i;
+      open &= ~(1u << i);
+    } else {
+      bad = true;
+    }
+    return ok;
+  }
+  __device__ __forceinline__ bool waiting(int i) const { return (open >> i) & 1u; }
   // block barrier that makes shared-memory writes visible to the MMAs and
   // orders this thread's TMEM reads before them; true if a wait gave up
   __device__ __forceinline__ bool sync() {
@@ -164,10 +185,12 @@ struct Cta {
     return stop;
   }
   __device__ __forceinline__ void finish(bool stopped) {
-    if (stopped) {
+    if (__syncthreads_or(stopped || bad)) {
       if (threadIdx.x == 0) atomicOr(&g_tc_error, 1u);
-      // MMAs committed but not waited for end (bounded) before the TMEM goes
-      for (int i = 0; i < BARS; ++i) mbar_wait(bar(i), (phases >> i) & 1u);
+      // MMAs committed but not waited for end (bounded) before the TMEM and
+      // the shared memory go
+      for (int i = 0; i < BARS; ++i)
+        if ((open >> i) & 1u) mbar_wait(bar(i), (phases >> i) & 1u);
     }
     tc_before();
     __syncthreads();
@@ -284,6 +307,7 @@ struct FwdRows {
   float* z;
   __nv_bfloat16 *h, *S1, *xcopy;
   int N, items, cin;
+  long long limit;
 };
 
 template <int MODE>
@@ -312,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_fwd_rows(FwdRows p) {
   const Op W{take(4 * kSmallLbo), kSmallLbo, kColSbo};
   const uint32_t stage = take(8 * kStageBytes) + warp * kStageBytes;
   Cta<128, 2> cta;
-  cta.start(bars, &slot);
+  cta.start(bars, &slot, p.limit);
   const uint32_t dG = cta.tmem, dW = cta.tmem + 32, dS = cta.tmem + 64;
   const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
 
@@ -374,16 +398,16 @@ __global__ void __launch_bounds__(kThreads, 3) k_fwd_rows(FwdRows p) {
       if (tid == 0) {
         if (MODE != 0) mma(dG, G, (uint32_t)t * 16 * kRowSbo, Wm, 0, kC, 2, false);
         mma(dW, A, 0, W, 0, kC, MODE != 0 ? 2 : 1, false);
-        commit(cta.bar(0));
       }
+      cta.commit(0);
       if (t + 1 < tiles) prefetch(item, t + 1);
       else prefetch(item + (int)gridDim.x, 0);
-      cta.wait(0);
-      if (MODE != 2 && t > 0) cta.wait(1);      // the transform has read hT
+      bool ok = cta.wait(0);
+      if (MODE != 2 && t > 0) ok = cta.wait(1) && ok;      // the transform has read hT
       const int wv = max(0, min(32, nv - quarter * 32));   // valid rows of this warp
       const bool valid = lane < wv;
       const long long wrow = row0 + quarter * 32;
-      {
+      if (ok) {
         float v[16], g[16];
         tmem_ld16(dW + lanes + half * 16, v);
         if (MODE != 0) tmem_ld16(dG + lanes + half * 16, g);
@@ -424,15 +448,12 @@ __global__ void __launch_bounds__(kThreads, 3) k_fwd_rows(FwdRows p) {
       }
       if (MODE != 2) {
         if ((stop = cta.sync())) break;
-        if (tid == 0) {
-          mma(dS, F1, (uint32_t)t * 16 * kColLbo, hT, 0, kC, 8, t > 0);
-          commit(cta.bar(1));
-        }
+        if (tid == 0) mma(dS, F1, (uint32_t)t * 16 * kColLbo, hT, 0, kC, 8, t > 0);
+        cta.commit(1);
       }
     }
     if (MODE != 2 && !stop) {
-      cta.wait(1);
-      if (quarter == 0) {
+      if (cta.wait(1) && quarter == 0) {
         uint32_t s[8];
         float v[16];
         tmem_ld16(dS + half * 16, v);
@@ -464,6 +485,7 @@ struct Spectral {
   float* S2;
   __nv_bfloat16* out;
   int N;
+  long long limit;
 };
 
 constexpr int kSlabK = 256;                                        // k of one slab
@@ -490,7 +512,7 @@ __global__ void __launch_bounds__(256) k_spectral(Spectral p) {
   float* s2 = reinterpret_cast<float*>(tc_smem + kSlabA + 2 * kTileA + kSlabB);
   float2* rt = reinterpret_cast<float2*>(s2 + kModes * kMixPitch) + warp * 32 * kMixPitch;
   Cta<128, 1> cta;
-  cta.start(bars, &slot);
+  cta.start(bars, &slot, p.limit);
   const __nv_bfloat16* X = p.X + (long long)b * K * (kKy * kC) + ky * kC;
 
   // A2 tiles of round r (rows 256 r .. 256 r + 255), 16-byte pieces along k
@@ -547,10 +569,9 @@ __global__ void __launch_bounds__(256) k_spectral(Spectral p) {
       scatter8(B, (i & 3) * 8, i >> 2, rb[q]);
     }
     if ((stop = cta.sync())) break;
-    if (tid == 0) {
+    if (tid == 0)
       mma(cta.tmem, A1, 0, B, 0, kC, min(kSlabK, ((K - s * kSlabK) + 15) / 16 * 16) / 16, s > 0);
-      commit(cta.bar(0));
-    }
+    cta.commit(0);
     if (s + 1 < slabs) { load_a1(s + 1); load_x(s + 1); }
     else load_a2(0);
   }
@@ -564,9 +585,9 @@ __global__ void __launch_bounds__(256) k_spectral(Spectral p) {
   };
   if (!stop) {
     load_mix(warp);
-    cta.wait(0);
+    const bool ok = cta.wait(0);
     store_a2();
-    if (warp < 2) {
+    if (ok && warp < 2) {
       float* g = p.S2 + ((long long)b * kModes + warp * 32 + lane) * (kKy * kC) + ky * kC;
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
@@ -618,10 +639,10 @@ __global__ void __launch_bounds__(256) k_spectral(Spectral p) {
       if (tid == 0) {
         mma(cta.tmem + 32, A2(0), 0, B, 0, kC, 4, false);
         mma(cta.tmem + 64, A2(1), 0, B, 0, kC, 4, false);
-        commit(cta.bar(0));
       }
+      cta.commit(0);
       if (r + 1 < rounds) load_a2(r + 1);
-      cta.wait(0);
+      if (!cta.wait(0)) continue;          // the next sync stops the CTA
       const int tile = warp >> 2;          // warps 0-3: first tile, 4-7: second
       const int row = r * 256 + tile * 128 + (warp & 3) * 32 + lane;
       uint32_t s[16];
@@ -701,7 +722,7 @@ struct Head {
   const float* dy;                      // backward from here
   __nv_bfloat16* dz;
   float *gQ1, *gb1, *gQ2, *gb2, *gb;    // gradients (accumulated)
-  long long rows;
+  long long rows, limit;
 };
 
 constexpr uint32_t kQ1Lbo = 16 * 144;                    // B: n = 128, k = 32
@@ -726,7 +747,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_head_fwd(Head p) {
   const Op Y{Q1.base + 4 * kQ1Lbo, kY1Lbo, kY1Sbo};
   const Op Q2{Y.base + 16 * kY1Sbo, kQ2Lbo, 144};
   Cta<128, 1> cta;
-  cta.start(bars, &slot);
+  cta.start(bars, &slot, p.limit);
   if (tid < kQ) bq1[tid] = p.bq1[tid];
   load_q1(Q1, p.Q1);
   for (int i = tid; i < 16 * kQ; i += kThreads) {
@@ -755,14 +776,12 @@ __global__ void __launch_bounds__(kThreads, 4) k_head_fwd(Head p) {
       sts16(A.chunk(i >> 2, i & 3), next[q]);
     }
     if ((stop = cta.sync())) break;
-    if (tid == 0) {
-      mma(cta.tmem, A, 0, Q1, 0, kQ, 2, false);
-      commit(cta.bar(0));
-    }
+    if (tid == 0) mma(cta.tmem, A, 0, Q1, 0, kQ, 2, false);
+    cta.commit(0);
     prefetch(t + gridDim.x);
-    cta.wait(0);
+    const int cols = cta.wait(0) ? 64 : 0;
 #pragma unroll 1
-    for (int c0 = half * 64; c0 < half * 64 + 64; c0 += 16) {
+    for (int c0 = half * 64; c0 < half * 64 + cols; c0 += 16) {
       float v[16];
       tmem_ld16(cta.tmem + lanes + c0, v);
       tmem_wait();
@@ -774,12 +793,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_head_fwd(Head p) {
       sts16(Y.chunk(row, c0 / 8 + 1), make_uint4(s[4], s[5], s[6], s[7]));
     }
     if ((stop = cta.sync())) break;
-    if (tid == 0) {
-      mma(cta.tmem, Y, 0, Q2, 0, 16, 8, false);     // z1 is read: its columns are free
-      commit(cta.bar(0));
-    }
-    cta.wait(0);
-    if (half == 0) {
+    if (tid == 0) mma(cta.tmem, Y, 0, Q2, 0, 16, 8, false);     // z1 is read: its columns are free
+    cta.commit(0);
+    if (cta.wait(0) && half == 0) {
       float v[16];
       tmem_ld16(cta.tmem + lanes, v);
       tmem_wait();
@@ -843,7 +859,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_head_bwd(Head p) {
   const Op Bw{take(16 * kBwLbo), kBwLbo, 144};
   const uint32_t stage = DZ.base + warp * kStageBytes;     // free when dh is read
   Cta<256, 1> cta;
-  cta.start(bars, &slot);
+  cta.start(bars, &slot, p.limit);
   const uint32_t dZ = cta.tmem, dY = cta.tmem + 64, dH = cta.tmem + 128, dAcc = cta.tmem + 160;
   const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
   if (tid < kQ) bq1[tid] = p.bq1[tid];
@@ -901,14 +917,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_head_bwd(Head p) {
     if (tid == 0) {
       mma(dZ, A, 0, Q1, 0, 64, 2, false);
       mma(dY, DY, 0, Q2t, 0, 64, 1, false);
-      commit(cta.bar(0));
     }
+    cta.commit(0);
     prefetch(t + gridDim.x);
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
-      cta.wait(0);
+      const int chunks = cta.wait(0) ? 2 : 0;
 #pragma unroll 1
-      for (int c = 2 * part; c < 2 * part + 2; ++c) {
+      for (int c = 2 * part; c < 2 * part + chunks; ++c) {
         float z[16], g[16];
         tmem_ld16(dZ + lanes + c * 16, z);
         tmem_ld16(dY + lanes + c * 16, g);
@@ -944,11 +960,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_head_bwd(Head p) {
           mma(dZ, A, 0, Q1, 8 * 144, 64, 2, false);
           mma(dY, DY, 0, Q2t, 8 * 144, 64, 1, false);
         }
-        commit(cta.bar(0));
       }
+      cta.commit(0);
     }
     if (stop) break;
-    cta.wait(0);
+    if (!cta.wait(0)) continue;            // the next sync stops the CTA
     const int wv = max(0, min(32, nv - quarter * 32));
     {
       float v[16];
@@ -1018,6 +1034,7 @@ struct BwdRows {
   __nv_bfloat16* dWm;
   float *gW, *gb;
   int N, items, cin;
+  long long limit;
 };
 
 constexpr uint32_t kZPitch = 144;          // FP32 row of 32 in shared memory
@@ -1048,7 +1065,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(BwdRows p) {
   const Op dS{MODE != 0 ? take(4 * kSmallLbo) : 0, kSmallLbo, kColSbo};
   const uint32_t zs = MODE == 1 ? take(128 * kZPitch) : 0;
   Cta<128, 2> cta;
-  cta.start(bars, &slot);
+  cta.start(bars, &slot, p.limit);
   const uint32_t tW = cta.tmem, tF = cta.tmem + 32, tM = cta.tmem + 64, tG = cta.tmem + 96;
   const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
   if (MODE != 2) load_modes(GT, p.GT, p.N, tiles * 16);
@@ -1080,7 +1097,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(BwdRows p) {
     if (MODE != 0 && t == 0) nextS = fetch_kn32(p.dS1 + (long long)item * (kM * kC));
   };
   prefetch(blockIdx.x, 0);
-  bool stop = false, first = true, pending = false;
+  bool stop = false, first = true;
   for (int item = blockIdx.x; item < p.items && !stop; item += gridDim.x) {
     if (MODE != 0) store_kn32(dS, nextS);
     for (int t = 0; t < tiles && !stop; ++t) {
@@ -1097,11 +1114,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(BwdRows p) {
         if (tid == 0) {
           mma(tW, A, 0, W, 0, kC, 2, false);
           mma(tF, F1T, (uint32_t)t * 16 * kRowSbo, dS, 0, kC, 2, false);
-          commit(cta.bar(0));
         }
+        cta.commit(0);
       }
       // the previous tile's gradient products have read L and dzT
-      if (pending) { cta.wait(1); pending = false; }
+      if (cta.waiting(1)) cta.wait(1);
       if (MODE != 2) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -1136,8 +1153,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(BwdRows p) {
         }
         __syncwarp();
       }
-      if (MODE != 0) {
-        cta.wait(0);
+      if (MODE != 0 && cta.wait(0)) {
         uint32_t hp[8];
         float v[16], f[16];
         tmem_ld16(tW + lanes + half * 16, v);
@@ -1182,15 +1198,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(BwdRows p) {
       if (tid == 0) {
         if (MODE != 2) mma(tM, GT, (uint32_t)t * 16 * kColLbo, dzT, 0, kC, 8, t > 0);
         mma(tG, L, 0, dzT, 0, kC, 8, !first);
-        commit(cta.bar(1));
       }
-      pending = true;
+      cta.commit(1);
       first = false;
     }
     if (MODE != 2 && !stop) {
-      cta.wait(1);
-      pending = false;
-      if (quarter == 0) {
+      if (cta.wait(1) && quarter == 0) {
         uint32_t s[8];
         float v[16];
         tmem_ld16(tM + half * 16, v);
@@ -1203,7 +1216,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_rows(BwdRows p) {
       }
     }
   }
-  if (pending && !stop) { cta.wait(1); pending = false; }
+  if (cta.waiting(1) && !stop) cta.wait(1);
+  if (!stop) stop = cta.sync();
   if (!first && !stop) {
     if (quarter == 0) {
       const int rows = MODE == 2 ? p.cin : kC;

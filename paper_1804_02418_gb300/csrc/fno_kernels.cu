@@ -280,17 +280,25 @@ __host__ __device__ constexpr uint32_t tc_idesc(int n) {
          ((uint32_t)(TC_M >> 4) << 24);
 }
 
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+// Bounded wait: gives up (false) once more than `limit` clock cycles have
+// passed.  The first probe does not block, so a limit shorter than an MMA's
+// latency gives up at once; later probes may suspend the thread for a while.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
+                                          long long limit = kTcSpinCycles) {
   const long long t0 = clock64();
-  while (true) {
-    uint32_t ok;
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  while (!ok) {
+    if (clock64() - t0 > limit) return false;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
         " selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (ok) return true;
-    if (clock64() - t0 > kTcSpinCycles) return false;
   }
+  return true;
 }
 
 // One operand of the tile: `rows` rows (M or N) of one K slab.
@@ -772,6 +780,7 @@ struct FusedLaunch {
   int sms;
   cudaError_t e;
   bool first;       // the first kernel of a pass starts after everything before it
+  long long limit;  // cycles a wait inside a kernel may take
   // CTAs that fit an SM by shared memory and tensor memory
   int slots(size_t smem, int cols) const {
     const int by_smem = (int)(228 * 1024 / (smem + 2048)), by_tmem = 512 / cols;
@@ -806,13 +815,14 @@ struct FusedLaunch {
 };
 
 int fused_start(const rlbm_fno_net* n, void* stream, FusedLaunch& f) {
-  if (!n || n->batch < 1 || n->batch > 65535 ||
+  if (!n || n->batch < 1 || n->batch > 65535 || n->wait_limit < 0 ||
       !rlbm_fno_fused_supported(n->N, fused::kC, fused::kQ, 16, 16, n->cin, 4, n->layers) ||
       (long long)n->batch * n->N > 0x7fffffffLL)
     return RLBM_EINVAL;
   f.st = static_cast<cudaStream_t>(stream);
   f.e = cudaSuccess;
   f.first = true;
+  f.limit = n->wait_limit > 0 ? n->wait_limit : kTcSpinCycles;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -1013,25 +1023,25 @@ int rlbm_fno_forward(const rlbm_fno_net* n, const void* x, void* stream) {
   fused::FwdRows in{};
   in.in = b16(x); in.F1 = b16(n->F1); in.W = b16(n->P); in.bias = n->bp;
   in.h = b16(n->h[0]); in.S1 = b16(n->S1); in.xcopy = b16(n->x);
-  in.N = n->N; in.items = items; in.cin = n->cin;
+  in.N = n->N; in.items = items; in.cin = n->cin; in.limit = f.limit;
   f.rows(fused::k_fwd_rows<0>, in, items, fused::fwd_smem<0>(T), 128);
   for (int l = 0; l < L; ++l) {
     fused::Spectral s{};
     s.A1 = b16(n->D); s.X = b16(n->S1); s.A2 = b16(n->Dinv);
     s.R = n->R + (long long)l * (fused::kModes / 2) * fused::kKy * C * C * 2;
-    s.S2 = n->S2[l]; s.out = b16(n->Wm); s.N = n->N;
+    s.S2 = n->S2[l]; s.out = b16(n->Wm); s.N = n->N; s.limit = f.limit;
     f.run(fused::k_spectral<false>, s, dim3(fused::kKy, (unsigned)n->batch), 256, fused::kSpectralSmem);
     fused::FwdRows w{};
     w.in = b16(n->h[l]); w.Wm = b16(n->Wm); w.G = b16(n->G); w.F1 = b16(n->F1);
     w.W = b16(n->W) + (long long)l * C * C; w.bias = n->b + (long long)l * C;
     w.z = n->z[l]; w.h = b16(n->h[l + 1]); w.S1 = b16(n->S1);
-    w.N = n->N; w.items = items;
+    w.N = n->N; w.items = items; w.limit = f.limit;
     if (l < L - 1) f.rows(fused::k_fwd_rows<1>, w, items, fused::fwd_smem<1>(T), 128);
     else f.rows(fused::k_fwd_rows<2>, w, items, fused::fwd_smem<2>(T), 128);
   }
   fused::Head h{};
   h.h = b16(n->h[L]); h.Q1 = b16(n->Q1); h.Q2 = b16(n->Q2); h.bq1 = n->bq1; h.bq2 = n->bq2;
-  h.y = n->y; h.rows = (long long)items * n->N;
+  h.y = n->y; h.rows = (long long)items * n->N; h.limit = f.limit;
   const long long tiles = (h.rows + 127) / 128;
   f.rows(fused::k_head_fwd, h, (int)(tiles < 0x7fffffff ? tiles : 0x7fffffff), fused::kHeadFwdSmem, 128);
   return f.e == cudaSuccess ? RLBM_OK : RLBM_ECUDA;
@@ -1048,12 +1058,12 @@ int rlbm_fno_backward(const rlbm_fno_net* n, void* stream) {
   h.dy = n->dy; h.dz = b16(n->dz);
   h.gQ1 = n->gQ1; h.gb1 = n->gbq1; h.gQ2 = n->gQ2; h.gb2 = n->gbq2;
   h.gb = n->gb + (long long)(L - 1) * C;
-  h.rows = (long long)items * n->N;
+  h.rows = (long long)items * n->N; h.limit = f.limit;
   const long long tiles = (h.rows + 127) / 128;
   f.rows(fused::k_head_bwd, h, (int)(tiles < 0x7fffffff ? tiles : 0x7fffffff), fused::kHeadBwdSmem, 256);
   for (int l = L - 1; l >= -1; --l) {
     fused::BwdRows w{};
-    w.dz = b16(n->dz); w.N = n->N; w.items = items; w.cin = n->cin;
+    w.dz = b16(n->dz); w.N = n->N; w.items = items; w.cin = n->cin; w.limit = f.limit;
     w.dWm = b16(n->dWm); w.GT = b16(n->GT); w.F1T = b16(n->F1T); w.dS1 = b16(n->dS1);
     if (l < L - 1) w.W = b16(n->W) + (long long)(l + 1) * C * C;
     if (l >= 0) {
@@ -1065,7 +1075,7 @@ int rlbm_fno_backward(const rlbm_fno_net* n, void* stream) {
       else f.rows(fused::k_bwd_rows<1>, w, items, fused::bwd_smem<1>(T), 128);
       fused::Spectral s{};
       s.A1 = b16(n->DinvT); s.X = b16(n->dWm); s.A2 = b16(n->DT);
-      s.R = n->R + l * nr; s.S2 = n->dU; s.out = b16(n->dS1); s.N = n->N;
+      s.R = n->R + l * nr; s.S2 = n->dU; s.out = b16(n->dS1); s.N = n->N; s.limit = f.limit;
       f.run(fused::k_spectral<true>, s, dim3(fused::kKy, (unsigned)n->batch), 256, fused::kSpectralSmem);
       const fused::MixGrad m{n->S2[l], n->dU, reinterpret_cast<float2*>(n->gR + l * nr), n->batch};
       f.run(fused::k_mix_grad, m, dim3((fused::kModes / 2) * fused::kKy), 256, 0);

@@ -66,7 +66,8 @@ class _Net(ctypes.Structure):
                    ("S2", ctypes.c_void_p * MAX_LAYERS)]
                 + [(k, ctypes.c_void_p) for k in (
                     "y", "dy", "dz", "dWm", "dS1", "dU", "gP", "gW", "gQ1", "gQ2", "gbp", "gb", "gR",
-                    "gbq1", "gbq2")])
+                    "gbq1", "gbq2")]
+                + [("wait_limit", ctypes.c_longlong)])
 
 
 _FNO_EXPORTS["rlbm_fno_fused_supported"] = (ctypes.c_int, [ctypes.c_int] * 8)
@@ -199,6 +200,7 @@ class FNO:
         # the default shape runs in fused kernels, which keep less per site and
         # move it less often; every other shape as a sequence of GEMMs
         self.fused = act == "bf16" and gemm_impl == "tc" and _fused_shape(self.lib, cfg)
+        self.wait_limit = 0     # cycles a wait in a fused kernel may take (0: about 2 s)
         if self.fused:
             self.F1T, self.DT, self.DinvT, self.GT = (
                 a.t().contiguous() for a in (self.F1, self.D, self.Dinv, self.G))
@@ -324,6 +326,7 @@ class FNO:
             n.h[l], n.z[l], n.S2[l] = (self.h16[l].data_ptr(), self.z[l].data_ptr(),
                                        self.S2[l].data_ptr())
         n.h[c.L] = self.h16[c.L].data_ptr()
+        n.wait_limit = self.wait_limit
         return n
 
     # -- forward ------------------------------------------------------------
