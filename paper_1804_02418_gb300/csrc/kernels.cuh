@@ -1029,12 +1029,12 @@ __device__ __forceinline__ void moments_body(const S* __restrict__ fin, const De
   if (dn_out) dn_out[(long long)y * s.ldx + x] = M.dn;
 }
 
-// Macroscopic state of site k of dense FP64 fields (n, u, T).  FP32
-// arithmetic takes n - 1 and T - 1 from the FP64 fields and forms gamma - 1
-// (relative error 2e-7 of a second-order quantity) itself: 8 operations on
-// the FP64 pipe instead of 26, which bounded k_init (FP16 storage
-// 4096 x 2048: 608 -> 159 us,
-// 268 MB in and 805 MB out).
+// Macroscopic state of site k of dense FP64 fields (n, u, T), formed in FP64
+// and rounded once: FP32 would lose 1 - u^2 for |u| near 1 (gamma off by 3 % at
+// 1 - u^2 = 1e-6, infinite at 1e-8).  17 FP64 operations and 6 conversions on
+// the FP64 pipe, which bounds k_init in FP32 arithmetic: FP16 storage
+// 4096 x 2048 361 us (268 MB in and 805 MB out; gamma in FP32 159 us, with
+// IEEE divisions and square root 608 us).
 template <typename R>
 __device__ __forceinline__ Macro<R> field_macro(const double* n, const double* ux,
                                                 const double* uy, const double* T, long long k,
@@ -1046,14 +1046,13 @@ __device__ __forceinline__ Macro<R> field_macro(const double* n, const double* u
   M.dn = R(nk - 1.0);
   M.dT = R(Tk - 1.0);
   M.deps = R(0);
-  const R u2 = fma(M.ux, M.ux, M.uy * M.uy);
-  M.gamma = qrsqrt(R(1) - u2);
-  M.gm1 = u2 * M.gamma * (M.gamma * qrcp(R(1) + M.gamma));
-  M.invT = qrcp(R(1) + M.dT);
-  // |u| < 1 in FP64 where FP32 rounding could decide it
-  const bool slow = sizeof(R) == 8 || !(u2 < R(0.99));
-  ok = (slow ? fma(vx, vx, vy * vy) < 1.0 : true) && positive(nk) && positive(Tk) &&
-       finite_bits(nk) && finite_bits(Tk);
+  const double u2 = fma(vx, vx, vy * vy), w = 1.0 - u2;
+  const double g = qrsqrt(w);
+  M.gamma = R(g);
+  M.gm1 = R(u2 * g * (g * qrcp(1.0 + g)));       // (gamma^2 - 1) / (gamma + 1)
+  if constexpr (sizeof(R) == 8) M.invT = qrcp(R(1) + M.dT);
+  else M.invT = R(1) / (R(1) + M.dT);
+  ok = positive(w) && positive(nk) && positive(Tk) && finite_bits(nk) && finite_bits(Tk);
   return M;
 }
 
