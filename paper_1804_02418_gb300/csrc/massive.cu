@@ -341,9 +341,10 @@ __device__ __forceinline__ bool mlandau_frame(const MMom<float>& m, float& deps,
 }
 __device__ __forceinline__ bool mlandau_frame(const MMom<double>& m, double& deps, double& ux, double& uy) {
   float d32, ux32, uy32;
-  mlandau_d32(trunc_f32(m.dE), trunc_f32(m.Mx), trunc_f32(m.My), trunc_f32(m.dPxx),
-              trunc_f32(m.dPxy), trunc_f32(m.dPyy), d32, ux32, uy32);
-  double d = finite_bits(d32) ? widen_f64(d32) : 0.0;
+  const bool conv32 = mlandau_d32(trunc_f32(m.dE), trunc_f32(m.Mx), trunc_f32(m.My),
+                                  trunc_f32(m.dPxx), trunc_f32(m.dPxy), trunc_f32(m.dPyy), d32,
+                                  ux32, uy32);
+  double d = conv32 ? widen_f64(d32) : 0.0;
   const double a0 = kH0 + m.dPxx + m.dE, c0 = kH0 + m.dPyy + m.dE, p2 = m.dPxy * m.dPxy;
   bool conv = false;
 #pragma unroll 1

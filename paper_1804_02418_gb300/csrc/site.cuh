@@ -495,10 +495,12 @@ __device__ __forceinline__ bool landau_frame(const Moments<float>& m, float& dep
 __device__ __forceinline__ bool landau_frame(const Moments<double>& m, double& deps, double& ux,
                                              double& uy) {
   float d32, ux32, uy32;
-  landau_d32(trunc_f32(m.dE), trunc_f32(m.Mx), trunc_f32(m.My), trunc_f32(m.dPxx),
-             trunc_f32(m.dPxy), trunc_f32(m.dPyy), d32, ux32, uy32);
-  // no use of an FP32 iteration that left the numbers: then from eps = E
-  double d = finite_bits(d32) ? widen_f64(d32) : 0.0;
+  const bool conv32 = landau_d32(trunc_f32(m.dE), trunc_f32(m.Mx), trunc_f32(m.My),
+                                 trunc_f32(m.dPxx), trunc_f32(m.dPxy), trunc_f32(m.dPyy), d32,
+                                 ux32, uy32);
+  // an FP32 iteration that did not converge (|u| near 1) may have left the
+  // root's side: then from eps = E
+  double d = conv32 ? widen_f64(d32) : 0.0;
   const double a0 = 3.0 + m.dPxx + m.dE, c0 = 3.0 + m.dPyy + m.dE, p2 = m.dPxy * m.dPxy;
   bool conv = false;
 #pragma unroll 1
