@@ -354,8 +354,8 @@ __device__ __forceinline__ bool mlandau_frame(const MMom<double>& m, double& dep
     ux = fma(c, m.Mx, -(m.dPxy * m.My)) * inv;
     uy = fma(a, m.My, -(m.dPxy * m.Mx)) * inv;
     const double g = fma(m.Mx, ux, fma(m.My, uy, d));
-    const float w = trunc_f32(fma(-ux, ux, fma(-uy, uy, 1.0)));
-    const double step = g * widen_f64(qrcp(w));
+    const double w = fma(-ux, ux, fma(-uy, uy, 1.0));
+    const double step = g * qrcp(w);
     d -= step;
     if (fabsf(trunc_f32(step)) <= 1e-8f * (float(kE0) + fabsf(trunc_f32(m.dE) + trunc_f32(d)))) {
       const double si = step * inv;
