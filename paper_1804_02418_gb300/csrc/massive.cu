@@ -943,10 +943,9 @@ __global__ void k_mset(R* __restrict__ dst, MGeom geo, const double* __restrict_
     const int i = (int)(t / nsite);
     const long long r = t - i * nsite;
     const int y = (int)(r / geo.nx), x = (int)(r - (long long)y * geo.nx);
-    // delta / f0 with 1 / f0 in two parts, rounded once (2 FP64 operations)
-    const double v = delta[t];
+    // delta / f0 with 1 / f0 in two parts
     dst[(long long)i * geo.plane + (long long)y * geo.ldx + x] =
-        (R)fma(v, mc<R>().if0[i], v * mc<R>().ifl[i]);
+        (R)over(delta[t], mc<R>().if0[i], mc<R>().ifl[i]);
   }
 }
 

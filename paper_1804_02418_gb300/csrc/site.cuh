@@ -110,12 +110,23 @@ constexpr unsigned kErrUnphysical = 2u;
 constexpr unsigned kErrNoConvergence = 4u;
 constexpr unsigned kErrTimeout = 8u;      // a bounded wait inside a kernel gave up
 
-// delta / w for a weight w: the product with 1 / w held as hi + lo, rounded
-// once (error below half an ulp and 2^-50 of one, as the division's, in 2
-// instead of about 10 FP64 operations).
+__device__ __forceinline__ bool finite_bits(float a) {
+  return (__float_as_uint(a) & 0x7f800000u) != 0x7f800000u;
+}
+__device__ __forceinline__ bool finite_bits(double a) {
+  return ((unsigned)__double2hiint(a) & 0x7ff00000u) != 0x7ff00000u;
+}
+
+// v / w for a weight w: the product with 1 / w held as hi + lo, rounded once
+// (error below half an ulp and 2^-50 of one, as the division's, in 2 instead
+// of about 10 FP64 operations).  An infinite v stays what it is: lo may have
+// the other sign or be 0.
+__device__ __forceinline__ double over(double v, double hi, double lo) {
+  return finite_bits(v) ? fma(v, hi, v * lo) : v;
+}
 template <class C>
 __device__ __forceinline__ double over_weight(double v, int kind, int j, const C& c) {
-  return fma(v, c.iwd[kind][j], v * c.iwl[kind][j]);
+  return over(v, c.iwd[kind][j], c.iwl[kind][j]);
 }
 
 // ---------------------------------------------------------------------------
@@ -299,12 +310,6 @@ __device__ __forceinline__ double as_f64(float a) {
   return (e - 0x00800000u) < 0x7f000000u || a == 0.f ? widen_f64(a) : double(a);
 }
 
-__device__ __forceinline__ bool finite_bits(float a) {
-  return (__float_as_uint(a) & 0x7f800000u) != 0x7f800000u;
-}
-__device__ __forceinline__ bool finite_bits(double a) {
-  return ((unsigned)__double2hiint(a) & 0x7ff00000u) != 0x7ff00000u;
-}
 // a > 0 (false for NaN) without a compare on the FP64 pipe; for numbers at
 // least 2^-1022
 __device__ __forceinline__ bool positive(float a) { return a > 0.f; }
