@@ -1053,6 +1053,8 @@ __device__ __forceinline__ Macro<R> field_macro(const double* n, const double* u
   if constexpr (sizeof(R) == 8) M.invT = qrcp(R(1) + M.dT);
   else M.invT = R(1) / (R(1) + M.dT);
   ok = positive(w) && positive(nk) && positive(Tk) && finite_bits(nk) && finite_bits(Tk);
+  // positive() takes no subnormal numbers
+  if (!ok) ok = w > 0.0 && nk > 0.0 && Tk > 0.0 && finite_bits(nk) && finite_bits(Tk);
   return M;
 }
 

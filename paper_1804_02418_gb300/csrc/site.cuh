@@ -310,8 +310,8 @@ __device__ __forceinline__ double as_f64(float a) {
   return (e - 0x00800000u) < 0x7f000000u || a == 0.f ? widen_f64(a) : double(a);
 }
 
-// a > 0 (false for NaN) without a compare on the FP64 pipe; for numbers at
-// least 2^-1022
+// a > 0 (false for NaN) without a compare on the FP64 pipe; for numbers that
+// are no subnormal ones (sums with 1 or 2)
 __device__ __forceinline__ bool positive(float a) { return a > 0.f; }
 __device__ __forceinline__ bool positive(double a) {
   const int hi = __double2hiint(a);

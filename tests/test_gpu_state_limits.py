@@ -32,3 +32,18 @@ def test_infinite_deviations_pass_through(lib, which):
         sv.set_state(d)
         got = sv.get_state()
     assert np.array_equal(got, d, equal_nan=True)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_subnormal_density_is_positive(lib, prec):
+    rlbm, _ = lib
+    n = np.ones((11, 11))
+    n[2, 3], n[4, 4] = 5e-324, 1e-310
+    z = np.zeros((11, 11))
+    with rlbm.Solver(W.Sample(11, 11), prec=prec) as sv:
+        sv.init(0, n, z, z, np.ones((11, 11)))
+        sv.check()
+        n[2, 3] = 0.0
+        sv.init(0, n, z, z, np.ones((11, 11)))
+        with pytest.raises(rlbm.RlbmError):
+            sv.check()
