@@ -713,6 +713,7 @@ struct WarpTiles {
   unsigned per_row, magic, count;   // magic = floor(2^32 / per_row)
   int evict_first;                  // L2 policy of the pulls (pull_policy)
   int reverse;                      // walk the tiles from the last to the first
+  int early;                        // let the next step's blocks be placed while this one runs
   __device__ __forceinline__ void row_of(unsigned t, unsigned& y, unsigned& r) const {
     // the product's high word is the quotient t / per_row or one below it
     y = __umulhi(t, magic);
@@ -723,7 +724,9 @@ struct WarpTiles {
 
 // Chained launches: a step kernel lets its successor start as soon as all of
 // its own blocks run, and waits for its predecessor's results only before
-// its first access to them.
+// its first access to them.  A small FP64 step does not (WarpTiles::early): the
+// next step's blocks would gather on the SMs that it leaves idle, several
+// to an SM, and share the FP64 units there.
 __device__ __forceinline__ void chain_release() {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
@@ -739,7 +742,7 @@ __device__ __forceinline__ void step_body(const S* __restrict__ fin, S* __restri
                                           const typename Codec<S>::R* __restrict__ ghost,
                                           const StepAux<typename Codec<S>::R>& aux, const C& qc,
                                           unsigned char* park) {
-  chain_release();
+  if (wt.early) chain_release();
   double r_du2 = 0.0, r_u2 = 0.0;
   const unsigned block = wt.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
   unsigned y, r;
@@ -764,7 +767,9 @@ __device__ __forceinline__ void step_body(const S* __restrict__ fin, S* __restri
 // sub-partitions (608) is bound by the chain of one warp: about 690 FP64
 // instructions.  Split, a warp runs about 320 (its third of the moments and
 // the relaxation; the Landau solve and the coefficients are repeated).
-// 64 x 64 sites: 22.9 -> 12.1 us per step.
+// 64 x 64 sites: 22.9 -> 12.1 us per step; eight such samples at once, each on
+// its own stream, 58 us per step of all (one thread per site, 1,026
+// operations: 66).
 template <typename S, int FORCE, int RES, int G, class C>
 __device__ __forceinline__ void split_group(const S* __restrict__ fin, const Tile<S>& tl,
                                             const StepOffsets& of, const DevSample& s, int x,
@@ -802,7 +807,6 @@ __device__ __forceinline__ void split_body(const S* __restrict__ fin, S* __restr
                                            const StepOffsets& of, const double* __restrict__ ghost,
                                            const StepAux<double>& aux, const C& qc,
                                            GroupSums<double>* part) {
-  chain_release();
   unsigned y, r;
   wt.row_of(wt.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x, y, r);
   const int x = (int)(r * 32 + threadIdx.x % 32), g = threadIdx.x / 32;

@@ -162,9 +162,7 @@ __device__ __forceinline__ double ld_pull(const double* p, uint64_t) {
 // Which group of an NS-way split holds class c (the rest vector: class 9).
 // The groups hold about the same number of pairs.
 __host__ __device__ constexpr int class_group(int ns, int c) {
-  return ns == 1 ? 0
-       : ns == 2 ? (c <= 3 || c == 9 ? 0 : 1)
-       : (c == 2 || c == 3 ? 0 : c == 6 || c == 0 ? 1 : c == 1 || c == 4 || c == 5 ? 2 : 3);
+  return ns == 1 || c <= 3 || c == 9 ? 0 : 1;
 }
 __host__ __device__ constexpr bool mine(int ns, int g, int p) {
   return class_group(ns, pair_class(p)) == g;
@@ -762,15 +760,15 @@ __device__ __forceinline__ uint64_t mpolicy(bool evict_first) {
 
 struct MLaunch {
   int reverse, evict_first;
+  int early;             // let the next step's blocks be placed while this one runs
 };
-
 
 // Warps take 32 consecutive sites of a row, two per block.
 template <typename R, bool FORCE>
 __device__ __forceinline__ void mstep_body(const R* __restrict__ src, R* __restrict__ dst,
                                            const MGeom& geo, const MOffsets& of, const MLaunch& ml,
                                            R inv_tau, R Fx, R Fy, unsigned* __restrict__ err) {
-  chain_release();
+  if (ml.early) chain_release();
   const unsigned per_row = (unsigned)(geo.nx + 31) / 32;
   const unsigned block = ml.reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
   const unsigned t = block * (kMThreads / 32) + threadIdx.x / 32;
@@ -803,11 +801,15 @@ k_mstep(const R* __restrict__ src, R* __restrict__ dst, const __grid_constant__ 
   mstep_body<R, FORCE>(src, dst, geo, of, ml, inv_tau, Fx, Fy, err);
 }
 
-// FP64, few sites: NS warps share 32 sites (consecutive in row-major order,
+// FP64, few sites: two warps share 32 sites (consecutive in row-major order,
 // across row ends), each with the populations of some classes.  A warp
 // instruction of the FP64 pipe takes 66 cycles of its SM sub-partition, so
 // below one warp per sub-partition a step lasts as long as one warp's chain.
-// 97 x 70 sites with a force: 78 -> 38 us per step.
+// 97 x 70 sites with a force: 78 -> 38 us per step.  Two and not four: four
+// repeat the Landau solve and the coefficients once more each, which pays for
+// one solver alone (64 x 64 28 us, two warps 34) but not where several share
+// the GPU (eight of 64 x 64, each on its own stream, per step of all: four 194
+// us, two 112, one thread per site 136).
 template <int NS, int G, bool FORCE>
 __device__ __forceinline__ void msplit_group(const double* __restrict__ src, double* __restrict__ dst,
                                              const MGeom& geo, const MOffsets& of, double inv_tau,
@@ -842,7 +844,6 @@ k_mstep_split(const double* __restrict__ src, double* __restrict__ dst,
               const __grid_constant__ MGeom geo, const __grid_constant__ MOffsets of,
               double inv_tau, double Fx, double Fy, unsigned* __restrict__ err) {
   __shared__ MMom<double> part[NS * 32];
-  chain_release();
   const long long n = (long long)blockIdx.x * 32 + threadIdx.x % 32;
   const bool in = n < (long long)geo.nx * geo.ny;
   const int y = in ? (int)(n / geo.nx) : 0, x = in ? (int)(n - (long long)y * geo.nx) : 0;
@@ -850,11 +851,7 @@ k_mstep_split(const double* __restrict__ src, double* __restrict__ dst,
   chain_wait();
   const int w = threadIdx.x / 32;
   if (w == 0) msplit_group<NS, 0, FORCE>(src, dst, geo, of, inv_tau, Fx, Fy, err, part, x, y, in, interior);
-  else if (w == 1) msplit_group<NS, 1, FORCE>(src, dst, geo, of, inv_tau, Fx, Fy, err, part, x, y, in, interior);
-  else if constexpr (NS == 4) {
-    if (w == 2) msplit_group<NS, 2, FORCE>(src, dst, geo, of, inv_tau, Fx, Fy, err, part, x, y, in, interior);
-    else msplit_group<NS, 3, FORCE>(src, dst, geo, of, inv_tau, Fx, Fy, err, part, x, y, in, interior);
-  }
+  else msplit_group<NS, 1, FORCE>(src, dst, geo, of, inv_tau, Fx, Fy, err, part, x, y, in, interior);
 }
 
 template <typename R>
@@ -1039,10 +1036,6 @@ void fill_consts(const Tables& t, MConsts<R>& c) {
   }
 }
 
-// Dynamic shared memory that leaves room for one / two blocks per SM: chained
-// launches would otherwise gather the next step's blocks on idle SMs.
-constexpr int kOnePerSm = 120 * 1024, kTwoPerSm = 80 * 1024;
-
 std::mutex g_upload_mu;
 bool g_uploaded[64];
 
@@ -1095,11 +1088,6 @@ int upload_tables(int dev) {
   fill_consts(t, hd);
   cudaError_t e = cudaMemcpyToSymbol(c_f, &hf, sizeof hf);
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_d, &hd, sizeof hd);
-  for (const void* k : {(const void*)k_mstep_split<4, false>, (const void*)k_mstep_split<4, true>})
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePerSm);
-  for (const void* k : {(const void*)k_mstep_split<2, false>, (const void*)k_mstep_split<2, true>,
-                        (const void*)k_mstep<double, false>, (const void*)k_mstep<double, true>})
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTwoPerSm);
   if (e != cudaSuccess) return fail(nullptr, RLBM_ECUDA, "constant upload: %s", cudaGetErrorString(e));
   g_uploaded[dev] = true;
   return RLBM_OK;
@@ -1149,10 +1137,10 @@ int launch_steps(rlbm_massive_ctx* c, int nsteps) {
   const size_t bytes = (size_t)c->geo.plane * kQm * c->elem;
   const long long warps = (long long)((c->geo.nx + 31) / 32) * c->geo.ny;
   const unsigned grid = (unsigned)((warps + kMThreads / 32 - 1) / (kMThreads / 32));
-  // FP64: four warps per 32 sites up to one such tile per SM, two up to two
-  // (one warp per SM sub-partition either way)
+  // FP64: two warps per 32 sites up to two such tiles per SM (one warp per SM
+  // sub-partition)
   const long long tiles = ((long long)c->geo.nx * c->geo.ny + 31) / 32;
-  const int ns = tiles <= c->sms ? 4 : tiles <= 2 * c->sms ? 2 : 1;
+  const bool split = tiles <= 2 * c->sms;
   for (int s = 0; s < nsteps; ++s) {
     const void* src = c->buf[c->cur];
     void* dst = c->buf[c->cur ^ 1];
@@ -1160,20 +1148,20 @@ int launch_steps(rlbm_massive_ctx* c, int nsteps) {
     // (launch_single in prec_impl.cuh)
     MLaunch ml;
     ml.evict_first = bytes <= 2 * c->l2;
+    // as in the massless step, FP64 of up to two blocks per SM keeps the next
+    // step's blocks from gathering on the SMs it leaves idle
+    ml.early = c->elem != 8 || grid > 2u * (unsigned)c->sms;
     ml.reverse = c->cur && bytes <= 4 * c->l2;
     if (c->elem == 8) {
       const double it = 1.0 / c->cfg.tau, fx = c->cfg.Fx, fy = c->cfg.Fy;
       const double* a = (const double*)src;
       double* b = (double*)dst;
-      if (ns == 4)
-        launch_chained(st, force ? k_mstep_split<4, true> : k_mstep_split<4, false>, (unsigned)tiles, 128,
-                       kOnePerSm, a, b, c->geo, c->of, it, fx, fy, c->err);
-      else if (ns == 2)
-        launch_chained(st, force ? k_mstep_split<2, true> : k_mstep_split<2, false>, (unsigned)tiles, 64,
-                       kTwoPerSm, a, b, c->geo, c->of, it, fx, fy, c->err);
+      if (split)
+        launch_chained(st, force ? k_mstep_split<2, true> : k_mstep_split<2, false>, (unsigned)tiles, 64, 0,
+                       a, b, c->geo, c->of, it, fx, fy, c->err);
       else
-        launch_chained(st, force ? k_mstep<double, true> : k_mstep<double, false>, grid, kMThreads,
-                       grid <= 2u * (unsigned)c->sms ? kTwoPerSm : 0, a, b, c->geo, c->of, ml, it, fx, fy, c->err);
+        launch_chained(st, force ? k_mstep<double, true> : k_mstep<double, false>, grid, kMThreads, 0, a, b,
+                       c->geo, c->of, ml, it, fx, fy, c->err);
     } else {
       const float it = (float)(1.0 / c->cfg.tau), fx = (float)c->cfg.Fx, fy = (float)c->cfg.Fy;
       launch_chained(st, force ? k_mstep<float, true> : k_mstep<float, false>, grid, kMThreads, 0,

@@ -51,12 +51,7 @@ __global__ void __maxnreg__(kStepRegs) k_step(const S* __restrict__ fin, S* __re
   step_body<S, FORCE, RES, BT>(fin, fout, s, wt, of, ghost, aux, c_qc, park_smem);
 }
 
-// FP64 samples of few sites (split_body).  The launches ask for more shared
-// memory than two blocks of an SM could have: otherwise the blocks of the next
-// step, placed while this one runs, gather on the SMs that it leaves idle
-// (64 x 64: 44 us per step instead of 12.1).
-constexpr size_t kSplitSmem = 120 * 1024;
-constexpr size_t kSpreadSmem = 80 * 1024;   // two blocks per SM
+// FP64 samples of few sites (split_body).
 template <int FORCE, int RES>
 __global__ void __launch_bounds__(96) k_step_split(const S* __restrict__ fin, S* __restrict__ fout,
                                                    const __grid_constant__ DevSample s,
@@ -104,39 +99,6 @@ cudaError_t allow_park_smem() {
   set((const void*)k_step_batch<2, 0, BX>);
   set((const void*)k_step_batch<2, 1, BX>);
   set((const void*)k_step_batch<2, 2, BX>);
-  return e;
-}
-
-cudaError_t allow_split_smem() {
-  cudaError_t e = cudaSuccess;
-  if constexpr (sizeof(S) == 8) {
-    auto set = [&](const void* fn) {
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSplitSmem);
-    };
-    set((const void*)k_step_split<0, 0>);
-    set((const void*)k_step_split<0, 1>);
-    set((const void*)k_step_split<0, 2>);
-    set((const void*)k_step_split<1, 0>);
-    set((const void*)k_step_split<1, 1>);
-    set((const void*)k_step_split<1, 2>);
-    set((const void*)k_step_split<2, 0>);
-    set((const void*)k_step_split<2, 1>);
-    set((const void*)k_step_split<2, 2>);
-    auto spread = [&](const void* fn) {
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpreadSmem);
-    };
-    spread((const void*)k_step<0, 0, kStepThreads>);
-    spread((const void*)k_step<0, 1, kStepThreads>);
-    spread((const void*)k_step<0, 2, kStepThreads>);
-    spread((const void*)k_step<1, 0, kStepThreads>);
-    spread((const void*)k_step<1, 1, kStepThreads>);
-    spread((const void*)k_step<1, 2, kStepThreads>);
-    spread((const void*)k_step<2, 0, kStepThreads>);
-    spread((const void*)k_step<2, 1, kStepThreads>);
-    spread((const void*)k_step<2, 2, kStepThreads>);
-  }
   return e;
 }
 
@@ -243,7 +205,6 @@ cudaError_t upload(const double p0[4], const double w[2][4], double scale) {
   if (e == cudaSuccess) e = allow_stage_smem<128>();
   if (e == cudaSuccess) e = allow_stage_smem<256>();
   if (e == cudaSuccess) e = allow_park_smem<256>();
-  if (e == cudaSuccess) e = allow_split_smem();
   return e;
 }
 
@@ -291,13 +252,7 @@ void launch_single_bt(const S* a, S* b, const DevSample& s, const WarpTiles& wt,
                       const StepOffsets& of, const R* g, int res, const StepAux<R>& aux,
                       cudaStream_t st) {
   const unsigned grid = (wt.count + BT / 32 - 1) / (BT / 32);
-  size_t pk = park_bytes<S>(BT);
-  if constexpr (sizeof(S) == 8) {
-    // at most two blocks per SM, one warp per FP64 sub-partition: without it
-    // the blocks of the next step, placed while this one runs, gather on the
-    // SMs it leaves idle (150 x 77 sites: 52 us per step instead of 29)
-    if (grid <= 2u * (unsigned)sm_count()) pk = kSpreadSmem;
-  }
+  const size_t pk = park_bytes<S>(BT);
   if (res == 0) launch_chained(k_step<F, 0, BT>, grid, BT, pk, st, a, b, s, wt, of, g, aux);
   else if (res == 1) launch_chained(k_step<F, 1, BT>, grid, BT, pk, st, a, b, s, wt, of, g, aux);
   else launch_chained(k_step<F, 2, BT>, grid, BT, pk, st, a, b, s, wt, of, g, aux);
@@ -319,6 +274,14 @@ void launch_single(const S* a, S* b, const DevSample& s, const R* g, int res, co
   const size_t bytes = (size_t)s.plane * kQ * sizeof(S), l2 = l2_bytes();
   wt.evict_first = bytes <= 2 * l2;
   wt.reverse = s.cur && bytes <= 4 * l2;
+  // FP64, up to two blocks per SM (one warp per FP64 sub-partition): the next
+  // step's blocks, placed while this one runs, would gather on the SMs it
+  // leaves idle.  Us per step, early / not: 64 x 64 44 / 13.4, 150 x 77 52 / 29.
+  // Room for one or two blocks per SM by a request for shared memory gives the
+  // same times, but keeps several small solvers on their own streams apart
+  // (eight of 64 x 64: 83 us per step of all, 58 so).
+  wt.early = sizeof(S) != 8 || (wt.count + kStepThreads / 32 - 1) / (kStepThreads / 32) >
+                                   2u * (unsigned)sm_count();
   StepOffsets of;
   for (int d = 0; d < kDirs; ++d) {
     of.pull_[d] = pull_offset<S>(d, s.plane, s.ldx);
@@ -328,10 +291,9 @@ void launch_single(const S* a, S* b, const DevSample& s, const R* g, int res, co
     // up to one tile per SM: a second one would share sub-partitions, and two
     // split chains take as long as one whole chain
     if (wt.count <= (unsigned)sm_count()) {
-      const size_t sm = kSplitSmem;
-      if (res == 0) launch_chained(k_step_split<F, 0>, wt.count, 96, sm, st, a, b, s, wt, of, g, aux);
-      else if (res == 1) launch_chained(k_step_split<F, 1>, wt.count, 96, sm, st, a, b, s, wt, of, g, aux);
-      else launch_chained(k_step_split<F, 2>, wt.count, 96, sm, st, a, b, s, wt, of, g, aux);
+      if (res == 0) launch_chained(k_step_split<F, 0>, wt.count, 96, 0, st, a, b, s, wt, of, g, aux);
+      else if (res == 1) launch_chained(k_step_split<F, 1>, wt.count, 96, 0, st, a, b, s, wt, of, g, aux);
+      else launch_chained(k_step_split<F, 2>, wt.count, 96, 0, st, a, b, s, wt, of, g, aux);
       return;
     }
   }
