@@ -178,10 +178,12 @@ int rlbm_sample_residuals(const rlbm_ctx* ctx, double* out);
  * its own kernel without timing.  With
  * rlbm_config.tune_cache the choice is read from / added to that file
  * (a JSON object {"<key>": {"bx": B, "grid": G, "staged": S}, ...}, the key
- * naming the GPU, the precision and the batch's geometry).  Needs an initialised state.  Writes the
- * choice to *bx, *grid and *staged (each may be NULL).  The staged kernels
- * bound every wait (about 1 s); a wait that gives up raises the error bit
- * that rlbm_check reports as RLBM_ETIMEOUT. */
+ * naming the GPU, the precision, the batch's geometry and the revision of the
+ * library's kernels: entries of another revision are kept and not used).
+ * Needs an initialised state.  Writes the choice to *bx, *grid and *staged
+ * (each may be NULL).  The staged kernels bound every wait (about 1 s); a wait
+ * that gives up raises the error bit that rlbm_check reports as
+ * RLBM_ETIMEOUT. */
 int rlbm_autotune(rlbm_ctx* ctx, int* bx, int* grid, int* staged);
 
 /* Sets the launch shape directly (same meaning as the rlbm_autotune outputs):

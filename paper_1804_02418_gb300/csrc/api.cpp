@@ -437,6 +437,10 @@ long long launches_per_step(const rlbm_ctx* c) {
   return c->bx == 0 ? (long long)c->samples.size() : 1;
 }
 
+// Revision of the step kernels and of the tuning rules: part of the tune
+// cache's keys, raised when the best shapes may have changed.
+constexpr int kTuneRevision = 2;
+
 std::string tune_key(const rlbm_ctx* c) {
   cudaDeviceProp p;
   cudaGetDeviceProperties(&p, c->device);
@@ -449,8 +453,8 @@ std::string tune_key(const rlbm_ctx* c) {
   char b[512];
   std::string name = p.name;
   for (auto& ch : name) if (ch == ' ') ch = '_';
-  snprintf(b, sizeof b, "%s|%s|n=%zu|sites=%lld|force=%d|h=%016llx", name.c_str(), c->ops->name,
-           c->samples.size(), c->total_sites, (int)c->force_any, h);
+  snprintf(b, sizeof b, "%s|%s|n=%zu|sites=%lld|force=%d|h=%016llx|k=%d", name.c_str(),
+           c->ops->name, c->samples.size(), c->total_sites, (int)c->force_any, h, kTuneRevision);
   return b;
 }
 
@@ -731,7 +735,8 @@ namespace {
 
 // The autotuner's cache file: one JSON object,
 //   {"<key>": {"bx": B, "grid": G, "staged": S}, ...}
-// (keys from tune_key: GPU name, precision, batch and geometry hash).
+// (keys from tune_key: GPU name, precision, batch, geometry hash and kernel
+// revision).
 struct TuneEntry {
   std::string key;
   int bx, grid, staged;
@@ -793,6 +798,59 @@ void write_tune_cache(const std::string& path, const std::vector<TuneEntry>& ent
   std::rename(tmp.c_str(), path.c_str());
 }
 
+// Times a step in every candidate shape (steps repeated from the same input
+// buffer: the state does not advance) and takes the fastest.
+int time_shapes(rlbm_ctx* c) {
+  struct Cand { int bx, grid, staged; };
+  std::vector<Cand> cands;
+  if (c->samples.size() == 1) cands.push_back({0, 0, 0});
+  for (int b = 0; b < 3; ++b) {
+    const int bx = kBxChoices[b];
+    cands.push_back({bx, 0, 0});                    // one block per tile
+    for (int m : {1, 2, 4, 8, 16}) {
+      const long long g = (long long)m * c->sm_count * (256 / bx);
+      if (g < c->ntiles[b]) cands.push_back({bx, (int)g, 0});
+    }
+    // staged pulls pay off when a block walks several tiles (prefetch)
+    for (int m : {1, 2, 4}) {
+      const long long g = (long long)m * c->sm_count * (256 / bx);
+      if (2 * g <= c->ntiles[b]) cands.push_back({bx, (int)g, 1});
+    }
+  }
+  cudaEvent_t e0, e1;
+  cudaEventCreate(&e0);
+  cudaEventCreate(&e1);
+  float best = 1e30f;
+  Cand pick = {c->bx, c->grid, c->staged};
+  const long long launches = c->launches;
+  for (const Cand& k : cands) {
+    cudaError_t e = cudaSuccess;
+    for (int w = 0; w < 2 && e == cudaSuccess; ++w)
+      e = launch_step(c, c->cur, 0, k.bx, k.grid, k.staged);
+    cudaEventRecord(e0, c->stream);
+    const int reps = 5;
+    for (int w = 0; w < reps && e == cudaSuccess; ++w)
+      e = launch_step(c, c->cur, 0, k.bx, k.grid, k.staged);
+    cudaEventRecord(e1, c->stream);
+    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    if (e != cudaSuccess) {
+      cudaEventDestroy(e0);
+      cudaEventDestroy(e1);
+      return cuda_fail(c, e, "autotune launch");
+    }
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    if (ms < best) { best = ms; pick = k; }
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  c->launches = launches;
+  c->bx = pick.bx;
+  c->grid = pick.grid;
+  c->staged = pick.staged;
+  return RLBM_OK;
+}
+
 }  // namespace
 
 int rlbm_autotune(rlbm_ctx* c, int* bx_out, int* grid_out, int* staged_out) {
@@ -823,54 +881,12 @@ int rlbm_autotune(rlbm_ctx* c, int* bx_out, int* grid_out, int* staged_out) {
     cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device);
     const bool own = c->samples.size() == 1 && c->ops->real_bytes == 4 &&
                      (size_t)c->samples[0].dev.plane * kQ * c->ops->elem_bytes <= 4 * (size_t)l2;
-    struct Cand { int bx, grid, staged; };
-    std::vector<Cand> cands;
-    if (c->samples.size() == 1) cands.push_back({0, 0, 0});
-    for (int b = 0; b < 3 && !own; ++b) {
-      const int bx = kBxChoices[b];
-      cands.push_back({bx, 0, 0});                    // one block per tile
-      for (int m : {1, 2, 4, 8, 16}) {
-        const long long g = (long long)m * c->sm_count * (256 / bx);
-        if (g < c->ntiles[b]) cands.push_back({bx, (int)g, 0});
-      }
-      // staged pulls pay off when a block walks several tiles (prefetch)
-      for (int m : {1, 2, 4}) {
-        const long long g = (long long)m * c->sm_count * (256 / bx);
-        if (2 * g <= c->ntiles[b]) cands.push_back({bx, (int)g, 1});
-      }
+    if (own) {
+      c->bx = c->grid = c->staged = 0;
+    } else {
+      const int r = time_shapes(c);
+      if (r) return r;
     }
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    float best = 1e30f;
-    Cand pick = {c->bx, c->grid, c->staged};
-    const long long launches = c->launches;
-    for (const Cand& k : cands) {
-      // repeated steps from the same input buffer: the state does not advance
-      cudaError_t e = cudaSuccess;
-      for (int w = 0; w < 2 && e == cudaSuccess; ++w)
-        e = launch_step(c, c->cur, 0, k.bx, k.grid, k.staged);
-      cudaEventRecord(e0, c->stream);
-      const int reps = 5;
-      for (int w = 0; w < reps && e == cudaSuccess; ++w)
-        e = launch_step(c, c->cur, 0, k.bx, k.grid, k.staged);
-      cudaEventRecord(e1, c->stream);
-      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-      if (e != cudaSuccess) {
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        return cuda_fail(c, e, "autotune launch");
-      }
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      if (ms < best) { best = ms; pick = k; }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    c->launches = launches;
-    c->bx = pick.bx;
-    c->grid = pick.grid;
-    c->staged = pick.staged;
     if (!c->tune_cache.empty()) {
       std::vector<TuneEntry> entries = read_tune_cache(c->tune_cache);
       bool replaced = false;
