@@ -617,7 +617,7 @@ int init_sample(rlbm_ctx* c, int sample, const double* n, const double* ux, cons
                              c->stream)
            : c->ops->init(dst, d, dp[0], dp[1], dp[2], dp[3], err, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "init kernel");
-    c->launches++;
+    c->launches += ce && c->ops->elem_bytes >= sizeof(float) ? 2 : 1;   // init_ce in prec_impl.cuh
   }
   c->sample_ready[sample] = 1;
   c->initialised = std::all_of(c->sample_ready.begin(), c->sample_ready.end(),
