@@ -366,7 +366,7 @@ cudaError_t init(void* fout, const DevSample& s, const double* n, const double* 
 cudaError_t init_ce(void* fout, void* scratch, const DevSample& s, const double* n,
                     const double* ux, const double* uy, const double* T, unsigned* err,
                     cudaStream_t st) {
-  if (sizeof(S) >= sizeof(float)) {
+  if constexpr (sizeof(S) >= sizeof(float)) {
     k_init<<<site_grid(s), kBX, 0, st>>>(static_cast<S*>(scratch), s, n, ux, uy, T, err);
     k_ce_from_eq<<<site_grid(s), kBX, 0, st>>>(static_cast<const S*>(scratch),
                                                static_cast<S*>(fout), s, ux, uy);
