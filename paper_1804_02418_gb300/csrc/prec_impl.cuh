@@ -134,17 +134,21 @@ __global__ void __launch_bounds__(kBX) k_init(S* __restrict__ fout, DevSample s,
   init_body<S>(fout, s, n, ux, uy, T, err, c_qc);
 }
 
-__global__ void __launch_bounds__(kBX) k_init_ce(S* __restrict__ fout, DevSample s,
+// The two forms of the Chapman-Enskog seed: templates, so that a module holds
+// only the one its storage type takes (seed).
+template <typename E>
+__global__ void __launch_bounds__(kBX) k_init_ce(E* __restrict__ fout, DevSample s,
                                                  const double* n, const double* ux,
                                                  const double* uy, const double* T,
                                                  unsigned* err) {
-  init_ce_body<S>(fout, s, n, ux, uy, T, err, c_qc);
+  init_ce_body<E>(fout, s, n, ux, uy, T, err, c_qc);
 }
 
-__global__ void __launch_bounds__(kBX) k_ce_from_eq(const S* __restrict__ eq, S* __restrict__ fout,
+template <typename E>
+__global__ void __launch_bounds__(kBX) k_ce_from_eq(const E* __restrict__ eq, E* __restrict__ fout,
                                                     DevSample s, const double* ux,
                                                     const double* uy) {
-  ce_from_eq_body<S>(eq, fout, s, ux, uy, c_qc);
+  ce_from_eq_body<E>(eq, fout, s, ux, uy, c_qc);
 }
 
 __global__ void __launch_bounds__(kBX) k_get(const S* __restrict__ fin, DevSample s, int d0,
@@ -363,16 +367,21 @@ cudaError_t init(void* fout, const DevSample& s, const double* n, const double* 
   return cudaGetLastError();
 }
 
+template <typename E>
+void seed(E* fout, E* scratch, const DevSample& s, const double* n, const double* ux,
+          const double* uy, const double* T, unsigned* err, cudaStream_t st) {
+  if constexpr (sizeof(E) >= sizeof(float)) {
+    k_init<<<site_grid(s), kBX, 0, st>>>(scratch, s, n, ux, uy, T, err);
+    k_ce_from_eq<E><<<site_grid(s), kBX, 0, st>>>(scratch, fout, s, ux, uy);
+  } else {
+    k_init_ce<E><<<site_grid(s), kBX, 0, st>>>(fout, s, n, ux, uy, T, err);
+  }
+}
+
 cudaError_t init_ce(void* fout, void* scratch, const DevSample& s, const double* n,
                     const double* ux, const double* uy, const double* T, unsigned* err,
                     cudaStream_t st) {
-  if constexpr (sizeof(S) >= sizeof(float)) {
-    k_init<<<site_grid(s), kBX, 0, st>>>(static_cast<S*>(scratch), s, n, ux, uy, T, err);
-    k_ce_from_eq<<<site_grid(s), kBX, 0, st>>>(static_cast<const S*>(scratch),
-                                               static_cast<S*>(fout), s, ux, uy);
-  } else {
-    k_init_ce<<<site_grid(s), kBX, 0, st>>>(static_cast<S*>(fout), s, n, ux, uy, T, err);
-  }
+  seed(static_cast<S*>(fout), static_cast<S*>(scratch), s, n, ux, uy, T, err, st);
   return cudaGetLastError();
 }
 
