@@ -569,9 +569,8 @@ struct EqCoeffs {
 template <typename R>
 __device__ __forceinline__ EqCoeffs<R> eq_coeffs(const Macro<R>& M, R nT, R nmT) {
   EqCoeffs<R> c;
-  const R tg = fma(M.dT, M.gamma, M.gamma);              // T gamma
   const R W = fma(M.dT, M.gamma, M.gm1);                 // T gamma - 1
-  const R X = tg * M.ux, Y = tg * M.uy;
+  const R X = fma(W, M.ux, M.ux), Y = fma(W, M.uy, M.uy);  // T gamma u, rounded once
   const R r2 = fma(X, X, Y * Y), W2 = W * W;
   const R h = fma(R(1.5), r2, R(1));                     // 1 + 3 r^2 / 2
   const R q0 = fma(-W, W2 + h, fma(R(0.5), r2, W2));
@@ -623,7 +622,8 @@ __device__ __forceinline__ ForceCoeffs<R> force_coeffs(const EqCoeffs<R>& c, R F
   return k;
 }
 
-// What a direction's cubic needs beside c: gt = gamma / tau, 1 - gt, gt u and F.
+// What a direction's cubic needs beside c: gt = gamma / tau, gt u and F; FP64
+// also 1 - gt.
 template <typename R>
 struct RelaxSite {
   R gt, omgt, gux, guy, Fx, Fy;

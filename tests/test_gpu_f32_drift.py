@@ -1,0 +1,57 @@
+"""FP32 storage: error of u against FP64 after many steps (GPU).
+
+Smooth fields of amplitude 1e-4 between walls, with a force and with the
+electric force, in FP32 and in FP64 from the same fields.  u gathers the
+roundings of each step's update; where a factor of order 1 (n / T, omega, T
+gamma) is rounded once, a step's relative error of a population's linear part
+is three roundings, at most 3 x 2^-24 = 1.8e-7 and 1e-7 in the mean square of
+independent ones, and the scheme damps them over about one relaxation time.
+Bound: 1.15e-7 without and 1.42e-7 with the electric force (whose gradient adds
+a rounding), between this and the forms with two roundings per factor.
+"""
+import numpy as np
+import pytest
+
+from paper_1804_02418_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rl():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1804_02418_gb300 import build, rlbm
+    build.build()
+    return rlbm
+
+
+def fields(nx, ny, seed):
+    g = np.random.default_rng(seed)
+    y, x = np.arange(ny)[:, None] * (2 * np.pi / ny), np.arange(nx)[None, :] * (2 * np.pi / nx)
+    out = []
+    for f in range(4):
+        a = np.zeros((ny, nx))
+        for _ in range(4):
+            a += g.uniform(-0.5, 0.5) * np.sin(g.integers(0, 4) * x + g.integers(0, 4) * y + g.uniform(0, 6.28))
+        out.append(np.ascontiguousarray(1e-4 * a + (1.0 if f in (0, 3) else 0.0)))
+    return out
+
+
+@pytest.mark.parametrize("inv_cg,force,tau,bound", [(0.0, 1e-6, 1.0, 1.15e-7), (0.1, 0.0, 0.8, 1.42e-7)])
+def test_velocity_error_of_fp32(rl, inv_cg, force, tau, bound):
+    err = []
+    for seed in (1, 2, 3, 4):
+        s = W.Sample(600, 300, tau=tau, Fx=force, inv_cg=inv_cg)
+        f = fields(600, 300, seed)
+        got = {}
+        for prec in ("f64", "f32"):
+            with rl.Solver(s, prec=prec) as sv:
+                sv.init(0, *f)
+                sv.step(50)
+                got[prec] = sv.moments()
+                sv.check()
+        a, b = np.stack(got["f32"][1:3]), np.stack(got["f64"][1:3])
+        err.append(np.linalg.norm(a - b) / np.linalg.norm(b))
+    assert np.mean(err) <= bound, err
