@@ -88,9 +88,10 @@ KERNEL_SOURCES = {
     "f32": ["kernels.cuh", "site.cuh", "prec_impl.cuh", "ops.h", "kernels_f32.cu"],
     "f16dev": ["kernels.cuh", "site.cuh", "prec_impl.cuh", "ops.h", "kernels_f16.cu"],
     "bf16dev": ["kernels.cuh", "site.cuh", "prec_impl.cuh", "ops.h", "kernels_bf16.cu"],
-    "massive_f32": ["massive.cu", "massive_tables.h", "massive_quadrature.cpp", "dd.h"],
-    "massive_f64": ["massive.cu", "massive_tables.h", "massive_quadrature.cpp", "dd.h"],
-    "massive_f32_force0": ["massive.cu", "massive_tables.h", "massive_quadrature.cpp", "dd.h"],
+    "massive_f32": ["massive.cu", "site.cuh", "massive_tables.h", "massive_quadrature.cpp", "dd.h"],
+    "massive_f64": ["massive.cu", "site.cuh", "massive_tables.h", "massive_quadrature.cpp", "dd.h"],
+    "massive_f32_force0": ["massive.cu", "site.cuh", "massive_tables.h", "massive_quadrature.cpp",
+                           "dd.h"],
 }
 
 

@@ -151,7 +151,9 @@ int rlbm_init(rlbm_ctx* ctx, int sample, const double* n, const double* ux,
  * sample.  Its non-equilibrium shear stress is the first-order (Navier-
  * Stokes) stress of the relaxation-time model, eta = (3/4) n T tau.  Same
  * arguments, layout and checks as rlbm_init (NULL fields: the rest state);
- * with the electric force on, the first step's density is n. */
+ * with the electric force on, the first step's density is n.  With FP64 and
+ * FP32 storage the sample's other population buffer, which the next step
+ * overwrites, serves as scratch. */
 int rlbm_init_ce(rlbm_ctx* ctx, int sample, const double* n, const double* ux,
                  const double* uy, const double* T, int device_ptrs);
 

@@ -3,12 +3,17 @@
 // a multiple of 8 from 32 to 512.  Included by fno_kernels.cu, whose tcgen05
 // helpers they use.  Other shapes run the operator as a sequence of GEMMs.
 //
-// What bounds the operator is memory traffic and the FP32 arithmetic of the
-// activations, not its contractions (60 GFLOP per training step at N = 256,
-// batch 8).  As a sequence of GEMMs a training step moved every activation
-// through HBM two to four times (z as FP32 written, read, written; z1 and
-// dz1, 268 MB each, three times) in 105 launches, 3.7 ms.  Here a CTA keeps a
-// canvas row in shared and tensor memory between the contractions:
+// The contractions (60 GFLOP per training step at N = 256, batch 8) do not
+// bound it.  The head kernels are bound by instruction issue (80 and 70 % of the
+// slots: one erff, backward also one expf, for each of 67 M values), the row
+// kernels by the latency of their phases (load, barrier, MMA, wait, epilogue,
+// one after the other; issue 55 and 47 %, shared-memory pipe 41 and 30 %, a
+// quarter to a third of the copy rate), k_spectral by one CTA's chain (issue
+// 19 %, 14 - 17 us whatever the batch).  As a sequence of GEMMs a training step
+// moved every activation through HBM two to four times (z as FP32 written,
+// read, written; z1 and dz1, 268 MB each, three times) in 105 launches, 3.7 ms.
+// Here a CTA keeps a canvas row in shared and tensor memory between the
+// contractions:
 //   k_fwd_rows     z_l = G Wm[b, x] + h W + b, h' = gelu(z_l), S1 = F1 h'
 //                  (the first: h_0 = x P + bp, S1 = F1 h_0)
 //   k_spectral     S2 = D S1[b], per-mode mixing, Wm[b] = Dinv U, one CTA per
@@ -24,8 +29,9 @@
 // then the additions of its epilogues), so outputs agree with it bit for bit;
 // only the order of the FP32 sums of weight and bias gradients differs.
 // Measured, GEMM sequence -> fused: training step 256 x 256, batch 8, 3.84 ->
-// 0.90 ms, 64 x 64, batch 4, 1.70 -> 0.22 ms (105 launches from Python -> 27,
-// the operator's 10 and 14 from one call per direction), inference 256 x 256, batch 1, 0.65 -> 0.105 ms.
+// 0.90 ms, 64 x 64, batch 4, 1.70 -> 0.23 ms (105 launches from Python -> 27,
+// the operator's 10 and 14 from one call per direction), inference 256 x 256,
+// batch 1, 0.65 -> 0.106 ms.
 
 namespace fused {
 
@@ -809,10 +815,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_head_fwd(Head p) {
 // ---------------------------------------------------------------------------
 // Head, backward: 128 sites per tile, the 128 projected channels in two
 // halves.  Per half: z1 = h Q1 + bq1 and dy1 = dy Q2^T (MMA), then per value
-// one erff and one expf for y1 = gelu(z1) and dz1 = dy1 gelu'(z1), which bound
-// the kernel (67 M values at N = 256, batch 8); dz1 and y1 transposed into
-// shared memory give the weight gradients: [dz1; y1]^T [h, dy] in one MMA
-// whose accumulators stay in TMEM for all tiles of the CTA.
+// one erff and one expf for y1 = gelu(z1) and dz1 = dy1 gelu'(z1); dz1 and y1
+// transposed into shared memory give the weight gradients: [dz1; y1]^T [h, dy]
+// in one MMA whose accumulators stay in TMEM for all tiles of the CTA.  Bound by
+// instruction issue (67 M values at N = 256, batch 8, 62 instructions each: 70 %
+// of the slots, 163 us).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kDyLbo = 128, kDySbo = 256;           // A: 128 rows, k = 16
 constexpr uint32_t kQ2tLbo = 16 * 144;                   // B: n = 128, k = 16

@@ -96,10 +96,11 @@ __device__ __forceinline__ T* byte_ptr(T* base, long long bytes) {
   return reinterpret_cast<T*>(reinterpret_cast<B*>(base) + bytes);
 }
 
-// L2 policy of the pulls.  Each stored value is read once per step and its
-// line is next written a step later, so when a buffer is not much larger than
-// the L2 the lines just read should leave first and the ones just written
-// (the next step's input) stay; see launch_single for the rule.
+// L2 policy of the pulls, FP32 storage (the other types' loads take none).
+// Each stored value is read once per step and its line is next written a step
+// later, so when a buffer is not much larger than the L2 the lines just read
+// should leave first and the ones just written (the next step's input) stay;
+// see launch_single for the rule.
 __device__ __forceinline__ uint64_t pull_policy(bool evict_first) {
   uint64_t a, b;
   asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(a));
@@ -718,7 +719,7 @@ __device__ __forceinline__ void site_step(const S* __restrict__ fin, const Tile<
 // Row segments of 32 sites ("warp tiles") of one sample, numbered row by row.
 struct WarpTiles {
   unsigned per_row, magic, count;   // magic = floor(2^32 / per_row)
-  int evict_first;                  // L2 policy of the pulls (pull_policy)
+  int evict_first;                  // L2 policy of the pulls (pull_policy; FP32 storage)
   int reverse;                      // walk the tiles from the last to the first
   int early;                        // let the next step's blocks be placed while this one runs
   __device__ __forceinline__ void row_of(unsigned t, unsigned& y, unsigned& r) const {
@@ -1138,7 +1139,8 @@ __device__ __forceinline__ void init_body(S* __restrict__ fout, const DevSample&
 // f^eq_i(s) where d lies outside (only the bounce-back at s reads it).  The
 // relation is affine with unit weight on f^eq, so it holds for the stored
 // relative deviations as well.  Each thread evaluates the equilibrium at its
-// own site and, for each direction, at the arrival site.
+// own site and, for each direction, at the arrival site.  For 16-bit storage
+// only; FP64 and FP32 take two passes (ce_from_eq_body).
 template <typename S, class C>
 __device__ __forceinline__ void init_ce_body(S* __restrict__ fout, const DevSample& s,
                                              const double* n, const double* ux,
@@ -1192,7 +1194,8 @@ __device__ __forceinline__ void init_ce_body(S* __restrict__ fout, const DevSamp
 // values init_ce_body forms in registers (16-bit storage would round them
 // twice).  init_ce_body evaluates the equilibrium coefficients at 13 sites per
 // site, about 1,300 FP64 operations more than the two passes: FP64 1024 x 512
-// about 1.7 ms -> 0.44 ms (0.28 + 0.16).
+// about 1.7 ms -> 0.44 ms (0.28 + 0.16); FP32 4096 x 2048 0.89 ms, where FP16
+// storage takes 4.6 ms.
 template <typename S, class C>
 __device__ __forceinline__ void ce_from_eq_body(const S* __restrict__ eq, S* __restrict__ fout,
                                                 const DevSample& s, const double* ux,

@@ -1144,7 +1144,7 @@ int launch_steps(rlbm_massive_ctx* c, int nsteps) {
   for (int s = 0; s < nsteps; ++s) {
     const void* src = c->buf[c->cur];
     void* dst = c->buf[c->cur ^ 1];
-    // order and L2 policy of the pulls: the rules of the massless step
+    // order and L2 policy of the pulls (FP32): the rules of the massless step
     // (launch_single in prec_impl.cuh)
     MLaunch ml;
     ml.evict_first = bytes <= 2 * c->l2;

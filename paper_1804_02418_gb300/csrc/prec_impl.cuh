@@ -269,7 +269,8 @@ void launch_single(const S* a, S* b, const DevSample& s, const R* g, int res, co
   wt.per_row = (unsigned)(s.nx + 31) / 32;
   wt.magic = wt.per_row > 1 ? (unsigned)((1ull << 32) / wt.per_row) : 0xffffffffu;
   wt.count = wt.per_row * (unsigned)s.ny;
-  // Both rules were measured on FP32 (us per step, neither / reversed /
+  // Both rules were measured on FP32 storage, the only type whose loads take
+  // the policy (us per step, neither / reversed /
   // reversed and evict-first): buffers of 48 MiB 14.7 / 14.7 / 14.0, 74 MiB
   // 24.6 / 23.2 / 20.9, 96 MiB (1024 x 512) 32.5 / 29.7 / 27.6, 144 MiB 46.6 /
   // 44.3 / 43.3, 192 MiB 60.9 / 58.3 / 57.8, 384 MiB 116.4 / 113.6 / 115.2,

@@ -166,7 +166,7 @@ template <> struct Codec<double> {
 };
 template <> struct Codec<float> {
   using R = float;
-  // policy: an L2 eviction policy (pull_policy)
+  // policy: an L2 eviction policy (pull_policy); the other types' loads take none
   __device__ static void load4(const float* p, uint64_t policy, float* o) {
     asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;\n"
                  : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]) : "l"(p), "l"(policy) : "memory");

@@ -148,7 +148,10 @@ class FNO:
     the FP32 buffers themselves.  Inputs to forward() are of the act type.
     With act = "bf16" and gemm_impl = "tc" the default shape (C 32, Cq 128,
     m1 = m2 = 16, N a multiple of 8 from 32 to 512) runs in the fused kernels
-    of rlbm_fno_forward / rlbm_fno_backward, which give the same results."""
+    of rlbm_fno_forward / rlbm_fno_backward, which give the same results.  They
+    keep what the backward pass reads (x16, h16, z, S2, y) and no other
+    intermediate: z1, y116, U, dy1, dz1, dh, dz, dS2 and their 16-bit forms exist
+    in the GEMM sequence only, where S1 is a list per layer."""
 
     def __init__(self, cfg: FNOConfig, batch: int, seed: int = 0, device="cuda",
                  gemm_impl: str = "tc", act: str = "bf16"):
