@@ -481,9 +481,9 @@ __device__ __forceinline__ void pair_cubics_paired(const int d, const EqCoeffs<f
     if (hx && hy) phi = fma2(S2(s.Fx), vx, mul2(S2(s.Fy), vy));
     else if (hx) phi = mul2(S2(s.Fx), vx);
     else phi = mul2(S2(s.Fy), vy);
-    o = add2(o, phi);
     R[0] = fma2(o, S2(c.e0), fma2(phi, S2(k.a0), S2(k.b0)));
     R[1] = fma2(o, e1, fma2(z, fma2(phi, S2(k.a1), S2(k.b1)), fma2(phi, S2(k.a2), S2(k.b2))));
+    o = add2(o, phi);
     R[2] = fma2(o, e2, mul2(z2, fma2(phi, S2(k.a3), S2(k.b3))));
   } else {
     R[0] = mul2(o, S2(c.e0));
@@ -541,10 +541,10 @@ __device__ __forceinline__ void collide_store_paired(float (&f)[kQ], const Tile<
 
   const float scl = sizeof(S) == 2 ? qc.enc_s : 1.f;
   // n / T = 1 + (n - T) / T: the rounding of 1 / T reaches the small term only.
-  // With o and X, Y each rounded once, the error of u against 64 bits (50 to 100
-  // steps, amplitude 1e-4) is 1.05e-7 at 1024 x 512 and 1.32e-7 with the electric
-  // force at 600 x 300; 1.16e-7 and 1.50e-7 with n / T, omega and T gamma u in
-  // two roundings each, at the same speed.
+  // With o and X, Y each rounded once and the force kept out of o, the error of
+  // u against 64 bits (50 to 100 steps, amplitude 1e-4) is 1.04e-7 at 1024 x 512
+  // and 1.29e-7 with the electric force at 600 x 300; 1.16e-7 and 1.50e-7
+  // otherwise, at the same speed.
   const float iTs = M.invT * scl, dnT = M.dn - M.dT;
   const EqCoeffs<float> c = eq_coeffs(M, fmaf(dnT, iTs, scl), dnT * iTs);
   const float Fx = lca ? fmaf(-s.inv_cg_f, egx, s.Fx_f) : s.Fx_f;

@@ -55,3 +55,21 @@ def test_velocity_error_of_fp32(rl, inv_cg, force, tau, bound):
         a, b = np.stack(got["f32"][1:3]), np.stack(got["f64"][1:3])
         err.append(np.linalg.norm(a - b) / np.linalg.norm(b))
     assert np.mean(err) <= bound, err
+
+
+def test_density_of_a_forced_box(rl):
+    """A closed box driven by a force, 2,000 steps from rest: at rest and in the
+    linear regime the update has to keep a population that is at its equilibrium
+    (omega + (1 - omega) = 1 whatever the force).  The error of n - 1 is then one
+    rounding of the stored deviations, 2^-24 = 6e-8; a factor off by up to 2^-25
+    in one direction adds as much again: bound 8e-8."""
+    s = W.Sample(256, 128, tau=1.5, Fx=2e-6, Fy=-1e-6)
+    got = {}
+    for prec in ("f64", "f32"):
+        with rl.Solver(s, prec=prec) as sv:
+            sv.init(0)
+            sv.step(2000)
+            got[prec] = sv.moments()[0]
+            sv.check()
+    err = np.linalg.norm(got["f32"] - got["f64"]) / np.linalg.norm(got["f64"] - 1.0)
+    assert err <= 8e-8, err
